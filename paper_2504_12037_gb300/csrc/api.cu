@@ -743,6 +743,35 @@ size_t tc_ws_floats(const tnvan_ctx* ctx, int batch) {
   return tot + (size_t)ctx->inst.size() * batch + 16;
 }
 
+// FP32 backward (k_bwd32.cu): its unit-major rows, the batch rounded up to the
+// 32 samples of a tile.
+size_t bwd32_ws_floats(const tnvan_ctx* ctx, int batch, Bwd32Ws* bw) {
+  const size_t ldb = ((size_t)batch + 31) & ~size_t(31);
+  size_t off = 0;
+  for (size_t k = 0; k < ctx->inst.size(); ++k) {
+    const Instance& in = ctx->inst[k];
+    if (bw) bw->off[k] = (long long)off;
+    off += ldb * 2 * (in.W.size() + in.H[0] + in.H[1]);
+  }
+  if (bw) bw->ldb = (long long)ldb;
+  return off;
+}
+
+// Weight blocks of an instance and the slices of the batch the FP32 weight
+// gradients run over: about four CTAs per SM over all instances (the kernel's
+// occupancy, one wave), slices of at least 64 samples.
+int bwd32_blocks(const Instance& in) {
+  int nb = 0;
+  for (int l = 0; l <= in.nh; ++l)
+    nb += ((in.dev.made.layer[l].nout + 63) / 64) * ((in.dev.made.layer[l].nin + 63) / 64);
+  return nb;
+}
+int bwd32_splits(const tnvan_ctx* ctx, int batch) {
+  int blocks = 0;
+  for (const Instance& in : ctx->inst) blocks += bwd32_blocks(in);
+  return std::max(1, std::min({608 / std::max(blocks, 1), (batch + 63) / 64, 256}));
+}
+
 #define TC_SPLITS 16
 
 // Backward of sum_b w_b log q(s_b) on the tensor cores (TF32 or BF16 operands,
@@ -1796,21 +1825,11 @@ static int ensure_grad_ws(tnvan_ctx* ctx, size_t floats) {
   return TNVAN_OK;
 }
 
-// Backward chunking: about two CTAs per SM over all instances.
-static int backward_chunk(const tnvan_ctx* ctx, int batch) {
-  const int n = (int)ctx->inst.size();
-  int per = std::max(1, 304 / std::max(n, 1));
-  int chunk = (batch + per - 1) / per;
-  chunk = ((chunk + 31) / 32) * 32;
-  return std::max(chunk, 32);
-}
-
+// Partial gradient rows of the FP32 backward.
 static size_t grad_ws_floats(const tnvan_ctx* ctx, int batch) {
-  const int chunk = backward_chunk(ctx, batch);
-  const int parts = (batch + chunk - 1) / chunk;
   long long maxp = 0;
   for (const Instance& in : ctx->inst) maxp = std::max(maxp, in.n_params);
-  return (size_t)parts * ctx->inst.size() * (size_t)maxp;
+  return (size_t)bwd32_splits(ctx, batch) * ctx->inst.size() * (size_t)maxp;
 }
 
 int tnvan_reserve(tnvan_ctx* ctx, int max_batch) {
@@ -1827,7 +1846,8 @@ int tnvan_reserve(tnvan_ctx* ctx, int max_batch) {
     rc = ensure_grad_ws(ctx, std::max(grad_ws_floats(ctx, std::max(max_batch, 1)),
                                       (size_t)splits * ctx->inst.size() * (size_t)maxp));
     if (rc) return rc;
-    rc = ensure_ws(ctx, tc_ws_floats(ctx, std::max(max_batch, 1)) * sizeof(float));
+    rc = ensure_ws(ctx, std::max(tc_ws_floats(ctx, std::max(max_batch, 1)),
+                                 bwd32_ws_floats(ctx, std::max(max_batch, 1), nullptr)) * sizeof(float));
     if (rc) return rc;
     int max_edges = 0, ctas = 0;
     for (const Instance& in : ctx->inst) {
@@ -2435,32 +2455,52 @@ int backward_impl(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* 
          "gradient reduce kernel");
     }
   }
-  const int chunk = backward_chunk(ctx, batch);
-  LaunchInfo lb;
-  if ((rc = fill_launch(ctx, betas, batch, chunk, lb))) return rc;
-  if (any_fused) {  // the SIMT backward leaves the fused instances out (no CTAs, not reduced)
-    int acc = 0;
+  if (simt) {
+    LaunchInfo lb;
+    if ((rc = fill_launch(ctx, betas, batch, 32, lb))) return rc;
+    const int splits = bwd32_splits(ctx, batch);
+    int n_run = 0, max_units = 0, max_blocks = 0, max_res = 0;
     for (int k = 0; k < lb.n_inst; ++k) {
+      const Instance& in = ctx->inst[k];
+      if ((fused_bits[k >> 5] >> (k & 31)) & 1u) continue;
+      ++n_run;
+      max_blocks = std::max(max_blocks, bwd32_blocks(in));
+      max_units = std::max(max_units, (int)in.W.size() + in.H[0] + in.H[1]);
+      max_res = std::max(max_res, bwd32_res_floats((int)in.W.size(), in.nh, in.H[0], in.H[1]));
+    }
+    // the networks this backward is sized for (any that fit 880 units of a 32-sample tile)
+    if (max_units > 880) return fail(ctx, TNVAN_E_CUDA, "backward kernel: invalid argument (%d units)", max_units);
+    // weights resident in shared memory, one CTA per SM, where they fit beside
+    // two tiles and every CTA has work for both of its halves
+    const int tiles = (batch + 31) / 32, per = std::max(1, 152 / std::max(n_run, 1));
+    const bool res = bwd32_smem_bytes(max_units, max_res) <= 227 * 1024 && tiles >= 2 * per;
+    int acc = 0;
+    for (int k = 0; k < lb.n_inst; ++k) {  // the fused instances are left out (no CTAs, not reduced)
       lb.tile_begin[k] = acc;
-      if (!((fused_bits[k >> 5] >> (k & 31)) & 1u)) acc += (batch + chunk - 1) / chunk;
+      if (!((fused_bits[k >> 5] >> (k & 31)) & 1u)) acc += res ? per : tiles;
     }
     lb.tile_begin[lb.n_inst] = acc;
     for (int j = 0; j < TNVAN_MAX_INST / 32; ++j) lb.skip[j] = fused_bits[j];
-  }
-  if (simt && (rc = ensure_grad_ws(ctx, grad_ws_floats(ctx, batch)))) return rc;
-  int smem = 0;
-  for (const Instance& in : ctx->inst)
-    smem = std::max(smem, (int)((2 * in.W.size() + 2 * in.H[0] + 2 * in.H[1]) * 33 * sizeof(float)));
-  if (simt) {
+    Bwd32Ws bw;
+    if ((rc = ensure_grad_ws(ctx, grad_ws_floats(ctx, batch)))) return rc;
+    if ((rc = ensure_ws(ctx, bwd32_ws_floats(ctx, batch, &bw) * sizeof(float)))) return rc;
+    bw.base = static_cast<float*>(ctx->d_ws);
     {
       PROF("backward", s);
-      CK(launch_backward(ctx->d_inst, lb, smem, precision, d_spins, d_logZR, d_logq, ctx->d_stats,
-                         ctx->d_grad_packed, (int)max_elems, s),
+      CK(launch_bwd32_delta(ctx->d_inst, lb, bw, res, bwd32_smem_bytes(max_units, res ? max_res : 0), d_spins, d_logZR,
+                            d_logq, ctx->d_stats, s),
          "backward kernel");
     }
     {
+      PROF("backward_wgrad", s);
+      CK(launch_bwd32_wgrad(ctx->d_inst, lb, bw, max_blocks, splits, ctx->d_grad_packed, max_elems, s),
+         "weight gradient kernel");
+    }
+    LaunchInfo lr = lb;
+    for (int k = 0; k <= lr.n_inst; ++k) lr.tile_begin[k] = k * splits;
+    {
       PROF("grad_reduce", s);
-      CK(launch_grad_reduce(ctx->d_inst, lb, ctx->d_grad_packed, (int)max_elems, d_grad_params, s, adam),
+      CK(launch_grad_reduce(ctx->d_inst, lr, ctx->d_grad_packed, (int)max_elems, d_grad_params, s, adam),
          "gradient reduce kernel");
     }
   }

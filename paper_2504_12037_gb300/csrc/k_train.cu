@@ -1,5 +1,5 @@
-// Reduction to F_q / log Z_IS (Eq. 9), REINFORCE backward of the network
-// (Eq. 10) and the Adam update (Algorithm 1 step (d)).
+// Reduction to F_q / log Z_IS (Eq. 9), the gradient's reduction over partial
+// rows and the Adam update (Algorithm 1 step (d)).
 #include <math.h>
 
 #include "common.cuh"
@@ -407,208 +407,6 @@ __global__ void merge_stats_kernel(const LaunchInfo li, int n_parts, const doubl
 cudaError_t launch_merge_stats(const LaunchInfo& li, int n_parts, const double* parts, double* stats,
                                cudaStream_t s) {
   merge_stats_kernel<<<(li.n_inst + 127) / 128, 128, 0, s>>>(li, n_parts, parts, stats);
-  return cudaGetLastError();
-}
-
-// ---------------------------------------------------------------------------
-// K2 + K3: teacher-forced forward and hand-written backward of
-//   sum_b w_b log q(s_b),   w_b = -(l_b - mean l) / (beta B)       (Eq. 10)
-// for a chunk of samples per CTA, 32 samples at a time (FP32 SIMT).
-//   d log q / d x_i = s_i sigmoid(-s_i x_i)
-// Shared memory, layout [unit][TP] with TP = 33:
-//   S [D], A1 [H1], A2 [H2], X/dX [D], dA2 [H2], dA1 [H1].
-// Weight-gradient partial sums of the chunk are accumulated in this CTA's
-// slice of `partials` (packed, degree-sorted layout, n_params floats).
-// ---------------------------------------------------------------------------
-#define BW_TS 32
-#define BW_TP 33
-
-// G[M][N] (+)= sum_t A[m][t] Bm[n][t];  gb[M] (+)= sum_t A[m][t].
-__device__ void outer_acc(float* __restrict__ G, float* __restrict__ gb, const float* A,
-                          const float* Bm, int M, int N, int TS, bool first, int tid, int nth) {
-  const int mb = (M + 3) >> 2, nb = (N + 3) >> 2;
-  for (int blk = tid; blk < mb * nb; blk += nth) {
-    const int i0 = (blk / nb) << 2, j0 = (blk % nb) << 2;
-    float acc[4][4];
-#pragma unroll
-    for (int r = 0; r < 4; ++r)
-#pragma unroll
-      for (int c = 0; c < 4; ++c) acc[r][c] = 0.f;
-    for (int t = 0; t < TS; ++t) {
-      float a[4], bb[4];
-#pragma unroll
-      for (int r = 0; r < 4; ++r) a[r] = (i0 + r < M) ? A[(i0 + r) * BW_TP + t] : 0.f;
-#pragma unroll
-      for (int c = 0; c < 4; ++c) bb[c] = (j0 + c < N) ? Bm[(j0 + c) * BW_TP + t] : 0.f;
-#pragma unroll
-      for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) acc[r][c] = fmaf(a[r], bb[c], acc[r][c]);
-    }
-#pragma unroll
-    for (int r = 0; r < 4; ++r)
-#pragma unroll
-      for (int c = 0; c < 4; ++c)
-        if (i0 + r < M && j0 + c < N) {
-          float* g = G + (long long)(i0 + r) * N + j0 + c;
-          *g = first ? acc[r][c] : *g + acc[r][c];
-        }
-  }
-  for (int m = tid; m < M; m += nth) {
-    float s = 0.f;
-    for (int t = 0; t < TS; ++t) s += A[m * BW_TP + t];
-    gb[m] = first ? s : gb[m] + s;
-  }
-}
-
-__device__ __forceinline__ float dot_row(const float* __restrict__ w, const float* col, int n) {
-  float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-  int j = 0;
-  for (; j + 4 <= n; j += 4) {
-    a0 = fmaf(__ldg(w + j), col[j * BW_TP], a0);
-    a1 = fmaf(__ldg(w + j + 1), col[(j + 1) * BW_TP], a1);
-    a2 = fmaf(__ldg(w + j + 2), col[(j + 2) * BW_TP], a2);
-    a3 = fmaf(__ldg(w + j + 3), col[(j + 3) * BW_TP], a3);
-  }
-  for (; j < n; ++j) a0 = fmaf(__ldg(w + j), col[j * BW_TP], a0);
-  return (a0 + a1) + (a2 + a3);
-}
-
-// sum_{i = i0}^{n-1} col[i] * w[i * stride]
-__device__ __forceinline__ float dot_strided(const float* __restrict__ w, long long stride,
-                                             const float* col, int i0, int n) {
-  float a0 = 0.f, a1 = 0.f;
-  int i = i0;
-  for (; i + 2 <= n; i += 2) {
-    a0 = fmaf(__ldg(w + i * stride), col[i * BW_TP], a0);
-    a1 = fmaf(__ldg(w + (i + 1) * stride), col[(i + 1) * BW_TP], a1);
-  }
-  if (i < n) a0 = fmaf(__ldg(w + i * stride), col[i * BW_TP], a0);
-  return a0 + a1;
-}
-
-__global__ void __launch_bounds__(256) backward_kernel(const InstDev* __restrict__ inst,
-                                                       const LaunchInfo li,
-                                                       const int8_t* __restrict__ spins,
-                                                       const double* __restrict__ logZR,
-                                                       const float* __restrict__ logq,
-                                                       const double* __restrict__ stats,
-                                                       float* __restrict__ partials,
-                                                       long long part_stride) {
-  extern __shared__ float sm[];
-  const int k = find_inst(li, blockIdx.x);
-  const InstDev& I = inst[k];
-  const MadeDev& md = I.made;
-  const int D = md.D, nh = md.nh, H1 = md.H1, H2 = md.H2, Hl = md.Hl;
-  const int tid = threadIdx.x, nth = blockDim.x;
-  const int t = tid & 31, q = tid >> 5, nq = nth >> 5;
-  const int chunk = li.tile;
-  const int c_idx = blockIdx.x - li.tile_begin[k];
-  const int b_lo = c_idx * chunk, b_hi = min(li.batch, b_lo + chunk);
-  float* S = sm;
-  float* A1 = S + D * BW_TP;
-  float* A2 = A1 + H1 * BW_TP;
-  float* X = A2 + H2 * BW_TP;
-  float* dA2 = X + D * BW_TP;
-  float* dA1 = dA2 + H2 * BW_TP;
-  const float* W1 = md.packed + md.layer[0].dst_off;
-  const float* b1 = W1 + (long long)H1 * D;
-  const float* W2 = nh >= 2 ? md.packed + md.layer[1].dst_off : nullptr;
-  const float* b2 = nh >= 2 ? W2 + (long long)H2 * H1 : nullptr;
-  const float* Wo = md.packed + md.layer[nh].dst_off;
-  const float* bo = Wo + (long long)D * Hl;
-  const float* src = nh == 0 ? S : (nh == 1 ? A1 : A2);
-  const int* deg1 = nh >= 1 ? md.layer[0].deg_out : nullptr;
-  const int* deg2 = nh >= 2 ? md.layer[1].deg_out : nullptr;
-  const int* cL = nh == 1 ? md.c1 : md.c2;
-  const double mean = stats[8 * k + 4];
-  const double beta = li.beta[k];
-  const double wscale = -1.0 / (beta * stats_batch(stats + 8 * k));
-  float* Gk = partials + (long long)blockIdx.x * part_stride;
-  const int8_t* sp = spins + I.spin_units * li.batch;
-  bool first = true;
-  for (int b0 = b_lo; b0 < b_hi; b0 += BW_TS) {
-    const int nv = min(BW_TS, b_hi - b0);
-    __syncthreads();
-    for (int e = tid; e < BW_TS * D; e += nth) {
-      const int tt = e / D, i = e % D;
-      S[i * BW_TP + tt] = tt < nv ? (float)sp[(long long)(b0 + tt) * D + i] : 0.f;
-    }
-    __syncthreads();
-    if (nh >= 1) {
-      for (int o = q; o < H1; o += nq)
-        A1[o * BW_TP + t] = fmaxf(__ldg(b1 + o) + dot_row(W1 + (long long)o * D, S + t, deg1[o]), 0.f);
-      __syncthreads();
-    }
-    if (nh >= 2) {
-      for (int o = q; o < H2; o += nq)
-        A2[o * BW_TP + t] =
-            fmaxf(__ldg(b2 + o) + dot_row(W2 + (long long)o * H1, A1 + t, md.c1[deg2[o]]), 0.f);
-      __syncthreads();
-    }
-    // output logits -> dX = w_b s_i sigmoid(-s_i x_i)
-    const bool valid = t < nv;
-    const float wb =
-        valid ? (float)(wscale * (logZR[(long long)k * li.batch + b0 + t] -
-                                  (double)logq[(long long)k * li.batch + b0 + t] - mean))
-              : 0.f;
-    for (int i = q; i < D; i += nq) {
-      const int nin = nh == 0 ? i : cL[i];
-      const float x = __ldg(bo + i) + dot_row(Wo + (long long)i * Hl, src + t, nin);
-      const float s = S[i * BW_TP + t];
-      X[i * BW_TP + t] = wb * s / (1.f + expf(s * x));
-    }
-    __syncthreads();
-    if (nh == 2) {
-      // dA2[o] = 1[h2 > 0] sum_{i >= deg2(o)} dX[i] Wo[i][o]
-      for (int o = q; o < H2; o += nq) {
-        const float h = A2[o * BW_TP + t];
-        dA2[o * BW_TP + t] = h > 0.f ? dot_strided(Wo + o, Hl, X + t, deg2[o], D) : 0.f;
-      }
-      __syncthreads();
-      // dA1[j] = 1[h1 > 0] sum_{o: deg2(o) >= deg1(j)} dA2[o] W2[o][j]
-      for (int j = q; j < H1; j += nq) {
-        const float h = A1[j * BW_TP + t];
-        const int o0 = md.c2[deg1[j] - 1];
-        dA1[j * BW_TP + t] = h > 0.f ? dot_strided(W2 + j, H1, dA2 + t, o0, H2) : 0.f;
-      }
-      __syncthreads();
-    } else if (nh == 1) {
-      for (int j = q; j < H1; j += nq) {
-        const float h = A1[j * BW_TP + t];
-        dA1[j * BW_TP + t] = h > 0.f ? dot_strided(Wo + j, Hl, X + t, deg1[j], D) : 0.f;
-      }
-      __syncthreads();
-    }
-    // weight gradients of this sub-tile
-    float* Go = Gk + md.layer[nh].dst_off;
-    outer_acc(Go, Go + (long long)D * Hl, X, src, D, Hl, BW_TS, first, tid, nth);
-    if (nh == 2) {
-      float* G2 = Gk + md.layer[1].dst_off;
-      outer_acc(G2, G2 + (long long)H2 * H1, dA2, A1, H2, H1, BW_TS, first, tid, nth);
-    }
-    if (nh >= 1) {
-      float* G1 = Gk + md.layer[0].dst_off;
-      outer_acc(G1, G1 + (long long)H1 * D, dA1, S, H1, D, BW_TS, first, tid, nth);
-    }
-    first = false;
-  }
-  if (first) {  // empty chunk: zero the slice
-    for (long long e = tid; e < md.n_params; e += nth) Gk[e] = 0.f;
-  }
-}
-
-cudaError_t launch_backward(const InstDev* d_inst, const LaunchInfo& li, int smem_bytes, int,
-                            const int8_t* spins, const double* logZR, const float* logq,
-                            const double* stats, float* partials, int part_stride,
-                            cudaStream_t s) {
-  const int nblk = li.tile_begin[li.n_inst];
-  if (nblk == 0) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(backward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       smem_bytes);
-  if (e != cudaSuccess) return e;
-  backward_kernel<<<nblk, 256, smem_bytes, s>>>(d_inst, li, spins, logZR, logq, stats, partials,
-                                                part_stride);
   return cudaGetLastError();
 }
 
