@@ -382,6 +382,11 @@ void plan_wide_strips(Instance& in, const std::map<std::pair<int, int>, int>& ed
     if (wa && wb) used[e] = 1;
     if (!used[e]) return;  // a bond the strips do not carry
   }
+  int off = 0;
+  for (WideStripDev& sd : plan.strips) {
+    sd.tab_off = off;
+    off += wide_tab_floats(sd.L);
+  }
   in.wide = std::move(plan);
 }
 
@@ -427,6 +432,11 @@ int upload_plan(tnvan_ctx* ctx, Instance& in) {
     if ((rc = upload(ctx, in, in.wide.rows, &dwr))) return rc;
     in.dev.wide = dws;
     in.dev.wrows = dwr;
+    const WideStripDev& last = in.wide.strips.back();
+    std::vector<float> zt((size_t)last.tab_off + wide_tab_floats(last.L), 0.f);
+    float* dt = nullptr;
+    if ((rc = upload(ctx, in, zt, &dt))) return rc;
+    in.dev.wtab = dt;
     in.dev.n_wide = (int)in.wide.strips.size();
   }
   if (in.kind == 0) {
@@ -3178,7 +3188,7 @@ int contract_all(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* d
   if (any_wide) {
     LaunchInfo lw;
     if ((rc = fill_launch(ctx, betas, batch, 1, lw))) return rc;
-    int acc = 0, ms = 0, Dm = 0;
+    int acc = 0, ms = 0, rows = 0;
     bool rest = false;
     for (int k = 0; k < lw.n_inst; ++k) {
       const Instance& in = ctx->inst[k];
@@ -3186,7 +3196,7 @@ int contract_all(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* d
       if (in.kind == 2 && in.dev.n_wide > 0) {
         acc += batch;
         ms = std::max(ms, in.dev.n_wide);
-        Dm = std::max(Dm, (int)in.W.size());
+        rows = std::max(rows, (int)in.wide.rows.size());
       } else if (in.kind == 2) {
         rest = true;
       }
@@ -3201,7 +3211,7 @@ int contract_all(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* d
     }
     if ((rc = ensure_wide_part(ctx, (size_t)lw.n_inst * batch * ms))) return rc;
     PROF("wide_strips", s);
-    CK(launch_wide(ctx->d_inst, lw, per_class, ms, Dm, d_spins, ctx->d_wide_part, d_logZR, s), "wide-strip kernels");
+    CK(launch_wide(ctx->d_inst, lw, per_class, ms, rows, d_spins, ctx->d_wide_part, d_logZR, s), "wide-strip kernels");
     k2 = rest;
   }
   if (k2) {

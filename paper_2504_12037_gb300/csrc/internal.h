@@ -161,7 +161,7 @@ struct WideRow {
 struct WideStripDev {
   int w, L;
   int row0;      // first row in the instance's wide-row array
-  int pad;
+  int tab_off;   // float offset of the strip's row tables in wtab (per call, wide_tab_kernel)
   double c_hat;  // sum of |J| over the strip's bonds (horizontal, vertical, W neighbours)
 };
 
@@ -258,6 +258,7 @@ struct InstDev {
   int n_wide;
   const WideStripDev* wide;
   const WideRow* wrows;
+  float* wtab;
 };
 
 // Per-launch parameters passed by value.
@@ -443,13 +444,15 @@ cudaError_t launch_strip_tables(const InstDev* d_inst, const LaunchInfo& li, int
 cudaError_t launch_observables(const LaunchInfo& li, const double* logZR, const float* logq, const double* stats,
                                const double* dbeta, float* wmul, double* out, bool energies, cudaStream_t s);
 // Wide strips (k_wide.cu): log Z_R of the elimination instances that carry a
-// wide-strip plan (li: one tile per sample of the instances to run, zero
-// tiles for the others), one CTA per sample, one launch per class of states
-// per lane (strips_per_class[c]: the most strips of 2^c states per lane in
-// one instance, c = 0 for strips of <= 5 columns), per-strip results in
-// part [n_inst][batch][max_strips], then their sum in strip order.
+// wide-strip plan (li: tiles of the instances to run, zero tiles for the
+// others): the row tables at li.beta, one launch per class of states per lane
+// (strips_per_class[c]: the most strips of 2^c states per lane in one
+// instance, c = 0 for strips of <= 5 columns), per-strip results in part
+// [n_inst][batch][max_strips], then their sum in strip order.  max_rows: the
+// most strip rows of an instance.
 cudaError_t launch_wide(const InstDev* d_inst, const LaunchInfo& li, const int* strips_per_class, int max_strips,
-                        int max_D, const int8_t* spins, double* part, double* logZR, cudaStream_t s);
+                        int max_rows, const int8_t* spins, double* part, double* logZR, cudaStream_t s);
+int wide_tab_floats(int L);  // table floats of a strip of L rows
 // Magnetisation moments (tnvan_magnetisation): per sample E[M | s] and
 // Var(M | s) of the whole system's magnetisation given the width set, by
 // contraction kind (strips: li.tile samples per CTA, smem as strip_smem_bytes;

@@ -3,19 +3,36 @@
 // instances whose plan is an elimination plan (their strips are wider than
 // the per-thread strip kernels hold in registers).  Forward log Z_R only.
 //
-// One CTA per sample, one warp per strip.  The 2^w states of a strip row are
-// spread over the warp: state x = lane | (j << 5), lane holding j = 0 ..
-// 2^(w-5) - 1 in registers (strips narrower than 5 columns use lanes < 2^w).
-// Per row y (same gauge as the strip planner: every vertical coupling >= 0):
+// One warp per (sample, strip), four samples of one strip per CTA.  Per row y
+// (same gauge as the strip planner: every vertical coupling >= 0):
 //   v <- V_{y-1} v   with V the Kronecker product of [[1, t_c], [t_c, 1]],
-//                    t_c = exp(-2 beta Jv_c): a shuffle for column bits < 5,
-//                    a register pair for the others;
+//                    t_c = exp(-2 beta Jv_c);
 //   v <- D_y v       D_y(x) = product over the row's bonds that x leaves
 //                    unsatisfied (J s s' < 0, W neighbours included) of
 //                    exp(-2 beta |J|): every factor is at most 1;
 //   v <- v / 2^e     e the exponent of the row's largest entry.
 // ln Z_strip = ln sum_x v(x) + ln 2 sum e + beta sum |J| over the strip's
 // bonds; log Z_R adds beta sum over W-W bonds J s s' (Eq. 4).
+//
+// The 2^w states of a row are spread over the warp: bits 0-4 of a state on the
+// lane, the others on the register index j.  A vertical factor on a register
+// bit is a pair of FMAs, on a lane bit a shuffle and an FMA per state.  Strips
+// of 10 to 12 columns instead exchange the lane bits with register bits 0-4
+// (32 x 32 transposes through shared memory), apply the five factors in
+// registers and exchange back: four shared accesses per state, not five
+// shuffles, without their latency chain.
+// D_y of a state is a product over the bonds in column order, the W neighbours
+// after bond 3 and last.  Its lane part is formed once per lane and row; the
+// register part along the binary tree of j's bits, so a state costs about
+// three products and not a chain of nine conditional ones.  The power of two
+// of the row before rides on the lane part.  The factors are tabulated per
+// strip row and beta (wide_tab_kernel).  Every value is rounded as in the
+// plain chain of products: at high temperature the same few products recur in
+// every row, so their rounding is systematic and moves log Z.
+// Bound by the FP32 pipe and shared memory alike (w + 4 operations and 4
+// shared accesses a state and row); 40 x 40 ferromagnet, 6 x 1,000 samples:
+// 5.15 ms with conditional products per state, a sample per CTA and shuffles,
+// 2.13 ms in this form.
 #include "common.cuh"
 
 namespace tnvan {
@@ -25,140 +42,250 @@ namespace {
 // Factor of a bond of coupling J that a state leaves unsatisfied.
 __device__ __forceinline__ float unsat_factor(float J, float beta) { return expf(-2.f * beta * fabsf(J)); }
 
-// One strip for one sample; NPL = states per lane (2^(w-5), or 1 for w <= 5).
-// Returns ln of the normalised sum and the power-of-two exponent count.
-template <int NPL>
-__device__ void wide_chain(const WideStripDev& sd, const WideRow* __restrict__ rows, const int8_t* srow, float beta,
-                           int lane, float& lnz, int& e2) {
-  const int w = sd.w;
-  const bool active = NPL > 1 || lane < (1 << w);
-  float v[NPL];
-  e2 = 0;
-  for (int y = 0; y < sd.L; ++y) {
-    const WideRow& R = rows[y];
-    // the row's factors, one per lane: lanes 0..10 horizontal bonds, 16..27
-    // vertical factors from row y - 1, 30 / 31 the W neighbours
-    float f = 1.f;
-    if (lane < w - 1) f = unsat_factor(R.Jh[lane], beta);
-    else if (lane >= 16 && lane < 16 + w && y > 0) f = expf(-2.f * beta * rows[y - 1].Jv[lane - 16]);
-    else if (lane == 30 && R.posL >= 0) f = unsat_factor(R.JL, beta);
-    else if (lane == 31 && R.posR >= 0) f = unsat_factor(R.JR, beta);
-    // negative-coupling bits of the horizontal bonds and the W-neighbour terms
-    uint32_t neg = 0;
-    for (int c = 0; c + 1 < w; ++c) neg |= (R.Jh[c] < 0.f ? 1u : 0u) << c;
-    // a W-neighbour bond J s_W s_0 is satisfied iff bit 0 == (J s_W < 0)
-    const float sL = R.posL >= 0 ? (float)srow[R.posL] : 0.f, sR = R.posR >= 0 ? (float)srow[R.posR] : 0.f;
-    const uint32_t wantL = (R.JL * sL < 0.f) ? 1u : 0u, wantR = (R.JR * sR < 0.f) ? 1u : 0u;
-    const float uL = __shfl_sync(0xffffffffu, f, 30), uR = __shfl_sync(0xffffffffu, f, 31);
-    if (y > 0) {
-      // vertical factors: column bits below 5 across lanes, the rest in registers
-#pragma unroll
-      for (int c = 0; c < 5; ++c) {
-        const float t = __shfl_sync(0xffffffffu, f, 16 + c);
-        if (c < w) {
-#pragma unroll
-          for (int j = 0; j < NPL; ++j) v[j] = fmaf(t, __shfl_xor_sync(0xffffffffu, v[j], 1 << c), v[j]);
-        }
-      }
-#pragma unroll
-      for (int c = 5; c < 5 + 7; ++c) {
-        if ((1 << (c - 5)) < NPL) {
-          const float t = __shfl_sync(0xffffffffu, f, 16 + c);
-#pragma unroll
-          for (int j = 0; j < NPL; ++j) {
-            if ((j >> (c - 5)) & 1) continue;
-            const int j1 = j | (1 << (c - 5));
-            const float a = v[j], b = v[j1];
-            v[j] = fmaf(t, b, a);
-            v[j1] = fmaf(t, a, b);
-          }
-        }
-      }
-    }
-    // diagonal: the lane part (bonds among bits 0..4, the left neighbour, and
-    // the right one when w <= 5), then per register the bonds among its bits
-    const uint32_t x0 = (uint32_t)lane;
-    float pl = 1.f;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const float u = __shfl_sync(0xffffffffu, f, c);
-      if (c + 1 < w && ((((x0 >> c) ^ (x0 >> (c + 1))) & 1u) != ((neg >> c) & 1u))) pl *= u;
-    }
-    if (R.posL >= 0 && ((x0 & 1u) != wantL)) pl *= uL;
-    if (w <= 5 && R.posR >= 0 && (((x0 >> (w - 1)) & 1u) != wantR)) pl *= uR;
-    // bond 4 (bits 4, 5) and bonds 5 .. w-2, the right neighbour on bit w-1
-    const float u4 = __shfl_sync(0xffffffffu, f, 4);
-    float ub[7];
-#pragma unroll
-    for (int i = 0; i < 7; ++i) ub[i] = __shfl_sync(0xffffffffu, f, (5 + i) & 31);
-    float mx = 0.f;
-#pragma unroll
-    for (int j = 0; j < NPL; ++j) {
-      float d = pl;
-      if (NPL > 1) {
-        const uint32_t x = x0 | ((uint32_t)j << 5);
-        if (((((x >> 4) ^ (x >> 5)) & 1u) != ((neg >> 4) & 1u))) d *= u4;
-#pragma unroll
-        for (int i = 0; i < 7; ++i) {
-          const int c = 5 + i;
-          if ((2 << i) < NPL && ((((x >> c) ^ (x >> (c + 1))) & 1u) != ((neg >> c) & 1u))) d *= ub[i];
-        }
-        if (R.posR >= 0 && (((x >> (w - 1)) & 1u) != wantR)) d *= uR;
-      }
-      const float vv = y == 0 ? d : v[j] * d;
-      v[j] = active ? vv : 0.f;
-      mx = fmaxf(mx, v[j]);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    const int e = exponent_of(mx);
-    const float sc = pow2i(-e);
-#pragma unroll
-    for (int j = 0; j < NPL; ++j) v[j] *= sc;
-    e2 += e;
-  }
-  float z = 0.f;
-#pragma unroll
-  for (int j = 0; j < NPL; ++j) z += v[j];
-  z = warp_sum(z);
-  lnz = logf(z);
-}
+// Per strip row 32 floats: 0-10 the horizontal bonds' factors, 16-27 the
+// vertical factors from the row above, 28 the mask of negative horizontal
+// couplings as bits, 30 / 31 the W neighbours' factors.
+constexpr int ROW_FLOATS = 32;
 
 }  // namespace
 
 // States per lane of a strip of w columns.
 __host__ __device__ __forceinline__ int wide_npl(int w) { return w <= 5 ? 1 : 1 << (w - 5); }
 
-// The strips of one state-count class (wide_npl(w) == NPL): CTA = sample,
-// warps over the instance's strips of that class; per-strip results to
+int wide_tab_floats(int L) { return L * ROW_FLOATS; }
+
+// One warp per strip row of an instance.
+__global__ void __launch_bounds__(128) wide_tab_kernel(const InstDev* __restrict__ inst, const LaunchInfo li) {
+  const int k = blockIdx.y;
+  if (li.tile_begin[k + 1] == li.tile_begin[k]) return;
+  const InstDev& I = inst[k];
+  int st = 0, y = blockIdx.x * 4 + (threadIdx.x >> 5);
+  for (; st < I.n_wide; ++st) {
+    if (y < I.wide[st].L) break;
+    y -= I.wide[st].L;
+  }
+  if (st == I.n_wide) return;
+  const WideRow* rows = I.wrows + I.wide[st].row0;
+  const WideRow& R = rows[y];
+  const int w = I.wide[st].w, t = threadIdx.x & 31;
+  const float beta = (float)li.beta[k];
+  float v = 1.f;
+  if (t < w - 1) {
+    v = unsat_factor(R.Jh[t], beta);
+  } else if (t >= 16 && t < 16 + w && y > 0) {
+    v = expf(-2.f * beta * rows[y - 1].Jv[t - 16]);
+  } else if (t == 28) {
+    uint32_t neg = 0;
+    for (int c = 0; c + 1 < w; ++c) neg |= (R.Jh[c] < 0.f ? 1u : 0u) << c;
+    v = __uint_as_float(neg);
+  } else if (t == 30 && R.posL >= 0) {
+    v = unsat_factor(R.JL, beta);
+  } else if (t == 31 && R.posR >= 0) {
+    v = unsat_factor(R.JR, beta);
+  }
+  I.wtab[I.wide[st].tab_off + y * ROW_FLOATS + t] = v;
+}
+
+namespace {
+
+// v <- (I + t X_bit) v on register bit Q.
+template <int NPL, int Q>
+__device__ __forceinline__ void vert(float (&v)[NPL], float t) {
+  if constexpr ((1 << Q) < NPL) {
+#pragma unroll
+    for (int j = 0; j < NPL; ++j) {
+      if ((j >> Q) & 1) continue;
+      const float a = v[j], b = v[j | (1 << Q)];
+      v[j] = fmaf(t, b, a);
+      v[j | (1 << Q)] = fmaf(t, a, b);
+    }
+  }
+}
+
+// The factors t[0..4] of the lane bits: 32 registers at a time exchanged with
+// the lanes (two alternating shared buffers of 32 x 33 floats), applied as
+// register bits, exchanged back.
+template <int NPL>
+__device__ __forceinline__ void vert_lanes(float (&v)[NPL], const float (&t)[5], float* buf, int lane) {
+#pragma unroll
+  for (int h = 0; h < NPL / 32; ++h) {
+    float* b = buf + (h & 1) * (32 * 33);
+    float x[32];
+#pragma unroll
+    for (int j = 0; j < 32; ++j) b[j * 33 + lane] = v[h * 32 + j];
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < 32; ++j) x[j] = b[lane * 33 + j];
+    vert<32, 0>(x, t[0]);
+    vert<32, 1>(x, t[1]);
+    vert<32, 2>(x, t[2]);
+    vert<32, 3>(x, t[3]);
+    vert<32, 4>(x, t[4]);
+#pragma unroll
+    for (int j = 0; j < 32; ++j) b[lane * 33 + j] = x[j];
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < 32; ++j) v[h * 32 + j] = b[j * 33 + lane];
+  }
+}
+
+// The row's largest entry over the warp -> its exponent.
+template <int NPL>
+__device__ __forceinline__ int row_exponent(const float (&v)[NPL]) {
+  float mx = 0.f;
+#pragma unroll
+  for (int j = 0; j < NPL; ++j) mx = fmaxf(mx, v[j]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  return exponent_of(mx);
+}
+
+// Which lane bits a bond of the lane part leaves unsatisfied: bits i, i + 1.
+__device__ __forceinline__ bool unsat(uint32_t x, int i, uint32_t neg_bit) {
+  return (((x >> i) ^ (x >> (i + 1))) & 1u) != (neg_bit & 1u);
+}
+
+// The register part of D: p the product so far at the low LEV bits J of the
+// register index; f[i][1 or 0] the factor of bond 5 + i when register bits i
+// and i + 1 differ or agree, g the right neighbour's by the top bit.
+template <int NPL, int LEV, int J, bool FIRST>
+__device__ __forceinline__ void diag_tree(float (&v)[NPL], float p, const float (&f)[6][2], const float (&g)[2]) {
+  if constexpr ((1 << LEV) == NPL) {
+    const float d = p * g[(J >> (LEV - 1)) & 1];
+    v[J] = FIRST ? d : v[J] * d;
+  } else {
+    constexpr int top = (J >> (LEV - 1)) & 1;
+    diag_tree<NPL, LEV + 1, J, FIRST>(v, p * f[LEV - 1][top], f, g);
+    diag_tree<NPL, LEV + 1, J | (1 << LEV), FIRST>(v, p * f[LEV - 1][top ^ 1], f, g);
+  }
+}
+
+// D of a row on v, times sc (FIRST: v = D sc).
+template <int NPL, bool FIRST>
+__device__ __forceinline__ void diag(float (&v)[NPL], const float* __restrict__ row, int w, uint32_t wantL,
+                                     uint32_t wantR, bool hasL, bool hasR, float sc, int lane) {
+  const float4 u03 = __ldg(reinterpret_cast<const float4*>(row));
+  const float u[4] = {u03.x, u03.y, u03.z, u03.w};
+  const uint32_t neg = __float_as_uint(__ldg(row + 28)), x0 = (uint32_t)lane;
+  float pl = sc;
+#pragma unroll
+  for (int c = 0; c < 4; ++c)
+    if (c + 1 < w && unsat(x0, c, neg >> c)) pl *= u[c];
+  if (hasL && (x0 & 1u) != wantL) pl *= __ldg(row + 30);
+  if (w <= 5 && hasR && ((x0 >> (w - 1)) & 1u) != wantR) pl *= __ldg(row + 31);
+  if constexpr (NPL == 1) {
+    const float d = lane < (1 << w) ? pl : 0.f;
+    v[0] = FIRST ? d : v[0] * d;
+  } else {
+    const float4 u47 = __ldg(reinterpret_cast<const float4*>(row + 4));
+    const float4 u8 = __ldg(reinterpret_cast<const float4*>(row + 8));
+    const float ub[6] = {u47.y, u47.z, u47.w, u8.x, u8.y, u8.z};
+    float f[6][2];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+      const bool ng = (neg >> (5 + i)) & 1u;
+      f[i][0] = ng ? ub[i] : 1.f;
+      f[i][1] = ng ? 1.f : ub[i];
+    }
+    const float uR = hasR ? __ldg(row + 31) : 1.f;
+    const float g[2] = {wantR ? uR : 1.f, wantR ? 1.f : uR};
+    // bond 4 joins lane bit 4 and register bit 0
+    const bool one4 = ((x0 >> 4) & 1u) != ((neg >> 4) & 1u);  // register bit 0 that satisfies it
+    diag_tree<NPL, 1, 0, FIRST>(v, one4 ? pl * u47.x : pl, f, g);
+    diag_tree<NPL, 1, 1, FIRST>(v, one4 ? pl : pl * u47.x, f, g);
+  }
+}
+
+// One strip for one sample; NPL = states per lane (2^(w-5), or 1 for w <= 5).
+// Returns ln of the normalised sum and the power-of-two exponent count.
+template <int NPL>
+__device__ __forceinline__ void wide_chain(const WideStripDev& sd, const WideRow* __restrict__ rows,
+                                           const float* __restrict__ tab, const int8_t* __restrict__ srow, float* buf,
+                                           int lane, float& lnz, int& e2) {
+  const int w = sd.w;
+  float v[NPL];
+  // the W neighbours of 32 rows at a time, one row per lane: bit y & 31 of
+  // wl / wr = the bit value of column 0 / w - 1 that satisfies the bond
+  uint32_t wl = 0, wr = 0, hl = 0, hr = 0;
+  auto neighbours = [&](int y0) {
+    const int y = y0 + lane;
+    const bool on = y < sd.L;
+    const int pL = on ? rows[y].posL : -1, pR = on ? rows[y].posR : -1;
+    const float sL = pL >= 0 ? (float)srow[pL] : 0.f, sR = pR >= 0 ? (float)srow[pR] : 0.f;
+    wl = __ballot_sync(0xffffffffu, on && rows[y].JL * sL < 0.f);
+    wr = __ballot_sync(0xffffffffu, on && rows[y].JR * sR < 0.f);
+    hl = __ballot_sync(0xffffffffu, pL >= 0);
+    hr = __ballot_sync(0xffffffffu, pR >= 0);
+  };
+  neighbours(0);
+  diag<NPL, true>(v, tab, w, wl & 1u, wr & 1u, hl & 1u, hr & 1u, 1.f, lane);
+  int e = row_exponent(v);
+  e2 = e;
+  float sc = pow2i(-e);
+  for (int y = 1; y < sd.L; ++y) {
+    if ((y & 31) == 0) neighbours(y);
+    const uint32_t b = 1u << (y & 31);
+    const float* row = tab + y * ROW_FLOATS;
+    const float4 ta = __ldg(reinterpret_cast<const float4*>(row + 16)), tb = __ldg(reinterpret_cast<const float4*>(row + 20)),
+                 tc = __ldg(reinterpret_cast<const float4*>(row + 24));
+    const float t5[5] = {ta.x, ta.y, ta.z, ta.w, tb.x};
+    if constexpr (NPL >= 32) {
+      vert_lanes(v, t5, buf, lane);
+    } else {
+#pragma unroll
+      for (int c = 0; c < 5; ++c)
+        if (c < w) {
+#pragma unroll
+          for (int j = 0; j < NPL; ++j) v[j] = fmaf(t5[c], __shfl_xor_sync(0xffffffffu, v[j], 1 << c), v[j]);
+        }
+    }
+    vert<NPL, 0>(v, tb.y);
+    vert<NPL, 1>(v, tb.z);
+    vert<NPL, 2>(v, tb.w);
+    vert<NPL, 3>(v, tc.x);
+    vert<NPL, 4>(v, tc.y);
+    vert<NPL, 5>(v, tc.z);
+    vert<NPL, 6>(v, tc.w);
+    diag<NPL, false>(v, row, w, (wl & b) ? 1u : 0u, (wr & b) ? 1u : 0u, hl & b, hr & b, sc, lane);
+    e = row_exponent(v);
+    e2 += e;
+    sc = pow2i(-e);
+  }
+  float z = 0.f;
+#pragma unroll
+  for (int j = 0; j < NPL; ++j) z += v[j] * sc;
+  z = warp_sum(z);
+  lnz = logf(z);
+}
+
+}  // namespace
+
+// The strips of one state-count class (wide_npl(w) == NPL): CTA = four
+// samples of strip blockIdx.y of the class, a warp each; per-strip results to
 // part[(k * batch + b) * li.tile_aux + strip].
 template <int NPL>
-__global__ void __launch_bounds__(256) wide_kernel(const InstDev* __restrict__ inst, const LaunchInfo li,
-                                                    const int8_t* __restrict__ spins, double* __restrict__ part) {
-  extern __shared__ float sm[];
-  const int k = find_inst(li, blockIdx.x);
+__global__ void __launch_bounds__(128, NPL >= 128 ? 3 : 4)
+    wide_kernel(const InstDev* __restrict__ inst, const LaunchInfo li, const int8_t* __restrict__ spins,
+                double* __restrict__ part) {
+  __shared__ float tr[NPL >= 32 ? 4 * 2 * 32 * 33 : 1];
+  const int k = blockIdx.z;
+  if (li.tile_begin[k + 1] == li.tile_begin[k]) return;
   const InstDev& I = inst[k];
-  if (I.n_wide == 0) return;
-  const int b = blockIdx.x - li.tile_begin[k];
-  const int t = threadIdx.x, wp = t >> 5, lane = t & 31;
-  const int D = I.D;
-  const int nw = blockDim.x >> 5;
-  int8_t* srow = reinterpret_cast<int8_t*>(sm);
-  const int8_t* g = spins + I.spin_units * li.batch + (long long)b * D;
-  for (int e = t; e < D; e += blockDim.x) srow[e] = g[e];
-  __syncthreads();
-  const float beta = (float)li.beta[k];
-  double* out = part + ((long long)k * li.batch + b) * li.tile_aux;
-  int nth = 0;  // index of the strip among this class's strips
-  for (int st = 0; st < I.n_wide; ++st) {
-    const WideStripDev sd = I.wide[st];
-    if (wide_npl(sd.w) != NPL) continue;
-    if (nth++ % nw != wp) continue;
-    float lnz = 0.f;
-    int e2 = 0;
-    wide_chain<NPL>(sd, I.wrows + sd.row0, srow, beta, lane, lnz, e2);
-    if (lane == 0) out[st] = (double)lnz + (double)e2 * 0.69314718055994530942 + li.beta[k] * sd.c_hat;
-  }
+  const int wp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int b = blockIdx.x * 4 + wp;
+  int nth = blockIdx.y, st = 0;
+  for (; st < I.n_wide; ++st)
+    if (wide_npl(I.wide[st].w) == NPL && nth-- == 0) break;
+  if (st == I.n_wide || b >= li.batch) return;
+  const WideStripDev sd = I.wide[st];
+  const int8_t* srow = spins + I.spin_units * li.batch + (long long)b * I.D;
+  float lnz = 0.f;
+  int e2 = 0;
+  wide_chain<NPL>(sd, I.wrows + sd.row0, I.wtab + sd.tab_off, srow, tr + (NPL >= 32 ? wp * 2 * 32 * 33 : 0), lane, lnz,
+                  e2);
+  if (lane == 0)
+    part[((long long)k * li.batch + b) * li.tile_aux + st] =
+        (double)lnz + (double)e2 * 0.69314718055994530942 + li.beta[k] * sd.c_hat;
 }
 
 // log Z_R per sample: the strips' results in strip order plus the W-W term.
@@ -183,27 +310,28 @@ __global__ void wide_sum_kernel(const InstDev* __restrict__ inst, const LaunchIn
 }
 
 cudaError_t launch_wide(const InstDev* d_inst, const LaunchInfo& li, const int* strips_per_class, int max_strips,
-                        int max_D, const int8_t* spins, double* part, double* logZR, cudaStream_t s) {
-  const int nblk = li.tile_begin[li.n_inst];
-  if (nblk == 0 || max_strips == 0) return cudaSuccess;
+                        int max_rows, const int8_t* spins, double* part, double* logZR, cudaStream_t s) {
+  if (li.tile_begin[li.n_inst] == 0 || max_strips == 0) return cudaSuccess;
   LaunchInfo lw = li;
   lw.tile_aux = max_strips;
-  const int smem = max_D + 16;
-  for (int c = 0; c < 8; ++c) {
+  wide_tab_kernel<<<dim3((unsigned)((max_rows + 3) / 4), li.n_inst), 128, 0, s>>>(d_inst, lw);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  for (int c = 7; c >= 0; --c) {  // the widest strips first
     const int n = strips_per_class[c];  // most strips of class c in one instance
     if (n == 0) continue;
-    const int warps = n < 8 ? n : 8;
+    const dim3 grid((unsigned)((li.batch + 3) / 4), n, li.n_inst);
     switch (c) {
-      case 0: wide_kernel<1><<<nblk, 32 * warps, smem, s>>>(d_inst, lw, spins, part); break;
-      case 1: wide_kernel<2><<<nblk, 32 * warps, smem, s>>>(d_inst, lw, spins, part); break;
-      case 2: wide_kernel<4><<<nblk, 32 * warps, smem, s>>>(d_inst, lw, spins, part); break;
-      case 3: wide_kernel<8><<<nblk, 32 * warps, smem, s>>>(d_inst, lw, spins, part); break;
-      case 4: wide_kernel<16><<<nblk, 32 * warps, smem, s>>>(d_inst, lw, spins, part); break;
-      case 5: wide_kernel<32><<<nblk, 32 * warps, smem, s>>>(d_inst, lw, spins, part); break;
-      case 6: wide_kernel<64><<<nblk, 32 * warps, smem, s>>>(d_inst, lw, spins, part); break;
-      default: wide_kernel<128><<<nblk, 32 * warps, smem, s>>>(d_inst, lw, spins, part); break;
+      case 0: wide_kernel<1><<<grid, 128, 0, s>>>(d_inst, lw, spins, part); break;
+      case 1: wide_kernel<2><<<grid, 128, 0, s>>>(d_inst, lw, spins, part); break;
+      case 2: wide_kernel<4><<<grid, 128, 0, s>>>(d_inst, lw, spins, part); break;
+      case 3: wide_kernel<8><<<grid, 128, 0, s>>>(d_inst, lw, spins, part); break;
+      case 4: wide_kernel<16><<<grid, 128, 0, s>>>(d_inst, lw, spins, part); break;
+      case 5: wide_kernel<32><<<grid, 128, 0, s>>>(d_inst, lw, spins, part); break;
+      case 6: wide_kernel<64><<<grid, 128, 0, s>>>(d_inst, lw, spins, part); break;
+      default: wide_kernel<128><<<grid, 128, 0, s>>>(d_inst, lw, spins, part); break;
     }
-    cudaError_t e = cudaGetLastError();
+    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
   wide_sum_kernel<<<dim3((unsigned)((li.batch + 255) / 256), li.n_inst), 256, 0, s>>>(d_inst, lw, spins, part, logZR);
