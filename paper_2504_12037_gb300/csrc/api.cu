@@ -742,6 +742,8 @@ int ensure_ws(tnvan_ctx* ctx, size_t bytes) {
   return TNVAN_OK;
 }
 
+size_t chain_ws_elems(const tnvan_ctx* ctx, int batch, ChainWs* cw);
+
 // Floats of the tensor-core backward workspace for `batch` samples.
 size_t tc_ws_floats(const tnvan_ctx* ctx, int batch) {
   // per instance: A1, A2, dX, dA2, dA1, w and the BF16 spins, each rounded up
@@ -750,7 +752,7 @@ size_t tc_ws_floats(const tnvan_ctx* ctx, int batch) {
   for (const Instance& in : ctx->inst)
     tot += (size_t)batch * (2 * in.H[0] + 2 * in.H[1] + in.W.size() + 1) + 6 * 16 +
            ((size_t)batch * ((in.W.size() + 7) & ~size_t(7)) + 1) / 2 + 16;
-  return tot + (size_t)ctx->inst.size() * batch + 16;
+  return std::max(tot + (size_t)ctx->inst.size() * batch + 16, (chain_ws_elems(ctx, batch, nullptr) + 1) / 2);
 }
 
 // FP32 backward (k_bwd32.cu): its unit-major rows, the batch rounded up to the
@@ -782,6 +784,38 @@ int bwd32_splits(const tnvan_ctx* ctx, int batch) {
   return std::max(1, std::min({608 / std::max(blocks, 1), (batch + 63) / 64, 256}));
 }
 
+// BF16 chain kernel (k_bwd_chain.cu): workspace in BF16 elements, and the
+// launch's ring depth and shared memory (false: some instance does not fit).
+size_t chain_ws_elems(const tnvan_ctx* ctx, int batch, ChainWs* cw) {
+  size_t off = 0;
+  for (size_t k = 0; k < ctx->inst.size(); ++k) {
+    const Instance& in = ctx->inst[k];
+    if (cw) cw->off[k] = (long long)off;
+    off += 2 * (size_t)batch * (((in.W.size() + 7) & ~size_t(7)) + ((in.H[0] + 7) & ~7) + ((in.H[1] + 7) & ~7));
+  }
+  return off;
+}
+template <class Skip>
+bool plan_bwd_chain(const tnvan_ctx* ctx, Skip skip, int* ns, int* max_n, int* smem) {
+  *max_n = 1;
+  for (size_t k = 0; k < ctx->inst.size(); ++k)
+    if (!skip((int)k)) {
+      const Instance& in = ctx->inst[k];
+      *max_n = std::max({*max_n, (int)in.W.size(), in.H[0], in.H[1]});
+    }
+  if (*max_n > 256) return false;
+  for (*ns = 4; *ns >= 2; --*ns) {
+    *smem = 0;
+    for (size_t k = 0; k < ctx->inst.size(); ++k)
+      if (!skip((int)k)) {
+        const Instance& in = ctx->inst[k];
+        *smem = std::max(*smem, bwd_chain_smem_bytes((int)in.W.size(), in.H[0], in.H[1], *max_n, *ns));
+      }
+    if (*smem <= 227 * 1024) return true;
+  }
+  return false;
+}
+
 #define TC_SPLITS 16
 
 // Backward of sum_b w_b log q(s_b) on the tensor cores (TF32 or BF16 operands,
@@ -804,7 +838,11 @@ int backward_tc(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* d_
     off += (cnt + 15) & ~size_t(15);
     return p;
   };
-  for (int k = 0; k < n; ++k) {
+  // BF16: the chain kernel where every instance fits it
+  int ns = 0, max_n = 0, smem = 0;
+  const bool chain = bf16 && plan_bwd_chain(ctx, skip, &ns, &max_n, &smem);
+  ChainWs cw;
+  for (int k = 0; k < n && !chain; ++k) {
     const Instance& in = ctx->inst[k];
     const size_t B = batch, D = in.W.size();
     bf[k].A1 = take(B * in.H[0]);
@@ -821,7 +859,7 @@ int backward_tc(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* d_
   const int IT = bf16 ? GT_BF16 : GT_F32;
   uint16_t* s16 = nullptr;
   std::vector<size_t> s16off(n, 0);
-  if (bf16) {
+  if (bf16 && !chain) {
     size_t tot16 = 0;
     for (int k = 0; k < n; ++k) {
       s16off[k] = tot16;
@@ -837,8 +875,9 @@ int backward_tc(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* d_
   for (int k = 0; k < n; ++k)
     if (skip(k)) li.skip[k >> 5] |= 1u << (k & 31);  // no BF16 spins for the fused instances
   // per-instance REINFORCE weights laid out [k][batch] in one contiguous buffer
-  float* wall = take((size_t)n * batch);
-  {
+  float* wall = nullptr;
+  if (!chain) {
+    wall = take((size_t)n * batch);
     PROF("reinforce_w", s);
     CK(launch_reinforce_w(ctx->d_inst, li, d_logZR, d_logq, ctx->d_stats, wall, d_spins, s16, s), "weights kernel");
   }
@@ -881,80 +920,96 @@ int backward_tc(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* d_
     return P;
   };
   const int B = batch;
-  // stage 1: A1 = relu(S W1^T + b1)
-  for (int k = 0; k < n; ++k) {
-    if (skip(k)) continue;
-    const Instance& in = ctx->inst[k];
-    const MadeDev& md = in.dev.made;
-    if (md.nh < 1) continue;
-    const int D = md.D;
-    const long long o1 = md.layer[0].dst_off;
-    GemmProblem P = base(B, md.H1, D, spin_op(k, false), op(wts(md, o1), D, 1, IT), EPI_BIAS_RELU, bf[k].A1, md.H1);
-    P.bias = md.packed + o1 + (long long)md.H1 * D;
-    probs.push_back(P);
-    max_m = std::max(max_m, B);
+  if (chain) {
+    chain_ws_elems(ctx, batch, &cw);
+    cw.base = reinterpret_cast<uint16_t*>(ws);
+    LaunchInfo lc;
+    if ((rc = fill_launch(ctx, betas, batch, 128, lc))) return rc;
+    int acc = 0;
+    for (int k = 0; k < n; ++k) {
+      lc.tile_begin[k] = acc;
+      if (!skip(k)) acc += (batch + 127) / 128;
+    }
+    lc.tile_begin[n] = acc;
+    PROF("bwd_chain", s);
+    CK(launch_bwd_chain(ctx->d_inst, lc, cw, ns, max_n, smem, d_spins, d_logZR, d_logq, ctx->d_stats, s),
+       "backward chain kernel");
+  } else {
+    // stage 1: A1 = relu(S W1^T + b1)
+    for (int k = 0; k < n; ++k) {
+      if (skip(k)) continue;
+      const Instance& in = ctx->inst[k];
+      const MadeDev& md = in.dev.made;
+      if (md.nh < 1) continue;
+      const int D = md.D;
+      const long long o1 = md.layer[0].dst_off;
+      GemmProblem P = base(B, md.H1, D, spin_op(k, false), op(wts(md, o1), D, 1, IT), EPI_BIAS_RELU, bf[k].A1, md.H1);
+      P.bias = md.packed + o1 + (long long)md.H1 * D;
+      probs.push_back(P);
+      max_m = std::max(max_m, B);
+    }
+    if ((rc = flush("gemm_fwd1"))) return rc;
+    // stage 2: A2 = relu(A1 W2^T + b2)
+    for (int k = 0; k < n; ++k) {
+      if (skip(k)) continue;
+      const MadeDev& md = ctx->inst[k].dev.made;
+      if (md.nh < 2) continue;
+      const long long o2 = md.layer[1].dst_off;
+      GemmProblem P = base(B, md.H2, md.H1, op(bf[k].A1, md.H1, 1, IT), op(wts(md, o2), md.H1, 1, IT),
+                           EPI_BIAS_RELU, bf[k].A2, md.H2);
+      P.bias = md.packed + o2 + (long long)md.H2 * md.H1;
+      probs.push_back(P);
+      max_m = std::max(max_m, B);
+    }
+    if ((rc = flush("gemm_fwd2"))) return rc;
+    // stage 3: dX = w_b s sigmoid(-s x), x = src Wo^T + bo
+    for (int k = 0; k < n; ++k) {
+      if (skip(k)) continue;
+      const Instance& in = ctx->inst[k];
+      const MadeDev& md = in.dev.made;
+      const int D = md.D, Hl = md.Hl;
+      const int8_t* S = d_spins + in.dev.spin_units * batch;
+      const long long oo = md.layer[md.nh].dst_off;
+      GemmOperand A = md.nh == 0 ? op(S, D, 1, GT_I8) : op(md.nh == 1 ? bf[k].A1 : bf[k].A2, Hl, 1, IT);
+      GemmProblem P = base(B, D, Hl, A, op(wts(md, oo), Hl, 1, IT), EPI_DX, bf[k].dX, D);
+      P.bias = md.packed + oo + (long long)D * Hl;
+      P.spins = S;
+      P.ld_spins = D;
+      P.row_w = wall + (size_t)k * batch;
+      probs.push_back(P);
+      max_m = std::max(max_m, B);
+    }
+    if ((rc = flush("gemm_out_dx"))) return rc;
+    // stage 4: delta of the last hidden layer = (dX Wo) * 1[h > 0]
+    for (int k = 0; k < n; ++k) {
+      if (skip(k)) continue;
+      const MadeDev& md = ctx->inst[k].dev.made;
+      if (md.nh < 1) continue;
+      const int D = md.D, Hl = md.Hl;
+      float* out = md.nh == 2 ? bf[k].dA2 : bf[k].dA1;
+      const float* mask = md.nh == 2 ? bf[k].A2 : bf[k].A1;
+      GemmProblem P = base(B, Hl, D, op(bf[k].dX, D, 1, IT), op(wts(md, md.layer[md.nh].dst_off), 1, Hl, IT), EPI_MASK,
+                           out, Hl);
+      P.mask = mask;
+      P.ld_mask = Hl;
+      probs.push_back(P);
+      max_m = std::max(max_m, B);
+    }
+    if ((rc = flush("gemm_bwd_last"))) return rc;
+    // stage 5: dA1 = (dA2 W2) * 1[h1 > 0]
+    for (int k = 0; k < n; ++k) {
+      if (skip(k)) continue;
+      const MadeDev& md = ctx->inst[k].dev.made;
+      if (md.nh < 2) continue;
+      GemmProblem P = base(B, md.H1, md.H2, op(bf[k].dA2, md.H2, 1, IT), op(wts(md, md.layer[1].dst_off), 1, md.H1, IT),
+                           EPI_MASK, bf[k].dA1, md.H1);
+      P.mask = bf[k].A1;
+      P.ld_mask = md.H1;
+      probs.push_back(P);
+      max_m = std::max(max_m, B);
+    }
+    if ((rc = flush("gemm_bwd_h1"))) return rc;
   }
-  if ((rc = flush("gemm_fwd1"))) return rc;
-  // stage 2: A2 = relu(A1 W2^T + b2)
-  for (int k = 0; k < n; ++k) {
-    if (skip(k)) continue;
-    const MadeDev& md = ctx->inst[k].dev.made;
-    if (md.nh < 2) continue;
-    const long long o2 = md.layer[1].dst_off;
-    GemmProblem P = base(B, md.H2, md.H1, op(bf[k].A1, md.H1, 1, IT), op(wts(md, o2), md.H1, 1, IT),
-                         EPI_BIAS_RELU, bf[k].A2, md.H2);
-    P.bias = md.packed + o2 + (long long)md.H2 * md.H1;
-    probs.push_back(P);
-    max_m = std::max(max_m, B);
-  }
-  if ((rc = flush("gemm_fwd2"))) return rc;
-  // stage 3: dX = w_b s sigmoid(-s x), x = src Wo^T + bo
-  for (int k = 0; k < n; ++k) {
-    if (skip(k)) continue;
-    const Instance& in = ctx->inst[k];
-    const MadeDev& md = in.dev.made;
-    const int D = md.D, Hl = md.Hl;
-    const int8_t* S = d_spins + in.dev.spin_units * batch;
-    const long long oo = md.layer[md.nh].dst_off;
-    GemmOperand A = md.nh == 0 ? op(S, D, 1, GT_I8) : op(md.nh == 1 ? bf[k].A1 : bf[k].A2, Hl, 1, IT);
-    GemmProblem P = base(B, D, Hl, A, op(wts(md, oo), Hl, 1, IT), EPI_DX, bf[k].dX, D);
-    P.bias = md.packed + oo + (long long)D * Hl;
-    P.spins = S;
-    P.ld_spins = D;
-    P.row_w = wall + (size_t)k * batch;
-    probs.push_back(P);
-    max_m = std::max(max_m, B);
-  }
-  if ((rc = flush("gemm_out_dx"))) return rc;
-  // stage 4: delta of the last hidden layer = (dX Wo) * 1[h > 0]
-  for (int k = 0; k < n; ++k) {
-    if (skip(k)) continue;
-    const MadeDev& md = ctx->inst[k].dev.made;
-    if (md.nh < 1) continue;
-    const int D = md.D, Hl = md.Hl;
-    float* out = md.nh == 2 ? bf[k].dA2 : bf[k].dA1;
-    const float* mask = md.nh == 2 ? bf[k].A2 : bf[k].A1;
-    GemmProblem P = base(B, Hl, D, op(bf[k].dX, D, 1, IT), op(wts(md, md.layer[md.nh].dst_off), 1, Hl, IT), EPI_MASK,
-                         out, Hl);
-    P.mask = mask;
-    P.ld_mask = Hl;
-    probs.push_back(P);
-    max_m = std::max(max_m, B);
-  }
-  if ((rc = flush("gemm_bwd_last"))) return rc;
-  // stage 5: dA1 = (dA2 W2) * 1[h1 > 0]
-  for (int k = 0; k < n; ++k) {
-    if (skip(k)) continue;
-    const MadeDev& md = ctx->inst[k].dev.made;
-    if (md.nh < 2) continue;
-    GemmProblem P = base(B, md.H1, md.H2, op(bf[k].dA2, md.H2, 1, IT), op(wts(md, md.layer[1].dst_off), 1, md.H1, IT),
-                         EPI_MASK, bf[k].dA1, md.H1);
-    P.mask = bf[k].A1;
-    P.ld_mask = md.H1;
-    probs.push_back(P);
-    max_m = std::max(max_m, B);
-  }
-  if ((rc = flush("gemm_bwd_h1"))) return rc;
   // stage 6: weight gradients, split over the batch into TC_SPLITS partial slices
   splits = std::max(1, std::min(TC_SPLITS, (batch + 127) / 128));
   float* part = ctx->d_grad_packed;
@@ -965,16 +1020,21 @@ int backward_tc(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* d_
     float* pk = part + (long long)k * splits * part_stride;
     for (int l = 0; l <= md.nh; ++l) {
       const LayerDev& L = md.layer[l];
-      const float* delta = l == md.nh ? bf[k].dX : (l == 1 ? bf[k].dA2 : bf[k].dA1);
-      GemmOperand act;
-      if (l == 0) act = spin_op(k, true);
-      else act = op(l == 1 ? bf[k].A1 : bf[k].A2, 1, L.nin, IT);
+      GemmOperand del, act;
+      if (chain) {
+        const ChainRows r = chain_rows(cw, k, batch, md.D, md.H1, md.H2);
+        del = l == md.nh ? op(r.X, 1, r.ldD, GT_BF16) : (l == 1 ? op(r.dA2, 1, r.ld2, GT_BF16) : op(r.dA1, 1, r.ld1, GT_BF16));
+        act = l == 0 ? op(r.S, 1, r.ldD, GT_BF16) : (l == 1 ? op(r.A1, 1, r.ld1, GT_BF16) : op(r.A2, 1, r.ld2, GT_BF16));
+      } else {
+        del = op(l == md.nh ? bf[k].dX : (l == 1 ? bf[k].dA2 : bf[k].dA1), 1, L.nout, IT);
+        act = l == 0 ? spin_op(k, true) : op(l == 1 ? bf[k].A1 : bf[k].A2, 1, L.nin, IT);
+      }
       for (int n0 = 0; n0 < L.nin; n0 += 128) {
         const bool last = n0 + 128 >= L.nin;
         const int nn = (L.nin + 1 <= 256) ? L.nin : std::min(128, L.nin - n0);
         GemmOperand actn = act;
         actn.ptr = static_cast<const char*>(act.ptr) + (size_t)n0 * (act.type == GT_F32 ? 4 : act.type == GT_BF16 ? 2 : 1);
-        GemmProblem P = base(L.nout, nn, B, op(delta, 1, L.nout, IT), actn, EPI_STORE,
+        GemmProblem P = base(L.nout, nn, B, del, actn, EPI_STORE,
                              pk + L.dst_off + n0, L.nin);
         P.split_stride = part_stride;
         if (last || L.nin + 1 <= 256) {

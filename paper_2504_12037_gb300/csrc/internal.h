@@ -520,6 +520,36 @@ cudaError_t launch_grad_reduce(const InstDev* d_inst, const LaunchInfo& li,
 // s16 != nullptr: also the spins as BF16 rows of r8(D) (the GEMM chain's operand)
 cudaError_t launch_reinforce_w(const InstDev* d_inst, const LaunchInfo& li, const double* logZR, const float* logq,
                                const double* stats, float* w, const int8_t* spins, uint16_t* s16, cudaStream_t s);
+// BF16 backward chain (k_bwd_chain.cu): row-major BF16 rows of every sample in
+// global memory, instance k's six arrays back to back at base + off[k].
+struct ChainWs {
+  uint16_t* base;
+  long long off[TNVAN_MAX_INST];
+};
+struct ChainRows {
+  uint16_t *S, *A1, *A2, *X, *dA2, *dA1;
+  int ldD, ld1, ld2;  // row lengths: the widths rounded up to 8, zeros beyond
+};
+__host__ __device__ inline ChainRows chain_rows(const ChainWs& w, int k, int batch, int D, int H1, int H2) {
+  ChainRows r;
+  r.ldD = (D + 7) & ~7;
+  r.ld1 = (H1 + 7) & ~7;
+  r.ld2 = (H2 + 7) & ~7;
+  const long long B = batch;
+  r.S = w.base + w.off[k];
+  r.A1 = r.S + B * r.ldD;
+  r.A2 = r.A1 + B * r.ld1;
+  r.X = r.A2 + B * r.ld2;
+  r.dA2 = r.X + B * r.ldD;
+  r.dA1 = r.dA2 + B * r.ld2;
+  return r;
+}
+int bwd_chain_smem_bytes(int D, int H1, int H2, int max_n, int ns);
+// li: tiles of 128 samples; ns weight stages in the ring (2 to 4); max_n: the
+// widest layer or width set (at most 256).
+cudaError_t launch_bwd_chain(const InstDev* d_inst, const LaunchInfo& li, const ChainWs& cw, int ns, int max_n,
+                             int smem_bytes, const int8_t* spins, const double* logZR, const float* logq,
+                             const double* stats, cudaStream_t s);
 cudaError_t launch_bwd_fused(const InstDev* d_inst, const LaunchInfo& li, int smem_bytes,
                              const int8_t* spins, const double* logZR, const float* logq,
                              const double* stats, float* partials, long long part_stride, int* status,

@@ -15,8 +15,8 @@
 // Bound by latency: five dependent products of 1 to 8 stages, each with an
 // epilogue of (columns / 2) values a thread.  As five GEMM launches (64 columns
 // a CTA, operands through global memory) with the weights' and spins' own
-// launch before them, CHAIN_WAS us for the 48-256-256-48 network and 3 x 4,096
-// samples; CHAIN_NOW us in this form.
+// launch before them, 134 us for the 48-256-256-48 network and 3 x 4,096
+// samples; 73 us in this form.
 #include <cuda_bf16.h>
 
 #include "common.cuh"
