@@ -110,8 +110,135 @@ __device__ __forceinline__ float group_max(float v, int GL) {
   return v;
 }
 
-// Component c for the sample whose tables start at A (entry e at A[e * RS];
-// with DB the beta-derivatives at dA[e * RS]); forward, live offsets.
+// The entries of one step's table for a sample (entry e of a table at A[e *
+// RS]; with DB the beta-derivatives at dA[e * RS]): fv the eliminated spin's
+// field factors, fr their beta-logarithmic derivatives, out the new table's
+// offset, COL the input offsets' column (0 live, 1 full), NIN the number of
+// input tables (-1: r.nin).  Returns the table's exponent; the table is
+// written scaled by 2^-exponent, ZERO also clears Ab at its entries.
+// A step is a chain of map, table and scale accesses whose latency sets the
+// time, so a lane's entries are taken GEN_U at a time with every load of a
+// batch independent, and tables of at most GEN_U entries a lane stay in
+// registers until their scale is known (one table write instead of a write, a
+// read and a write).
+#define GEN_U 4
+template <bool DB, int NIN, int COL, bool ZERO>
+__device__ __forceinline__ int step_table(const StepRec& r, const GenDev& G, const float (&fv)[2], const float (&fr)[2],
+                                          float* A, float* dA, float* Ab, int RS, int out, int lane, int GL) {
+  const int M = 1 << r.m, E = 2 * M;
+  const float* pp = G.pp + r.ppo;
+  const float* pd = G.pp + G.n_pp + r.ppo;
+  const unsigned short* mp = G.map + r.mo;
+  const bool regs = M <= GL * GEN_U;
+  int io[NIN > 0 ? NIN : 1];
+#pragma unroll
+  for (int i = 0; i < NIN; ++i) io[i] = r.io[3 * i + COL];
+  float av[GEN_U], dv[GEN_U];
+  float mx = 0.f;
+  for (int x0 = lane; x0 < M; x0 += GL * GEN_U) {
+    float p[GEN_U][2], rr[GEN_U][2];
+#pragma unroll
+    for (int u = 0; u < GEN_U; ++u) {
+      const int x = x0 + u * GL < M ? x0 + u * GL : x0;
+#pragma unroll
+      for (int sg = 0; sg < 2; ++sg) {
+        p[u][sg] = pp[x | (sg << r.m)];
+        rr[u][sg] = DB ? pd[x | (sg << r.m)] : 0.f;
+      }
+    }
+    if constexpr (NIN >= 0) {
+      float val[NIN > 0 ? NIN : 1][GEN_U][2], dval[NIN > 0 ? NIN : 1][GEN_U][2];
+#pragma unroll
+      for (int i = 0; i < NIN; ++i)
+#pragma unroll
+        for (int u = 0; u < GEN_U; ++u) {
+          const int x = x0 + u * GL < M ? x0 + u * GL : x0;
+#pragma unroll
+          for (int sg = 0; sg < 2; ++sg) {
+            const int q = (io[i] + mp[i * E + (x | (sg << r.m))]) * RS;
+            val[i][u][sg] = A[q];
+            if (DB) dval[i][u][sg] = dA[q];
+          }
+        }
+#pragma unroll
+      for (int u = 0; u < GEN_U; ++u)
+#pragma unroll
+        for (int sg = 0; sg < 2; ++sg) {
+          p[u][sg] = fv[sg] * p[u][sg];
+          if (DB) rr[u][sg] = fr[sg] + rr[u][sg];
+#pragma unroll
+          for (int i = 0; i < NIN; ++i) {
+            p[u][sg] *= val[i][u][sg];
+            if (DB) rr[u][sg] += dval[i][u][sg] / val[i][u][sg];
+          }
+        }
+    } else {
+#pragma unroll
+      for (int u = 0; u < GEN_U; ++u) {
+        const int x = x0 + u * GL < M ? x0 + u * GL : x0;
+#pragma unroll
+        for (int sg = 0; sg < 2; ++sg) {
+          p[u][sg] = fv[sg] * p[u][sg];
+          if (DB) rr[u][sg] = fr[sg] + rr[u][sg];
+          for (int i = 0; i < r.nin; ++i) {
+            const int q = (r.io[3 * i + COL] + mp[i * E + (x | (sg << r.m))]) * RS;
+            const float v = A[q];
+            p[u][sg] *= v;
+            if (DB) rr[u][sg] += dA[q] / v;
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < GEN_U; ++u) {
+      const int x = x0 + u * GL;
+      av[u] = __fadd_rn(p[u][0], p[u][1]);  // the products' own rounding: not contracted into the last one
+      if (DB) dv[u] = fmaf(p[u][1], rr[u][1], p[u][0] * rr[u][0]);
+      if (x >= M) continue;
+      mx = fmaxf(mx, av[u]);
+      if (!regs) {
+        A[(out + x) * RS] = av[u];
+        if (DB) dA[(out + x) * RS] = dv[u];
+      }
+    }
+  }
+  mx = group_max(mx, GL);
+  const int e = exponent_of(mx);
+  const float sc = pow2i(-e);
+  if (regs) {
+#pragma unroll
+    for (int u = 0; u < GEN_U; ++u) {
+      const int x = lane + u * GL;
+      if (x >= M) continue;
+      A[(out + x) * RS] = av[u] * sc;
+      if (DB) dA[(out + x) * RS] = dv[u] * sc;
+      if (ZERO) Ab[(out + x) * RS] = 0.f;
+    }
+  } else {
+#pragma unroll 4
+    for (int x = lane; x < M; x += GL) {
+      A[(out + x) * RS] *= sc;
+      if (DB) dA[(out + x) * RS] *= sc;
+      if (ZERO) Ab[(out + x) * RS] = 0.f;
+    }
+  }
+  return e;
+}
+
+template <bool DB, int COL, bool ZERO>
+__device__ __forceinline__ int step_table_any(const StepRec& r, const GenDev& G, const float (&fv)[2],
+                                              const float (&fr)[2], float* A, float* dA, float* Ab, int RS, int out,
+                                              int lane, int GL) {
+  switch (r.nin) {  // the same for every lane
+    case 0: return step_table<DB, 0, COL, ZERO>(r, G, fv, fr, A, dA, Ab, RS, out, lane, GL);
+    case 1: return step_table<DB, 1, COL, ZERO>(r, G, fv, fr, A, dA, Ab, RS, out, lane, GL);
+    case 2: return step_table<DB, 2, COL, ZERO>(r, G, fv, fr, A, dA, Ab, RS, out, lane, GL);
+    case 3: return step_table<DB, 3, COL, ZERO>(r, G, fv, fr, A, dA, Ab, RS, out, lane, GL);
+    default: return step_table<DB, -1, COL, ZERO>(r, G, fv, fr, A, dA, Ab, RS, out, lane, GL);
+  }
+}
+
+// Component c for the sample whose tables start at A; forward, live offsets.
 // Adds log Z_c (and with DB its beta-derivative) to lz / dl on lane 0 of the
 // group.
 template <bool DB>
@@ -125,9 +252,11 @@ __device__ __forceinline__ void run_component(const GenDev& G, int c, const int8
   // both added to the FP64 result once per component
   int esum = 0;
   float hs = 0.f, hc = 0.f;
+  // the next step's record and field are read ahead of this step's tables
+  StepRec r = nsteps > 0 ? step_at(G, g0) : StepRec{};
+  float h = nsteps > 0 ? field_of(G, r.fb, r.fc, s) : 0.f;
   for (int st = 0; st < nsteps; ++st) {
-    const StepRec r = step_at(G, g0 + st);
-    const float h = field_of(G, r.fb, r.fc, s);
+    const StepRec rn = step_at(G, g0 + (st + 1 < nsteps ? st + 1 : st));
     const float ah = fabsf(h);
     {
       const float y = ah - hc;
@@ -137,40 +266,10 @@ __device__ __forceinline__ void run_component(const GenDev& G, int c, const int8
     }
     const float fv[2] = {expf(beta * (h - ah)), expf(beta * (-h - ah))};
     const float fr[2] = {h - ah, -h - ah};
-    const int M = 1 << r.m, E = 2 * M;
-    const float* pp = G.pp + r.ppo;
-    const float* pd = G.pp + G.n_pp + r.ppo;
-    const unsigned short* mp = G.map + r.mo;
-    const int out = r.out_live;
-    float mx = 0.f;
-    for (int x = lane; x < M; x += GL) {
-      float acc = 0.f, dacc = 0.f;
-#pragma unroll
-      for (int sg = 0; sg < 2; ++sg) {
-        const int ext = x | (sg << r.m);
-        float p = fv[sg] * pp[ext];
-        float rr = DB ? fr[sg] + pd[ext] : 0.f;
-        for (int i = 0; i < r.nin; ++i) {
-          const int a = (r.io[3 * i] + mp[i * E + ext]) * RS;
-          const float val = A[a];
-          p *= val;
-          if (DB) rr += dA[a] / val;
-        }
-        acc += p;
-        if (DB) dacc = fmaf(p, rr, dacc);
-      }
-      A[(out + x) * RS] = acc;
-      if (DB) dA[(out + x) * RS] = dacc;
-      mx = fmaxf(mx, acc);
-    }
-    mx = group_max(mx, GL);
-    const int e = exponent_of(mx);
-    const float sc = pow2i(-e);
-    for (int x = lane; x < M; x += GL) {
-      A[(out + x) * RS] *= sc;
-      if (DB) dA[(out + x) * RS] *= sc;
-    }
-    esum += e;
+    const float hn = field_of(G, rn.fb, rn.fc, s);
+    esum += step_table_any<DB, 0, false>(r, G, fv, fr, A, dA, nullptr, RS, r.out_live, lane, GL);
+    r = rn;
+    h = hn;
     __syncwarp();
   }
   if (lane == 0) {
@@ -334,9 +433,95 @@ __global__ void __launch_bounds__(128) general_tab_kernel(const InstDev* __restr
 // row per CTA, and the rows added per instance in a fixed order: the result
 // does not depend on scheduling.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void acc_edge(float* acc_w, int e, float v, bool lane0) {
-  v = warp_sum(v);
-  if (lane0 && e >= 0) acc_w[e] += v;
+// Four bond sums at once (their shuffles overlap).
+__device__ __forceinline__ void acc_edges(float* acc_w, const int (&e)[4], float (&v)[4], bool lane0) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v[j] += __shfl_xor_sync(0xffffffffu, v[j], o);
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+    if (lane0 && e[j] >= 0) acc_w[e[j]] += v[j];
+}
+
+// The product terms of one step in the reverse sweep: g(x, sigma) into gb, its
+// sums with sigma (gs) and with sigma sigma_u of the first NPU bonds (gp), in
+// the order of x; loads GEN_U entries at a time.
+template <int NIN, int NPU>
+__device__ __forceinline__ void step_g(const StepRec& r, const GenDev& G, const float (&fv)[2], const float* A,
+                                       const float* Ab, float* gb, int RS, int out, float scl, const int* pos, int np,
+                                       int lane, int GL, float& gs, float (&gp)[TNVAN_MAX_ELIM_W]) {
+  const int M = 1 << r.m, E = 2 * M;
+  const float* pp = G.pp + r.ppo;
+  const unsigned short* mp = G.map + r.mo;
+  int io[NIN > 0 ? NIN : 1];
+#pragma unroll
+  for (int i = 0; i < NIN; ++i) io[i] = r.io[3 * i + 1];
+  for (int x0 = lane; x0 < M; x0 += GL * GEN_U) {
+    float p[GEN_U][2], abx[GEN_U];
+#pragma unroll
+    for (int u = 0; u < GEN_U; ++u) {
+      const int x = x0 + u * GL < M ? x0 + u * GL : x0;
+      abx[u] = Ab[(out + x) * RS];
+#pragma unroll
+      for (int sg = 0; sg < 2; ++sg) p[u][sg] = pp[x | (sg << r.m)];
+    }
+    if constexpr (NIN >= 0) {
+      float val[NIN > 0 ? NIN : 1][GEN_U][2];
+#pragma unroll
+      for (int i = 0; i < NIN; ++i)
+#pragma unroll
+        for (int u = 0; u < GEN_U; ++u) {
+          const int x = x0 + u * GL < M ? x0 + u * GL : x0;
+#pragma unroll
+          for (int sg = 0; sg < 2; ++sg) val[i][u][sg] = A[(io[i] + mp[i * E + (x | (sg << r.m))]) * RS];
+        }
+#pragma unroll
+      for (int u = 0; u < GEN_U; ++u)
+#pragma unroll
+        for (int sg = 0; sg < 2; ++sg) {
+          p[u][sg] = fv[sg] * p[u][sg];
+#pragma unroll
+          for (int i = 0; i < NIN; ++i) p[u][sg] *= val[i][u][sg];
+        }
+    } else {
+#pragma unroll
+      for (int u = 0; u < GEN_U; ++u) {
+        const int x = x0 + u * GL < M ? x0 + u * GL : x0;
+#pragma unroll
+        for (int sg = 0; sg < 2; ++sg) {
+          p[u][sg] = fv[sg] * p[u][sg];
+          for (int i = 0; i < r.nin; ++i) p[u][sg] *= A[(r.io[3 * i + 1] + mp[i * E + (x | (sg << r.m))]) * RS];
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < GEN_U; ++u) {
+      const int x = x0 + u * GL;
+      if (x >= M) continue;
+      const float ab = abx[u] * scl;
+#pragma unroll
+      for (int sg = 0; sg < 2; ++sg) {
+        const float g = ab * p[u][sg];
+        gb[(x | (sg << r.m)) * RS] = g;
+        gs = fmaf(g, sg ? -1.f : 1.f, gs);
+#pragma unroll
+        for (int j = 0; j < NPU; ++j)
+          if (j < np) gp[j] = fmaf(g, (((x >> pos[j]) & 1) == sg) ? 1.f : -1.f, gp[j]);
+      }
+    }
+  }
+}
+template <int NPU>
+__device__ __forceinline__ void step_g_any(const StepRec& r, const GenDev& G, const float (&fv)[2], const float* A,
+                                           const float* Ab, float* gb, int RS, int out, float scl, const int* pos,
+                                           int np, int lane, int GL, float& gs, float (&gp)[TNVAN_MAX_ELIM_W]) {
+  switch (r.nin) {  // the same for every lane
+    case 0: step_g<0, NPU>(r, G, fv, A, Ab, gb, RS, out, scl, pos, np, lane, GL, gs, gp); break;
+    case 1: step_g<1, NPU>(r, G, fv, A, Ab, gb, RS, out, scl, pos, np, lane, GL, gs, gp); break;
+    case 2: step_g<2, NPU>(r, G, fv, A, Ab, gb, RS, out, scl, pos, np, lane, GL, gs, gp); break;
+    default: step_g<-1, NPU>(r, G, fv, A, Ab, gb, RS, out, scl, pos, np, lane, GL, gs, gp); break;
+  }
 }
 
 __global__ void __launch_bounds__(128) general_dJ_kernel(const InstDev* __restrict__ inst,
@@ -382,32 +567,14 @@ __global__ void __launch_bounds__(128) general_dJ_kernel(const InstDev* __restri
     const int nsteps = H[0], fin = H[2];
     const int g0 = G.comp_step0[c];
     // forward: tables and their scales
+    const float fr[2] = {0.f, 0.f};
     for (int st = 0; st < nsteps; ++st) {
       const StepRec r = step_at(G, g0 + st);
       const float h = field_of(G, r.fb, r.fc, s);
       const float ah = fabsf(h);
       const float fv[2] = {expf(beta * (h - ah)), expf(beta * (-h - ah))};
-      const int M = 1 << r.m, E = 2 * M;
-      const float* pp = G.pp + r.ppo;
-      const unsigned short* mp = G.map + r.mo;
-      const int out = r.out_full;
-      float mx = 0.f;
-      for (int x = lane; x < M; x += GL) {
-        float accv = 0.f;
-        for (int sg = 0; sg < 2; ++sg) {
-          const int ext = x | (sg << r.m);
-          float pr = fv[sg] * pp[ext];
-          for (int i = 0; i < r.nin; ++i) pr *= A[(r.io[3 * i + 1] + mp[i * E + ext]) * RS];
-          accv += pr;
-        }
-        A[(out + x) * RS] = accv;
-        Ab[(out + x) * RS] = 0.f;
-        mx = fmaxf(mx, accv);
-      }
-      mx = group_max(mx, GL);
-      const float scl = pow2i(-exponent_of(mx));
-      for (int x = lane; x < M; x += GL) A[(out + x) * RS] *= scl;
-      if (lane == 0) sc[st * RS] = scl;
+      const int e = step_table_any<false, 1, true>(r, G, fv, fr, A, nullptr, Ab, RS, r.out_full, lane, GL);
+      if (lane == 0) sc[st * RS] = pow2i(-e);
       __syncwarp();
     }
     if (lane == 0) Ab[fin * RS] = 1.f / A[fin * RS];
@@ -418,10 +585,8 @@ __global__ void __launch_bounds__(128) general_dJ_kernel(const InstDev* __restri
       const float h = field_of(G, r.fb, r.fc, s);
       const float ah = fabsf(h);
       const float fv[2] = {expf(beta * (h - ah)), expf(beta * (-h - ah))};
-      const int M = 1 << r.m, E = 2 * M;
-      const float* pp = G.pp + r.ppo;
+      const int E = 2 << r.m;
       const unsigned short* mp = G.map + r.mo;
-      const int out = r.out_full;
       const float scl = sc[st * RS];
       constexpr int MW = TNVAN_MAX_ELIM_W;
       const int np = min(r.npair, MW);  // at most MW neighbours remain
@@ -432,20 +597,8 @@ __global__ void __launch_bounds__(128) general_dJ_kernel(const InstDev* __restri
       float gp[MW];         // sum g sigma_v sigma_u per pair
 #pragma unroll
       for (int j = 0; j < MW; ++j) gp[j] = 0.f;
-      for (int x = lane; x < M; x += GL) {
-        const float abx = Ab[(out + x) * RS] * scl;
-        for (int sg = 0; sg < 2; ++sg) {
-          const int ext = x | (sg << r.m);
-          float pr = fv[sg] * pp[ext];
-          for (int i = 0; i < r.nin; ++i) pr *= A[(r.io[3 * i + 1] + mp[i * E + ext]) * RS];
-          const float g = abx * pr;
-          gb[ext * RS] = g;
-          gs = fmaf(g, sg ? -1.f : 1.f, gs);
-#pragma unroll
-          for (int j = 0; j < MW; ++j)
-            if (j < np) gp[j] = fmaf(g, (((x >> pos[j]) & 1) == sg) ? 1.f : -1.f, gp[j]);
-        }
-      }
+      if (np <= 4) step_g_any<4>(r, G, fv, A, Ab, gb, RS, r.out_full, scl, pos, np, lane, GL, gs, gp);
+      else step_g_any<MW>(r, G, fv, A, Ab, gb, RS, r.out_full, scl, pos, np, lane, GL, gs, gp);
       __syncwarp();
       // input adjoints: each entry gathers the g of the extended indices that
       // read it (inverse map), lanes split the entries
@@ -453,18 +606,45 @@ __global__ void __launch_bounds__(128) general_dJ_kernel(const InstDev* __restri
         const int in = r.io[3 * i + 1], kk = r.io[3 * i + 2];
         const int R = E >> kk;
         const unsigned short* inv = mp + (r.nin + i) * E;
+#pragma unroll 2
         for (int e = lane; e < (1 << kk); e += GL) {
           const float av = A[(in + e) * RS];
-          if (av > 0.f) {
-            float sum = 0.f;
-            for (int f = 0; f < R; ++f) sum += gb[inv[e * R + f] * RS];
-            Ab[(in + e) * RS] += sum / av;
+          float sum = 0.f;
+          for (int f = 0; f + 4 <= R; f += 4) {  // in index order, four loads in flight
+            float q[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) q[j] = gb[inv[e * R + f + j] * RS];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) sum += q[j];
           }
+          if (R < 4)
+            for (int f = 0; f < R; ++f) sum += gb[inv[e * R + f] * RS];
+          if (av > 0.f) Ab[(in + e) * RS] += sum / av;
         }
       }
-      for (int f = r.fb; f < r.fb + r.fc; ++f)
-        acc_edge(acc_w, G.fld[2 * f + 1], wscale * gs * (float)s[G.fld[2 * f]], lane0);
-      for (int j = 0; j < np; ++j) acc_edge(acc_w, G.pairE[r.pr[2 * j]], wscale * gp[j], lane0);
+      for (int f0 = 0; f0 < r.fc; f0 += 4) {
+        int ee[4];
+        float v[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int f = r.fb + f0 + j;
+          ee[j] = f0 + j < r.fc ? G.fld[2 * f + 1] : -1;
+          v[j] = f0 + j < r.fc ? wscale * gs * (float)s[G.fld[2 * f]] : 0.f;
+        }
+        acc_edges(acc_w, ee, v, lane0);
+      }
+#pragma unroll
+      for (int j0 = 0; j0 < MW; j0 += 4) {
+        if (j0 >= np) break;
+        int ee[4];
+        float v[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          ee[j] = j0 + j < np ? G.pairE[r.pr[2 * (j0 + j)]] : -1;
+          v[j] = wscale * gp[j0 + j];
+        }
+        acc_edges(acc_w, ee, v, lane0);
+      }
       __syncwarp();
     }
   }
