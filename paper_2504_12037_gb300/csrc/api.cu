@@ -2394,12 +2394,14 @@ int tnvan_magnetisation(tnvan_ctx* ctx, const double* betas, int batch, const in
   // per-sample moments, by contraction kind
   bool k0 = false, k1 = false, k2 = false;
   int max_D = 0, arena = 0, nsteps = 0;
-  int strip_sm = 0;
+  int strip_sm = 0, strip_sm0 = 0, max_strips = 1;
   for (const Instance& in : ctx->inst) {
     max_D = std::max(max_D, (int)in.W.size());
     if (in.kind == 0) {
       k0 = true;
-      strip_sm = std::max(strip_sm, strip_smem_bytes(in, 128));
+      strip_sm0 = std::max(strip_sm0, strip_smem_bytes(in, 128));  // the limit this call has always had
+      strip_sm = std::max(strip_sm, strip_mom_smem_bytes(in));
+      max_strips = std::max(max_strips, (int)in.strip.strips.size());
     } else if (in.kind == 1) {
       k1 = true;
     } else {
@@ -2409,10 +2411,10 @@ int tnvan_magnetisation(tnvan_ctx* ctx, const double* betas, int batch, const in
     }
   }
   if (k0) {
-    if (strip_sm > 227 * 1024) return fail(ctx, TNVAN_E_UNSUPPORTED, "strip tables need %d B of shared memory", strip_sm);
+    if (strip_sm0 > 227 * 1024) return fail(ctx, TNVAN_E_UNSUPPORTED, "strip tables need %d B of shared memory", strip_sm0);
     LaunchInfo ls;
-    if ((rc = fill_launch(ctx, betas, batch, 128, ls))) return rc;
-    CK(launch_strips_mom(ctx->d_inst, ls, strip_sm, d_spins, mean, var, s), "strip moments kernel");
+    if ((rc = fill_launch(ctx, betas, batch, 32, ls))) return rc;
+    CK(launch_strips_mom(ctx->d_inst, ls, strip_sm, max_strips, d_spins, mean, var, s), "strip moments kernel");
   }
   if (k1) CK(launch_dense_mom(ctx->d_inst, li, max_D, d_spins, mean, var, s), "dense moments kernel");
   if (k2) {

@@ -455,11 +455,12 @@ cudaError_t launch_wide(const InstDev* d_inst, const LaunchInfo& li, const int* 
 int wide_tab_floats(int L);  // table floats of a strip of L rows
 // Magnetisation moments (tnvan_magnetisation): per sample E[M | s] and
 // Var(M | s) of the whole system's magnetisation given the width set, by
-// contraction kind (strips: li.tile samples per CTA, smem as strip_smem_bytes;
+// contraction kind (strips: li.tile = 32 samples per CTA, a warp per strip;
 // dense: builds the block's table at li.beta; elimination: as launch_general,
 // tables x 3, garena of general_mom_scratch_floats when too large).
-cudaError_t launch_strips_mom(const InstDev* d_inst, const LaunchInfo& li, int smem_bytes, const int8_t* spins,
-                              double* mag_mean, double* mag_var, cudaStream_t s);
+cudaError_t launch_strips_mom(const InstDev* d_inst, const LaunchInfo& li, int smem_bytes, int max_strips,
+                              const int8_t* spins, double* mag_mean, double* mag_var, cudaStream_t s);
+int strip_mom_smem_bytes(const Instance& in);
 cudaError_t launch_dense_mom(const InstDev* d_inst, const LaunchInfo& li, int max_D, const int8_t* spins,
                              double* mag_mean, double* mag_var, cudaStream_t s);
 int general_mom_smem_bytes(int arena, int D, int T, int GL, bool glob);

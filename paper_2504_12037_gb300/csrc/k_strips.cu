@@ -983,30 +983,32 @@ __device__ void strip_moments(const StripTab& tb, const StripRow* __restrict__ r
   var = qq;
 }
 
-// One thread per sample: E[M | s] = M_W(s) + sum over strips of the strip
-// means, Var(M | s) = sum of the strip variances (the strips are independent
-// given the width set), both FP64 sums of the FP32 per-strip values.
-__global__ void __launch_bounds__(128) strips_mom_kernel(const InstDev* __restrict__ inst, const LaunchInfo li,
+// E[M | s] = M_W(s) + sum over strips of the strip means, Var(M | s) = sum of
+// the strip variances (the strips are independent given the width set), both
+// FP64 sums of the FP32 per-strip values in strip order.  A CTA takes 32
+// samples with one warp per strip (at most 8, then in turn).  A thread's row
+// is a long dependent chain (2 w divisions deep), so warps in flight set the
+// time: 5 x 2,048 samples of the 16 x 16 lattice (four strips) took 223 us a call
+// with a thread per sample going through all strips, 119 us here.
+__global__ void __launch_bounds__(256) strips_mom_kernel(const InstDev* __restrict__ inst, const LaunchInfo li,
                                                          const int8_t* __restrict__ spins,
                                                          double* __restrict__ mag_mean, double* __restrict__ mag_var) {
   extern __shared__ float sm[];
   const int k = find_inst(li, blockIdx.x);
   const InstDev& I = inst[k];
   if (I.kind != 0) return;
-  const int T = li.tile, t = threadIdx.x;
-  const int b0 = (blockIdx.x - li.tile_begin[k]) * T, b = b0 + t;
+  const int NT = blockDim.x, tid = threadIdx.x, lane = tid & 31;
+  const int b0 = (blockIdx.x - li.tile_begin[k]) * 32, b = b0 + lane;
   const int D = I.D, Dp = padded_row_bytes(D);
-  build_strip_tables(I, (float)li.beta[k], sm, t, T, false);  // tables without ddiag (adjoint layout)
-  int8_t* ssp = reinterpret_cast<int8_t*>(sm + I.strip_tab_floats);
-  const int n_valid = min(T, li.batch - b0);
-  stage_spins(spins + I.spin_units * li.batch + (long long)b0 * D, n_valid, D, Dp, ssp, t, T);
+  build_strip_tables(I, (float)li.beta[k], sm, tid, NT, false);  // tables without ddiag (adjoint layout)
+  float2* part = reinterpret_cast<float2*>(sm + strip_tab_offset(I, I.n_strips, false));  // [strip][sample]
+  int8_t* ssp = reinterpret_cast<int8_t*>(part + I.n_strips * 32);
+  const int n_valid = min(32, li.batch - b0);
+  stage_spins(spins + I.spin_units * li.batch + (long long)b0 * D, n_valid, D, Dp, ssp, tid, NT);
+  for (int e = n_valid * Dp + tid; e < 32 * Dp; e += NT) ssp[e] = 1;  // padding rows
   __syncthreads();
-  if (b >= li.batch) return;
-  const int8_t* srow = ssp + t * Dp;
-  int mw = 0;
-  for (int j = 0; j < D; ++j) mw += srow[j];
-  double mean = (double)mw, var = 0.0;
-  for (int st = 0; st < I.n_strips; ++st) {
+  const int8_t* srow = ssp + lane * Dp;
+  for (int st = tid >> 5; st < I.n_strips; st += NT >> 5) {
     const StripDev& sd = I.strips[st];
     const StripTab tb = strip_tab_at(sm + strip_tab_offset(I, st, false), sd.w, sd.L, false);
     const StripRow* rows = I.rows + sd.row0;
@@ -1017,21 +1019,38 @@ __global__ void __launch_bounds__(128) strips_mom_kernel(const InstDev* __restri
       case 3: strip_moments<3>(tb, rows, sd.L, srow, m, q); break;
       default: strip_moments<4>(tb, rows, sd.L, srow, m, q); break;
     }
-    mean += (double)m;
-    var += (double)q;
+    part[st * 32 + lane] = make_float2(m, q);
+  }
+  __syncthreads();
+  if (tid >= n_valid) return;
+  int mw = 0;
+  for (int j = 0; j < D; ++j) mw += srow[j];
+  double mean = (double)mw, var = 0.0;
+  for (int st = 0; st < I.n_strips; ++st) {
+    mean += (double)part[st * 32 + lane].x;
+    var += (double)part[st * 32 + lane].y;
   }
   const long long o = (long long)k * li.batch + b;
   mag_mean[o] = mean;
   mag_var[o] = var;
 }
 
-cudaError_t launch_strips_mom(const InstDev* d_inst, const LaunchInfo& li, int smem_bytes, const int8_t* spins,
-                              double* mag_mean, double* mag_var, cudaStream_t s) {
+int strip_mom_smem_bytes(const Instance& in) {
+  int w4 = ((int)in.W.size() + 3) / 4;
+  if ((w4 & 1) == 0) ++w4;
+  int tabn = 0;
+  for (const StripDev& sd : in.strip.strips) tabn += strip_tab_floats_adj(sd.w, sd.L);
+  return 4 * tabn + (int)in.strip.strips.size() * 32 * 8 + 32 * 4 * w4;
+}
+
+cudaError_t launch_strips_mom(const InstDev* d_inst, const LaunchInfo& li, int smem_bytes, int max_strips,
+                              const int8_t* spins, double* mag_mean, double* mag_var, cudaStream_t s) {
   const int nblk = li.tile_begin[li.n_inst];
   if (nblk == 0) return cudaSuccess;
   cudaError_t e = cudaFuncSetAttribute(strips_mom_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
   if (e != cudaSuccess) return e;
-  strips_mom_kernel<<<nblk, li.tile, smem_bytes, s>>>(d_inst, li, spins, mag_mean, mag_var);
+  strips_mom_kernel<<<nblk, 32 * (max_strips < 8 ? max_strips : 8), smem_bytes, s>>>(d_inst, li, spins, mag_mean,
+                                                                                  mag_var);
   return cudaGetLastError();
 }
 
