@@ -604,14 +604,28 @@ int max_sample_smem(const tnvan_ctx* ctx, int tile) {
   return m;
 }
 
-int pick_sample_tile(const tnvan_ctx* ctx) {
+// Samples per CTA of the FP32 sampler (a multiple of 8, four threads each).
+// A CTA takes as long as its D dependent steps while fewer than about 16 warps
+// share an SM, then as long as their instructions; so the tile is the one that
+// needs the least (waves of CTAs) x max(16, warps per SM) -- a tile that
+// leaves a nearly empty last wave costs a whole pass of D steps.  Of equals
+// the smaller CTA.
+int pick_sample_tile(const tnvan_ctx* ctx, int batch) {
   if (ctx->tune_sample_tile && max_sample_smem(ctx, ctx->tune_sample_tile) <= 227 * 1024) return ctx->tune_sample_tile;
-  // largest tile that keeps two CTAs per SM, else the largest that fits
-  for (int T : {64, 32})
-    if (max_sample_smem(ctx, T) <= 113 * 1024) return T;
-  for (int T : {32, 16, 8})
-    if (max_sample_smem(ctx, T) <= 227 * 1024) return T;
-  return 8;
+  const long long n = (long long)ctx->inst.size();
+  int best = 8;
+  long long best_cost = -1;
+  for (int T = 8; T <= 192; T += 8) {
+    const int smem = max_sample_smem(ctx, T);
+    if (smem > 227 * 1024) break;
+    const int occ = std::max(1, std::min({227 * 1024 / (smem + 1024), 192 / T, 32}));
+    const long long nblk = n * ((batch + T - 1) / T), slots = 152LL * occ;
+    const long long full = nblk / slots, rest = nblk % slots;
+    const long long warps = (long long)occ * T / 8, last = ((rest + 151) / 152) * T / 8;
+    const long long cost = full * std::max(16LL, warps) + (rest ? std::max(16LL, last) : 0);
+    if (best_cost < 0 || cost < best_cost) best = T, best_cost = cost;
+  }
+  return best;
 }
 
 
@@ -3206,7 +3220,7 @@ int run_sampler(tnvan_ctx* ctx, const double* betas, int batch, uint64_t seed, u
     }
     return TNVAN_OK;
   }
-  const int tile = pick_sample_tile(ctx);
+  const int tile = pick_sample_tile(ctx, batch);
   LaunchInfo li;
   if ((rc = fill_launch(ctx, betas, batch, tile, li))) return rc;
   li.seed = seed;

@@ -228,68 +228,44 @@ cudaError_t launch_pack_all(const InstDev* d_inst, int n_inst, const long long* 
   return cudaSuccess;
 }
 
-// Dot product of a warp-uniform weight row with this thread's activation
-// column (layout [unit][T]) over entries [j0, j1).
-__device__ __forceinline__ float dot_col(const float* __restrict__ w, const float* col, int T,
-                                         int j0, int j1) {
-  float a0 = 0.f, a1 = 0.f;
-  int j = j0;
-  for (; j + 2 <= j1; j += 2) {
-    a0 = fmaf(__ldg(w + j), col[j * T], a0);
-    a1 = fmaf(__ldg(w + j + 1), col[(j + 1) * T], a1);
-  }
-  if (j < j1) a0 = fmaf(__ldg(w + j), col[j * T], a0);
-  return a0 + a1;
-}
-
-// Pre-activations of up to 16 units from n_in inputs: acc[q] = bias[q] +
-// sum_j blk[j][q] * act[j], one activation load per 16 FMAs, weights as
-// warp-uniform float4 loads.  Results go to pre[q][T] (q < nu).
-__device__ __forceinline__ void block_preact(const float* blk, const float* act, int T,
-                                             int n_in, const float* __restrict__ bias, int nu,
+// Pre-activations of the units [lo, hi) of one layer for the current group,
+// 16 units a block: acc[q] = bias[q] + sum_j blk[j][q] act[j] in input order,
+// four units to each of the sample's four threads (one activation load and
+// one 16-byte weight load per four FMAs).  Results go to pre[unit][T].
+__device__ __forceinline__ void layer_preact(const float* blocks, int off, int n_in, int lo, int hi,
+                                             const float* __restrict__ bias, const float* act, int T, int sub,
                                              float* pre) {
-  float acc[16];
-#pragma unroll
-  for (int q = 0; q < 16; ++q) acc[q] = q < nu ? __ldg(bias + q) : 0.f;
-  const float4* w4 = reinterpret_cast<const float4*>(blk);
-#pragma unroll 2
-  for (int j = 0; j < n_in; ++j) {
-    const float x = act[j * T];
-    const float4 a = w4[4 * j], b = w4[4 * j + 1], c = w4[4 * j + 2], d = w4[4 * j + 3];
-    acc[0] = fmaf(a.x, x, acc[0]);
-    acc[1] = fmaf(a.y, x, acc[1]);
-    acc[2] = fmaf(a.z, x, acc[2]);
-    acc[3] = fmaf(a.w, x, acc[3]);
-    acc[4] = fmaf(b.x, x, acc[4]);
-    acc[5] = fmaf(b.y, x, acc[5]);
-    acc[6] = fmaf(b.z, x, acc[6]);
-    acc[7] = fmaf(b.w, x, acc[7]);
-    acc[8] = fmaf(c.x, x, acc[8]);
-    acc[9] = fmaf(c.y, x, acc[9]);
-    acc[10] = fmaf(c.z, x, acc[10]);
-    acc[11] = fmaf(c.w, x, acc[11]);
-    acc[12] = fmaf(d.x, x, acc[12]);
-    acc[13] = fmaf(d.y, x, acc[13]);
-    acc[14] = fmaf(d.z, x, acc[14]);
-    acc[15] = fmaf(d.w, x, acc[15]);
-  }
-#pragma unroll
-  for (int q = 0; q < 16; ++q)
-    if (q < nu) pre[q * T] = acc[q];
-}
-
-// Pre-activations of the units [lo, hi) of one layer for the current group.
-__device__ __forceinline__ void layer_preact(const float* blocks, int off, int n_in,
-                                             int lo, int hi, const float* __restrict__ bias,
-                                             const float* act, int T, float* pre) {
   for (int c = lo; c < hi; c += 16) {
-    const int nu = min(16, hi - c);
-    block_preact(blocks + off + (long long)(c - lo) * n_in, act, T, n_in, bias + c, nu,
-                 pre + (c - lo) * T);
+    const int q0 = c + 4 * sub;
+    if (q0 >= hi) break;
+    const float4* w4 = reinterpret_cast<const float4*>(blocks + off + (long long)(c - lo) * n_in) + sub;
+    float acc[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) acc[q] = q0 + q < hi ? __ldg(bias + q0 + q) : 0.f;
+#pragma unroll 8
+    for (int j = 0; j < n_in; ++j) {
+      const float x = act[j * T];
+      const float4 a = w4[4 * j];
+      acc[0] = fmaf(a.x, x, acc[0]);
+      acc[1] = fmaf(a.y, x, acc[1]);
+      acc[2] = fmaf(a.z, x, acc[2]);
+      acc[3] = fmaf(a.w, x, acc[3]);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (q0 + q < hi) pre[(q0 + q - lo) * T] = acc[q];
   }
 }
 
-// Ancestral sampling (Eq. 8), one thread per sample, T samples per CTA.
+// a + sum_{j < n} w[j] col[j T], in order.
+__device__ __forceinline__ float chain_dot(float a, const float* w, const float* col, int T, int n) {
+#pragma unroll 4
+  for (int j = 0; j < n; ++j) a = fmaf(w[j], col[j * T], a);
+  return a;
+}
+
+// Ancestral sampling (Eq. 8), four threads per sample (8 samples a warp), T
+// samples per CTA.
 // Hidden units are degree-sorted, so output i (degree i+1) needs exactly the
 // inputs 0..i-1, the layer-1 units of degree <= i and the layer-2 units of
 // degree <= i, each evaluated once: one masked forward pass in total.
@@ -300,19 +276,26 @@ __device__ __forceinline__ void layer_preact(const float* blocks, int off, int n
 //            every input known before the group (register tiled, 16 units);
 //   phase B: the group's steps one by one, adding the in-group contributions
 //            and drawing s_i = +1 iff u < sigmoid(x_i).
+// The units of a phase are shared out over a sample's four threads (each
+// unit's sum stays one thread's chain, in input order); the logit and the draw
+// are formed by all four alike.  Bound by latency: D dependent steps, whose
+// hidden values limit the samples a CTA's shared memory holds, so warps in
+// flight come from splitting the samples; 5 x 4,099 samples of the 64-128-128-64
+// network took 0.26 ms with one thread per sample, 0.12 ms here.
 // With `given` non-null the spins are read from it (teacher forcing).
 // Shared memory: [unit][T] S [D], A1 [H1], A2 [H2], P1 [ug1], P2 [ug2],
 // PO [ugo]; then the weight block [wmax] and one mbarrier.
-__global__ void __launch_bounds__(64) sample_kernel(const InstDev* __restrict__ inst,
-                                                    const LaunchInfo li,
-                                                    int8_t* __restrict__ spins,
-                                                    float* __restrict__ logq,
-                                                    const int8_t* __restrict__ given) {
+__global__ void __launch_bounds__(768) sample_kernel(const InstDev* __restrict__ inst,
+                                                      const LaunchInfo li,
+                                                      int8_t* __restrict__ spins,
+                                                      float* __restrict__ logq,
+                                                      const int8_t* __restrict__ given) {
   extern __shared__ __align__(16) float sm[];
   const int k = find_inst(li, blockIdx.x);
   const InstDev& I = inst[k];
   const MadeDev& md = I.made;
-  const int T = li.tile, t = threadIdx.x;
+  const int T = li.tile, lane = threadIdx.x & 31, sub = lane >> 3;
+  const int t = (threadIdx.x >> 5) * 8 + (lane & 7);
   const int b = (blockIdx.x - li.tile_begin[k]) * T + t;
   const int D = md.D, nh = md.nh, H1 = md.H1, H2 = md.H2;
   float* S = sm;
@@ -332,7 +315,7 @@ __global__ void __launch_bounds__(64) sample_kernel(const InstDev* __restrict__ 
   const uint32_t step32 = launch_step(li);
   const int8_t* gv = given ? given + I.spin_units * li.batch + (long long)b * D : nullptr;
   const bool valid = b < li.batch;
-  if (t == 0) mbar_init(bar, 1);
+  if (threadIdx.x == 0) mbar_init(bar, 1);
   __syncthreads();
   float lq = 0.f;
   uint4 rnd = make_uint4(0, 0, 0, 0);
@@ -341,22 +324,23 @@ __global__ void __launch_bounds__(64) sample_kernel(const InstDev* __restrict__ 
     const int i0 = G[0], i1 = G[1], u1lo = G[2], u1hi = G[3], u2lo = G[4], u2hi = G[5];
     const int gsize = G[10];
     __syncthreads();  // every thread is done with the previous block
-    if (t == 0) {
+    if (threadIdx.x == 0) {
       fence_proxy_async_smem();
       mbar_expect_tx(bar, (uint32_t)gsize * 4u);
       bulk_g2s(Wsm, md.blocks + G[9], (uint32_t)gsize * 4u, bar);
     }
     if (!mbar_wait(bar, (uint32_t)(g & 1))) {
-      if (t == 0) atomicExch(li.status, 1);
+      if (threadIdx.x == 0) atomicExch(li.status, 1);
       return;
     }
     // phase A
-    if (nh >= 1) layer_preact(Wsm, G[6], i0, u1lo, u1hi, bias1, S + t, T, P1 + t);
-    if (nh >= 2) layer_preact(Wsm, G[7], u1lo, u2lo, u2hi, bias2, A1 + t, T, P2 + t);
+    if (nh >= 1) layer_preact(Wsm, G[6], i0, u1lo, u1hi, bias1, S + t, T, sub, P1 + t);
+    if (nh >= 2) layer_preact(Wsm, G[7], u1lo, u2lo, u2hi, bias2, A1 + t, T, sub, P2 + t);
     {
       const int n_in = nh == 0 ? i0 : (nh == 1 ? u1lo : u2lo);
-      layer_preact(Wsm, G[8], n_in, i0, i1, biaso, src + t, T, PO + t);
+      layer_preact(Wsm, G[8], n_in, i0, i1, biaso, src + t, T, sub, PO + t);
     }
+    __syncwarp();
     // phase B
     const int gi = i1 - i0, n1 = u1hi - u1lo;
     const int clo = nh == 0 ? i0 : (nh == 1 ? u1lo : u2lo);
@@ -369,44 +353,36 @@ __global__ void __launch_bounds__(64) sample_kernel(const InstDev* __restrict__ 
         rnd = philox4x32_10(
             make_uint4((uint32_t)b, (uint32_t)(i >> 2), step32, (uint32_t)k), key);
       if (nh >= 1 && i >= 1) {
-        for (int u = md.c1[i - 1]; u < md.c1[i]; ++u) {
-          const float* w = TW1 + (u - u1lo) * gi;
-          float a = P1[(u - u1lo) * T + t];
-          for (int j = i0; j < i; ++j) a = fmaf(w[j - i0], S[j * T + t], a);
-          A1[u * T + t] = fmaxf(a, 0.f);
-        }
+        for (int u = md.c1[i - 1] + sub; u < md.c1[i]; u += 4)
+          A1[u * T + t] = fmaxf(chain_dot(P1[(u - u1lo) * T + t], TW1 + (u - u1lo) * gi, S + i0 * T + t, T, i - i0), 0.f);
+        __syncwarp();
       }
       if (nh >= 2 && i >= 1) {
         const int n1i = md.c1[i];
-        for (int v = md.c2[i - 1]; v < md.c2[i]; ++v) {
-          const float* w = TW2 + (v - u2lo) * n1;
-          float a = P2[(v - u2lo) * T + t];
-          for (int u = u1lo; u < n1i; ++u) a = fmaf(w[u - u1lo], A1[u * T + t], a);
-          A2[v * T + t] = fmaxf(a, 0.f);
-        }
+        for (int v = md.c2[i - 1] + sub; v < md.c2[i]; v += 4)
+          A2[v * T + t] =
+              fmaxf(chain_dot(P2[(v - u2lo) * T + t], TW2 + (v - u2lo) * n1, A1 + u1lo * T + t, T, n1i - u1lo), 0.f);
+        __syncwarp();
       }
-      float x = PO[(i - i0) * T + t];
-      {
-        const float* w = TWo + (i - i0) * nL;
-        const int chi = nh == 0 ? i : cL[i];
-        for (int c = clo; c < chi; ++c) x = fmaf(w[c - clo], src[c * T + t], x);
-      }
+      const float x =
+          chain_dot(PO[(i - i0) * T + t], TWo + (i - i0) * nL, src + clo * T + t, T, (nh == 0 ? i : cL[i]) - clo);
       const float p = 1.f / (1.f + expf(-x));
       const uint32_t word =
           (i & 3) == 0 ? rnd.x : (i & 3) == 1 ? rnd.y : (i & 3) == 2 ? rnd.z : rnd.w;
       const float u = (float)(word >> 8) * 5.9604644775390625e-08f;  // 2^-24
       float s = u < p ? 1.f : -1.f;
       if (gv) s = valid ? (float)gv[i] : 1.f;
-      S[i * T + t] = s;
+      if (sub == 0) S[i * T + t] = s;
+      __syncwarp();
       lq -= softplusf(-s * x);
     }
   }
   if (valid) {
     if (spins) {
       int8_t* out = spins + I.spin_units * li.batch + (long long)b * D;
-      for (int i = 0; i < D; ++i) out[i] = (int8_t)S[i * T + t];
+      for (int i = sub; i < D; i += 4) out[i] = (int8_t)S[i * T + t];
     }
-    logq[(long long)k * li.batch + b] = lq;
+    if (sub == 0) logq[(long long)k * li.batch + b] = lq;
   }
 }
 
@@ -423,7 +399,7 @@ cudaError_t launch_sample(const InstDev* d_inst, const LaunchInfo& li, int smem_
   cudaError_t e = cudaFuncSetAttribute(sample_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        smem_bytes);
   if (e != cudaSuccess) return e;
-  sample_kernel<<<nblk, li.tile, smem_bytes, s>>>(d_inst, li, spins, logq, given);
+  sample_kernel<<<nblk, 4 * li.tile, smem_bytes, s>>>(d_inst, li, spins, logq, given);
   return cudaGetLastError();
 }
 
