@@ -259,14 +259,134 @@ __device__ __forceinline__ void slot_group(const int* G, const float* TWb, int g
 #undef TNVAN_SLOT_STEP
 }
 
+// One step of a full group in the slot form, in registers alone (see
+// slot_group_full); given: the step's spin is s_in, else u decides it.
+template <int U, int Q, bool GIVEN>
+__device__ __forceinline__ void full_step(const float* TW1, const float* TW2, const float* TWo, const float* B1,
+                                          const float* B2, const float* BO, const uint32_t (&r1)[8 * U],
+                                          const uint32_t (&r2)[8 * U], const uint32_t (&ro)[8], float (&h1)[8 * U],
+                                          float (&h2)[8 * U], float (&sg)[8], float u, uint32_t& gbits, float& lq) {
+  constexpr int S = 8 * U;
+#pragma unroll
+  for (int a = 0; a < U; ++a) {
+    const int r = Q * U + a;
+    h1[r] = bf16_round(fmaxf(slot_dot<Q, 8>(TW1 + r * 8, sg, __uint_as_float(r1[r]) + B1[r]), 0.f));
+  }
+#pragma unroll
+  for (int a = 0; a < U; ++a) {
+    const int r = Q * U + a;
+    h2[r] = bf16_round(fmaxf(slot_dot<(Q + 1) * U, S>(TW2 + r * S, h1, __uint_as_float(r2[r]) + B2[r]), 0.f));
+  }
+  const float x = slot_dot<(Q + 1) * U, S>(TWo + Q * S, h2, __uint_as_float(ro[Q]) + BO[Q]);
+  const float ex = __expf(-fabsf(x));
+  if (!GIVEN) {
+    const float rcp = __frcp_rn(1.f + ex);
+    const float pr = x >= 0.f ? rcp : ex * rcp;
+    const bool up = u < pr;
+    sg[Q] = up ? 1.f : -1.f;
+    gbits |= (up ? 1u : 0u) << Q;
+  }
+  lq -= fmaxf(-sg[Q] * x, 0.f) + __logf(1.f + ex);
+}
+
+// A full group of 8 steps in the slot form (i0 a multiple of 4): the same
+// arithmetic as slot_group, every sum in the same order, as one branch-free
+// run of register arithmetic.  The steps are a chain (a step's spin enters the
+// next steps' hidden units), but most of a step's products only need earlier
+// steps' values: with no branch and no shared-memory store between the steps
+// (fold tiles, spin tile and random words are written before or after), the
+// weights' loads and those products are scheduled under the chain's own
+// latency.  338 us for the 64-instance workload (65,536 samples, 2 x 128
+// units) with a branch and stores per step, 271 us here; log q of 3 x 5,003 given
+// configurations of 256 spins 182 and 105 us.
+template <int U, bool GIVEN>
+__device__ __forceinline__ void slot_group_full(const int* G, const float* TWb, int i0, int w1, int w2, uint32_t tP1,
+                                                uint32_t tP2, uint32_t tPO, bool p1ok, bool init2, bool inito,
+                                                unsigned char* sH1, unsigned char* sH2, unsigned char* sS, uint32_t rb1,
+                                                uint32_t rb2, uint32_t rbS, int b, uint32_t step32, int k, uint2 key,
+                                                const int8_t* gv, bool valid, SlotState& st) {
+  constexpr int S = 8 * U;
+  uint32_t r1[S], r2[S], ro[8];
+#pragma unroll
+  for (int j = 0; j < S; ++j) r1[j] = r2[j] = 0u;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) ro[q] = 0u;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const int ua = G[13 + q], nu = G[14 + q] - ua, va = G[22 + q], nv = G[23 + q] - va;
+#pragma unroll
+    for (int a = 0; a < U; ++a) {
+      if (p1ok && a < nu) tmem_ld1_nowait(tP1 + (uint32_t)(ua + a - w1), r1[q * U + a]);
+      if (init2 && a < nv) tmem_ld1_nowait(tP2 + (uint32_t)(va + a), r2[q * U + a]);
+    }
+    if (inito) tmem_ld1_nowait(tPO + (uint32_t)(i0 + q), ro[q]);
+  }
+  // the group's random numbers, or its given spins
+  float u[8], sg[8];
+  if (GIVEN) {
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      sg[q] = !valid || gv[i0 + q] > 0 ? 1.f : -1.f;
+      st.gbits |= (sg[q] > 0.f ? 1u : 0u) << q;
+      u[q] = 0.f;
+    }
+  } else {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const uint4 rnd = philox4x32_10(make_uint4((uint32_t)b, (uint32_t)((i0 >> 2) + h), step32, (uint32_t)k), key);
+      u[4 * h] = (float)(rnd.x >> 8) * 5.9604644775390625e-08f;
+      u[4 * h + 1] = (float)(rnd.y >> 8) * 5.9604644775390625e-08f;
+      u[4 * h + 2] = (float)(rnd.z >> 8) * 5.9604644775390625e-08f;
+      u[4 * h + 3] = (float)(rnd.w >> 8) * 5.9604644775390625e-08f;
+    }
+  }
+  tmem_wait_all();
+#pragma unroll
+  for (int j = 0; j < S; ++j) {
+    tie(r1[j]);
+    tie(r2[j]);
+  }
+#pragma unroll
+  for (int q = 0; q < 8; ++q) tie(ro[q]);
+  const float* TW2 = TWb + G[8];
+  const float* TWo = TWb + G[9];
+  const float* B1 = TWb + G[10];
+  const float* B2 = TWb + G[11];
+  const float* BO = TWb + G[12];
+  float h1[S], h2[S];
+#define TNVAN_FULL_STEP(QQ) \
+  full_step<U, QQ, GIVEN>(TWb, TW2, TWo, B1, B2, BO, r1, r2, ro, h1, h2, sg, u[QQ], st.gbits, st.lq);
+  TNVAN_FULL_STEP(0)
+  TNVAN_FULL_STEP(1)
+  TNVAN_FULL_STEP(2)
+  TNVAN_FULL_STEP(3)
+  TNVAN_FULL_STEP(4)
+  TNVAN_FULL_STEP(5)
+  TNVAN_FULL_STEP(6)
+  TNVAN_FULL_STEP(7)
+#undef TNVAN_FULL_STEP
+  // fold tiles and spin tile
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const int ua = G[13 + q], nu = G[14 + q] - ua, va = G[22 + q], nv = G[23 + q] - va;
+#pragma unroll
+    for (int a = 0; a < U; ++a) {
+      if (a < nu) st_bf16(sH1, rb1 + 16u * (uint32_t)(ua - w1 + a), h1[q * U + a]);
+      if (a < nv) st_bf16(sH2, rb2 + 16u * (uint32_t)(va - w2 + a), h2[q * U + a]);
+    }
+    st_bf16(sS, rbS + 16u * (uint32_t)(i0 + q), sg[q]);
+  }
+}
+
 __host__ __device__ inline int sample_tcg_tmem_cols(int D, int H2, int tcw1) {
   D = (D + 15) & ~15;
   return tcw1 + H2 + D <= 256 ? 256 : 512;
 }
 
 // ANY_STREAMED: some instance of the launch streams its weights (the
-// resident-only instantiation carries none of that code).
-template <bool ANY_STREAMED>
+// resident-only instantiation carries none of that code).  GIVEN: log q of
+// the configurations `given` (teacher forcing) instead of drawing.
+template <bool ANY_STREAMED, bool GIVEN>
 __global__ void __launch_bounds__(128, 2) sample_tcg_kernel(const InstDev* __restrict__ inst,
                                                            const LaunchInfo li, const TcgOrder ord, int plan,
                                                            int8_t* __restrict__ spins, float* __restrict__ logq,
@@ -371,7 +491,7 @@ __global__ void __launch_bounds__(128, 2) sample_tcg_kernel(const InstDev* __res
   const uint32_t id2 = tc::idesc(128, H2, 1u) | idA, ido = tc::idesc(128, Dp, 1u) | idA;
   const uint2 key = make_uint2((uint32_t)li.seed, (uint32_t)(li.seed >> 32));
   const uint32_t step32 = launch_step(li);
-  const int8_t* gv = given ? given + I.spin_units * li.batch + (long long)b * D : nullptr;
+  const int8_t* gv = GIVEN ? given + I.spin_units * li.batch + (long long)b * D : nullptr;
   uint32_t phase = 0;
   bool ok = true;
   bool p1ok = false, init2 = false, inito = false;  // accumulator holds data
@@ -574,7 +694,14 @@ __global__ void __launch_bounds__(128, 2) sample_tcg_kernel(const InstDev* __res
       }
     } else {
       SlotState st{rnd, 0u, lq};
-      if (P.slot_u == 2)
+#define TNVAN_FULL_GROUP(UU)                                                                                       \
+  slot_group_full<UU, GIVEN>(G, TWb, i0, w1, w2, tP1, tP2, tPO, p1ok, init2, inito, sH1, sH2, sS, rb1, rb2, rbS, b, \
+                             step32, k, key, gv, valid, st)
+      if (gi == 8 && (i0 & 3) == 0) {
+        if (P.slot_u == 2) TNVAN_FULL_GROUP(2);
+        else if (P.slot_u == 3) TNVAN_FULL_GROUP(3);
+        else TNVAN_FULL_GROUP(4);
+      } else if (P.slot_u == 2)
         slot_group<2>(G, TWb, gi, i0, w1, w2, tP1, tP2, tPO, p1ok, init2, inito, sH1, sH2, sS, rb1, rb2, rbS, b,
                       step32, k, key, gv, valid, st);
       else if (P.slot_u == 3)
@@ -583,6 +710,7 @@ __global__ void __launch_bounds__(128, 2) sample_tcg_kernel(const InstDev* __res
       else
         slot_group<4>(G, TWb, gi, i0, w1, w2, tP1, tP2, tPO, p1ok, init2, inito, sH1, sH2, sS, rb1, rb2, rbS, b,
                       step32, k, key, gv, valid, st);
+#undef TNVAN_FULL_GROUP
       rnd = st.rnd;
       lq = st.lq;
       // the group's spin bits (at most 8, from bit i0) into the 128-bit mask
@@ -658,7 +786,7 @@ __global__ void __launch_bounds__(128, 2) sample_tcg_kernel(const InstDev* __res
     if (t == 0) atomicExch(li.status, 4);
   }
   if (ok && valid) {
-    if (spins) {
+    if (!GIVEN && spins) {
       int8_t* row = spins + I.spin_units * li.batch + (long long)b * D;
       // rows of more than 128 spins: from the spin tile
       auto up_at = [&](int ii) {
@@ -700,7 +828,8 @@ cudaError_t launch_sample_tcg(const InstDev* d_inst, const LaunchInfo& li, const
   if (blk_end < 0) blk_end = li.tile_begin[li.n_inst];
   const int nblk = blk_end - blk_begin;
   if (nblk <= 0) return cudaSuccess;
-  auto kern = streamed ? sample_tcg_kernel<true> : sample_tcg_kernel<false>;
+  auto kern = given ? (streamed ? sample_tcg_kernel<true, true> : sample_tcg_kernel<false, true>)
+                    : (streamed ? sample_tcg_kernel<true, false> : sample_tcg_kernel<false, false>);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
   if (e != cudaSuccess) return e;
   LaunchInfo lc = li;
