@@ -1,5 +1,6 @@
 // Reduction to F_q / log Z_IS (Eq. 9), the gradient's reduction over partial
 // rows and the Adam update (Algorithm 1 step (d)).
+#include <limits.h>
 #include <math.h>
 
 #include "common.cuh"
@@ -186,9 +187,10 @@ __device__ __forceinline__ FF ff_from_double(double x) {
 }
 __device__ __forceinline__ double ff_to_double(FF x) { return (double)x.hi + (double)x.lo; }
 
-// s1, s2: float-float sums of l - K and (l - K)^2; m, se: the maximum of the
-// importance weights' logs and the sum of exp(l - m), in FP64 (Eq. 9's log Z_IS
-// is a logsumexp of the l_b, kept in FP64 throughout).
+// s1, s2: float-float sums of l - K and (l - K)^2; se: the sum of exp(l - e ln 2)
+// in FP64, e an integer (m, once a chunk's sums are written) near its largest
+// l / ln 2 (Eq. 9's log Z_IS is a logsumexp of the l_b, kept in FP64
+// throughout).
 struct TupleFF {
   int n, bad;
   FF s1, s2;
@@ -213,27 +215,45 @@ __device__ __forceinline__ TupleFF ld_tuple_ff(const double* slot) {
   return TupleFF{__ldcg(q), __ldcg(q + 1), FF{__ldcg(f + 2), __ldcg(f + 3)}, FF{__ldcg(f + 4), __ldcg(f + 5)},
                  __ldcg(slot + 3), __ldcg(slot + 4)};
 }
-// Block-wide reductions over the 256 threads (8 warps); `red` holds 8 values.
-__device__ __forceinline__ double block_max(double v, double* red) {
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  double r = red[0];
-  for (int w = 1; w < 8; ++w) r = fmax(r, red[w]);
-  __syncthreads();
-  return r;
+// Floats as integers of the same order (and back).
+__device__ __forceinline__ int ordered(float f) {
+  const int i = __float_as_int(f);
+  return i ^ ((i >> 31) & 0x7FFFFFFF);
+}
+__device__ __forceinline__ float from_ordered(int i) { return __int_as_float(i ^ ((i >> 31) & 0x7FFFFFFF)); }
+
+// Sums of two lanes' tuples against the same maximum.
+__device__ __forceinline__ void add_lane(TupleFF& r, int o) {
+  r.n += __shfl_xor_sync(0xffffffffu, r.n, o);
+  r.bad += __shfl_xor_sync(0xffffffffu, r.bad, o);
+  r.s1 = ff_add(r.s1, shfl_ff(r.s1, o));
+  r.s2 = ff_add(r.s2, shfl_ff(r.s2, o));
+  r.se += __shfl_xor_sync(0xffffffffu, r.se, o);
 }
 
-// Each CTA reduces a chunk in two passes over its samples: the chunk's
-// largest l first (compares only), then per sample one FP64 exp(l - max) and
-// the float-float moment sums; the CTA's warps are summed in a fixed order.
-// The last CTA of an instance rescales the n_part (<= 64) chunk sums to the
-// instance's largest l, one FP64 exp per chunk in parallel lanes, and adds
-// them in a fixed tree, so the result does not depend on which CTA finishes
-// last.  Only two exps lie on any thread's path: FP64 is a narrow unit on
-// this part, and a running maximum with a rescale at every merge would put
-// one exp per merge level on the critical path.
-__global__ void __launch_bounds__(256) reduce_kernel(const LaunchInfo li, int n_part, const double* __restrict__ logZR,
+// ln 2 times an integer, the exponent of the exponentials' common scale
+// (formed the same way wherever a scale is taken off again).
+__device__ __forceinline__ double scale_log(int e) { return (double)e * 0.69314718055994530942; }
+
+// Each CTA (64 to 256 threads) reduces a chunk in two passes over its samples:
+// the chunk's largest l first (in FP32: it only picks a power of two 2^e near
+// exp(max l)), then per sample one FP64 exp(l - e ln 2) and the float-float
+// moment sums, merged over lanes and warps by a fixed tree.  The last CTA of an
+// instance takes the n_part (<= 64) chunk sums to the largest e -- an exact
+// power of two each -- and adds them in a fixed tree, so the result does not
+// depend on which CTA finishes last.  Bound by a chain of latencies (loads, one
+// exp, about ten float-float additions, the hand-over between CTAs, one log):
+// FP64 is a narrow unit on this part, so small batches are spread over CTAs of
+// 64 samples, maxima are integer warp reductions, chunks are rescaled without
+// exponentials, and what depends on the batch size alone (its log, reciprocals)
+// comes from the host.  1,024 samples: 14.8 us with FP64 maxima, an exp per
+// chunk and one thread merging the warps, 11 us here (3 x 4,096: 15.1 and
+// 11).
+struct BatchConsts {  // of n samples: 1 / n, 1 / (n - 1) (0 for n = 1), ln n, 1 / sqrt n
+  double inv_n, inv_n1, ln_n, rsqrt_n;
+};
+__global__ void __launch_bounds__(256) reduce_kernel(const LaunchInfo li, int n_part, const BatchConsts bc,
+                                                     const double* __restrict__ logZR,
                                                      const float* __restrict__ logq, double* __restrict__ part,
                                                      double* __restrict__ stats, int* __restrict__ counters,
                                                      int k0) {
@@ -245,18 +265,27 @@ __global__ void __launch_bounds__(256) reduce_kernel(const LaunchInfo li, int n_
   const FF negK = ff_neg(K);
   const int chunk = (B + n_part - 1) / n_part;
   const int lo = p * chunk, hi = min(B, lo + chunk);
-  __shared__ double redd[8];
+  const int l = threadIdx.x & 31, nw = blockDim.x >> 5;
+  __shared__ int redi[8];
   __shared__ TupleFF red[8];
   __shared__ int last;
   // pass 1: the chunk's largest finite l
-  double mx = -INFINITY;
+  float mf = -INFINITY;
   for (int b = lo + threadIdx.x; b < hi; b += blockDim.x) {
     const double ld = logZR[base + b] - (double)logq[base + b];
-    if (isfinite(ld)) mx = fmax(mx, ld);
+    if (isfinite(ld)) mf = fmaxf(mf, (float)ld);
   }
-  mx = block_max(mx, redd);
-  // pass 2: exp sums against that maximum, moment sums, counts
-  TupleFF acc = {0, 0, {0.f, 0.f}, {0.f, 0.f}, mx, 0.0};
+  int mi = __reduce_max_sync(0xffffffffu, ordered(mf));
+  if (l == 0) redi[threadIdx.x >> 5] = mi;
+  __syncthreads();
+  mi = redi[0];
+  for (int w = 1; w < nw; ++w) mi = max(mi, redi[w]);
+  // no finite l: any scale (the sums stay zero)
+  const float top = from_ordered(mi);
+  const int e2 = top > -INFINITY ? (int)fminf(fmaxf(ceilf(top * 1.44269504f), -1e9f), 1e9f) : 0;
+  const double mx = scale_log(e2);
+  // pass 2: exp sums at that scale, moment sums, counts
+  TupleFF acc = {0, 0, {0.f, 0.f}, {0.f, 0.f}, 0.0, 0.0};
   for (int b = lo + threadIdx.x; b < hi; b += blockDim.x) {
     const double z = logZR[base + b];
     const float q = logq[base + b];
@@ -271,69 +300,65 @@ __global__ void __launch_bounds__(256) reduce_kernel(const LaunchInfo li, int n_
     acc.se += exp(ld - mx);
     acc.n += 1;
   }
-  for (int o = 16; o > 0; o >>= 1) {
-    acc.n += __shfl_xor_sync(0xffffffffu, acc.n, o);
-    acc.bad += __shfl_xor_sync(0xffffffffu, acc.bad, o);
-    acc.s1 = ff_add(acc.s1, shfl_ff(acc.s1, o));
-    acc.s2 = ff_add(acc.s2, shfl_ff(acc.s2, o));
-    acc.se += __shfl_xor_sync(0xffffffffu, acc.se, o);
-  }
-  const int l = threadIdx.x & 31;
+  for (int o = 16; o > 0; o >>= 1) add_lane(acc, o);
   if (l == 0) red[threadIdx.x >> 5] = acc;
   __syncthreads();
-  if (threadIdx.x == 0) {  // the CTA's warps in order
-    TupleFF r = red[0];
-    for (int w = 1; w < 8; ++w) {
-      r.n += red[w].n;
-      r.bad += red[w].bad;
-      r.s1 = ff_add(r.s1, red[w].s1);
-      r.s2 = ff_add(r.s2, red[w].s2);
-      r.se += red[w].se;
+  if (threadIdx.x < 32) {
+    TupleFF r = red[l < nw ? l : 0];
+    if (l >= nw) r = TupleFF{0, 0, {0.f, 0.f}, {0.f, 0.f}, 0.0, 0.0};
+    for (int o = 4; o > 0; o >>= 1) add_lane(r, o);
+    if (l == 0) {
+      r.m = (double)e2;
+      st_tuple_ff(part + ((long long)k * n_part + p) * 6, r);
+      __threadfence();
+      last = atomicAdd(counters + k, 1) == n_part - 1;
     }
-    st_tuple_ff(part + ((long long)k * n_part + p) * 6, r);
-    __threadfence();
-    last = atomicAdd(counters + k, 1) == n_part - 1;
   }
   __syncthreads();
   if (!last || threadIdx.x >= 32) return;
+  const double inv_beta = 1.0 / li.beta[k];
   __threadfence();
   // the instance's chunks: lane l holds chunks l and l + 32
-  TupleFF r = {0, 0, {0.f, 0.f}, {0.f, 0.f}, -INFINITY, 0.0};
+  TupleFF r = {0, 0, {0.f, 0.f}, {0.f, 0.f}, 0.0, 0.0};
   TupleFF r2 = r;
   if (l < n_part) r = ld_tuple_ff(part + ((long long)k * n_part + l) * 6);
   if (l + 32 < n_part) r2 = ld_tuple_ff(part + ((long long)k * n_part + l + 32) * 6);
-  double M = fmax(r.n ? r.m : -INFINITY, r2.n ? r2.m : -INFINITY);
-  for (int o = 16; o > 0; o >>= 1) M = fmax(M, __shfl_xor_sync(0xffffffffu, M, o));
-  double se = (r.n ? r.se * exp(r.m - M) : 0.0) + (r2.n ? r2.se * exp(r2.m - M) : 0.0);
-  int n_ = r.n + r2.n, bad_ = r.bad + r2.bad;
-  FF s1 = ff_add(r.s1, r2.s1), s2 = ff_add(r.s2, r2.s2);
-  for (int o = 16; o > 0; o >>= 1) {
-    n_ += __shfl_xor_sync(0xffffffffu, n_, o);
-    bad_ += __shfl_xor_sync(0xffffffffu, bad_, o);
-    s1 = ff_add(s1, shfl_ff(s1, o));
-    s2 = ff_add(s2, shfl_ff(s2, o));
-    se += __shfl_xor_sync(0xffffffffu, se, o);
+  const int ea = r.n ? (int)r.m : INT_MIN, eb = r2.n ? (int)r2.m : INT_MIN;
+  const int E = __reduce_max_sync(0xffffffffu, max(ea, eb));
+  r.se = r.n ? scalbn(r.se, max(ea - E, -2000)) : 0.0;
+  if (n_part > 32) {
+    r.se += r2.n ? scalbn(r2.se, max(eb - E, -2000)) : 0.0;
+    r.n += r2.n;
+    r.bad += r2.bad;
+    r.s1 = ff_add(r.s1, r2.s1);
+    r.s2 = ff_add(r.s2, r2.s2);
   }
-  // FP64 statistics; the transcendental tails in parallel lanes
-  const double beta = li.beta[k];
+  for (int o = 16; o > 0; o >>= 1) add_lane(r, o);
+  const int n_ = r.n, bad_ = r.bad;
+  // FP64 statistics
+  double inv_n = bc.inv_n, inv_n1 = bc.inv_n1, ln_n = bc.ln_n, rsqrt_n = bc.rsqrt_n;
   const double n = (double)n_;
-  const double s1d = ff_to_double(s1), s2d = ff_to_double(s2);
-  const double mean_d = s1d / n;
-  const double var = n_ > 1 ? fmax(s2d - s1d * mean_d, 0.0) / (n - 1.0) : 0.0;
-  double f = 0.0;
-  if (l == 1) f = log(se);
-  else if (l == 2) f = log(n);
-  else if (l == 3) f = sqrt(var);
-  else if (l == 4) f = sqrt(n);
-  const double lse = __shfl_sync(0xffffffffu, f, 1), ln_n = __shfl_sync(0xffffffffu, f, 2);
-  const double sd = __shfl_sync(0xffffffffu, f, 3), sn = __shfl_sync(0xffffffffu, f, 4);
+  if (bad_) {  // some l_b left out
+    inv_n = 1.0 / n;
+    inv_n1 = n_ > 1 ? 1.0 / (n - 1.0) : 0.0;
+    ln_n = log(n);
+    rsqrt_n = 1.0 / sqrt(n);
+  }
+  const double s1d = ff_to_double(r.s1), s2d = ff_to_double(r.s2);
+  const double mean_d = s1d * inv_n;
+  const double var = fmax(s2d - s1d * mean_d, 0.0) * inv_n1;
+  double f = l == 0 ? r.se : var;  // log of one lane's value, square root of the others'
+  if (l == 0) f = log(f);
+  else f = sqrt(f);
+  const double sd = __shfl_sync(0xffffffffu, f, 1);
   if (l != 0) return;
-  const double mean = ff_to_double(K) + mean_d;
-  const double lz = M + lse - ln_n;
+  const double nan = __longlong_as_double(0x7FF8000000000000ll);
+  const double mean = n_ ? ff_to_double(K) + mean_d : nan;
+  const double lz = n_ ? scale_log(E) + f - ln_n : nan;
   double* st = stats + 8 * k;
-  st[0] = -mean / beta;
-  st[1] = -lz / beta;
-  st[2] = sd / (beta * sn);
+  st[0] = -mean * inv_beta;
+  st[1] = -lz * inv_beta;
+  st[2] = sd * inv_beta * rsqrt_n;
   st[3] = lz;
   st[4] = mean;
   st[5] = (double)bad_;
@@ -346,13 +371,17 @@ cudaError_t launch_reduce(const InstDev*, const LaunchInfo& li, const double* lo
                           const float* logq, double* stats, int* counters, cudaStream_t s, int k0, int k1) {
   if (k1 < 0) k1 = li.n_inst;
   if (k1 <= k0) return cudaSuccess;
-  // n_part: chunks of >= 256 samples, at most 64 per instance
-  int n_part = (li.batch + 255) / 256;
+  // chunks of >= 64 samples, at most 64 per instance; a thread per sample up to 256
+  int n_part = (li.batch + 63) / 64;
   if (n_part > 64) n_part = 64;
   if (n_part < 1) n_part = 1;
+  const int chunk = (li.batch + n_part - 1) / n_part;
+  const int threads = chunk <= 64 ? 64 : (chunk <= 128 ? 128 : 256);
   // partial tuples live right after the stats block
   double* part = stats + 8 * TNVAN_MAX_INST;
-  reduce_kernel<<<dim3(n_part, k1 - k0), 256, 0, s>>>(li, n_part, logZR, logq, part, stats, counters, k0);
+  const double n = li.batch;
+  const BatchConsts bc = {1.0 / n, n > 1.0 ? 1.0 / (n - 1.0) : 0.0, log(n), 1.0 / sqrt(n)};
+  reduce_kernel<<<dim3(n_part, k1 - k0), threads, 0, s>>>(li, n_part, bc, logZR, logq, part, stats, counters, k0);
   return cudaGetLastError();
 }
 
