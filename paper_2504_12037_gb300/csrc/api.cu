@@ -805,7 +805,7 @@ size_t chain_ws_elems(const tnvan_ctx* ctx, int batch, ChainWs* cw) {
   for (size_t k = 0; k < ctx->inst.size(); ++k) {
     const Instance& in = ctx->inst[k];
     if (cw) cw->off[k] = (long long)off;
-    off += 2 * (size_t)batch * (((in.W.size() + 7) & ~size_t(7)) + ((in.H[0] + 7) & ~7) + ((in.H[1] + 7) & ~7));
+    off += (size_t)((batch + 127) / 128) * ChainTile((int)in.W.size(), in.H[0], in.H[1]).elems;
   }
   return off;
 }
@@ -837,7 +837,7 @@ bool plan_bwd_chain(const tnvan_ctx* ctx, Skip skip, int* ns, int* max_n, int* s
 // gradients (bias gradients ride along as an extra column of ones).
 int backward_tc(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* d_spins,
                 const double* d_logZR, const float* d_logq, bool bf16, int part_stride,
-                cudaStream_t s, bool skip_fused) {
+                cudaStream_t s, bool skip_fused, int* splits_out) {
   int rc;
   const int n = (int)ctx->inst.size();
   // instances the fused backward handles in the same call are left out
@@ -945,9 +945,26 @@ int backward_tc(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* d_
       if (!skip(k)) acc += (batch + 127) / 128;
     }
     lc.tile_begin[n] = acc;
-    PROF("bwd_chain", s);
-    CK(launch_bwd_chain(ctx->d_inst, lc, cw, ns, max_n, smem, d_spins, d_logZR, d_logq, ctx->d_stats, s),
-       "backward chain kernel");
+    {
+      PROF("bwd_chain", s);
+      CK(launch_bwd_chain(ctx->d_inst, lc, cw, ns, max_n, smem, d_spins, d_logZR, d_logq, ctx->d_stats, s),
+         "backward chain kernel");
+    }
+    // weight gradients: one wave of CTAs (128 rows of a weight matrix and a
+    // slice of the batch each), every slice at least one tile of 128 samples
+    acc = 0;
+    for (int k = 0; k < n; ++k) {
+      lc.tile_begin[k] = acc;
+      const MadeDev& md = ctx->inst[k].dev.made;
+      for (int l = 0; l <= md.nh && !skip(k); ++l) acc += (md.layer[l].nout + 127) / 128;
+    }
+    lc.tile_begin[n] = acc;
+    const int occ = std::max(1, std::min(227 * 1024 / (chain_wgrad_smem_bytes(max_n) + 1024), 512 / std::max(32, 2 * max_n)));
+    *splits_out = std::max(1, std::min({TC_SPLITS, (batch + 127) / 128, 152 * occ / std::max(acc, 1)}));
+    PROF("gemm_wgrad", s);
+    CK(launch_chain_wgrad(ctx->d_inst, lc, cw, *splits_out, max_n, ctx->d_grad_packed, part_stride, s),
+       "weight gradient kernel");
+    return TNVAN_OK;
   } else {
     // stage 1: A1 = relu(S W1^T + b1)
     for (int k = 0; k < n; ++k) {
@@ -1025,7 +1042,7 @@ int backward_tc(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* d_
     if ((rc = flush("gemm_bwd_h1"))) return rc;
   }
   // stage 6: weight gradients, split over the batch into TC_SPLITS partial slices
-  splits = std::max(1, std::min(TC_SPLITS, (batch + 127) / 128));
+  splits = *splits_out;
   float* part = ctx->d_grad_packed;
   for (int k = 0; k < n; ++k) {
     if (skip(k)) continue;
@@ -1034,15 +1051,8 @@ int backward_tc(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* d_
     float* pk = part + (long long)k * splits * part_stride;
     for (int l = 0; l <= md.nh; ++l) {
       const LayerDev& L = md.layer[l];
-      GemmOperand del, act;
-      if (chain) {
-        const ChainRows r = chain_rows(cw, k, batch, md.D, md.H1, md.H2);
-        del = l == md.nh ? op(r.X, 1, r.ldD, GT_BF16) : (l == 1 ? op(r.dA2, 1, r.ld2, GT_BF16) : op(r.dA1, 1, r.ld1, GT_BF16));
-        act = l == 0 ? op(r.S, 1, r.ldD, GT_BF16) : (l == 1 ? op(r.A1, 1, r.ld1, GT_BF16) : op(r.A2, 1, r.ld2, GT_BF16));
-      } else {
-        del = op(l == md.nh ? bf[k].dX : (l == 1 ? bf[k].dA2 : bf[k].dA1), 1, L.nout, IT);
-        act = l == 0 ? spin_op(k, true) : op(l == 1 ? bf[k].A1 : bf[k].A2, 1, L.nin, IT);
-      }
+      const GemmOperand del = op(l == md.nh ? bf[k].dX : (l == 1 ? bf[k].dA2 : bf[k].dA1), 1, L.nout, IT);
+      const GemmOperand act = l == 0 ? spin_op(k, true) : op(l == 1 ? bf[k].A1 : bf[k].A2, 1, L.nin, IT);
       for (int n0 = 0; n0 < L.nin; n0 += 128) {
         const bool last = n0 + 128 >= L.nin;
         const int nn = (L.nin + 1 <= 256) ? L.nin : std::min(128, L.nin - n0);
@@ -1382,6 +1392,18 @@ int tnvan_set_made(tnvan_ctx* ctx, int instance, int n_hidden, const int32_t* wi
     if (e2 != cudaSuccess) return fail(ctx, TNVAN_E_NOMEM, "cudaMalloc(weight tiles): %s", cudaGetErrorString(e2));
     in.dev_allocs.push_back(wt);
     md.wtiles = static_cast<uint16_t*>(wt);
+  }
+  md.ctiles = nullptr;
+  if (std::max({D, H[0], H[1]}) <= 256) {  // the backward chain's limit
+    size_t n = 0;
+    for (int l = 0; l <= n_hidden; ++l)
+      n += (size_t)((md.layer[l].nout + 15) & ~15) * ((md.layer[l].nin + 15) & ~15);
+    void* ct = nullptr;
+    cudaError_t e2 = cudaMalloc(&ct, n * sizeof(uint16_t));
+    if (e2 == cudaSuccess) e2 = cudaMemset(ct, 0, n * sizeof(uint16_t));  // the padding stays zero
+    if (e2 != cudaSuccess) return fail(ctx, TNVAN_E_NOMEM, "cudaMalloc(weight tiles): %s", cudaGetErrorString(e2));
+    in.dev_allocs.push_back(ct);
+    md.ctiles = static_cast<uint16_t*>(ct);
   }
   md.c1 = dbuf + o_c1;
   md.c2 = dbuf + o_c2;
@@ -2136,7 +2158,8 @@ int tnvan_train_step(tnvan_ctx* ctx, const double* betas, int batch, uint64_t se
     any_fused = any_fused || in.dev.made.fused_ok;
   }
   any_fused = any_fused && precision == TNVAN_BF16;  // the fused backward reads the BF16 tiles
-  if ((rc = pack_network(ctx, sampler_pack_mask(ctx, precision) | PACK_FLAT | (any_fused ? PACK_TILES : 0), s)))
+  if ((rc = pack_network(ctx, sampler_pack_mask(ctx, precision) | PACK_FLAT | (any_fused ? PACK_TILES : 0) |
+                                  (precision == TNVAN_BF16 && !all_fused ? PACK_CHAIN : 0), s)))
     return rc;
   // the overlapped schedule runs each chunk's Eq. 9 reduction (statistics
   // and the backward's baseline) behind its adjoint, and the d/dJ reduction (it reads only the adjoint's partial
@@ -2498,7 +2521,9 @@ int backward_impl(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* 
     any_fused = any_fused || in.dev.made.fused_ok;
   }
   any_fused = any_fused && precision == TNVAN_BF16;
-  if (pack && (rc = pack_network(ctx, PACK_FLAT | (any_fused ? PACK_TILES : 0), s))) return rc;
+  if (pack && (rc = pack_network(ctx, PACK_FLAT | (any_fused ? PACK_TILES : 0) |
+                                         (precision == TNVAN_BF16 && !all_fused ? PACK_CHAIN : 0), s)))
+    return rc;
   if (!stats_ready) {
     PROF("reduce", s);
     CK(launch_reduce(ctx->d_inst, li, d_logZR, d_logq, ctx->d_stats, ctx->d_status + 4, s), "reduce kernel");
@@ -2526,10 +2551,10 @@ int backward_impl(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* 
   // GEMM chain or (tuned, where faster) the FP32 SIMT backward
   const bool simt = precision == TNVAN_FP32 || (!all_fused && ctx->tune_bwd_form == 2);
   if (!all_fused && !simt) {
-    const int splits = std::max(1, std::min(TC_SPLITS, (batch + 127) / 128));
+    int splits = std::max(1, std::min(TC_SPLITS, (batch + 127) / 128));
     if ((rc = ensure_grad_ws(ctx, (size_t)splits * ctx->inst.size() * (size_t)max_elems))) return rc;
     if ((rc = backward_tc(ctx, betas, batch, d_spins, d_logZR, d_logq, precision == TNVAN_BF16,
-                          (int)max_elems, s, any_fused)))
+                          (int)max_elems, s, any_fused, &splits)))
       return rc;
     LaunchInfo lr;
     if ((rc = fill_launch(ctx, betas, batch, 1, lr))) return rc;

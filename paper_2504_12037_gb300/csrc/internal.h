@@ -122,6 +122,7 @@ struct MadeDev {
   long long n_blk;
   int fused_ok;           // eligible for the fused BF16 tcgen05 backward
   int sample_tc_ok;       // eligible for the BF16 tcgen05 sampler
+  uint16_t* ctiles;       // BF16 K-major tiles of every layer, [r16(nout)][r16(nin)] each (the backward chain; padding zero)
   uint16_t* wtiles;       // BF16 K-major tiles W1 [H1 x D] | W2 [H2 x H1] | Wo [D x H2] (fused kernels)
   long long n_params;     // size of the natural layout
   long long param_off;    // offset in the all-instances packed gradient layout
@@ -401,7 +402,7 @@ struct tnvan_ctx {
 namespace tnvan {
 
 // Kernel launchers (defined in the .cu files).  All return a cudaError_t.
-enum { PACK_FLAT = 1, PACK_TILES = 2, PACK_SIMT = 4, PACK_TC = 8, PACK_TCG = 16 };
+enum { PACK_FLAT = 1, PACK_TILES = 2, PACK_SIMT = 4, PACK_TC = 8, PACK_TCG = 16, PACK_CHAIN = 32 };
 __host__ __device__ long long pack_elems(const MadeDev& md, int mask);
 cudaError_t launch_pack_all(const InstDev* d_inst, int n_inst, const long long* counts, int mask, cudaStream_t s);
 cudaError_t launch_sample(const InstDev* d_inst, const LaunchInfo& li, int smem_bytes,
@@ -521,36 +522,40 @@ cudaError_t launch_grad_reduce(const InstDev* d_inst, const LaunchInfo& li,
 // s16 != nullptr: also the spins as BF16 rows of r8(D) (the GEMM chain's operand)
 cudaError_t launch_reinforce_w(const InstDev* d_inst, const LaunchInfo& li, const double* logZR, const float* logq,
                                const double* stats, float* w, const int8_t* spins, uint16_t* s16, cudaStream_t s);
-// BF16 backward chain (k_bwd_chain.cu): row-major BF16 rows of every sample in
-// global memory, instance k's six arrays back to back at base + off[k].
+// BF16 backward chain (k_bwd_chain.cu): per 128 samples one block of BF16 tiles
+// in global memory, instance k's blocks back to back at base + off[k].
 struct ChainWs {
   uint16_t* base;
   long long off[TNVAN_MAX_INST];
 };
-struct ChainRows {
-  uint16_t *S, *A1, *A2, *X, *dA2, *dA1;
-  int ldD, ld1, ld2;  // row lengths: the widths rounded up to 8, zeros beyond
+// Element offsets of a block's tiles, each [128 samples][width rounded up to
+// 16] in K-major core matrices of 8 samples x 8 units (zeros past the width
+// and the batch).
+struct ChainTile {
+  int S, A1, A2, X, dA2, dA1, elems;
+  __host__ __device__ ChainTile(int D, int H1, int H2) {
+    const int d = 128 * ((D + 15) & ~15), a = 128 * ((H1 + 15) & ~15), b = 128 * ((H2 + 15) & ~15);
+    S = 0;
+    A1 = S + d;
+    A2 = A1 + a;
+    X = A2 + b;
+    dA2 = X + d;
+    dA1 = dA2 + b;
+    elems = dA1 + a;
+  }
 };
-__host__ __device__ inline ChainRows chain_rows(const ChainWs& w, int k, int batch, int D, int H1, int H2) {
-  ChainRows r;
-  r.ldD = (D + 7) & ~7;
-  r.ld1 = (H1 + 7) & ~7;
-  r.ld2 = (H2 + 7) & ~7;
-  const long long B = batch;
-  r.S = w.base + w.off[k];
-  r.A1 = r.S + B * r.ldD;
-  r.A2 = r.A1 + B * r.ld1;
-  r.X = r.A2 + B * r.ld2;
-  r.dA2 = r.X + B * r.ldD;
-  r.dA1 = r.dA2 + B * r.ld2;
-  return r;
-}
 int bwd_chain_smem_bytes(int D, int H1, int H2, int max_n, int ns);
 // li: tiles of 128 samples; ns weight stages in the ring (2 to 4); max_n: the
 // widest layer or width set (at most 256).
 cudaError_t launch_bwd_chain(const InstDev* d_inst, const LaunchInfo& li, const ChainWs& cw, int ns, int max_n,
                              int smem_bytes, const int8_t* spins, const double* logZR, const float* logq,
                              const double* stats, cudaStream_t s);
+// Weight and bias gradients from the chain's tiles: li.tile_begin counts the
+// instances' 128-row blocks of weight matrices; slice z of instance k into
+// partial row k * splits + z.
+cudaError_t launch_chain_wgrad(const InstDev* d_inst, const LaunchInfo& li, const ChainWs& cw, int splits, int max_n,
+                               float* partials, long long part_stride, cudaStream_t s);
+int chain_wgrad_smem_bytes(int max_n);
 cudaError_t launch_bwd_fused(const InstDev* d_inst, const LaunchInfo& li, int smem_bytes,
                              const int8_t* spins, const double* logZR, const float* logq,
                              const double* stats, float* partials, long long part_stride, int* status,

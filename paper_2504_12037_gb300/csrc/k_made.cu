@@ -60,6 +60,7 @@ __device__ __forceinline__ void store_tile(const MadeDev& md, int l, int r, int 
 //              entry, so the tiles need no segment of their own
 //   PACK_TILES BF16 tiles in the tensor cores' canonical K-major layout (no
 //              swizzle): W1 [H1 x D], W2 [H2 x H1], Wo [D x H2]
+//   PACK_CHAIN (with PACK_FLAT) BF16 tiles of every layer for the backward chain
 //   PACK_SIMT  the blocked SIMT sampler's weight blocks
 //   PACK_TCG   the grouped tensor-core sampler plans' triangle tiles (one
 //              plan, or all, per pack_tc_plan)
@@ -75,6 +76,21 @@ __device__ __forceinline__ void pack_one(const MadeDev& md, int mask, long long 
         uint32_t u = __float_as_uint(v);
         u += 0x7fffu + ((u >> 16) & 1u);  // round to nearest even
         md.packed16[e] = (uint16_t)(u >> 16);
+        if ((mask & PACK_CHAIN) && md.ctiles) {
+          int j = (int)e, off = 0;
+          for (int l = 0; l < md.n_layers; ++l) {
+            const LayerDev& L = md.layer[l];
+            const int nw = L.nout * L.nin, cp = (L.nin + 15) & ~15;
+            if (j < nw) {
+              const int r = j / L.nin, c = j - r * L.nin;
+              md.ctiles[off + (r >> 3) * cp * 8 + (c >> 3) * 64 + (r & 7) * 8 + (c & 7)] = (uint16_t)(u >> 16);
+              break;
+            }
+            off += ((L.nout + 15) & ~15) * cp;
+            j -= nw + L.nout;
+            if (j < 0) break;  // a bias
+          }
+        }
       }
       if (tiles) {  // weights of layer l at [dst_off, dst_off + nout * nin), row-major
         int j = (int)e;
