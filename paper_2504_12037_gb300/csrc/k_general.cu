@@ -41,6 +41,13 @@ struct StepRec {
   const int* pr;  // n_pair x (pair id, position of the neighbour in the out scope)
 };
 
+// What a sweep needs of a step: sizes, offsets (out and in[] live or full) and
+// the sample's field on the eliminated spin; f the record's place in fprog.
+struct Step {
+  int m, nin, ppo, mo, out, in[3], f;
+  float h;
+};
+
 __device__ __forceinline__ StepRec step_at(const GenDev& G, int g) {
   const int* F = G.fprog + G.fstep[g];
   StepRec r;
@@ -63,6 +70,45 @@ __device__ __forceinline__ float field_of(const GenDev& G, int fb, int fc, const
   float h = 0.f;
   for (int f = fb; f < fb + fc; ++f) h = fmaf(G.fldJ[f], (float)s[G.fld[2 * f]], h);
   return h;
+}
+
+// The next GL steps of a sweep, one per lane of the group: their records and
+// fields are chains of dependent loads, walked by the lanes in parallel once
+// per GL steps and handed out by shuffles.  COL: 0 live, 1 full offsets.
+struct StepBlock {
+  int pk, ppo, mo, out, in0, in1, in2, f;
+  float h;
+};
+template <int COL>
+__device__ __forceinline__ StepBlock load_block(const GenDev& G, int g, const int8_t* s) {
+  StepBlock b;
+  b.f = G.fstep[g];
+  const int* F = G.fprog + b.f;
+  const int nin = F[3];
+  b.pk = F[0] | (nin << 8);
+  b.ppo = F[5];
+  b.mo = F[6];
+  b.out = F[7 + COL];
+  b.in0 = nin > 0 ? F[9 + COL] : 0;
+  b.in1 = nin > 1 ? F[12 + COL] : 0;
+  b.in2 = nin > 2 ? F[15 + COL] : 0;
+  b.h = field_of(G, F[1], F[2], s);
+  return b;
+}
+__device__ __forceinline__ Step block_step(const StepBlock& b, int j, int GL) {
+  Step r;
+  const int pk = __shfl_sync(0xffffffffu, b.pk, j, GL);
+  r.m = pk & 255;
+  r.nin = pk >> 8;
+  r.ppo = __shfl_sync(0xffffffffu, b.ppo, j, GL);
+  r.mo = __shfl_sync(0xffffffffu, b.mo, j, GL);
+  r.out = __shfl_sync(0xffffffffu, b.out, j, GL);
+  r.in[0] = __shfl_sync(0xffffffffu, b.in0, j, GL);
+  r.in[1] = __shfl_sync(0xffffffffu, b.in1, j, GL);
+  r.in[2] = __shfl_sync(0xffffffffu, b.in2, j, GL);
+  r.f = __shfl_sync(0xffffffffu, b.f, j, GL);
+  r.h = __shfl_sync(0xffffffffu, b.h, j, GL);
+  return r;
 }
 
 // Bond products of every step at this call's beta: one CTA per (step,
@@ -123,22 +169,21 @@ __device__ __forceinline__ float group_max(float v, int GL) {
 // read and a write).
 #define GEN_U 4
 template <bool DB, int NIN, int COL, bool ZERO>
-__device__ __forceinline__ int step_table(const StepRec& r, const GenDev& G, const float (&fv)[2], const float (&fr)[2],
-                                          float* A, float* dA, float* Ab, int RS, int out, int lane, int GL) {
+__device__ __forceinline__ int step_table(const Step& r, const GenDev& G, const float (&fv)[2], const float (&fr)[2],
+                                          float* A, float* dA, float* Ab, int RS, int lane, int GL) {
+  constexpr int U = DB && NIN >= 3 ? GEN_U / 2 : GEN_U;  // within 128 registers
+  const int out = r.out;
   const int M = 1 << r.m, E = 2 * M;
   const float* pp = G.pp + r.ppo;
   const float* pd = G.pp + G.n_pp + r.ppo;
   const unsigned short* mp = G.map + r.mo;
-  const bool regs = M <= GL * GEN_U;
-  int io[NIN > 0 ? NIN : 1];
-#pragma unroll
-  for (int i = 0; i < NIN; ++i) io[i] = r.io[3 * i + COL];
-  float av[GEN_U], dv[GEN_U];
+  const bool regs = M <= GL * U;
+  float av[U], dv[U];
   float mx = 0.f;
-  for (int x0 = lane; x0 < M; x0 += GL * GEN_U) {
-    float p[GEN_U][2], rr[GEN_U][2];
+  for (int x0 = lane; x0 < M; x0 += GL * U) {
+    float p[U][2], rr[U][2];
 #pragma unroll
-    for (int u = 0; u < GEN_U; ++u) {
+    for (int u = 0; u < U; ++u) {
       const int x = x0 + u * GL < M ? x0 + u * GL : x0;
 #pragma unroll
       for (int sg = 0; sg < 2; ++sg) {
@@ -147,21 +192,21 @@ __device__ __forceinline__ int step_table(const StepRec& r, const GenDev& G, con
       }
     }
     if constexpr (NIN >= 0) {
-      float val[NIN > 0 ? NIN : 1][GEN_U][2], dval[NIN > 0 ? NIN : 1][GEN_U][2];
+      float val[NIN > 0 ? NIN : 1][U][2], dval[NIN > 0 ? NIN : 1][U][2];
 #pragma unroll
       for (int i = 0; i < NIN; ++i)
 #pragma unroll
-        for (int u = 0; u < GEN_U; ++u) {
+        for (int u = 0; u < U; ++u) {
           const int x = x0 + u * GL < M ? x0 + u * GL : x0;
 #pragma unroll
           for (int sg = 0; sg < 2; ++sg) {
-            const int q = (io[i] + mp[i * E + (x | (sg << r.m))]) * RS;
+            const int q = (r.in[i] + mp[i * E + (x | (sg << r.m))]) * RS;
             val[i][u][sg] = A[q];
             if (DB) dval[i][u][sg] = dA[q];
           }
         }
 #pragma unroll
-      for (int u = 0; u < GEN_U; ++u)
+      for (int u = 0; u < U; ++u)
 #pragma unroll
         for (int sg = 0; sg < 2; ++sg) {
           p[u][sg] = fv[sg] * p[u][sg];
@@ -174,14 +219,14 @@ __device__ __forceinline__ int step_table(const StepRec& r, const GenDev& G, con
         }
     } else {
 #pragma unroll
-      for (int u = 0; u < GEN_U; ++u) {
+      for (int u = 0; u < U; ++u) {
         const int x = x0 + u * GL < M ? x0 + u * GL : x0;
 #pragma unroll
         for (int sg = 0; sg < 2; ++sg) {
           p[u][sg] = fv[sg] * p[u][sg];
           if (DB) rr[u][sg] = fr[sg] + rr[u][sg];
           for (int i = 0; i < r.nin; ++i) {
-            const int q = (r.io[3 * i + COL] + mp[i * E + (x | (sg << r.m))]) * RS;
+            const int q = (G.fprog[r.f + 9 + 3 * i + COL] + mp[i * E + (x | (sg << r.m))]) * RS;
             const float v = A[q];
             p[u][sg] *= v;
             if (DB) rr[u][sg] += dA[q] / v;
@@ -190,7 +235,7 @@ __device__ __forceinline__ int step_table(const StepRec& r, const GenDev& G, con
       }
     }
 #pragma unroll
-    for (int u = 0; u < GEN_U; ++u) {
+    for (int u = 0; u < U; ++u) {
       const int x = x0 + u * GL;
       av[u] = __fadd_rn(p[u][0], p[u][1]);  // the products' own rounding: not contracted into the last one
       if (DB) dv[u] = fmaf(p[u][1], rr[u][1], p[u][0] * rr[u][0]);
@@ -207,7 +252,7 @@ __device__ __forceinline__ int step_table(const StepRec& r, const GenDev& G, con
   const float sc = pow2i(-e);
   if (regs) {
 #pragma unroll
-    for (int u = 0; u < GEN_U; ++u) {
+    for (int u = 0; u < U; ++u) {
       const int x = lane + u * GL;
       if (x >= M) continue;
       A[(out + x) * RS] = av[u] * sc;
@@ -226,15 +271,15 @@ __device__ __forceinline__ int step_table(const StepRec& r, const GenDev& G, con
 }
 
 template <bool DB, int COL, bool ZERO>
-__device__ __forceinline__ int step_table_any(const StepRec& r, const GenDev& G, const float (&fv)[2],
-                                              const float (&fr)[2], float* A, float* dA, float* Ab, int RS, int out,
-                                              int lane, int GL) {
+__device__ __forceinline__ int step_table_any(const Step& r, const GenDev& G, const float (&fv)[2],
+                                              const float (&fr)[2], float* A, float* dA, float* Ab, int RS, int lane,
+                                              int GL) {
   switch (r.nin) {  // the same for every lane
-    case 0: return step_table<DB, 0, COL, ZERO>(r, G, fv, fr, A, dA, Ab, RS, out, lane, GL);
-    case 1: return step_table<DB, 1, COL, ZERO>(r, G, fv, fr, A, dA, Ab, RS, out, lane, GL);
-    case 2: return step_table<DB, 2, COL, ZERO>(r, G, fv, fr, A, dA, Ab, RS, out, lane, GL);
-    case 3: return step_table<DB, 3, COL, ZERO>(r, G, fv, fr, A, dA, Ab, RS, out, lane, GL);
-    default: return step_table<DB, -1, COL, ZERO>(r, G, fv, fr, A, dA, Ab, RS, out, lane, GL);
+    case 0: return step_table<DB, 0, COL, ZERO>(r, G, fv, fr, A, dA, Ab, RS, lane, GL);
+    case 1: return step_table<DB, 1, COL, ZERO>(r, G, fv, fr, A, dA, Ab, RS, lane, GL);
+    case 2: return step_table<DB, 2, COL, ZERO>(r, G, fv, fr, A, dA, Ab, RS, lane, GL);
+    case 3: return step_table<DB, 3, COL, ZERO>(r, G, fv, fr, A, dA, Ab, RS, lane, GL);
+    default: return step_table<DB, -1, COL, ZERO>(r, G, fv, fr, A, dA, Ab, RS, lane, GL);
   }
 }
 
@@ -252,12 +297,12 @@ __device__ __forceinline__ void run_component(const GenDev& G, int c, const int8
   // both added to the FP64 result once per component
   int esum = 0;
   float hs = 0.f, hc = 0.f;
-  // the next step's record and field are read ahead of this step's tables
-  StepRec r = nsteps > 0 ? step_at(G, g0) : StepRec{};
-  float h = nsteps > 0 ? field_of(G, r.fb, r.fc, s) : 0.f;
+  StepBlock blk;
   for (int st = 0; st < nsteps; ++st) {
-    const StepRec rn = step_at(G, g0 + (st + 1 < nsteps ? st + 1 : st));
-    const float ah = fabsf(h);
+    const int j = st & (GL - 1);
+    if (j == 0) blk = load_block<0>(G, g0 + min(st + lane, nsteps - 1), s);
+    const Step r = block_step(blk, j, GL);
+    const float h = r.h, ah = fabsf(h);
     {
       const float y = ah - hc;
       const float t2 = hs + y;
@@ -266,10 +311,7 @@ __device__ __forceinline__ void run_component(const GenDev& G, int c, const int8
     }
     const float fv[2] = {expf(beta * (h - ah)), expf(beta * (-h - ah))};
     const float fr[2] = {h - ah, -h - ah};
-    const float hn = field_of(G, rn.fb, rn.fc, s);
-    esum += step_table_any<DB, 0, false>(r, G, fv, fr, A, dA, nullptr, RS, r.out_live, lane, GL);
-    r = rn;
-    h = hn;
+    esum += step_table_any<DB, 0, false>(r, G, fv, fr, A, dA, nullptr, RS, lane, GL);
     __syncwarp();
   }
   if (lane == 0) {
@@ -297,7 +339,7 @@ __device__ __forceinline__ void stage_spins(int8_t* ssp, const int8_t* gsp, int 
 
 // li.tile = samples per CTA (S); blockDim.x = S * GL.
 template <bool DB>
-__global__ void __launch_bounds__(128) general_kernel(const InstDev* __restrict__ inst,
+__global__ void __launch_bounds__(128, 4) general_kernel(const InstDev* __restrict__ inst,
                                                       const LaunchInfo li, int arena_floats, int GL,
                                                       const int8_t* __restrict__ spins,
                                                       double* __restrict__ logZR,
@@ -448,15 +490,13 @@ __device__ __forceinline__ void acc_edges(float* acc_w, const int (&e)[4], float
 // sums with sigma (gs) and with sigma sigma_u of the first NPU bonds (gp), in
 // the order of x; loads GEN_U entries at a time.
 template <int NIN, int NPU>
-__device__ __forceinline__ void step_g(const StepRec& r, const GenDev& G, const float (&fv)[2], const float* A,
-                                       const float* Ab, float* gb, int RS, int out, float scl, const int* pos, int np,
+__device__ __forceinline__ void step_g(const Step& r, const GenDev& G, const float (&fv)[2], const float* A,
+                                       const float* Ab, float* gb, int RS, float scl, const int* pos, int np,
                                        int lane, int GL, float& gs, float (&gp)[TNVAN_MAX_ELIM_W]) {
+  const int out = r.out;
   const int M = 1 << r.m, E = 2 * M;
   const float* pp = G.pp + r.ppo;
   const unsigned short* mp = G.map + r.mo;
-  int io[NIN > 0 ? NIN : 1];
-#pragma unroll
-  for (int i = 0; i < NIN; ++i) io[i] = r.io[3 * i + 1];
   for (int x0 = lane; x0 < M; x0 += GL * GEN_U) {
     float p[GEN_U][2], abx[GEN_U];
 #pragma unroll
@@ -474,7 +514,7 @@ __device__ __forceinline__ void step_g(const StepRec& r, const GenDev& G, const 
         for (int u = 0; u < GEN_U; ++u) {
           const int x = x0 + u * GL < M ? x0 + u * GL : x0;
 #pragma unroll
-          for (int sg = 0; sg < 2; ++sg) val[i][u][sg] = A[(io[i] + mp[i * E + (x | (sg << r.m))]) * RS];
+          for (int sg = 0; sg < 2; ++sg) val[i][u][sg] = A[(r.in[i] + mp[i * E + (x | (sg << r.m))]) * RS];
         }
 #pragma unroll
       for (int u = 0; u < GEN_U; ++u)
@@ -491,7 +531,7 @@ __device__ __forceinline__ void step_g(const StepRec& r, const GenDev& G, const 
 #pragma unroll
         for (int sg = 0; sg < 2; ++sg) {
           p[u][sg] = fv[sg] * p[u][sg];
-          for (int i = 0; i < r.nin; ++i) p[u][sg] *= A[(r.io[3 * i + 1] + mp[i * E + (x | (sg << r.m))]) * RS];
+          for (int i = 0; i < r.nin; ++i) p[u][sg] *= A[(G.fprog[r.f + 9 + 3 * i + 1] + mp[i * E + (x | (sg << r.m))]) * RS];
         }
       }
     }
@@ -513,18 +553,18 @@ __device__ __forceinline__ void step_g(const StepRec& r, const GenDev& G, const 
   }
 }
 template <int NPU>
-__device__ __forceinline__ void step_g_any(const StepRec& r, const GenDev& G, const float (&fv)[2], const float* A,
-                                           const float* Ab, float* gb, int RS, int out, float scl, const int* pos,
-                                           int np, int lane, int GL, float& gs, float (&gp)[TNVAN_MAX_ELIM_W]) {
+__device__ __forceinline__ void step_g_any(const Step& r, const GenDev& G, const float (&fv)[2], const float* A,
+                                           const float* Ab, float* gb, int RS, float scl, const int* pos, int np,
+                                           int lane, int GL, float& gs, float (&gp)[TNVAN_MAX_ELIM_W]) {
   switch (r.nin) {  // the same for every lane
-    case 0: step_g<0, NPU>(r, G, fv, A, Ab, gb, RS, out, scl, pos, np, lane, GL, gs, gp); break;
-    case 1: step_g<1, NPU>(r, G, fv, A, Ab, gb, RS, out, scl, pos, np, lane, GL, gs, gp); break;
-    case 2: step_g<2, NPU>(r, G, fv, A, Ab, gb, RS, out, scl, pos, np, lane, GL, gs, gp); break;
-    default: step_g<-1, NPU>(r, G, fv, A, Ab, gb, RS, out, scl, pos, np, lane, GL, gs, gp); break;
+    case 0: step_g<0, NPU>(r, G, fv, A, Ab, gb, RS, scl, pos, np, lane, GL, gs, gp); break;
+    case 1: step_g<1, NPU>(r, G, fv, A, Ab, gb, RS, scl, pos, np, lane, GL, gs, gp); break;
+    case 2: step_g<2, NPU>(r, G, fv, A, Ab, gb, RS, scl, pos, np, lane, GL, gs, gp); break;
+    default: step_g<-1, NPU>(r, G, fv, A, Ab, gb, RS, scl, pos, np, lane, GL, gs, gp); break;
   }
 }
 
-__global__ void __launch_bounds__(128) general_dJ_kernel(const InstDev* __restrict__ inst,
+__global__ void __launch_bounds__(128, 4) general_dJ_kernel(const InstDev* __restrict__ inst,
                                                          const LaunchInfo li, int arena_floats, int max_steps,
                                                          int gmax, int GL, const int8_t* __restrict__ spins,
                                                          float* __restrict__ part, int part_stride,
@@ -568,42 +608,48 @@ __global__ void __launch_bounds__(128) general_dJ_kernel(const InstDev* __restri
     const int g0 = G.comp_step0[c];
     // forward: tables and their scales
     const float fr[2] = {0.f, 0.f};
+    StepBlock blk;
     for (int st = 0; st < nsteps; ++st) {
-      const StepRec r = step_at(G, g0 + st);
-      const float h = field_of(G, r.fb, r.fc, s);
-      const float ah = fabsf(h);
+      const int j = st & (GL - 1);
+      if (j == 0) blk = load_block<1>(G, g0 + min(st + lane, nsteps - 1), s);
+      const Step r = block_step(blk, j, GL);
+      const float h = r.h, ah = fabsf(h);
       const float fv[2] = {expf(beta * (h - ah)), expf(beta * (-h - ah))};
-      const int e = step_table_any<false, 1, true>(r, G, fv, fr, A, nullptr, Ab, RS, r.out_full, lane, GL);
+      const int e = step_table_any<false, 1, true>(r, G, fv, fr, A, nullptr, Ab, RS, lane, GL);
       if (lane == 0) sc[st * RS] = pow2i(-e);
       __syncwarp();
     }
     if (lane == 0) Ab[fin * RS] = 1.f / A[fin * RS];
     __syncwarp();
     // backward
-    for (int st = nsteps - 1; st >= 0; --st) {
-      const StepRec r = step_at(G, g0 + st);
-      const float h = field_of(G, r.fb, r.fc, s);
-      const float ah = fabsf(h);
+    for (int st = nsteps - 1, j0 = 0; st >= 0; --st, ++j0) {
+      const int jb = j0 & (GL - 1);
+      if (jb == 0) blk = load_block<1>(G, g0 + max(st - lane, 0), s);
+      const Step r = block_step(blk, jb, GL);
+      const int* F = G.fprog + r.f;
+      const int fb = F[1], fc = F[2], npair = F[4];
+      const int* pr = F + 9 + 3 * r.nin;
+      const float h = r.h, ah = fabsf(h);
       const float fv[2] = {expf(beta * (h - ah)), expf(beta * (-h - ah))};
       const int E = 2 << r.m;
       const unsigned short* mp = G.map + r.mo;
       const float scl = sc[st * RS];
       constexpr int MW = TNVAN_MAX_ELIM_W;
-      const int np = min(r.npair, MW);  // at most MW neighbours remain
+      const int np = min(npair, MW);  // at most MW neighbours remain
       int pos[MW];
 #pragma unroll
-      for (int j = 0; j < MW; ++j) pos[j] = j < np ? r.pr[2 * j + 1] : 0;
+      for (int j = 0; j < MW; ++j) pos[j] = j < np ? pr[2 * j + 1] : 0;
       float gs = 0.f;       // sum g sigma_v
       float gp[MW];         // sum g sigma_v sigma_u per pair
 #pragma unroll
       for (int j = 0; j < MW; ++j) gp[j] = 0.f;
-      if (np <= 4) step_g_any<4>(r, G, fv, A, Ab, gb, RS, r.out_full, scl, pos, np, lane, GL, gs, gp);
-      else step_g_any<MW>(r, G, fv, A, Ab, gb, RS, r.out_full, scl, pos, np, lane, GL, gs, gp);
+      if (np <= 4) step_g_any<4>(r, G, fv, A, Ab, gb, RS, scl, pos, np, lane, GL, gs, gp);
+      else step_g_any<MW>(r, G, fv, A, Ab, gb, RS, scl, pos, np, lane, GL, gs, gp);
       __syncwarp();
       // input adjoints: each entry gathers the g of the extended indices that
       // read it (inverse map), lanes split the entries
       for (int i = 0; i < r.nin; ++i) {
-        const int in = r.io[3 * i + 1], kk = r.io[3 * i + 2];
+        const int in = F[9 + 3 * i + 1], kk = F[9 + 3 * i + 2];
         const int R = E >> kk;
         const unsigned short* inv = mp + (r.nin + i) * E;
 #pragma unroll 2
@@ -622,26 +668,26 @@ __global__ void __launch_bounds__(128) general_dJ_kernel(const InstDev* __restri
           if (av > 0.f) Ab[(in + e) * RS] += sum / av;
         }
       }
-      for (int f0 = 0; f0 < r.fc; f0 += 4) {
+      for (int f0 = 0; f0 < fc; f0 += 4) {
         int ee[4];
         float v[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          const int f = r.fb + f0 + j;
-          ee[j] = f0 + j < r.fc ? G.fld[2 * f + 1] : -1;
-          v[j] = f0 + j < r.fc ? wscale * gs * (float)s[G.fld[2 * f]] : 0.f;
+          const int f = fb + f0 + j;
+          ee[j] = f0 + j < fc ? G.fld[2 * f + 1] : -1;
+          v[j] = f0 + j < fc ? wscale * gs * (float)s[G.fld[2 * f]] : 0.f;
         }
         acc_edges(acc_w, ee, v, lane0);
       }
 #pragma unroll
-      for (int j0 = 0; j0 < MW; j0 += 4) {
-        if (j0 >= np) break;
+      for (int p0 = 0; p0 < MW; p0 += 4) {
+        if (p0 >= np) break;
         int ee[4];
         float v[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          ee[j] = j0 + j < np ? G.pairE[r.pr[2 * (j0 + j)]] : -1;
-          v[j] = wscale * gp[j0 + j];
+          ee[j] = p0 + j < np ? G.pairE[pr[2 * (p0 + j)]] : -1;
+          v[j] = wscale * gp[p0 + j];
         }
         acc_edges(acc_w, ee, v, lane0);
       }
