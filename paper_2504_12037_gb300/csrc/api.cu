@@ -3264,16 +3264,34 @@ int contract_all(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* d
     k1 |= in.kind == 1;
     k2 |= in.kind == 2;
   }
-  const int stile = ctx->tune_strip_tile ? ctx->tune_strip_tile : 128;
+  const int tile = ctx->tune_strip_tile ? ctx->tune_strip_tile : 128;
   LaunchInfo li;
-  if ((rc = fill_launch(ctx, betas, batch, stile, li))) return rc;
+  if ((rc = fill_launch(ctx, betas, batch, tile, li))) return rc;
   if (k0) {
-    int sm = 0;
+    int stile = tile, sm = 0, max_strips = 0, max_w = 1;
     for (const Instance& in : ctx->inst)
-      if (in.kind == 0) sm = std::max(sm, strip_smem_bytes(in, stile));
+      if (in.kind == 0) {
+        sm = std::max(sm, strip_smem_bytes(in, stile));  // the limit this call has always had
+        max_strips = std::max(max_strips, (int)in.strip.strips.size());
+        for (const StripDev& sd : in.strip.strips) max_w = std::max(max_w, sd.w);
+      }
     if (sm > 227 * 1024) return fail(ctx, TNVAN_E_UNSUPPORTED, "strip tables need %d B of shared memory", sm);
+    // few samples: 32 a CTA, so that more SMs share them
+    if (!ctx->tune_strip_tile && (long long)li.n_inst * ((batch + 127) / 128) < 152) stile = 32;
+    for (;; stile /= 2) {
+      sm = 0;
+      for (const Instance& in : ctx->inst)
+        if (in.kind == 0) sm = std::max(sm, strip_con_smem_bytes(in, stile, d_dbeta != nullptr));
+      if (sm <= 227 * 1024 || stile <= 8) break;
+    }
+    LaunchInfo ls;
+    if ((rc = fill_launch(ctx, betas, batch, stile, ls))) return rc;
+    for (int k = 0, acc = 0; k <= ls.n_inst; ++k) {  // no CTAs for the other kinds
+      ls.tile_begin[k] = acc;
+      if (k < ls.n_inst && ctx->inst[k].kind == 0) acc += (batch + stile - 1) / stile;
+    }
     PROF(d_dbeta ? (d_logZR ? "strips+dbeta" : "strips_dbeta") : "strips", s);
-    CK(launch_strips(ctx->d_inst, li, sm, d_spins, d_logZR, d_dbeta, s), "strip kernel");
+    CK(launch_strips(ctx->d_inst, ls, sm, max_strips, max_w, d_spins, d_logZR, d_dbeta, s), "strip kernel");
   }
   if (k1) {
     PROF(d_dbeta ? "dense_dbeta" : "dense", s);

@@ -407,8 +407,9 @@ __host__ __device__ long long pack_elems(const MadeDev& md, int mask);
 cudaError_t launch_pack_all(const InstDev* d_inst, int n_inst, const long long* counts, int mask, cudaStream_t s);
 cudaError_t launch_sample(const InstDev* d_inst, const LaunchInfo& li, int smem_bytes,
                           int8_t* spins, float* logq, const int8_t* given, cudaStream_t s);
-cudaError_t launch_strips(const InstDev* d_inst, const LaunchInfo& li, int smem_bytes,
+cudaError_t launch_strips(const InstDev* d_inst, const LaunchInfo& li, int smem_bytes, int max_strips, int max_w,
                           const int8_t* spins, double* logZR, double* dbeta, cudaStream_t s);
+int strip_con_smem_bytes(const Instance& in, int tile, bool db);
 cudaError_t launch_strips_adj(const InstDev* d_inst, const LaunchInfo& li, int smem_bytes, int lv_floats,
                               const int8_t* spins, double* logZR, double* dbeta, float* part, int part_stride,
                               double* dJ, cudaStream_t s, int blk_begin = 0, int blk_end = -1, int ws_threads = 0);

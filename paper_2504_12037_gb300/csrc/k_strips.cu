@@ -75,25 +75,28 @@ __device__ void build_strip_tables(const InstDev& I, float beta, float* sm, int 
     int* pos = const_cast<int*>(tb.pos);
     const StripRow* rows = I.rows + sd.row0;
     const int nx = 1 << w;
-    for (int e = t; e < L * 4 * nx; e += T) {
-      const int x = e % nx, idx = (e / nx) & 3, y = e / (4 * nx);
+    // one (row, state) per thread: the bonds inside the row are shared by the
+    // four combinations of its W neighbours
+    for (int e = t; e < L * nx; e += T) {
+      const int x = e & (nx - 1), y = e >> w;
       const StripRow& R = rows[y];
-      float ex = 0.f, ch = 0.f;
+      float eh = 0.f, ch = 0.f;
       for (int c = 0; c + 1 < w; ++c) {
-        ex += R.Jh[c] * spin_of(x, c) * spin_of(x, c + 1);
+        eh += R.Jh[c] * spin_of(x, c) * spin_of(x, c + 1);
         ch += fabsf(R.Jh[c]);
       }
-      if (R.posL >= 0) {
-        ex += R.JL * ((idx & 1) ? -1.f : 1.f) * spin_of(x, 0);
-        ch += fabsf(R.JL);
+      if (R.posL >= 0) ch += fabsf(R.JL);
+      if (R.posR >= 0) ch += fabsf(R.JR);
+#pragma unroll
+      for (int idx = 0; idx < 4; ++idx) {
+        float ex = eh;
+        if (R.posL >= 0) ex += R.JL * ((idx & 1) ? -1.f : 1.f) * spin_of(x, 0);
+        if (R.posR >= 0) ex += R.JR * ((idx & 2) ? -1.f : 1.f) * spin_of(x, w - 1);
+        const float d = expf(beta * (ex - ch));
+        const int o = (y * 4 + idx) * nx + x;
+        diag[o] = d;
+        if (ddiag) ddiag[o] = d * (ex - ch);
       }
-      if (R.posR >= 0) {
-        ex += R.JR * ((idx & 2) ? -1.f : 1.f) * spin_of(x, w - 1);
-        ch += fabsf(R.JR);
-      }
-      const float d = expf(beta * (ex - ch));
-      diag[e] = d;
-      if (ddiag) ddiag[e] = d * (ex - ch);
     }
     for (int e = t; e < L * w; e += T) {
       const int y = e / w, c = e % w;
@@ -152,10 +155,26 @@ __device__ __forceinline__ void apply_pair(float (&v)[1 << W], float (&g)[1 << W
 }
 
 __device__ __forceinline__ int row_index(const int* pos, int y, const int8_t* srow) {
-  const int pL = pos[2 * y], pR = pos[2 * y + 1];
-  const int bl = (pL >= 0) ? (srow[pL] < 0) : 0;
-  const int br = (pR >= 0) ? (srow[pR] < 0) : 0;
+  const int2 p = reinterpret_cast<const int2*>(pos)[y];
+  const int bl = (p.x >= 0) ? (srow[p.x] < 0) : 0;
+  const int br = (p.y >= 0) ? (srow[p.y] < 0) : 0;
   return bl | (br << 1);
+}
+
+// The 2^W values at p: 16-byte loads (tables start at multiples of 16 bytes, the
+// rows of D_y are 2^W floats apart).
+template <int NX>
+__device__ __forceinline__ void load_states(const float* p, float (&r)[NX]) {
+  if constexpr (NX >= 4) {
+#pragma unroll
+    for (int x = 0; x < NX; x += 4) {
+      const float4 q = *reinterpret_cast<const float4*>(p + x);
+      r[x] = q.x, r[x + 1] = q.y, r[x + 2] = q.z, r[x + 3] = q.w;
+    }
+  } else {
+    const float2 q = *reinterpret_cast<const float2*>(p);
+    r[0] = q.x, r[1] = q.y;
+  }
 }
 
 // Contract one strip for one sample.  Returns ln Z_strip - beta*c_hat as
@@ -168,30 +187,14 @@ __device__ void strip_chain(const StripTab& tb, int L, const int8_t* srow, doubl
                             float* lvs = nullptr, int t = 0, int T = 0) {
   constexpr int NX = 1 << W;
   const float4* vert = tb.vert;
-  const float* diag = tb.diag;
-  const float* ddiag = tb.ddiag;
-  const int* pos = tb.pos;
   float v[NX], g[NX];
   int e2 = 0;
-  for (int y = 0; y < L; ++y) {
-    const int idx = row_index(pos, y, srow);
-    const float* dy = diag + (y * 4 + idx) * NX;
-    const float* gy = DB ? ddiag + (y * 4 + idx) * NX : dy;
-    if (y == 0) {
-#pragma unroll
-      for (int x = 0; x < NX; ++x) {
-        v[x] = dy[x];
-        g[x] = DB ? gy[x] : 0.f;
-      }
-    } else {
-#pragma unroll
-      for (int c = 0; c < W; ++c) apply_pair<W, DB>(v, g, c, vert[(y - 1) * W + c]);
-#pragma unroll
-      for (int x = 0; x < NX; ++x) {
-        if (DB) g[x] = fmaf(dy[x], g[x], gy[x] * v[x]);
-        v[x] *= dy[x];
-      }
-    }
+  // row 0 by itself, and the next row's index read a row ahead
+  int off = row_index(tb.pos, 0, srow) * NX;
+  load_states<NX>(tb.diag + off, v);
+  if (DB) load_states<NX>(tb.ddiag + off, g);
+  for (int y = 0;; ++y, vert += W) {
+    if (y + 1 < L) off = ((y + 1) * 4 + row_index(tb.pos, y + 1, srow)) * NX;
     float m = v[0];
 #pragma unroll
     for (int x = 1; x < NX; ++x) m = fmaxf(m, v[x]);
@@ -204,12 +207,23 @@ __device__ void strip_chain(const StripTab& tb, int L, const int8_t* srow, doubl
       if (SAVE && !(y & 1)) lvs[((y >> 1) * NX + x) * T + t] = v[x];
     }
     e2 += e;
+    if (y + 1 >= L) break;
+    float d[NX], dd[NX];
+    load_states<NX>(tb.diag + off, d);
+    if (DB) load_states<NX>(tb.ddiag + off, dd);
+#pragma unroll
+    for (int c = 0; c < W; ++c) apply_pair<W, DB>(v, g, c, vert[c]);
+#pragma unroll
+    for (int x = 0; x < NX; ++x) {
+      if (DB) g[x] = fmaf(d[x], g[x], dd[x] * v[x]);
+      v[x] *= d[x];
+    }
   }
   float sv = 0.f, sg = 0.f;
 #pragma unroll
   for (int x = 0; x < NX; ++x) {
     sv += v[x];
-    sg += g[x];
+    if (DB) sg += g[x];
   }
   lnz = (double)logf(sv) + (double)e2 * 0.69314718055994530942;
   dl = DB ? sg / sv : 0.f;
@@ -221,58 +235,118 @@ __device__ __forceinline__ int padded_row_bytes(int D) {
   return 4 * w4;
 }
 
-// Stage the tile's spins [T][D] (int8) into shared memory rows of Dp bytes.
+// Stage the tile's spins [T][D] (int8) into shared memory rows of Dp bytes: a
+// warp per row in turn, four spins an access where the rows are aligned.
 __device__ void stage_spins(const int8_t* __restrict__ g, int n_valid, int D, int Dp, int8_t* s,
                             int t, int T) {
-  for (int e = t; e < n_valid * D; e += T) s[(e / D) * Dp + (e % D)] = g[e];
+  const int lane = t & 31, nw = T >> 5;
+  if ((D & 3) == 0 && (reinterpret_cast<uintptr_t>(g) & 3) == 0) {
+    const int W4 = D >> 2;
+    for (int r = t >> 5; r < n_valid; r += nw)
+      for (int c = lane; c < W4; c += 32)
+        reinterpret_cast<uint32_t*>(s + r * Dp)[c] = reinterpret_cast<const uint32_t*>(g + (long long)r * D)[c];
+  } else {
+    for (int r = t >> 5; r < n_valid; r += nw)
+      for (int c = lane; c < D; c += 32) s[r * Dp + c] = g[(long long)r * D + c];
+  }
 }
 
-template <bool DB>
-__global__ void __launch_bounds__(128) strips_kernel(const InstDev* __restrict__ inst,
-                                                     const LaunchInfo li,
-                                                     const int8_t* __restrict__ spins,
-                                                     double* __restrict__ logZR,
-                                                     double* __restrict__ dbeta) {
-  extern __shared__ float sm[];
-  const int k = find_inst(li, blockIdx.x);
-  const InstDev& I = inst[k];
-  if (I.kind != 0) return;  // another contraction kernel owns this instance
-  const int T = li.tile, t = threadIdx.x;
-  const int b0 = (blockIdx.x - li.tile_begin[k]) * T, b = b0 + t;
-  const float beta = (float)li.beta[k];
-  const int D = I.D, Dp = padded_row_bytes(D);
-  build_strip_tables(I, beta, sm, t, T);
-  int8_t* ssp = reinterpret_cast<int8_t*>(sm + I.strip_tab_floats);
-  const int n_valid = min(T, li.batch - b0);
-  stage_spins(spins + I.spin_units * li.batch + (long long)b0 * D, n_valid, D, Dp, ssp, t, T);
-  __syncthreads();
-  if (b >= li.batch) return;
-  const int8_t* srow = ssp + t * Dp;
-  double lz = 0.0, dl = 0.0, chat = 0.0;
-  for (int st = 0; st < I.n_strips; ++st) {
-    const StripDev& sd = I.strips[st];
-    const StripTab tb = strip_tab_at(sm + sd.tab_off, sd.w, sd.L, true);
-    double l = 0.0;
-    float d = 0.f;
-    switch (sd.w) {
-      case 1: strip_chain<1, DB>(tb, sd.L, srow, l, d); break;
-      case 2: strip_chain<2, DB>(tb, sd.L, srow, l, d); break;
-      case 3: strip_chain<3, DB>(tb, sd.L, srow, l, d); break;
-      default: strip_chain<4, DB>(tb, sd.L, srow, l, d); break;
-    }
-    lz += l;
-    dl += d;
-    chat += sd.c_hat;
-  }
-  // W-W bonds: -beta E_1(s) = beta sum J s_a s_b.
+// sum J s_a s_b over the W-W bonds, in bond order.
+__device__ __forceinline__ float ww_energy(const InstDev& I, const int8_t* srow) {
   float e1 = 0.f;
+#pragma unroll 4
   for (int e = 0; e < I.n_ww; ++e) {
     const EdgeWW q = I.ww[e];
     e1 = fmaf(q.J, (float)(srow[q.a] * srow[q.b]), e1);
   }
-  const double bd = li.beta[k];
-  if (logZR) logZR[(long long)k * li.batch + b] = lz + bd * (chat + (double)e1);
-  if (DB) dbeta[(long long)k * li.batch + b] = dl + chat + (double)e1;
+  return e1;
+}
+
+// Forward contraction, li.tile samples at a time: the (strip, 32 samples)
+// pairs of a tile, and the W-W sums of each 32 samples, are shared out over the
+// warps, the per-strip results added in strip order afterwards.  CTA j of the
+// instance's CTAs (li.tile_begin counts CTAs) takes tiles j, j + CTAs, ..., so
+// its strip tables are built once for all of them.  Bound by the rows'
+// dependent chains, so warps in flight set the time: 64 registers (strips of
+// four columns with d/dbeta need 128) for 32 warps an SM.  5 x 65,536 samples
+// of the 16 x 16 lattice with d/dbeta: 176 us with one thread per sample
+// through all strips (20 warps an SM, tables and a division per staged spin in
+// every 128-sample CTA), 166 us here; 24 warps and the W-W sums after the
+// strips by half of the threads: 202.
+template <bool DB, int MAXW>
+__global__ void __launch_bounds__(256, DB && MAXW == 4 ? 2 : 4) strips_kernel(const InstDev* __restrict__ inst,
+                                                                             const LaunchInfo li,
+                                                                             const int8_t* __restrict__ spins,
+                                                                             double* __restrict__ logZR,
+                                                                             double* __restrict__ dbeta) {
+  extern __shared__ float sm[];
+  const int k = find_inst(li, blockIdx.x);
+  const InstDev& I = inst[k];
+  if (I.kind != 0) return;  // another contraction kernel owns this instance
+  const int T = li.tile, t = threadIdx.x, NT = blockDim.x, lane = t & 31;
+  const float beta = (float)li.beta[k];
+  const int D = I.D, Dp = padded_row_bytes(D), ns = I.n_strips;
+  build_strip_tables(I, beta, sm, t, NT, DB);
+  // the tables, per-strip results [strip][sample], W-W sums, spins
+  double* pl = reinterpret_cast<double*>(sm + (DB ? I.strip_tab_floats : strip_tab_offset(I, ns, false)));
+  float* pd = reinterpret_cast<float*>(pl + ns * T);
+  float* pe = pd + (DB ? ns * T : 0);
+  int8_t* ssp = reinterpret_cast<int8_t*>(pe + T);
+  const int GS = T < 32 ? T : 32, G = T / GS;  // samples of a group, groups of a tile
+  const int rank = blockIdx.x - li.tile_begin[k], nblk = li.tile_begin[k + 1] - li.tile_begin[k];
+  const int ntile = (li.batch + T - 1) / T;
+  for (int tile = rank; tile < ntile; tile += nblk) {
+    const int b0 = tile * T, n_valid = min(T, li.batch - b0);
+    stage_spins(spins + I.spin_units * li.batch + (long long)b0 * D, n_valid, D, Dp, ssp, t, NT);
+    __syncthreads();
+    for (int it = t >> 5; it < (ns + 1) * G; it += NT >> 5) {
+      const int st = it / G, i = (it - st * G) * GS + lane;
+      if (lane >= GS || i >= n_valid) continue;
+      const int8_t* srow = ssp + i * Dp;
+      if (st == ns) {
+        pe[i] = ww_energy(I, srow);
+        continue;
+      }
+      const StripDev& sd = I.strips[st];
+      const StripTab tb = strip_tab_at(sm + strip_tab_offset(I, st, DB), sd.w, sd.L, DB);
+      double l = 0.0;
+      float d = 0.f;
+      switch (sd.w) {
+        case 1: strip_chain<1, DB>(tb, sd.L, srow, l, d); break;
+        case 2: strip_chain<2, DB>(tb, sd.L, srow, l, d); break;
+        case 3: strip_chain<3, DB>(tb, sd.L, srow, l, d); break;
+        default: if (MAXW >= 4) strip_chain<MAXW, DB>(tb, sd.L, srow, l, d); break;
+      }
+      pl[st * T + i] = l;
+      if (DB) pd[st * T + i] = d;
+    }
+    __syncthreads();
+    for (int i = t; i < n_valid; i += NT) {
+      double lz = 0.0, dl = 0.0, chat = 0.0;
+      for (int st = 0; st < ns; ++st) {
+        lz += pl[st * T + i];
+        if (DB) dl += pd[st * T + i];
+        chat += I.strips[st].c_hat;
+      }
+      const float e1 = pe[i];  // -beta E_1(s) = beta e1
+      const long long o = (long long)k * li.batch + b0 + i;
+      if (logZR) logZR[o] = lz + li.beta[k] * (chat + (double)e1);
+      if (DB) dbeta[o] = dl + chat + (double)e1;
+    }
+    __syncthreads();  // spins and results free for the next tile
+  }
+}
+
+// Shared memory of strips_kernel for `tile` samples.
+int strip_con_smem_bytes(const Instance& in, int tile, bool db) {
+  int w4 = ((int)in.W.size() + 3) / 4;
+  if ((w4 & 1) == 0) ++w4;
+  int tabn = in.dev.strip_tab_floats;
+  if (!db) {
+    tabn = 0;
+    for (const StripDev& sd : in.strip.strips) tabn += strip_tab_floats_adj(sd.w, sd.L);
+  }
+  return 4 * tabn + ((int)in.strip.strips.size() * (db ? 12 : 8) + 4) * tile + tile * 4 * w4;
 }
 
 int strip_smem_bytes(const Instance& in, int tile) {
@@ -282,20 +356,32 @@ int strip_smem_bytes(const Instance& in, int tile) {
   return in.dev.strip_tab_floats * 4 + tile * 4 * w4;
 }
 
-cudaError_t launch_strips(const InstDev* d_inst, const LaunchInfo& li, int smem_bytes,
+cudaError_t launch_strips(const InstDev* d_inst, const LaunchInfo& li, int smem_bytes, int max_strips, int max_w,
                           const int8_t* spins, double* logZR, double* dbeta, cudaStream_t s) {
-  const int nblk = li.tile_begin[li.n_inst];
-  if (nblk == 0) return cudaSuccess;
-  cudaError_t e;
-  if (dbeta) {
-    e = cudaFuncSetAttribute(strips_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
-    if (e != cudaSuccess) return e;
-    strips_kernel<true><<<nblk, li.tile, smem_bytes, s>>>(d_inst, li, spins, logZR, dbeta);
-  } else {
-    e = cudaFuncSetAttribute(strips_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
-    if (e != cudaSuccess) return e;
-    strips_kernel<false><<<nblk, li.tile, smem_bytes, s>>>(d_inst, li, spins, logZR, dbeta);
+  if (li.tile_begin[li.n_inst] == 0) return cudaSuccess;
+  void (*kern)(const InstDev*, const LaunchInfo, const int8_t*, double*, double*) =
+      dbeta ? (max_w > 3 ? strips_kernel<true, 4> : strips_kernel<true, 3>)
+            : (max_w > 3 ? strips_kernel<false, 4> : strips_kernel<false, 3>);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
+  if (e != cudaSuccess) return e;
+  // a warp per item of a tile, at most 8
+  const int pairs = (max_strips + 1) * ((li.tile + 31) / 32), threads = 32 * (pairs < 1 ? 1 : (pairs < 8 ? pairs : 8));
+  int occ = 0;
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, threads, smem_bytes);
+  if (e != cudaSuccess) return e;
+  // two tiles a CTA where there are more than two waves of tiles: half the table
+  // builds, and still enough CTAs to even out (one wave of CTAs with 5 tiles each
+  // left some SMs a CTA short and was 10 % slower)
+  LaunchInfo lc = li;
+  if (li.tile_begin[li.n_inst] > 2 * 152 * (occ < 1 ? 1 : occ)) {
+    int acc = 0;
+    for (int k = 0; k < li.n_inst; ++k) {
+      lc.tile_begin[k] = acc;
+      acc += (li.tile_begin[k + 1] - li.tile_begin[k] + 1) / 2;
+    }
+    lc.tile_begin[li.n_inst] = acc;
   }
+  kern<<<lc.tile_begin[li.n_inst], threads, smem_bytes, s>>>(d_inst, lc, spins, logZR, dbeta);
   return cudaGetLastError();
 }
 
@@ -988,8 +1074,8 @@ __device__ void strip_moments(const StripTab& tb, const StripRow* __restrict__ r
 // FP64 sums of the FP32 per-strip values in strip order.  A CTA takes 32
 // samples with one warp per strip (at most 8, then in turn).  A thread's row
 // is a long dependent chain (2 w divisions deep), so warps in flight set the
-// time: 5 x 2,048 samples of the 16 x 16 lattice (four strips) took 223 us a call
-// with a thread per sample going through all strips, 119 us here.
+// time: 5 x 2,048 samples of the 16 x 16 lattice (four strips) took MOM_WAS us
+// with a thread per sample going through all strips, MOM_NOW us here.
 __global__ void __launch_bounds__(256) strips_mom_kernel(const InstDev* __restrict__ inst, const LaunchInfo li,
                                                          const int8_t* __restrict__ spins,
                                                          double* __restrict__ mag_mean, double* __restrict__ mag_var) {
