@@ -1146,6 +1146,7 @@ int tnvan_destroy(tnvan_ctx* ctx) {
   if (ctx->prof_ref) cudaEventDestroy(ctx->prof_ref);
   for (float* p : ctx->d_gen_scratch)
     if (p) cudaFree(p);
+  for (float* p : ctx->gen_scratch_old) cudaFree(p);
   delete ctx;
   return TNVAN_OK;
 }
@@ -1889,16 +1890,49 @@ bool gen_tables_global(int S, F smem) {
 
 // Global table scratch of the elimination kernels (which: 0 forward, 1
 // reverse sweep); grows only, kept for the context's lifetime.
-static int ensure_gen_scratch(tnvan_ctx* ctx, int which, size_t floats) {
-  if (floats <= ctx->gen_scratch_floats[which]) return TNVAN_OK;
-  if (ctx->d_gen_scratch[which]) cudaFree(ctx->d_gen_scratch[which]);
-  ctx->d_gen_scratch[which] = nullptr;
-  ctx->gen_scratch_floats[which] = 0;
-  cudaError_t e = cudaMalloc(&ctx->d_gen_scratch[which], floats * sizeof(float));
-  if (e != cudaSuccess)
-    return fail(ctx, TNVAN_E_NOMEM, "cudaMalloc(elimination tables, %zu floats): %s", floats, cudaGetErrorString(e));
-  ctx->gen_scratch_floats[which] = floats;
+static bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) == cudaSuccess) return st != cudaStreamCaptureStatusNone;
+  cudaGetLastError();  // the legacy stream beside a capture
+  return true;
+}
+static int ensure_gen_scratch(tnvan_ctx* ctx, int which, size_t floats, cudaStream_t s) {
+  if (floats > ctx->gen_scratch_floats[which]) {
+    // a captured graph may hold the old buffer: kept until the context goes
+    if (ctx->d_gen_scratch[which] && ctx->gen_scratch_captured[which])
+      ctx->gen_scratch_old.push_back(ctx->d_gen_scratch[which]);
+    else if (ctx->d_gen_scratch[which])
+      cudaFree(ctx->d_gen_scratch[which]);
+    ctx->d_gen_scratch[which] = nullptr;
+    ctx->gen_scratch_floats[which] = 0;
+    ctx->gen_scratch_captured[which] = false;
+    cudaError_t e = cudaMalloc(&ctx->d_gen_scratch[which], floats * sizeof(float));
+    if (e != cudaSuccess)
+      return fail(ctx, TNVAN_E_NOMEM, "cudaMalloc(elimination tables, %zu floats): %s", floats, cudaGetErrorString(e));
+    ctx->gen_scratch_floats[which] = floats;
+  }
+  if (!ctx->gen_scratch_captured[which]) ctx->gen_scratch_captured[which] = capturing(s);
   return TNVAN_OK;
+}
+// The same for a form that has another to fall back on: false where the buffer
+// would have to grow inside a capture or cannot.
+static bool try_gen_scratch(tnvan_ctx* ctx, int which, size_t floats, cudaStream_t s) {
+  if (floats > ctx->gen_scratch_floats[which]) {
+    if (capturing(s)) return false;
+    float* p = nullptr;  // the old buffer stays until the new one is there
+    if (cudaMalloc(&p, floats * sizeof(float)) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    if (ctx->d_gen_scratch[which] && ctx->gen_scratch_captured[which])
+      ctx->gen_scratch_old.push_back(ctx->d_gen_scratch[which]);
+    else if (ctx->d_gen_scratch[which])
+      cudaFree(ctx->d_gen_scratch[which]);
+    ctx->d_gen_scratch[which] = p;
+    ctx->gen_scratch_floats[which] = floats;
+    ctx->gen_scratch_captured[which] = false;
+  }
+  return ensure_gen_scratch(ctx, which, floats, s) == TNVAN_OK;
 }
 
 // Per-strip results of the wide-strip kernels [n_inst][batch][strips]; grows only.
@@ -2464,7 +2498,7 @@ int tnvan_magnetisation(tnvan_ctx* ctx, const double* betas, int batch, const in
     CK(launch_general_pp(ctx->d_inst, lg, nsteps, s), "elimination bond products");
     float* gs = nullptr;
     if (glob) {
-      if ((rc = ensure_gen_scratch(ctx, 0, general_mom_scratch_floats(lg, arena, GL)))) return rc;
+      if ((rc = ensure_gen_scratch(ctx, 0, general_mom_scratch_floats(lg, arena, GL), s))) return rc;
       gs = ctx->d_gen_scratch[0];
     }
     CK(launch_general_mom(ctx->d_inst, lg, sm, arena, GL, d_spins, mean, var, gs, s), "elimination moments kernel");
@@ -3367,17 +3401,54 @@ int contract_all(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* d
     for (const Instance& in : ctx->inst)
       if (in.kind == 2 && in.g_ntab > 0 && in.g_ntab <= batch)
         lg.gen_tab = std::max(lg.gen_tab, in.g_ntab);
-    float* gs = nullptr;
-    if (glob) {
-      if ((rc = ensure_gen_scratch(ctx, 0, general_scratch_floats(lg, arena, GL, db)))) return rc;
-      gs = ctx->d_gen_scratch[0];
+    // The lane = sample form, 32 samples a CTA and a warp per table entry up to
+    // the mean table size, is one CTA's chain of steps long whatever the batch;
+    // the lane-group form spends more instructions, but on small tables the
+    // barriers cost more than those (n = 500 of degree 3 with d/dbeta, 4,096
+    // samples: width 8, 12.8 entries on average, 717 against 1,060; width 4, 495
+    // against 434; width 2, 518 against 408 us).  So: tables of 8 entries on
+    // average (4 without derivatives).  With derivatives outside shared memory
+    // (one CTA an SM and slower steps) or small tables only while the CTAs last
+    // two rounds: 32,768 samples, width 8 with d/dbeta, 4,888 against 2,419 us;
+    // width 4 without, 1,374 against 694.
+    int steps = 0, W = 2, place = 0;
+    double mean = 1;
+    for (const Instance& in : ctx->inst)
+      if (in.kind == 2) {
+        steps = std::max(steps, in.g_max_steps);
+        mean = std::max(mean, in.g_mean_entries);
+      }
+    while (2 * W <= 8 && 2 * W <= mean) W *= 2;
+    for (int p : {db ? 3 : 1, 1})
+      if (!place && general_rows_smem_bytes(arena, steps, Dm, db, p) <= 224 * 1024) place = p;
+    LaunchInfo lw;
+    if ((rc = fill_launch(ctx, betas, batch, 32, lw))) return rc;
+    lw.gen_tab = lg.gen_tab;
+    int acc = 0;
+    for (int k = 0; k < lw.n_inst; ++k) {  // as lg: no tiles for what the wide-strip kernel has contracted
+      lw.tile_begin[k] = acc;
+      if (lg.tile_begin[k + 1] > lg.tile_begin[k]) acc += (batch + 31) / 32;
     }
+    lw.tile_begin[lw.n_inst] = acc;
+    bool by_rows = mean >= (db ? 8 : 4) && place && (acc <= 2 * 152 || (mean >= 8 && place == (db ? 3 : 1)));
+    const size_t scr_rows = by_rows ? general_rows_scratch_floats(arena, steps, db, place, acc) : 0;
+    if (scr_rows) by_rows = try_gen_scratch(ctx, 0, scr_rows, s);
+    if (glob && (!by_rows || lg.gen_tab > 0) &&
+        (rc = ensure_gen_scratch(ctx, 0, general_scratch_floats(lg, arena, GL, db), s)))
+      return rc;
+    float* gs = ctx->d_gen_scratch[0];
     if (lg.gen_tab > 0) {
       PROF("general_tables", s);
-      CK(launch_general_tables(ctx->d_inst, lg, sm, db, GL, gs, s), "general tables kernel");
+      CK(launch_general_tables(ctx->d_inst, lg, sm, db, GL, glob ? gs : nullptr, s), "general tables kernel");
     }
     PROF(d_dbeta ? "general_dbeta" : "general", s);
-    CK(launch_general(ctx->d_inst, lg, sm, GL, d_spins, d_logZR, d_dbeta, gs, s), "general kernel");
+    if (by_rows)
+      CK(launch_general_rows(ctx->d_inst, lw, general_rows_smem_bytes(arena, steps, Dm, db, place), W, arena, steps,
+                             place, d_spins, d_logZR, d_dbeta, gs, s),
+         "general kernel");
+    else
+      CK(launch_general(ctx->d_inst, lg, sm, GL, d_spins, d_logZR, d_dbeta, glob ? gs : nullptr, s),
+         "general kernel");
   }
   return TNVAN_OK;
 }
@@ -3463,9 +3534,35 @@ int run_adjoint(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* d_
         lg.wmul = wmul;
         const int stride = (me + 3) & ~3;
         if ((rc = ensure_dj_part(ctx, (size_t)lg.tile_begin[lg.n_inst] * stride))) return rc;
+        // lane = sample where the sum order allows it (4 or 8 lanes per sample)
+        // and the sums fit; small tables only while its CTAs last two rounds
+        // (n = 500 of degree 3, 16,384 samples, whole backward: width 8, 7.9 ms
+        // against 9.8 in lane groups; width 2, 4.4 against 2.8)
+        const int rows_sm = general_rows_dJ_smem_bytes(Dm, me, gmax, GL);
+        double mean = 1;
+        for (const Instance& in : ctx->inst)
+          if (in.kind == 2) mean = std::max(mean, in.g_mean_entries);
+        const long long n_rows = (long long)lg.n_inst * ((batch + 31) / 32);
+        const size_t scr_rows = general_rows_dJ_scratch_floats(arena, steps, (int)n_rows);
+        const bool by_rows = GL >= 4 && rows_sm <= 220 * 1024 && (mean >= 4 || n_rows <= 2 * 152) &&
+                             try_gen_scratch(ctx, 1, scr_rows, s);
+        if (by_rows) {
+          LaunchInfo lw;
+          if ((rc = fill_launch(ctx, betas, batch, 32, lw))) return rc;
+          lw.wmul = wmul;
+          {
+            PROF("general_pp", s);
+            CK(launch_general_pp(ctx->d_inst, lg, nsteps, s), "elimination bond products");
+          }
+          PROF("general_dJ", s);
+          CK(launch_general_rows_dJ(ctx->d_inst, lw, lg, rows_sm, GL, arena, steps, gmax, d_spins,
+                                    ctx->d_dj_part, stride, d_dJ, ctx->d_gen_scratch[1], s),
+             "general adjoint kernel");
+          return TNVAN_OK;
+        }
         float* gs = nullptr;
         if (glob) {
-          if ((rc = ensure_gen_scratch(ctx, 1, general_dJ_scratch_floats(per, T, GL, lg.tile_begin[lg.n_inst]))))
+          if ((rc = ensure_gen_scratch(ctx, 1, general_dJ_scratch_floats(per, T, GL, lg.tile_begin[lg.n_inst]), s)))
             return rc;
           gs = ctx->d_gen_scratch[1];
         }

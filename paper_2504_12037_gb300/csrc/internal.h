@@ -393,6 +393,8 @@ struct tnvan_ctx {
   size_t dj_part_floats = 0;
   float* d_gen_scratch[2] = {nullptr, nullptr};  // global elimination tables: forward, reverse sweep
   size_t gen_scratch_floats[2] = {0, 0};
+  bool gen_scratch_captured[2] = {false, false};  // a captured graph may hold the buffer
+  std::vector<float*> gen_scratch_old;            // such buffers, outgrown
   double* d_wide_part = nullptr;  // per-strip log Z of the wide-strip kernels
   size_t wide_part_n = 0;
   void* d_obs = nullptr;             // tnvan_observables: weights, d/dbeta, sums
@@ -429,6 +431,21 @@ cudaError_t launch_general(const InstDev* d_inst, const LaunchInfo& li, int smem
 cudaError_t launch_general_dJ(const InstDev* d_inst, const LaunchInfo& li, int smem_bytes, int arena, int steps,
                               int gmax, int GL, const int8_t* spins, float* part, int part_stride, double* dJ,
                               float* garena, cudaStream_t s);
+// The same with lane = sample, 32 samples and W warps per CTA (li.tile = 32;
+// steps: the most elimination steps of an instance; place: bit 0 tables in
+// shared memory, bit 1 their derivatives too).  The reverse sweep keeps the sums
+// of the lane-group form with W = 4 or 8 lanes per sample; lr: that form's tiles
+// of 128 / W samples, whose rows of bond sums it fills.
+cudaError_t launch_general_rows(const InstDev* d_inst, const LaunchInfo& li, int smem_bytes, int W, int arena,
+                                int steps, int place, const int8_t* spins, double* logZR, double* dbeta, float* gscr,
+                                cudaStream_t s);
+int general_rows_smem_bytes(int arena, int steps, int D, bool db, int place);
+size_t general_rows_scratch_floats(int arena, int steps, bool db, int place, int nblk);
+cudaError_t launch_general_rows_dJ(const InstDev* d_inst, const LaunchInfo& li, const LaunchInfo& lr, int smem_bytes,
+                                   int W, int arena, int steps, int gmax, const int8_t* spins, float* part,
+                                   int part_stride, double* dJ, float* gscr, cudaStream_t s);
+int general_rows_dJ_smem_bytes(int D, int n_edges, int gmax, int W);
+size_t general_rows_dJ_scratch_floats(int arena, int steps, int nblk);
 // bond products of every elimination step at li.beta (before the kernels above)
 cudaError_t launch_general_pp(const InstDev* d_inst, const LaunchInfo& li, int max_steps, cudaStream_t s);
 int general_dJ_smem_bytes(int per_sample, int D, int n_edges, int T, int GL, bool glob);

@@ -80,26 +80,32 @@ struct StepBlock {
   float h;
 };
 template <int COL>
-__device__ __forceinline__ StepBlock load_block(const GenDev& G, int g, const int8_t* s) {
+__device__ __forceinline__ StepBlock load_block(const GenDev& G, int g) {
   StepBlock b;
   b.f = G.fstep[g];
   const int* F = G.fprog + b.f;
   const int nin = F[3];
-  b.pk = F[0] | (nin << 8);
+  b.pk = F[0] | (nin << 8) | (nin > 0 ? F[11] << 16 : 0) | (nin > 1 ? F[14] << 20 : 0) | (nin > 2 ? F[17] << 24 : 0);
   b.ppo = F[5];
   b.mo = F[6];
   b.out = F[7 + COL];
   b.in0 = nin > 0 ? F[9 + COL] : 0;
   b.in1 = nin > 1 ? F[12 + COL] : 0;
   b.in2 = nin > 2 ? F[15 + COL] : 0;
-  b.h = field_of(G, F[1], F[2], s);
+  b.h = 0.f;
+  return b;
+}
+template <int COL>
+__device__ __forceinline__ StepBlock load_block(const GenDev& G, int g, const int8_t* s) {
+  StepBlock b = load_block<COL>(G, g);
+  b.h = field_of(G, G.fprog[b.f + 1], G.fprog[b.f + 2], s);
   return b;
 }
 __device__ __forceinline__ Step block_step(const StepBlock& b, int j, int GL) {
   Step r;
   const int pk = __shfl_sync(0xffffffffu, b.pk, j, GL);
   r.m = pk & 255;
-  r.nin = pk >> 8;
+  r.nin = (pk >> 8) & 255;
   r.ppo = __shfl_sync(0xffffffffu, b.ppo, j, GL);
   r.mo = __shfl_sync(0xffffffffu, b.mo, j, GL);
   r.out = __shfl_sync(0xffffffffu, b.out, j, GL);
@@ -109,6 +115,12 @@ __device__ __forceinline__ Step block_step(const StepBlock& b, int j, int GL) {
   r.f = __shfl_sync(0xffffffffu, b.f, j, GL);
   r.h = __shfl_sync(0xffffffffu, b.h, j, GL);
   return r;
+}
+
+// Spins of the inputs of the group's step j.
+__device__ __forceinline__ void next_widths(const StepBlock& b, int j, int (&kk)[3]) {
+  const int pk = __shfl_sync(0xffffffffu, b.pk, j);
+  kk[0] = (pk >> 16) & 15, kk[1] = (pk >> 20) & 15, kk[2] = (pk >> 24) & 15;
 }
 
 // Bond products of every step at this call's beta: one CTA per (step,
@@ -168,10 +180,16 @@ __device__ __forceinline__ float group_max(float v, int GL) {
 // registers until their scale is known (one table write instead of a write, a
 // read and a write).
 #define GEN_U 4
-template <bool DB, int NIN, int COL, bool ZERO>
+// Launches of more CTAs than this take one entry at a time in half of the
+// registers instead: there the CTAs in flight hide the latency, and the batch's
+// dropped entries are only instructions (n = 500 of degree 3, width 4, with
+// d/dbeta: 32,768 samples in 1,024 CTAs 1,068 us four at a time, 653 one at a
+// time; 4,096 samples in 256 CTAs 434 us four at a time, 526 one at a time).
+#define GEN_FEW (2 * 152)
+template <bool DB, int NIN, int COL, bool ZERO, int U0>
 __device__ __forceinline__ int step_table(const Step& r, const GenDev& G, const float (&fv)[2], const float (&fr)[2],
                                           float* A, float* dA, float* Ab, int RS, int lane, int GL) {
-  constexpr int U = DB && NIN >= 3 ? GEN_U / 2 : GEN_U;  // within 128 registers
+  constexpr int U = DB && NIN >= 3 && U0 > 1 ? U0 / 2 : U0;  // within 128 registers
   const int out = r.out;
   const int M = 1 << r.m, E = 2 * M;
   const float* pp = G.pp + r.ppo;
@@ -206,7 +224,9 @@ __device__ __forceinline__ int step_table(const Step& r, const GenDev& G, const 
           }
         }
 #pragma unroll
-      for (int u = 0; u < U; ++u)
+      for (int u = 0; u < U; ++u) {
+        // no divisions for what is dropped (M and GL are powers of two: the same for all lanes with an entry)
+        if (DB && u * GL >= M) continue;
 #pragma unroll
         for (int sg = 0; sg < 2; ++sg) {
           p[u][sg] = fv[sg] * p[u][sg];
@@ -217,10 +237,12 @@ __device__ __forceinline__ int step_table(const Step& r, const GenDev& G, const 
             if (DB) rr[u][sg] += dval[i][u][sg] / val[i][u][sg];
           }
         }
+      }
     } else {
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        const int x = x0 + u * GL < M ? x0 + u * GL : x0;
+        const int x = x0 + u * GL;
+        if (u * GL >= M) continue;
 #pragma unroll
         for (int sg = 0; sg < 2; ++sg) {
           p[u][sg] = fv[sg] * p[u][sg];
@@ -237,9 +259,10 @@ __device__ __forceinline__ int step_table(const Step& r, const GenDev& G, const 
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int x = x0 + u * GL;
+      av[u] = dv[u] = 0.f;
+      if (u * GL >= M) continue;
       av[u] = __fadd_rn(p[u][0], p[u][1]);  // the products' own rounding: not contracted into the last one
       if (DB) dv[u] = fmaf(p[u][1], rr[u][1], p[u][0] * rr[u][0]);
-      if (x >= M) continue;
       mx = fmaxf(mx, av[u]);
       if (!regs) {
         A[(out + x) * RS] = av[u];
@@ -270,23 +293,23 @@ __device__ __forceinline__ int step_table(const Step& r, const GenDev& G, const 
   return e;
 }
 
-template <bool DB, int COL, bool ZERO>
+template <bool DB, int COL, bool ZERO, int U0>
 __device__ __forceinline__ int step_table_any(const Step& r, const GenDev& G, const float (&fv)[2],
                                               const float (&fr)[2], float* A, float* dA, float* Ab, int RS, int lane,
                                               int GL) {
   switch (r.nin) {  // the same for every lane
-    case 0: return step_table<DB, 0, COL, ZERO>(r, G, fv, fr, A, dA, Ab, RS, lane, GL);
-    case 1: return step_table<DB, 1, COL, ZERO>(r, G, fv, fr, A, dA, Ab, RS, lane, GL);
-    case 2: return step_table<DB, 2, COL, ZERO>(r, G, fv, fr, A, dA, Ab, RS, lane, GL);
-    case 3: return step_table<DB, 3, COL, ZERO>(r, G, fv, fr, A, dA, Ab, RS, lane, GL);
-    default: return step_table<DB, -1, COL, ZERO>(r, G, fv, fr, A, dA, Ab, RS, lane, GL);
+    case 0: return step_table<DB, 0, COL, ZERO, U0>(r, G, fv, fr, A, dA, Ab, RS, lane, GL);
+    case 1: return step_table<DB, 1, COL, ZERO, U0>(r, G, fv, fr, A, dA, Ab, RS, lane, GL);
+    case 2: return step_table<DB, 2, COL, ZERO, U0>(r, G, fv, fr, A, dA, Ab, RS, lane, GL);
+    case 3: return step_table<DB, 3, COL, ZERO, U0>(r, G, fv, fr, A, dA, Ab, RS, lane, GL);
+    default: return step_table<DB, -1, COL, ZERO, U0>(r, G, fv, fr, A, dA, Ab, RS, lane, GL);
   }
 }
 
 // Component c for the sample whose tables start at A; forward, live offsets.
 // Adds log Z_c (and with DB its beta-derivative) to lz / dl on lane 0 of the
 // group.
-template <bool DB>
+template <bool DB, int U0>
 __device__ __forceinline__ void run_component(const GenDev& G, int c, const int8_t* s, float* A, float* dA, int RS,
                                               int lane, int GL, float beta, double& lz, double& dl) {
   const int* H = G.fprog + G.fhdr[c];
@@ -311,7 +334,7 @@ __device__ __forceinline__ void run_component(const GenDev& G, int c, const int8
     }
     const float fv[2] = {expf(beta * (h - ah)), expf(beta * (-h - ah))};
     const float fr[2] = {h - ah, -h - ah};
-    esum += step_table_any<DB, 0, false>(r, G, fv, fr, A, dA, nullptr, RS, lane, GL);
+    esum += step_table_any<DB, 0, false, U0>(r, G, fv, fr, A, dA, nullptr, RS, lane, GL);
     __syncwarp();
   }
   if (lane == 0) {
@@ -338,8 +361,8 @@ __device__ __forceinline__ void stage_spins(int8_t* ssp, const int8_t* gsp, int 
 }
 
 // li.tile = samples per CTA (S); blockDim.x = S * GL.
-template <bool DB>
-__global__ void __launch_bounds__(128, 4) general_kernel(const InstDev* __restrict__ inst,
+template <bool DB, int U0>
+__global__ void __launch_bounds__(128, U0 > 1 ? 4 : 8) general_kernel(const InstDev* __restrict__ inst,
                                                       const LaunchInfo li, int arena_floats, int GL,
                                                       const int8_t* __restrict__ spins,
                                                       double* __restrict__ logZR,
@@ -375,10 +398,266 @@ __global__ void __launch_bounds__(128, 4) general_kernel(const InstDev* __restri
       lz += G.tab_lz[cr[4] + x];
       if (DB) dl += G.tab_db[cr[4] + x];
     } else {
-      run_component<DB>(G, c, s, A, dA, RS, lane, GL, beta, lz, dl);
+      run_component<DB, U0>(G, c, s, A, dA, RS, lane, GL, beta, lz, dl);
     }
   }
   if (lane != 0 || b >= li.batch) return;
+  float e1 = 0.f;
+  for (int e = 0; e < I.n_ww; ++e) {
+    const EdgeWW q = I.ww[e];
+    e1 = fmaf(q.J, (float)(s[q.a] * s[q.b]), e1);
+  }
+  const double chf = G.c_hat;
+  const long long o = (long long)k * li.batch + b;
+  if (logZR) logZR[o] = lz + li.beta[k] * (chf + (double)e1);
+  if (DB) dbeta[o] = dl + chf + (double)e1;
+}
+
+// ---------------------------------------------------------------------------
+// The same contraction with lane = sample: a CTA takes 32 samples, its W warps
+// share out each table's entries (warp w takes x = w, w + W, ...), tables are
+// [entry][32 samples].  Every index (step record, map, bond product) is then
+// the same for a warp's lanes and every table access one 128-byte row, where
+// the lane-group form spends a warp's instructions on 32 / GL samples and, on
+// the many small tables, leaves most lanes idle: 426 M warp instructions against
+// 199 M for 4,096 samples of the n = 500 graph.  Costs two barriers a step.
+// Bound by the steps' dependent chain: one CTA lasts ~400 steps whatever the
+// batch.  Each entry's arithmetic, and so every result, is that of step_table.
+// ---------------------------------------------------------------------------
+#define G2_MAXW 8
+// floats of a CTA: tables, fields of every step, and with d/dbeta the tables'
+// derivatives
+__host__ __device__ __forceinline__ size_t g2_main_floats(int arena, int steps) { return (size_t)(arena + steps) * 32; }
+
+// The entries x = el, el + W, ... of a step's table, the table's maximum taken
+// over the CTA's warps (red: two buffers of [warps][32], used in turn).
+template <bool DB, int NIN, int COL, bool ZERO>
+__device__ __forceinline__ int step_rows(const Step& r, const GenDev& G, const float (&fv)[2], const float (&fr)[2],
+                                         float* A, float* dA, float* Ab, int el, int W, int lane, float* red) {
+  constexpr int U = DB && NIN >= 3 ? GEN_U / 2 : GEN_U;
+  const int M = 1 << r.m, E = 2 * M;
+  const float* pp = G.pp + r.ppo;
+  const float* pd = G.pp + G.n_pp + r.ppo;
+  const unsigned short* mp = G.map + r.mo;
+  const bool regs = M <= W * U;
+  float* out = A + r.out * 32;
+  float* dout = DB ? dA + r.out * 32 : nullptr;
+  float av[U], dv[U];
+  float mx = 0.f;
+  for (int x0 = el; x0 < M; x0 += W * U) {
+    float p[U][2], rr[U][2];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int x = x0 + u * W < M ? x0 + u * W : x0;
+#pragma unroll
+      for (int sg = 0; sg < 2; ++sg) {
+        p[u][sg] = __ldg(pp + (x | (sg << r.m)));
+        rr[u][sg] = DB ? __ldg(pd + (x | (sg << r.m))) : 0.f;
+      }
+    }
+    if constexpr (NIN >= 0) {
+      float val[NIN > 0 ? NIN : 1][U][2], dval[NIN > 0 ? NIN : 1][U][2];
+#pragma unroll
+      for (int i = 0; i < NIN; ++i)
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int x = x0 + u * W < M ? x0 + u * W : x0;
+#pragma unroll
+          for (int sg = 0; sg < 2; ++sg) {
+            const int q = (r.in[i] + __ldg(mp + i * E + (x | (sg << r.m)))) * 32;
+            val[i][u][sg] = A[q];
+            if (DB) dval[i][u][sg] = dA[q];
+          }
+        }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if (DB && x0 + u * W >= M) continue;  // no divisions for what is dropped (the same for the whole warp)
+#pragma unroll
+        for (int sg = 0; sg < 2; ++sg) {
+          p[u][sg] = fv[sg] * p[u][sg];
+          if (DB) rr[u][sg] = fr[sg] + rr[u][sg];
+#pragma unroll
+          for (int i = 0; i < NIN; ++i) {
+            p[u][sg] *= val[i][u][sg];
+            if (DB) rr[u][sg] += dval[i][u][sg] / val[i][u][sg];
+          }
+        }
+      }
+    } else {
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int x = x0 + u * W;
+        if (x >= M) continue;
+#pragma unroll
+        for (int sg = 0; sg < 2; ++sg) {
+          p[u][sg] = fv[sg] * p[u][sg];
+          if (DB) rr[u][sg] = fr[sg] + rr[u][sg];
+          for (int i = 0; i < r.nin; ++i) {
+            const int q = (G.fprog[r.f + 9 + 3 * i + COL] + mp[i * E + (x | (sg << r.m))]) * 32;
+            const float v = A[q];
+            p[u][sg] *= v;
+            if (DB) rr[u][sg] += dA[q] / v;
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int x = x0 + u * W;
+      av[u] = dv[u] = 0.f;
+      if (x >= M) continue;
+      av[u] = __fadd_rn(p[u][0], p[u][1]);  // the products' own rounding: not contracted into the last one
+      if (DB) dv[u] = fmaf(p[u][1], rr[u][1], p[u][0] * rr[u][0]);
+      mx = fmaxf(mx, av[u]);
+      if (!regs) {
+        out[x * 32] = av[u];
+        if (DB) dout[x * 32] = dv[u];
+      }
+    }
+  }
+  if (W > 1) {
+    red[el * 32 + lane] = mx;
+    __syncthreads();
+    mx = red[lane];
+    const int nw = min(W, M);  // warps that held entries
+    for (int w = 1; w < nw; ++w) mx = fmaxf(mx, red[w * 32 + lane]);
+  }
+  const int e = exponent_of(mx);
+  const float sc = pow2i(-e);
+  if (regs) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int x = el + u * W;
+      if (x >= M) continue;
+      out[x * 32] = av[u] * sc;
+      if (DB) dout[x * 32] = dv[u] * sc;
+      if (ZERO) Ab[(r.out + x) * 32] = 0.f;
+    }
+  } else {
+#pragma unroll 4
+    for (int x = el; x < M; x += W) {
+      out[x * 32] *= sc;
+      if (DB) dout[x * 32] *= sc;
+      if (ZERO) Ab[(r.out + x) * 32] = 0.f;
+    }
+  }
+  return e;
+}
+template <bool DB, int COL, bool ZERO>
+__device__ __forceinline__ int step_rows_any(const Step& r, const GenDev& G, const float (&fv)[2],
+                                             const float (&fr)[2], float* A, float* dA, float* Ab, int el, int W,
+                                             int lane, float* red) {
+  switch (r.nin) {
+    case 0: return step_rows<DB, 0, COL, ZERO>(r, G, fv, fr, A, dA, Ab, el, W, lane, red);
+    case 1: return step_rows<DB, 1, COL, ZERO>(r, G, fv, fr, A, dA, Ab, el, W, lane, red);
+    case 2: return step_rows<DB, 2, COL, ZERO>(r, G, fv, fr, A, dA, Ab, el, W, lane, red);
+    case 3: return step_rows<DB, 3, COL, ZERO>(r, G, fv, fr, A, dA, Ab, el, W, lane, red);
+    default: return step_rows<DB, -1, COL, ZERO>(r, G, fv, fr, A, dA, Ab, el, W, lane, red);
+  }
+}
+
+// The fields of component steps [g0, g0 + nsteps) into h[step * 32] (this
+// sample's column), the steps shared out over the warps.
+__device__ __forceinline__ void step_fields(const GenDev& G, int g0, int nsteps, const int8_t* s, float* h, int el,
+                                            int W) {
+#pragma unroll 2
+  for (int st = el; st < nsteps; st += W) {
+    const int* F = G.fprog + G.fstep[g0 + st];
+    h[st * 32] = field_of(G, F[1], F[2], s);
+  }
+}
+
+// A read that only brings its line into L1; landed() ends its wait.
+__device__ __forceinline__ int touch(const void* p) {
+  int v;
+  asm volatile("ld.global.b32 %0, [%1];" : "=r"(v) : "l"(reinterpret_cast<uintptr_t>(p) & ~(uintptr_t)3));
+  return v;
+}
+__device__ __forceinline__ void landed(int v) { asm volatile("" ::"r"(v)); }
+
+// li.tile = 32; place: bit 0 tables and fields in shared memory, bit 1 the
+// derivatives too, else in this CTA's slice of gscr.
+template <bool DB>
+__global__ void __launch_bounds__(32 * G2_MAXW, 2) general_rows_kernel(const InstDev* __restrict__ inst,
+                                                                       const LaunchInfo li, int arena, int steps,
+                                                                       int place, const int8_t* __restrict__ spins,
+                                                                       double* __restrict__ logZR,
+                                                                       double* __restrict__ dbeta,
+                                                                       float* __restrict__ gscr) {
+  extern __shared__ float sm[];
+  __shared__ float red[2][G2_MAXW * 32];
+  const int k = find_inst(li, blockIdx.x);
+  const InstDev& I = inst[k];
+  if (I.kind != 2) return;
+  const int lane = threadIdx.x & 31, el = threadIdx.x >> 5, W = blockDim.x >> 5;
+  const int b0 = (blockIdx.x - li.tile_begin[k]) * 32, b = b0 + lane;
+  const float beta = (float)li.beta[k];
+  const int D = I.D, Dp = padded_bytes(D);
+  const size_t mf = g2_main_floats(arena, steps), df = (size_t)arena * 32;
+  const size_t per = ((place & 1) ? 0 : mf) + (DB && !(place & 2) ? df : 0);
+  float* sp = sm;
+  float* gp = gscr + (size_t)blockIdx.x * per;
+  float* A;
+  if (place & 1) A = sp, sp += mf;
+  else A = gp, gp += mf;
+  float* dA = nullptr;
+  if (DB) {
+    if (place & 2) dA = sp, sp += df;
+    else dA = gp;
+  }
+  float* h = A + (size_t)arena * 32 + lane;
+  A += lane;
+  if (DB) dA += lane;
+  int8_t* ssp = reinterpret_cast<int8_t*>(sp);
+  const GenDev& G = I.gen;
+  stage_spins(ssp, spins + I.spin_units * li.batch + (long long)b0 * D, min(32, li.batch - b0), 32, D, Dp);
+  __syncthreads();
+  const int8_t* s = ssp + lane * Dp;
+  const bool tab = li.gen_tab && G.n_tab > 0 && G.n_tab <= li.batch;  // tables built for this call
+  double lz = 0.0, dl = 0.0;
+  int par = 0;
+  for (int c = 0; c < G.n_comp; ++c) {
+    const int* cr = G.ctab + 5 * c;
+    if (tab && cr[4] >= 0) {  // a tabulated component: one lookup
+      const int x = boundary_index(G, cr, s);
+      lz += G.tab_lz[cr[4] + x];
+      if (DB) dl += G.tab_db[cr[4] + x];
+      continue;
+    }
+    const int* H = G.fprog + G.fhdr[c];
+    const int nsteps = H[0], fin = H[1], g0 = G.comp_step0[c];
+    step_fields(G, g0, nsteps, s, h, el, W);
+    __syncthreads();
+    int esum = 0;
+    float hs = 0.f, hc = 0.f;  // as run_component
+    StepBlock blk, nxt = load_block<0>(G, g0 + min(lane, nsteps - 1));
+    for (int st = 0; st < nsteps; ++st) {
+      const int j = st & 31;
+      if (j == 0) {
+        blk = nxt;
+        nxt = load_block<0>(G, g0 + min(st + 32 + lane, nsteps - 1));
+      }
+      const Step r = block_step(blk, j, 32);
+      const float hv = h[st * 32], ah = fabsf(hv);
+      {
+        const float y = ah - hc;
+        const float t2 = hs + y;
+        hc = (t2 - hs) - y;
+        hs = t2;
+      }
+      const float fv[2] = {expf(beta * (hv - ah)), expf(beta * (-hv - ah))};
+      const float fr[2] = {hv - ah, -hv - ah};
+      esum += step_rows_any<DB, 0, false>(r, G, fv, fr, A, dA, nullptr, el, W, lane, red[par]);
+      par ^= 1;
+      __syncthreads();
+    }
+    const double hsum = (double)hs - (double)hc;
+    const float z = A[fin * 32];
+    lz += (double)beta * hsum + (double)esum * 0.69314718055994530942 + (double)logf(z);
+    if (DB) dl += hsum + (double)(dA[fin * 32] / z);
+    __syncthreads();  // the tables and fields are free for the next component
+  }
+  if (el != 0 || b >= li.batch) return;
   float e1 = 0.f;
   for (int e = 0; e < I.n_ww; ++e) {
     const EdgeWW q = I.ww[e];
@@ -449,7 +728,7 @@ __global__ void __launch_bounds__(128) general_tab_kernel(const InstDev* __restr
       for (int j = 0; j < cr[2]; ++j) s[G.bpos[cr[3] + j]] = ((x >> j) & 1) ? -1 : 1;
     __syncwarp();
     double lz = 0.0, dl = 0.0;
-    run_component<DB>(G, want, s, A, dA, RS, lane, GL, beta, lz, dl);
+    run_component<DB, GEN_U>(G, want, s, A, dA, RS, lane, GL, beta, lz, dl);
     if (mine && live && lane == 0) {
       G.tab_lz[g] = lz;
       if (DB) G.tab_db[g] = dl;
@@ -489,7 +768,7 @@ __device__ __forceinline__ void acc_edges(float* acc_w, const int (&e)[4], float
 // The product terms of one step in the reverse sweep: g(x, sigma) into gb, its
 // sums with sigma (gs) and with sigma sigma_u of the first NPU bonds (gp), in
 // the order of x; loads GEN_U entries at a time.
-template <int NIN, int NPU>
+template <int NIN, int NPU, int U0>
 __device__ __forceinline__ void step_g(const Step& r, const GenDev& G, const float (&fv)[2], const float* A,
                                        const float* Ab, float* gb, int RS, float scl, const int* pos, int np,
                                        int lane, int GL, float& gs, float (&gp)[TNVAN_MAX_ELIM_W]) {
@@ -497,37 +776,39 @@ __device__ __forceinline__ void step_g(const Step& r, const GenDev& G, const flo
   const int M = 1 << r.m, E = 2 * M;
   const float* pp = G.pp + r.ppo;
   const unsigned short* mp = G.map + r.mo;
-  for (int x0 = lane; x0 < M; x0 += GL * GEN_U) {
-    float p[GEN_U][2], abx[GEN_U];
+  for (int x0 = lane; x0 < M; x0 += GL * U0) {
+    float p[U0][2], abx[U0];
 #pragma unroll
-    for (int u = 0; u < GEN_U; ++u) {
+    for (int u = 0; u < U0; ++u) {
       const int x = x0 + u * GL < M ? x0 + u * GL : x0;
       abx[u] = Ab[(out + x) * RS];
 #pragma unroll
       for (int sg = 0; sg < 2; ++sg) p[u][sg] = pp[x | (sg << r.m)];
     }
     if constexpr (NIN >= 0) {
-      float val[NIN > 0 ? NIN : 1][GEN_U][2];
+      float val[NIN > 0 ? NIN : 1][U0][2];
 #pragma unroll
       for (int i = 0; i < NIN; ++i)
 #pragma unroll
-        for (int u = 0; u < GEN_U; ++u) {
+        for (int u = 0; u < U0; ++u) {
           const int x = x0 + u * GL < M ? x0 + u * GL : x0;
 #pragma unroll
           for (int sg = 0; sg < 2; ++sg) val[i][u][sg] = A[(r.in[i] + mp[i * E + (x | (sg << r.m))]) * RS];
         }
 #pragma unroll
-      for (int u = 0; u < GEN_U; ++u)
+      for (int u = 0; u < U0; ++u) {
 #pragma unroll
         for (int sg = 0; sg < 2; ++sg) {
           p[u][sg] = fv[sg] * p[u][sg];
 #pragma unroll
           for (int i = 0; i < NIN; ++i) p[u][sg] *= val[i][u][sg];
         }
+      }
     } else {
 #pragma unroll
-      for (int u = 0; u < GEN_U; ++u) {
-        const int x = x0 + u * GL < M ? x0 + u * GL : x0;
+      for (int u = 0; u < U0; ++u) {
+        const int x = x0 + u * GL;
+        if (u * GL >= M) continue;
 #pragma unroll
         for (int sg = 0; sg < 2; ++sg) {
           p[u][sg] = fv[sg] * p[u][sg];
@@ -536,9 +817,9 @@ __device__ __forceinline__ void step_g(const Step& r, const GenDev& G, const flo
       }
     }
 #pragma unroll
-    for (int u = 0; u < GEN_U; ++u) {
+    for (int u = 0; u < U0; ++u) {
       const int x = x0 + u * GL;
-      if (x >= M) continue;
+      if (u * GL >= M) continue;
       const float ab = abx[u] * scl;
 #pragma unroll
       for (int sg = 0; sg < 2; ++sg) {
@@ -552,19 +833,20 @@ __device__ __forceinline__ void step_g(const Step& r, const GenDev& G, const flo
     }
   }
 }
-template <int NPU>
+template <int NPU, int U0>
 __device__ __forceinline__ void step_g_any(const Step& r, const GenDev& G, const float (&fv)[2], const float* A,
                                            const float* Ab, float* gb, int RS, float scl, const int* pos, int np,
                                            int lane, int GL, float& gs, float (&gp)[TNVAN_MAX_ELIM_W]) {
   switch (r.nin) {  // the same for every lane
-    case 0: step_g<0, NPU>(r, G, fv, A, Ab, gb, RS, scl, pos, np, lane, GL, gs, gp); break;
-    case 1: step_g<1, NPU>(r, G, fv, A, Ab, gb, RS, scl, pos, np, lane, GL, gs, gp); break;
-    case 2: step_g<2, NPU>(r, G, fv, A, Ab, gb, RS, scl, pos, np, lane, GL, gs, gp); break;
-    default: step_g<-1, NPU>(r, G, fv, A, Ab, gb, RS, scl, pos, np, lane, GL, gs, gp); break;
+    case 0: step_g<0, NPU, U0>(r, G, fv, A, Ab, gb, RS, scl, pos, np, lane, GL, gs, gp); break;
+    case 1: step_g<1, NPU, U0>(r, G, fv, A, Ab, gb, RS, scl, pos, np, lane, GL, gs, gp); break;
+    case 2: step_g<2, NPU, U0>(r, G, fv, A, Ab, gb, RS, scl, pos, np, lane, GL, gs, gp); break;
+    default: step_g<-1, NPU, U0>(r, G, fv, A, Ab, gb, RS, scl, pos, np, lane, GL, gs, gp); break;
   }
 }
 
-__global__ void __launch_bounds__(128, 4) general_dJ_kernel(const InstDev* __restrict__ inst,
+template <int U0>
+__global__ void __launch_bounds__(128, U0 > 1 ? 4 : 8) general_dJ_kernel(const InstDev* __restrict__ inst,
                                                          const LaunchInfo li, int arena_floats, int max_steps,
                                                          int gmax, int GL, const int8_t* __restrict__ spins,
                                                          float* __restrict__ part, int part_stride,
@@ -615,7 +897,7 @@ __global__ void __launch_bounds__(128, 4) general_dJ_kernel(const InstDev* __res
       const Step r = block_step(blk, j, GL);
       const float h = r.h, ah = fabsf(h);
       const float fv[2] = {expf(beta * (h - ah)), expf(beta * (-h - ah))};
-      const int e = step_table_any<false, 1, true>(r, G, fv, fr, A, nullptr, Ab, RS, lane, GL);
+      const int e = step_table_any<false, 1, true, U0>(r, G, fv, fr, A, nullptr, Ab, RS, lane, GL);
       if (lane == 0) sc[st * RS] = pow2i(-e);
       __syncwarp();
     }
@@ -643,8 +925,8 @@ __global__ void __launch_bounds__(128, 4) general_dJ_kernel(const InstDev* __res
       float gp[MW];         // sum g sigma_v sigma_u per pair
 #pragma unroll
       for (int j = 0; j < MW; ++j) gp[j] = 0.f;
-      if (np <= 4) step_g_any<4>(r, G, fv, A, Ab, gb, RS, scl, pos, np, lane, GL, gs, gp);
-      else step_g_any<MW>(r, G, fv, A, Ab, gb, RS, scl, pos, np, lane, GL, gs, gp);
+      if (np <= 4) step_g_any<4, U0>(r, G, fv, A, Ab, gb, RS, scl, pos, np, lane, GL, gs, gp);
+      else step_g_any<MW, U0>(r, G, fv, A, Ab, gb, RS, scl, pos, np, lane, GL, gs, gp);
       __syncwarp();
       // input adjoints: each entry gathers the g of the extended indices that
       // read it (inverse map), lanes split the entries
@@ -703,6 +985,290 @@ __global__ void __launch_bounds__(128, 4) general_dJ_kernel(const InstDev* __res
   }
 }
 
+// ---------------------------------------------------------------------------
+// The reverse sweep with lane = sample (see general_rows_kernel), 32 samples
+// and 16 warps per CTA.  general_dJ_kernel's order of every sum is kept, so
+// d/dJ has the same bits in both forms: a bond's sum over a step's entries is
+// made of W (4 or 8, that kernel's lanes per sample) chains x = w, w + W, ...,
+// each added over the 32 / W samples of a group, then over the chains by the
+// same tree, the groups' rows in turn into one row per 128 / W samples.
+//
+// Tables and adjoints (1.3 MB for 32 samples of the n = 500 graph) stay in
+// global memory, i.e. L2, so a step is a chain of dependent L2 reads: record ->
+// maps -> tables -> g -> adjoints.  The next step's record, bond products, maps
+// and table rows are therefore read into L1 a step ahead (touch), and all 16
+// warps share out the extended indices, the bonds and the gathered entries.
+// 4,096 samples of the n = 500 graph, width 8: 1,769 us against 2,380 in the
+// lane-group form; without the reads ahead and with W warps only, 2,287.
+// ---------------------------------------------------------------------------
+#define G2_DJ_WARPS 16
+
+// Touch what step r will read: threads 0-31 bond products, 32-127 n_maps maps
+// of its extended indices, 128 and 129 its record, and each thread a row of its
+// inputs' tables (T) and, with ADJ, of their adjoints.
+struct Touched {
+  int a, b, c;
+};
+template <bool ADJ>
+__device__ __forceinline__ Touched touch_step(const GenDev& G, const Step& r, const int (&kk)[3], int n_maps,
+                                              const float* A, const float* Ab, int t) {
+  const int E = 2 << r.m;
+  Touched v = {0, 0, 0};
+  if (t < 32) {
+    if (t * 32 < E + 32) v.a = touch(G.pp + r.ppo + min(t * 32, E - 1));
+  } else if (t < 128) {
+    const int nm = n_maps * E, o = (t - 32) * 64;
+    if (nm > 0 && o < nm + 64) v.a = touch(G.map + r.mo + min(o, nm - 1));
+  } else if (ADJ && t < 130) {
+    v.a = touch(G.fprog + r.f + (t == 128 ? 0 : 8));
+  }
+  int q = t;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    if (i >= r.nin) break;
+    const int n = 1 << kk[i];
+    if (q >= 0 && q < n) {
+      v.b = touch(A + (r.in[i] + q) * 32);
+      if (ADJ) v.c = touch(Ab + (r.in[i] + q) * 32);
+    }
+    q -= n;
+  }
+  return v;
+}
+
+// g of the extended indices ext = w0, w0 + NW, ... of a step, into gb.
+template <int NIN>
+__device__ __forceinline__ void rows_g(const Step& r, const GenDev& G, const float (&fv)[2], const float* A,
+                                       const float* Ab, float* gb, float scl, int w0, int NW) {
+  const int M = 1 << r.m, E = 2 * M;
+  const float* pp = G.pp + r.ppo;
+  const unsigned short* mp = G.map + r.mo;
+  for (int e0 = w0; e0 < E; e0 += NW * GEN_U) {
+    float p[GEN_U], ab[GEN_U], val[NIN > 0 ? NIN : 1][GEN_U];
+#pragma unroll
+    for (int u = 0; u < GEN_U; ++u) {
+      const int ext = e0 + u * NW;
+      p[u] = ab[u] = 0.f;
+#pragma unroll
+      for (int i = 0; i < NIN; ++i) val[i][u] = 0.f;
+      if (ext >= E) continue;
+      p[u] = __ldg(pp + ext);
+      ab[u] = Ab[(r.out + (ext & (M - 1))) * 32];
+#pragma unroll
+      for (int i = 0; i < NIN; ++i) val[i][u] = A[(r.in[i] + __ldg(mp + i * E + ext)) * 32];
+    }
+#pragma unroll
+    for (int u = 0; u < GEN_U; ++u) {
+      const int ext = e0 + u * NW;
+      if (ext >= E) continue;
+      float v = ((ext >> r.m) & 1 ? fv[1] : fv[0]) * p[u];
+      if constexpr (NIN >= 0) {
+#pragma unroll
+        for (int i = 0; i < NIN; ++i) v *= val[i][u];
+      } else {
+        for (int i = 0; i < r.nin; ++i) v *= A[(G.fprog[r.f + 9 + 3 * i + 1] + mp[i * E + ext]) * 32];
+      }
+      gb[ext * 32] = (ab[u] * scl) * v;
+    }
+  }
+}
+
+// A bond value's sum over the samples of each group of 32 / W: at the groups'
+// first lanes.
+template <int W>
+__device__ __forceinline__ float group_samples(float v) {
+#pragma unroll
+  for (int o = 16; o >= W; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o / W);
+  return v;
+}
+
+// The W chains of a step's sum of g times a sign: that of the eliminated spin
+// (pos < 0), or of its product with out-scope spin pos.
+template <int W>
+__device__ __forceinline__ void bond_chains(const float* gb, int m, int pos, float (&v)[W]) {
+  const int M = 1 << m;
+#pragma unroll
+  for (int w = 0; w < W; ++w) v[w] = 0.f;
+  for (int x0 = 0; x0 < M; x0 += W) {
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+      const int x = x0 + w;
+      if (x >= M) break;
+      const int bit = pos < 0 ? 0 : (x >> pos) & 1;
+      v[w] = fmaf(gb[x * 32], bit == 0 ? 1.f : -1.f, v[w]);
+      v[w] = fmaf(gb[(x + M) * 32], bit == 1 ? 1.f : -1.f, v[w]);
+    }
+  }
+}
+// The chains, each times mul and added over the groups' samples, added up; into
+// edge e of each group's row (ne4 floats).
+template <int W>
+__device__ __forceinline__ void bond_add(const float (&v)[W], float wscale, float sgn, bool signed_, float* acc,
+                                         int ne4, int e, int lane) {
+  float u[W];
+#pragma unroll
+  for (int w = 0; w < W; ++w) {
+    const float q = wscale * v[w];
+    u[w] = group_samples<W>(signed_ ? q * sgn : q);
+  }
+  if (W == 8) {
+#pragma unroll
+    for (int w = 0; w < 4; ++w) u[w] += u[w + W / 2];
+  }
+  u[0] += u[2];
+  u[1] += u[3];
+  const float sum = u[0] + u[1];
+  if (e >= 0 && (lane & (32 / W - 1)) == 0) acc[lane / (32 / W) * ne4 + e] += sum;
+}
+
+// Dynamic shared memory: g values [gmax][32], bond sums [W][n_edges], spins.
+// Tables, adjoints, scales and fields ((2 arena + 2 steps) x 32 floats) in this
+// CTA's slice of gscr.
+template <int W>
+__global__ void __launch_bounds__(32 * G2_DJ_WARPS, 1) general_rows_dJ_kernel(
+    const InstDev* __restrict__ inst, const LaunchInfo li, int arena, int steps, int gmax,
+    const int8_t* __restrict__ spins, float* __restrict__ part, int part_stride, float* __restrict__ gscr) {
+  extern __shared__ float sm[];
+  __shared__ float red[2][G2_DJ_WARPS * 32];
+  const int k = find_inst(li, blockIdx.x);
+  const InstDev& I = inst[k];
+  if (I.kind != 2) return;
+  constexpr int NW = G2_DJ_WARPS;
+  const int t = threadIdx.x, lane = t & 31, wi = t >> 5;
+  const int c_idx = blockIdx.x - li.tile_begin[k];
+  const int b0 = c_idx * 32, b = b0 + lane;
+  const float beta = (float)li.beta[k];
+  const int D = I.D, Dp = padded_bytes(D), ne = I.n_edges, ne4 = (ne + 3) & ~3;
+  float* A0 = gscr + (size_t)blockIdx.x * (size_t)(2 * arena + 2 * steps) * 32;
+  float* A = A0 + lane;
+  float* Ab0 = A0 + (size_t)arena * 32;
+  float* Ab = Ab0 + lane;
+  float* sc = Ab + (size_t)arena * 32;
+  float* h = sc + (size_t)steps * 32;
+  float* gb = sm + lane;
+  float* acc = sm + gmax * 32;  // [W groups][ne4]
+  int8_t* ssp = reinterpret_cast<int8_t*>(acc + W * ne4);
+  const GenDev& G = I.gen;
+  for (int e = t; e < W * ne4; e += 32 * NW) acc[e] = 0.f;
+  stage_spins(ssp, spins + I.spin_units * li.batch + (long long)b0 * D, min(32, li.batch - b0), 32, D, Dp);
+  __syncthreads();
+  const int8_t* s = ssp + lane * Dp;
+  // per-sample weight of the bond sums (importance multipliers when given)
+  const float wscale =
+      b < li.batch ? beta / (float)li.batch * (li.wmul ? li.wmul[(long long)k * li.batch + b] : 1.f) : 0.f;
+  int par = 0;
+  for (int c = 0; c < G.n_comp; ++c) {
+    const int* H = G.fprog + G.fhdr[c];
+    const int nsteps = H[0], fin = H[2], g0 = G.comp_step0[c];
+    step_fields(G, g0, nsteps, s, h, wi, NW);
+    __syncthreads();
+    const float fr[2] = {0.f, 0.f};
+    int kk[3];
+    {
+      StepBlock blk = load_block<1>(G, g0 + min(lane, nsteps - 1)), nxt = blk;
+      float hv = h[0];
+      for (int st = 0; st < nsteps; ++st) {
+        const int j = st & 31;
+        if (j == 0) {
+          blk = nxt;
+          nxt = load_block<1>(G, g0 + min(st + 32 + lane, nsteps - 1));
+        }
+        const Step r = block_step(blk, j, 32);
+        const Step rn = block_step(j == 31 ? nxt : blk, (j + 1) & 31, 32);
+        next_widths(j == 31 ? nxt : blk, (j + 1) & 31, kk);
+        const float hn = h[min(st + 1, nsteps - 1) * 32], ah = fabsf(hv);
+        const Touched tc = touch_step<false>(G, rn, kk, rn.nin, A0, Ab0, t);
+        const float fv[2] = {expf(beta * (hv - ah)), expf(beta * (-hv - ah))};
+        const int e = step_rows_any<false, 1, true>(r, G, fv, fr, A, nullptr, Ab, wi, NW, lane, red[par]);
+        par ^= 1;
+        if (wi == 0) sc[st * 32] = pow2i(-e);
+        hv = hn;
+        landed(tc.a), landed(tc.b);
+        __syncthreads();
+      }
+    }
+    if (wi == 0) Ab[fin * 32] = 1.f / A[fin * 32];
+    __syncthreads();
+    StepBlock blk, nxt = load_block<1>(G, g0 + max(nsteps - 1 - lane, 0));
+    float hv = h[(nsteps - 1) * 32], scl = sc[(nsteps - 1) * 32];
+    for (int st = nsteps - 1, j0 = 0; st >= 0; --st, ++j0) {
+      const int jb = j0 & 31;
+      if (jb == 0) {
+        blk = nxt;
+        nxt = load_block<1>(G, g0 + max(st - 32 - lane, 0));
+      }
+      const Step r = block_step(blk, jb, 32);
+      const Step rn = block_step(jb == 31 ? nxt : blk, (jb + 1) & 31, 32);
+      next_widths(jb == 31 ? nxt : blk, (jb + 1) & 31, kk);
+      const float hn = h[max(st - 1, 0) * 32], scn = sc[max(st - 1, 0) * 32], ah = fabsf(hv);
+      const Touched tc = touch_step<true>(G, rn, kk, 2 * rn.nin, A0, Ab0, t);
+      const int* F = G.fprog + r.f;
+      const int fb = F[1], fc = F[2], np = min(F[4], TNVAN_MAX_ELIM_W);
+      const int* pr = F + 9 + 3 * r.nin;
+      const float fv[2] = {expf(beta * (hv - ah)), expf(beta * (-hv - ah))};
+      switch (r.nin) {
+        case 0: rows_g<0>(r, G, fv, A, Ab, gb, scl, wi, NW); break;
+        case 1: rows_g<1>(r, G, fv, A, Ab, gb, scl, wi, NW); break;
+        case 2: rows_g<2>(r, G, fv, A, Ab, gb, scl, wi, NW); break;
+        default: rows_g<-1>(r, G, fv, A, Ab, gb, scl, wi, NW); break;
+      }
+      __syncthreads();
+      // bonds, a warp each from the last warp on: one for the fields (if any),
+      // one for each pair
+      const int nq = np + (fc > 0);
+      for (int q = NW - 1 - wi; q < nq; q += NW) {
+        float v[W];
+        const int j = q - (fc > 0);
+        if (j < 0) {
+          bond_chains<W>(gb, r.m, -1, v);
+          for (int f = 0; f < fc; ++f)
+            bond_add<W>(v, wscale, (float)s[G.fld[2 * (fb + f)]], true, acc, ne4, G.fld[2 * (fb + f) + 1], lane);
+        } else {
+          bond_chains<W>(gb, r.m, pr[2 * j + 1], v);
+          bond_add<W>(v, wscale, 1.f, false, acc, ne4, G.pairE[pr[2 * j]], lane);
+        }
+      }
+      // input adjoints: each entry gathers the g of the extended indices that read it
+      const int E = 2 << r.m;
+      const unsigned short* mp = G.map + r.mo;
+      for (int i = 0; i < r.nin; ++i) {
+        const int in = F[9 + 3 * i + 1], ki = F[9 + 3 * i + 2];
+        const int R = E >> ki;
+        const unsigned short* inv = mp + (r.nin + i) * E;
+#pragma unroll 2
+        for (int e = wi; e < (1 << ki); e += NW) {
+          const float av = A[(in + e) * 32];
+          float sum = 0.f;
+          for (int f = 0; f + 4 <= R; f += 4) {  // in index order, four loads in flight
+            float q[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) q[j] = gb[__ldg(inv + e * R + f + j) * 32];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) sum += q[j];
+          }
+          if (R < 4)
+            for (int f = 0; f < R; ++f) sum += gb[inv[e * R + f] * 32];
+          if (av > 0.f) Ab[(in + e) * 32] += sum / av;
+        }
+      }
+      hv = hn, scl = scn;
+      landed(tc.a), landed(tc.b), landed(tc.c);
+      __syncthreads();
+    }
+  }
+  // one row per 128 / W samples: its four groups in turn
+  const int rows = W / 4, n_rows = (li.batch + 128 / W - 1) / (128 / W);
+  const long long row0 = (long long)k * n_rows + (long long)c_idx * rows;
+  for (int q = 0; q < rows && c_idx * rows + q < n_rows; ++q) {
+    float* row = part + (row0 + q) * part_stride;
+    for (int e = t; e < ne; e += 32 * NW) {
+      float v = 0.f;
+      for (int w = 0; w < 4; ++w) v += acc[(4 * q + w) * ne4 + e];
+      row[e] = v;
+    }
+  }
+}
+
 __global__ void general_dJ_reduce_kernel(const InstDev* __restrict__ inst, const LaunchInfo li,
                                          const float* __restrict__ part, int part_stride,
                                          double* __restrict__ dJ) {
@@ -739,18 +1305,62 @@ cudaError_t launch_general_dJ(const InstDev* d_inst, const LaunchInfo& li, int s
                               float* garena, cudaStream_t s) {
   const int nblk = li.tile_begin[li.n_inst];
   if (nblk == 0) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(general_dJ_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
+  auto kern = nblk <= GEN_FEW ? general_dJ_kernel<GEN_U> : general_dJ_kernel<1>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
   if (e != cudaSuccess) return e;
-  general_dJ_kernel<<<nblk, li.tile * GL, smem_bytes, s>>>(d_inst, li, arena, steps, gmax, GL, spins, part,
-                                                           part_stride, garena);
+  kern<<<nblk, li.tile * GL, smem_bytes, s>>>(d_inst, li, arena, steps, gmax, GL, spins, part, part_stride, garena);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   general_dJ_reduce_kernel<<<dim3(4, li.n_inst), 256, 0, s>>>(d_inst, li, part, part_stride, dJ);
   return cudaGetLastError();
 }
 
+int general_rows_smem_bytes(int arena, int steps, int D, bool db, int place) {
+  int w4 = (D + 3) / 4;
+  if ((w4 & 1) == 0) ++w4;
+  return (int)(4 * (((place & 1) ? g2_main_floats(arena, steps) : 0) + (db && (place & 2) ? (size_t)arena * 32 : 0))) +
+         32 * 4 * w4;
+}
+size_t general_rows_scratch_floats(int arena, int steps, bool db, int place, int nblk) {
+  return (((place & 1) ? 0 : g2_main_floats(arena, steps)) + (db && !(place & 2) ? (size_t)arena * 32 : 0)) * nblk;
+}
+cudaError_t launch_general_rows(const InstDev* d_inst, const LaunchInfo& li, int smem_bytes, int W, int arena,
+                                int steps, int place, const int8_t* spins, double* logZR, double* dbeta, float* gscr,
+                                cudaStream_t s) {
+  const int nblk = li.tile_begin[li.n_inst];
+  if (nblk == 0) return cudaSuccess;
+  auto kern = dbeta ? general_rows_kernel<true> : general_rows_kernel<false>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
+  if (e != cudaSuccess) return e;
+  kern<<<nblk, 32 * W, smem_bytes, s>>>(d_inst, li, arena, steps, place, spins, logZR, dbeta, gscr);
+  return cudaGetLastError();
+}
+
+int general_rows_dJ_smem_bytes(int D, int n_edges, int gmax, int W) {
+  int w4 = (D + 3) / 4;
+  if ((w4 & 1) == 0) ++w4;
+  return 4 * (gmax * 32 + W * ((n_edges + 3) & ~3)) + 32 * 4 * w4;
+}
+size_t general_rows_dJ_scratch_floats(int arena, int steps, int nblk) {
+  return (size_t)(2 * arena + 2 * steps) * 32 * nblk;
+}
+cudaError_t launch_general_rows_dJ(const InstDev* d_inst, const LaunchInfo& li, const LaunchInfo& lr, int smem_bytes,
+                                   int W, int arena, int steps, int gmax, const int8_t* spins, float* part,
+                                   int part_stride, double* dJ, float* gscr, cudaStream_t s) {
+  const int nblk = li.tile_begin[li.n_inst];
+  if (nblk == 0) return cudaSuccess;
+  auto kern = W == 8 ? general_rows_dJ_kernel<8> : general_rows_dJ_kernel<4>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
+  if (e != cudaSuccess) return e;
+  kern<<<nblk, 32 * G2_DJ_WARPS, smem_bytes, s>>>(d_inst, li, arena, steps, gmax, spins, part, part_stride, gscr);
+  e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  general_dJ_reduce_kernel<<<dim3(4, lr.n_inst), 256, 0, s>>>(d_inst, lr, part, part_stride, dJ);
+  return cudaGetLastError();
+}
+
 // The components' tables at this call's betas (li.gen_tab: the largest
-// table; general_kernel then looks them up).
+// table; the contraction kernels then look them up).
 cudaError_t launch_general_tables(const InstDev* d_inst, const LaunchInfo& li, int smem_bytes, bool db, int GL,
                                   float* garena, cudaStream_t s) {
   if (li.gen_tab <= 0) return cudaSuccess;
@@ -791,17 +1401,12 @@ cudaError_t launch_general(const InstDev* d_inst, const LaunchInfo& li, int smem
   if (nblk == 0) return cudaSuccess;
   // li.seed carries the arena size (floats) for this launch
   const int arena = (int)(li.seed & 0xffffffffull);
-  cudaError_t e;
-  if (dbeta) {
-    e = cudaFuncSetAttribute(general_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
-    if (e != cudaSuccess) return e;
-    general_kernel<true><<<nblk, li.tile * GL, smem_bytes, s>>>(d_inst, li, arena, GL, spins, logZR, dbeta, garena);
-  } else {
-    e = cudaFuncSetAttribute(general_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
-    if (e != cudaSuccess) return e;
-    general_kernel<false><<<nblk, li.tile * GL, smem_bytes, s>>>(d_inst, li, arena, GL, spins, logZR, dbeta,
-                                                                 garena);
-  }
+  const bool few = nblk <= GEN_FEW;
+  auto kern = dbeta ? (few ? general_kernel<true, GEN_U> : general_kernel<true, 1>)
+                    : (few ? general_kernel<false, GEN_U> : general_kernel<false, 1>);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
+  if (e != cudaSuccess) return e;
+  kern<<<nblk, li.tile * GL, smem_bytes, s>>>(d_inst, li, arena, GL, spins, logZR, dbeta, garena);
   return cudaGetLastError();
 }
 
