@@ -519,6 +519,20 @@ int upload_plan(tnvan_ctx* ctx, Instance& in) {
     g.fld = fld;
     g.fldJ = fj;
     g.c_hat = in.g_chat;
+    int *lt = nullptr, *ltl = nullptr, *lb = nullptr, *lbl = nullptr, *li_ = nullptr, *lr = nullptr;
+    if ((rc = upload(ctx, in, in.glt, &lt))) return rc;
+    if ((rc = upload(ctx, in, in.gltl, &ltl))) return rc;
+    if ((rc = upload(ctx, in, in.glb, &lb))) return rc;
+    if ((rc = upload(ctx, in, in.glbl, &lbl))) return rc;
+    if ((rc = upload(ctx, in, in.glin, &li_))) return rc;
+    if ((rc = upload(ctx, in, in.glroot, &lr))) return rc;
+    g.n_lev = in.gl_levels;
+    g.ltask = lt;
+    g.llev = ltl;
+    g.btask = lb;
+    g.blev = lbl;
+    g.lin = li_;
+    g.lroot = lr;
     int *ct = nullptr, *bp = nullptr, *tc = nullptr;
     if ((rc = upload(ctx, in, in.gctab, &ct))) return rc;
     if ((rc = upload(ctx, in, in.gbpos, &bp))) return rc;
@@ -1935,6 +1949,33 @@ static bool try_gen_scratch(tnvan_ctx* ctx, int which, size_t floats, cudaStream
   return ensure_gen_scratch(ctx, which, floats, s) == TNVAN_OK;
 }
 
+static bool try_dj_part(tnvan_ctx* ctx, size_t floats, cudaStream_t s) {
+  if (floats <= ctx->dj_part_floats) return true;
+  if (capturing(s)) return false;
+  if (ensure_dj_part(ctx, floats) == TNVAN_OK) return true;
+  cudaGetLastError();
+  return false;
+}
+
+// What the level kernels of a launch need: the largest over the instances.
+struct LevelPlan {
+  int live = 0, total = 0, gmax = 0, red = 0, tasks = 0, steps = 0;
+};
+static LevelPlan level_plan(const tnvan_ctx* ctx) {
+  LevelPlan p;
+  for (const Instance& in : ctx->inst) {
+    if (in.kind != 2) continue;
+    p.live = std::max(p.live, in.gl_live);
+    p.total = std::max(p.total, in.gl_total);
+    p.gmax = std::max(p.gmax, in.gl_gmax);
+    p.red = std::max(p.red, in.gl_red);
+    p.tasks = std::max(p.tasks, in.gl_tasks);
+    p.steps = std::max(p.steps, (int)in.gfstep.size());
+  }
+  return p;
+}
+constexpr int LEVEL_SMEM = 216 * 1024;  // and 8 KB of their own
+
 // Per-strip results of the wide-strip kernels [n_inst][batch][strips]; grows only.
 static int ensure_wide_part(tnvan_ctx* ctx, size_t n) {
   if (n <= ctx->wide_part_n) return TNVAN_OK;
@@ -1992,7 +2033,8 @@ int tnvan_reserve(tnvan_ctx* ctx, int max_batch) {
     int max_edges = 0, ctas = 0;
     for (const Instance& in : ctx->inst) {
       max_edges = std::max(max_edges, in.m);
-      ctas += (std::max(max_batch, 1) + 127) / 128;
+      // elimination instances: up to 8 rows per 32 samples
+      ctas += in.kind == 2 ? 8 * ((std::max(max_batch, 1) + 31) / 32) : (std::max(max_batch, 1) + 127) / 128;
     }
     rc = ensure_dj_part(ctx, (size_t)ctas * ((max_edges + 3) & ~3));
     if (rc) return rc;
@@ -3401,39 +3443,34 @@ int contract_all(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* d
     for (const Instance& in : ctx->inst)
       if (in.kind == 2 && in.g_ntab > 0 && in.g_ntab <= batch)
         lg.gen_tab = std::max(lg.gen_tab, in.g_ntab);
-    // The lane = sample form, 32 samples a CTA and a warp per table entry up to
-    // the mean table size, is one CTA's chain of steps long whatever the batch;
-    // the lane-group form spends more instructions, but on small tables the
-    // barriers cost more than those (n = 500 of degree 3 with d/dbeta, 4,096
-    // samples: width 8, 12.8 entries on average, 717 against 1,060; width 4, 495
-    // against 434; width 2, 518 against 408 us).  So: tables of 8 entries on
-    // average (4 without derivatives).  With derivatives outside shared memory
-    // (one CTA an SM and slower steps) or small tables only while the CTAs last
-    // two rounds: 32,768 samples, width 8 with d/dbeta, 4,888 against 2,419 us;
-    // width 4 without, 1,374 against 694.
-    int steps = 0, W = 2, place = 0;
-    double mean = 1;
-    for (const Instance& in : ctx->inst)
-      if (in.kind == 2) {
-        steps = std::max(steps, in.g_max_steps);
-        mean = std::max(mean, in.g_mean_entries);
-      }
-    while (2 * W <= 8 && 2 * W <= mean) W *= 2;
-    for (int p : {db ? 3 : 1, 1})
-      if (!place && general_rows_smem_bytes(arena, steps, Dm, db, p) <= 224 * 1024) place = p;
+    // By levels where the kernel's buffers can be had (a capture allocates
+    // nothing), whatever the sizes: from 33 to 32,768 samples of random regular
+    // graphs (n = 128 to 500, widths 1 to 8) 1.1 to 6 times faster than groups of
+    // lanes, with one exception: d/dbeta of tables of 4 to 8 entries on average
+    // over more than four rounds of CTAs (n = 500, width 4, 32,768 samples: 803 us
+    // by levels, 653 in lane groups).
+    const LevelPlan lp = level_plan(ctx);
     LaunchInfo lw;
     if ((rc = fill_launch(ctx, betas, batch, 32, lw))) return rc;
     lw.gen_tab = lg.gen_tab;
     int acc = 0;
-    for (int k = 0; k < lw.n_inst; ++k) {  // as lg: no tiles for what the wide-strip kernel has contracted
+    for (int k = 0; k < lw.n_inst; ++k) {  // no tiles for other kinds and what the wide-strip kernel has contracted
       lw.tile_begin[k] = acc;
-      if (lg.tile_begin[k + 1] > lg.tile_begin[k]) acc += (batch + 31) / 32;
+      if (ctx->inst[k].kind == 2 && lg.tile_begin[k + 1] > lg.tile_begin[k]) acc += (batch + 31) / 32;
     }
     lw.tile_begin[lw.n_inst] = acc;
-    bool by_rows = mean >= (db ? 8 : 4) && place && (acc <= 2 * 152 || (mean >= 8 && place == (db ? 3 : 1)));
-    const size_t scr_rows = by_rows ? general_rows_scratch_floats(arena, steps, db, place, acc) : 0;
-    if (scr_rows) by_rows = try_gen_scratch(ctx, 0, scr_rows, s);
-    if (glob && (!by_rows || lg.gen_tab > 0) &&
+    int place = db ? 3 : 1, lsm = 0;
+    for (;; place >>= 1) {
+      lsm = general_levels_smem_bytes(lp.live, lp.red, Dm, db, place);
+      if (lsm <= LEVEL_SMEM || !place) break;
+    }
+    double mean = 1;
+    for (const Instance& in : ctx->inst)
+      if (in.kind == 2) mean = std::max(mean, in.g_mean_entries);
+    const bool by_levels =
+        lsm <= LEVEL_SMEM && !(db && mean >= 4 && mean < 8 && acc > 4 * 152) &&
+        try_gen_scratch(ctx, 0, general_levels_scratch_floats(lp.live, lp.steps, db, place, acc, lp.tasks, lsm), s);
+    if (glob && (!by_levels || lg.gen_tab > 0) &&
         (rc = ensure_gen_scratch(ctx, 0, general_scratch_floats(lg, arena, GL, db), s)))
       return rc;
     float* gs = ctx->d_gen_scratch[0];
@@ -3442,9 +3479,9 @@ int contract_all(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* d
       CK(launch_general_tables(ctx->d_inst, lg, sm, db, GL, glob ? gs : nullptr, s), "general tables kernel");
     }
     PROF(d_dbeta ? "general_dbeta" : "general", s);
-    if (by_rows)
-      CK(launch_general_rows(ctx->d_inst, lw, general_rows_smem_bytes(arena, steps, Dm, db, place), W, arena, steps,
-                             place, d_spins, d_logZR, d_dbeta, gs, s),
+    if (by_levels)
+      CK(launch_general_levels(ctx->d_inst, lw, lsm, lp.live, lp.steps, lp.red, lp.tasks, place, d_spins, d_logZR,
+                               d_dbeta, gs, s),
          "general kernel");
     else
       CK(launch_general(ctx->d_inst, lg, sm, GL, d_spins, d_logZR, d_dbeta, glob ? gs : nullptr, s),
@@ -3533,33 +3570,37 @@ int run_adjoint(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* d_
         if ((rc = fill_launch(ctx, betas, batch, T, lg))) return rc;
         lg.wmul = wmul;
         const int stride = (me + 3) & ~3;
-        if ((rc = ensure_dj_part(ctx, (size_t)lg.tile_begin[lg.n_inst] * stride))) return rc;
-        // lane = sample where the sum order allows it (4 or 8 lanes per sample)
-        // and the sums fit; small tables only while its CTAs last two rounds
-        // (n = 500 of degree 3, 16,384 samples, whole backward: width 8, 7.9 ms
-        // against 9.8 in lane groups; width 2, 4.4 against 2.8)
-        const int rows_sm = general_rows_dJ_smem_bytes(Dm, me, gmax, GL);
-        double mean = 1;
-        for (const Instance& in : ctx->inst)
-          if (in.kind == 2) mean = std::max(mean, in.g_mean_entries);
-        const long long n_rows = (long long)lg.n_inst * ((batch + 31) / 32);
-        const size_t scr_rows = general_rows_dJ_scratch_floats(arena, steps, (int)n_rows);
-        const bool by_rows = GL >= 4 && rows_sm <= 220 * 1024 && (mean >= 4 || n_rows <= 2 * 152) &&
-                             try_gen_scratch(ctx, 1, scr_rows, s);
-        if (by_rows) {
-          LaunchInfo lw;
-          if ((rc = fill_launch(ctx, betas, batch, 32, lw))) return rc;
-          lw.wmul = wmul;
+        // by levels where the sum order allows it (2, 4 or 8 lanes per sample) and
+        // the kernel's buffers can be had
+        const LevelPlan lp = level_plan(ctx);
+        LaunchInfo lw;
+        if ((rc = fill_launch(ctx, betas, batch, 32, lw))) return rc;
+        lw.wmul = wmul;
+        int acc = 0;
+        for (int k = 0; k <= lw.n_inst; ++k) {
+          lw.tile_begin[k] = acc;
+          if (k < lw.n_inst && ctx->inst[k].kind == 2) acc += (batch + 31) / 32;
+        }
+        int place = 7, lsm = 0;
+        for (;; place >>= 1) {
+          lsm = general_levels_dJ_smem_bytes(lp.total, lp.live, lp.gmax, lp.red, Dm, place);
+          if (lsm <= LEVEL_SMEM || !place) break;
+        }
+        if (GL >= 2 && lsm <= LEVEL_SMEM && try_dj_part(ctx, (size_t)acc * GL * stride, s) &&
+            try_gen_scratch(ctx, 1,
+                            general_levels_dJ_scratch_floats(lp.total, lp.live, lp.gmax, lp.steps, place, acc, lp.tasks, lsm),
+                            s)) {
           {
             PROF("general_pp", s);
             CK(launch_general_pp(ctx->d_inst, lg, nsteps, s), "elimination bond products");
           }
           PROF("general_dJ", s);
-          CK(launch_general_rows_dJ(ctx->d_inst, lw, lg, rows_sm, GL, arena, steps, gmax, d_spins,
-                                    ctx->d_dj_part, stride, d_dJ, ctx->d_gen_scratch[1], s),
+          CK(launch_general_levels_dJ(ctx->d_inst, lw, lsm, GL, lp.total, lp.live, lp.gmax, lp.steps, lp.red, lp.tasks,
+                                      place, me, d_spins, ctx->d_dj_part, stride, d_dJ, ctx->d_gen_scratch[1], s),
              "general adjoint kernel");
           return TNVAN_OK;
         }
+        if ((rc = ensure_dj_part(ctx, (size_t)lg.tile_begin[lg.n_inst] * stride))) return rc;
         float* gs = nullptr;
         if (glob) {
           if ((rc = ensure_gen_scratch(ctx, 1, general_dJ_scratch_floats(per, T, GL, lg.tile_begin[lg.n_inst]), s)))
@@ -3625,6 +3666,147 @@ int plan_dense(tnvan_ctx* ctx, Instance& in, const std::vector<int>& pos) {
 //   n_in x { in_off, k, pos_0 .. pos_{k-1} }  (pos in the extended scope out+{v})
 //   n_pair x { pair_id, pos_u }                (pos of the neighbour in the out scope)
 // fld: per W-neighbour bond of an R spin, (AR position, edge id); fldJ its coupling.
+// Level schedule of the compiled steps (GenDev::ltask ff.).  Each table has one
+// consumer, so the steps of all components form trees; a step's level is its
+// distance from the leaves' side counted from the roots (as late as possible),
+// so a step's consumer is always in the next level: tables live for two levels
+// only, even levels' from the arena's start, odd levels' from its end.  Steps are
+// cut into tasks of C entries, C the level's entries over the CTA's 16 warps
+// within 4 and 16 (a sixteenth of the step if that is more): with 16 throughout
+// the levels of one or two steps kept a few warps busy (n = 500 graph of width 8,
+// 4,096 samples: d/dbeta 351 and 338 us, reverse sweep 480 and 464).  Tasks of a
+// level: cut steps first, then by falling work, as warps take them in turn.
+static int level_chunk(long entries) {
+  int c = 4;
+  while (c < 16 && 2 * c * 16 <= entries) c *= 2;
+  return c;
+}
+void plan_levels(Instance& in, const std::vector<int>& prog, const std::vector<int>& ctab,
+                 const std::vector<int>& step_off, const std::vector<int>& comp_step0, const std::vector<int>& F,
+                 const std::vector<int>& fs) {
+  const int S = (int)step_off.size(), nc = (int)comp_step0.size() - 1;
+  std::vector<int> parent(S, -1), depth(S, 0), comp(S, 0);
+  std::vector<std::vector<int>> inputs(S);
+  for (int c = 0; c < nc; ++c) {
+    std::map<int, int> maker;  // full offset -> step
+    for (int st = comp_step0[c]; st < comp_step0[c + 1]; ++st) {
+      const int r = step_off[st];
+      comp[st] = c;
+      int q = r + 7;
+      for (int i = 0; i < prog[r + 5]; ++i) {
+        const int from = maker[prog[q]];
+        parent[from] = st;
+        inputs[st].push_back(from);
+        q += 2 + prog[q + 1];
+      }
+      maker[prog[r + 4]] = st;
+    }
+  }
+  int deepest = 0;
+  for (int st = S - 1; st >= 0; --st) {  // a consumer comes after its inputs
+    depth[st] = parent[st] < 0 ? 0 : depth[parent[st]] + 1;
+    deepest = std::max(deepest, depth[st]);
+  }
+  const int L = S ? deepest + 1 : 0;
+  std::vector<std::vector<int>> lev(L);
+  for (int st = 0; st < S; ++st) lev[deepest - depth[st]].push_back(st);
+  std::vector<int> live(S), full(S), goff(S), size(L + 1, 0), m(S);
+  int total = 0, arena = 0, gmax = 0;
+  for (int l = 0; l < L; ++l)
+    for (int st : lev[l]) {
+      m[st] = F[fs[st]];
+      full[st] = total;
+      goff[st] = 2 * size[l];
+      live[st] = size[l];
+      total += 1 << m[st];
+      size[l] += 1 << m[st];
+    }
+  for (int l = 0; l < L; ++l) {
+    arena = std::max(arena, size[l] + size[l + 1]);
+    gmax = std::max(gmax, 2 * size[l]);
+  }
+  for (int l = 1; l < L; l += 2)
+    for (int st : lev[l]) live[st] += arena - size[l];
+  std::vector<int> T, B, LT, BT, lin, root;
+  int red_max = 0;
+  for (int l = 0; l < L; ++l) {
+    struct Task { int st, x0, nx, ch, nch; long work; };
+    std::vector<Task> ts;
+    for (int st : lev[l]) {
+      const int M = 1 << m[st], C = std::max(level_chunk(size[l]), M / 16), n = M <= C ? 1 : M / C;
+      for (int j = 0; j < n; ++j)
+        ts.push_back(Task{st, j * (M / n), M / n, j, n, (long)(M / n) * (2 + (long)inputs[st].size()) + 8});
+    }
+    std::stable_sort(ts.begin(), ts.end(), [](const Task& a, const Task& b) {
+      return (a.nch > 1) != (b.nch > 1) ? a.nch > 1 : a.work > b.work;
+    });
+    int red = 0, cut = 0;
+    std::map<int, int> slot;
+    LT.push_back((int)T.size() / TNVAN_LTASK);
+    for (const Task& t : ts)
+      if (t.nch > 1) {
+        ++cut;
+        if (!slot.count(t.st)) slot[t.st] = red, red += t.nch;
+      }
+    red_max = std::max(red_max, red);
+    LT.push_back(LT.back() + cut);
+    LT.push_back(LT[LT.size() - 2] + (int)ts.size());
+    for (const Task& t : ts) {
+      const int st = t.st, f = fs[st], nin = F[f + 3];
+      const bool tabbed = ctab[5 * comp[st] + 4] >= 0;
+      int r[TNVAN_LTASK] = {m[st] | (nin << 8) | ((tabbed ? 1 : 0) << 16), st, F[f + 5], F[f + 6], live[st], full[st],
+                            t.x0, t.nx, F[f + 1], F[f + 2], t.nch > 1 ? slot[st] : -1, t.nch | (t.ch << 16), goff[st],
+                            (int)lin.size()};
+      for (int i = 0; i < nin; ++i) {
+        if (i < 3) r[14 + i] = live[inputs[st][i]], r[17 + i] = full[inputs[st][i]];
+        lin.push_back(live[inputs[st][i]]);
+        lin.push_back(full[inputs[st][i]]);
+      }
+      T.insert(T.end(), r, r + TNVAN_LTASK);
+    }
+    // the reverse sweep's tasks of this level: bonds and gathers
+    struct Back { int r[TNVAN_BTASK]; long work; };
+    std::vector<Back> bs;
+    const int gc = level_chunk(l > 0 ? size[l - 1] : 0);
+    for (int st : lev[l]) {
+      const int f = fs[st], nin = F[f + 3], M = 1 << m[st], E = 2 * M;
+      if (F[f + 2] > 0) bs.push_back(Back{{0, m[st], goff[st], F[f + 1], F[f + 2], 0, 0, 0}, E + 40L * F[f + 2]});
+      const int* pr = F.data() + f + 9 + 3 * nin;
+      for (int j = 0; j < F[f + 4]; ++j)
+        bs.push_back(Back{{1, m[st], goff[st], pr[2 * j + 1], pr[2 * j], 0, 0, 0}, E + 40L});
+      for (int i = 0; i < nin; ++i) {
+        const int from = inputs[st][i], n = 1 << F[f + 9 + 3 * i + 2], R = E / n, C = std::max(gc, n / 16);
+        for (int e0 = 0; e0 < n; e0 += C)
+          bs.push_back(Back{{2 | (R << 8), std::min(C, n - e0), goff[st], live[from], full[from],
+                             F[f + 6] + (nin + i) * E + e0 * R, e0, 0},
+                            (long)std::min(C, n - e0) * (3 * R + 8)});
+      }
+    }
+    std::stable_sort(bs.begin(), bs.end(), [](const Back& a, const Back& b) { return a.work > b.work; });
+    BT.push_back((int)B.size() / TNVAN_BTASK);
+    BT.push_back(BT.back() + (int)bs.size());
+    for (const Back& b : bs) B.insert(B.end(), b.r, b.r + TNVAN_BTASK);
+  }
+  for (int c = 0; c < nc; ++c) {
+    const int st = comp_step0[c + 1] - 1;  // the component's last step
+    root.push_back(live[st]);
+    root.push_back(full[st]);
+  }
+  in.glt.swap(T);
+  in.glb.swap(B);
+  in.gltl.swap(LT);
+  in.glbl.swap(BT);
+  in.glin.swap(lin);
+  in.glroot.swap(root);
+  in.gl_levels = L;
+  in.gl_live = (arena + 3) & ~3;
+  in.gl_total = total;
+  in.gl_gmax = gmax;
+  in.gl_red = red_max;
+  // (tasks of a level, rounded up over the levels)
+  in.gl_tasks = L ? ((int)in.glt.size() / TNVAN_LTASK + L - 1) / L : 0;
+}
+
 int plan_general(tnvan_ctx* ctx, Instance& in, const std::vector<int>& pos, const std::vector<int>& rank) {
   auto comps = r_components(in, pos);
   std::vector<std::vector<std::pair<int, int>>> adj(in.n);  // (neighbour, edge)
@@ -3912,6 +4094,7 @@ int plan_general(tnvan_ctx* ctx, Instance& in, const std::vector<int>& pos, cons
       for (size_t st = 0; st < step_off.size(); ++st) tot += (double)(1 << prog[step_off[st] + 3]);
       in.g_mean_entries = step_off.empty() ? 1.0 : tot / (double)step_off.size();
     }
+    plan_levels(in, prog, ctab, step_off, comp_step0, F, fs);
     in.gfprog.swap(F);
     in.gfhdr.swap(fh);
     in.gfstep.swap(fs);

@@ -224,6 +224,19 @@ struct GenDev {
   double c_hat;          // constant log-offset / beta
   // components with at most TNVAN_TAB_MAX_K width-set neighbours can be
   // tabulated: log Z_c (and d/dbeta) over every boundary configuration
+  // Level schedule: levels of steps that only need earlier levels' tables, as
+  // tasks of one warp.  llev[3 l]: first task, end of those of cut steps, end;
+  // blev[2 l]: first and end of the reverse sweep's tasks.  ltask (24 ints):
+  //   m | n_in << 8 | tabulated << 16, step, pp_off, map_off, out (level arena),
+  //   out (all tables), x0, entries, fld_begin, fld_count, first slot of the cut
+  //   step's maxima (-1: not cut), tasks of the step | this one << 16, g offset
+  //   in the level, lin offset, 3 x input (level arena), 3 x input (all tables).
+  // btask (8 ints): 0, m, g offset, fld_begin, fld_count | 1, m, g offset, pos_u,
+  //   pair_id | 2 | R << 8, entries, g offset, input (level arena), input (all
+  //   tables), its inverse map from entry e0 on, e0.
+  // lin: per input (level arena, all tables); lroot: the same per final table.
+  int n_lev;
+  const int *ltask, *llev, *btask, *blev, *lin, *lroot;
   const int* ctab;       // [n_comp][5]: program header, program end, k, boundary list offset,
                          // table offset (-1: not tabulated)
   const int* bpos;       // boundary lists (AR positions of the W neighbours), bit j of the index = spin j
@@ -234,6 +247,8 @@ struct GenDev {
   double* tab_db;        // [n_tab] its beta-derivative
 };
 #define TNVAN_TAB_MAX_K 12
+#define TNVAN_LTASK 24
+#define TNVAN_BTASK 8
 
 struct InstDev {
   int kind;  // 0 strips, 1 dense, 2 general
@@ -328,6 +343,8 @@ struct Instance {
   std::vector<int> gfprog, gfhdr, gfstep;  // compiled step records (GenDev::fprog)
   std::vector<unsigned short> gmap;       // input index maps (GenDev::map)
   int g_npp = 0;
+  std::vector<int> glt, gltl, glb, glbl, glin, glroot;  // level schedule (GenDev)
+  int gl_levels = 0, gl_live = 0, gl_total = 0, gl_gmax = 0, gl_red = 0, gl_tasks = 0;
   double g_mean_entries = 1;  // mean table size (entries) of the elimination steps
   int g_max_steps = 0;
   std::vector<int> gctab, gbpos, gtabc;  // component tables (GenDev)
@@ -431,21 +448,23 @@ cudaError_t launch_general(const InstDev* d_inst, const LaunchInfo& li, int smem
 cudaError_t launch_general_dJ(const InstDev* d_inst, const LaunchInfo& li, int smem_bytes, int arena, int steps,
                               int gmax, int GL, const int8_t* spins, float* part, int part_stride, double* dJ,
                               float* garena, cudaStream_t s);
-// The same with lane = sample, 32 samples and W warps per CTA (li.tile = 32;
-// steps: the most elimination steps of an instance; place: bit 0 tables in
-// shared memory, bit 1 their derivatives too).  The reverse sweep keeps the sums
-// of the lane-group form with W = 4 or 8 lanes per sample; lr: that form's tiles
-// of 128 / W samples, whose rows of bond sums it fills.
-cudaError_t launch_general_rows(const InstDev* d_inst, const LaunchInfo& li, int smem_bytes, int W, int arena,
-                                int steps, int place, const int8_t* spins, double* logZR, double* dbeta, float* gscr,
-                                cudaStream_t s);
-int general_rows_smem_bytes(int arena, int steps, int D, bool db, int place);
-size_t general_rows_scratch_floats(int arena, int steps, bool db, int place, int nblk);
-cudaError_t launch_general_rows_dJ(const InstDev* d_inst, const LaunchInfo& li, const LaunchInfo& lr, int smem_bytes,
-                                   int W, int arena, int steps, int gmax, const int8_t* spins, float* part,
-                                   int part_stride, double* dJ, float* gscr, cudaStream_t s);
-int general_rows_dJ_smem_bytes(int D, int n_edges, int gmax, int W);
-size_t general_rows_dJ_scratch_floats(int arena, int steps, int nblk);
+// The same by levels of the elimination trees, lane = sample, tiles of 32 (li);
+// live, total, gmax, red_slots, tasks, steps: the instances' largest gl_* and
+// steps; place: what lies in shared memory (see the kernels).  The reverse sweep
+// keeps the sums of the lane-group form with W = 2, 4 or 8 lanes per sample; part:
+// W rows per tile.
+cudaError_t launch_general_levels(const InstDev* d_inst, const LaunchInfo& li, int smem_bytes, int live, int steps,
+                                  int red_slots, int tasks, int place, const int8_t* spins, double* logZR,
+                                  double* dbeta, float* gscr, cudaStream_t s);
+int general_levels_smem_bytes(int live, int red_slots, int D, bool db, int place);
+size_t general_levels_scratch_floats(int live, int steps, bool db, int place, int nblk, int tasks, int smem_bytes);
+cudaError_t launch_general_levels_dJ(const InstDev* d_inst, const LaunchInfo& li, int smem_bytes, int W, int total,
+                                     int live, int gmax, int steps, int red_slots, int tasks, int place, int max_edges,
+                                     const int8_t* spins, float* part, int part_stride, double* dJ, float* gscr,
+                                     cudaStream_t s);
+int general_levels_dJ_smem_bytes(int total, int live, int gmax, int red_slots, int D, int place);
+size_t general_levels_dJ_scratch_floats(int total, int live, int gmax, int steps, int place, int nblk, int tasks,
+                                        int smem_bytes);
 // bond products of every elimination step at li.beta (before the kernels above)
 cudaError_t launch_general_pp(const InstDev* d_inst, const LaunchInfo& li, int max_steps, cudaStream_t s);
 int general_dJ_smem_bytes(int per_sample, int D, int n_edges, int T, int GL, bool glob);

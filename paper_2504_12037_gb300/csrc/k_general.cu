@@ -85,7 +85,7 @@ __device__ __forceinline__ StepBlock load_block(const GenDev& G, int g) {
   b.f = G.fstep[g];
   const int* F = G.fprog + b.f;
   const int nin = F[3];
-  b.pk = F[0] | (nin << 8) | (nin > 0 ? F[11] << 16 : 0) | (nin > 1 ? F[14] << 20 : 0) | (nin > 2 ? F[17] << 24 : 0);
+  b.pk = F[0] | (nin << 8);
   b.ppo = F[5];
   b.mo = F[6];
   b.out = F[7 + COL];
@@ -105,7 +105,7 @@ __device__ __forceinline__ Step block_step(const StepBlock& b, int j, int GL) {
   Step r;
   const int pk = __shfl_sync(0xffffffffu, b.pk, j, GL);
   r.m = pk & 255;
-  r.nin = (pk >> 8) & 255;
+  r.nin = pk >> 8;
   r.ppo = __shfl_sync(0xffffffffu, b.ppo, j, GL);
   r.mo = __shfl_sync(0xffffffffu, b.mo, j, GL);
   r.out = __shfl_sync(0xffffffffu, b.out, j, GL);
@@ -115,12 +115,6 @@ __device__ __forceinline__ Step block_step(const StepBlock& b, int j, int GL) {
   r.f = __shfl_sync(0xffffffffu, b.f, j, GL);
   r.h = __shfl_sync(0xffffffffu, b.h, j, GL);
   return r;
-}
-
-// Spins of the inputs of the group's step j.
-__device__ __forceinline__ void next_widths(const StepBlock& b, int j, int (&kk)[3]) {
-  const int pk = __shfl_sync(0xffffffffu, b.pk, j);
-  kk[0] = (pk >> 16) & 15, kk[1] = (pk >> 20) & 15, kk[2] = (pk >> 24) & 15;
 }
 
 // Bond products of every step at this call's beta: one CTA per (step,
@@ -414,45 +408,60 @@ __global__ void __launch_bounds__(128, U0 > 1 ? 4 : 8) general_kernel(const Inst
 }
 
 // ---------------------------------------------------------------------------
-// The same contraction with lane = sample: a CTA takes 32 samples, its W warps
-// share out each table's entries (warp w takes x = w, w + W, ...), tables are
-// [entry][32 samples].  Every index (step record, map, bond product) is then
-// the same for a warp's lanes and every table access one 128-byte row, where
-// the lane-group form spends a warp's instructions on 32 / GL samples and, on
-// the many small tables, leaves most lanes idle: 426 M warp instructions against
-// 199 M for 4,096 samples of the n = 500 graph.  Costs two barriers a step.
-// Bound by the steps' dependent chain: one CTA lasts ~400 steps whatever the
-// batch.  Each entry's arithmetic, and so every result, is that of step_table.
+// Elimination by levels, lane = sample: 32 samples a CTA (tiles in turn), its
+// warps take the tasks of one level after the other.  A table has one consumer,
+// so the steps form a tree whose levels only need the level before: a plan of
+// ~400 steps has ~30 levels (n = 500 of degree 3), and a step done by one warp
+// needs no barrier inside (a lane only touches its own sample's column).  One
+// step after the other, with any split of a step's entries, the chain of ~400
+// steps' dependent reads and barriers set the time: 4,096 samples of that graph
+// at width 8 take 193 us (338 with d/dbeta) by levels, 433 (717) step by step
+// with the warps sharing a step's entries.  Every index is the same for a warp's
+// lanes and every table access one 128-byte row.  A large step is cut into
+// several tasks; their common scale follows after the level's barrier.  Tables
+// of two neighbouring levels at a time are live (130 KB of shared memory for
+// that graph).  What bounds it now: the levels' barriers (half of the stalls)
+// and the plan's first reads from L2.  Each entry's arithmetic, and so every
+// result, is that of step_table.
 // ---------------------------------------------------------------------------
-#define G2_MAXW 8
-// floats of a CTA: tables, fields of every step, and with d/dbeta the tables'
-// derivatives
-__host__ __device__ __forceinline__ size_t g2_main_floats(int arena, int steps) { return (size_t)(arena + steps) * 32; }
+#define LV_U 4
 
-// The entries x = el, el + W, ... of a step's table, the table's maximum taken
-// over the CTA's warps (red: two buffers of [warps][32], used in turn).
-template <bool DB, int NIN, int COL, bool ZERO>
-__device__ __forceinline__ int step_rows(const Step& r, const GenDev& G, const float (&fv)[2], const float (&fr)[2],
-                                         float* A, float* dA, float* Ab, int el, int W, int lane, float* red) {
-  constexpr int U = DB && NIN >= 3 ? GEN_U / 2 : GEN_U;
-  const int M = 1 << r.m, E = 2 * M;
-  const float* pp = G.pp + r.ppo;
-  const float* pd = G.pp + G.n_pp + r.ppo;
-  const unsigned short* mp = G.map + r.mo;
-  const bool regs = M <= W * U;
-  float* out = A + r.out * 32;
-  float* dout = DB ? dA + r.out * 32 : nullptr;
-  float av[U], dv[U];
-  float mx = 0.f;
-  for (int x0 = el; x0 < M; x0 += W * U) {
+// Scratch floats of a CTA of the level kernels.
+__host__ __device__ __forceinline__ size_t general_levels_cta_floats(int live, int steps, bool db, int place) {
+  return (size_t)steps * 64 + ((place & 1) ? 0 : (size_t)live * 32) + (db && !(place & 2) ? (size_t)live * 32 : 0);
+}
+__host__ __device__ __forceinline__ size_t general_levels_dJ_cta_floats(int total, int live, int gmax, int steps,
+                                                                        int place) {
+  return (size_t)steps * 64 + ((place & 1) ? 0 : (size_t)gmax * 32) + ((place & 2) ? 0 : (size_t)live * 32) +
+         ((place & 4) ? 0 : (size_t)total * 32);
+}
+
+// A task's record, one int a lane; field i.
+__device__ __forceinline__ int field(int rec, int i) { return __shfl_sync(0xffffffffu, rec, i); }
+
+// The entries x0 .. x0 + nx - 1 of a step's table (in: the inputs' tables;
+// nin >= 4: through lin), unscaled where nx > U or the step is cut.  Returns
+// the largest.  fin: scale them here, by the returned maximum.
+template <bool DB, int NIN, int U>
+__device__ __forceinline__ float level_entries(const GenDev& G, int m, int nin, int ppo, int mo, int out, const int (&in)[3],
+                                               const int* lin, int x0, int nx, const float (&fv)[2],
+                                               const float (&fr)[2], float* A, float* dA, bool fin) {
+  const int E = 2 << m, x1 = x0 + nx;
+  const float* pp = G.pp + ppo;
+  const float* pd = G.pp + G.n_pp + ppo;
+  const unsigned short* mp = G.map + mo;
+  float* oA = A + out * 32;
+  float* oD = DB ? dA + out * 32 : nullptr;
+  float av[U], dv[U], mx = 0.f;
+  for (int xb = x0; xb < x1; xb += U) {
     float p[U][2], rr[U][2];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const int x = x0 + u * W < M ? x0 + u * W : x0;
+      const int x = min(xb + u, x1 - 1);
 #pragma unroll
       for (int sg = 0; sg < 2; ++sg) {
-        p[u][sg] = __ldg(pp + (x | (sg << r.m)));
-        rr[u][sg] = DB ? __ldg(pd + (x | (sg << r.m))) : 0.f;
+        p[u][sg] = __ldg(pp + (x | (sg << m)));
+        rr[u][sg] = DB ? __ldg(pd + (x | (sg << m))) : 0.f;
       }
     }
     if constexpr (NIN >= 0) {
@@ -461,17 +470,17 @@ __device__ __forceinline__ int step_rows(const Step& r, const GenDev& G, const f
       for (int i = 0; i < NIN; ++i)
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-          const int x = x0 + u * W < M ? x0 + u * W : x0;
+          const int x = min(xb + u, x1 - 1);
 #pragma unroll
           for (int sg = 0; sg < 2; ++sg) {
-            const int q = (r.in[i] + __ldg(mp + i * E + (x | (sg << r.m)))) * 32;
+            const int q = (in[i] + __ldg(mp + i * E + (x | (sg << m)))) * 32;
             val[i][u][sg] = A[q];
             if (DB) dval[i][u][sg] = dA[q];
           }
         }
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        if (DB && x0 + u * W >= M) continue;  // no divisions for what is dropped (the same for the whole warp)
+        if (DB && u >= nx) continue;  // no divisions for what is dropped
 #pragma unroll
         for (int sg = 0; sg < 2; ++sg) {
           p[u][sg] = fv[sg] * p[u][sg];
@@ -486,14 +495,13 @@ __device__ __forceinline__ int step_rows(const Step& r, const GenDev& G, const f
     } else {
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        const int x = x0 + u * W;
-        if (x >= M) continue;
+        const int x = min(xb + u, x1 - 1);
 #pragma unroll
         for (int sg = 0; sg < 2; ++sg) {
           p[u][sg] = fv[sg] * p[u][sg];
           if (DB) rr[u][sg] = fr[sg] + rr[u][sg];
-          for (int i = 0; i < r.nin; ++i) {
-            const int q = (G.fprog[r.f + 9 + 3 * i + COL] + mp[i * E + (x | (sg << r.m))]) * 32;
+          for (int i = 0; i < nin; ++i) {
+            const int q = (lin[2 * i] + mp[i * E + (x | (sg << m))]) * 32;
             const float v = A[q];
             p[u][sg] *= v;
             if (DB) rr[u][sg] += dA[q] / v;
@@ -503,68 +511,34 @@ __device__ __forceinline__ int step_rows(const Step& r, const GenDev& G, const f
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const int x = x0 + u * W;
-      av[u] = dv[u] = 0.f;
-      if (x >= M) continue;
+      const int x = xb + u;
       av[u] = __fadd_rn(p[u][0], p[u][1]);  // the products' own rounding: not contracted into the last one
       if (DB) dv[u] = fmaf(p[u][1], rr[u][1], p[u][0] * rr[u][0]);
+      if (x >= x1) continue;
       mx = fmaxf(mx, av[u]);
-      if (!regs) {
-        out[x * 32] = av[u];
-        if (DB) dout[x * 32] = dv[u];
+      if (nx > U || !fin) {
+        oA[x * 32] = av[u];
+        if (DB) oD[x * 32] = dv[u];
       }
     }
   }
-  if (W > 1) {
-    red[el * 32 + lane] = mx;
-    __syncthreads();
-    mx = red[lane];
-    const int nw = min(W, M);  // warps that held entries
-    for (int w = 1; w < nw; ++w) mx = fmaxf(mx, red[w * 32 + lane]);
-  }
-  const int e = exponent_of(mx);
-  const float sc = pow2i(-e);
-  if (regs) {
+  if (!fin) return mx;
+  const float sc = pow2i(-exponent_of(mx));
+  if (nx <= U) {
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const int x = el + u * W;
-      if (x >= M) continue;
-      out[x * 32] = av[u] * sc;
-      if (DB) dout[x * 32] = dv[u] * sc;
-      if (ZERO) Ab[(r.out + x) * 32] = 0.f;
+      if (u >= nx) continue;
+      oA[(x0 + u) * 32] = av[u] * sc;
+      if (DB) oD[(x0 + u) * 32] = dv[u] * sc;
     }
   } else {
 #pragma unroll 4
-    for (int x = el; x < M; x += W) {
-      out[x * 32] *= sc;
-      if (DB) dout[x * 32] *= sc;
-      if (ZERO) Ab[(r.out + x) * 32] = 0.f;
+    for (int x = x0; x < x1; ++x) {
+      oA[x * 32] *= sc;
+      if (DB) oD[x * 32] *= sc;
     }
   }
-  return e;
-}
-template <bool DB, int COL, bool ZERO>
-__device__ __forceinline__ int step_rows_any(const Step& r, const GenDev& G, const float (&fv)[2],
-                                             const float (&fr)[2], float* A, float* dA, float* Ab, int el, int W,
-                                             int lane, float* red) {
-  switch (r.nin) {
-    case 0: return step_rows<DB, 0, COL, ZERO>(r, G, fv, fr, A, dA, Ab, el, W, lane, red);
-    case 1: return step_rows<DB, 1, COL, ZERO>(r, G, fv, fr, A, dA, Ab, el, W, lane, red);
-    case 2: return step_rows<DB, 2, COL, ZERO>(r, G, fv, fr, A, dA, Ab, el, W, lane, red);
-    case 3: return step_rows<DB, 3, COL, ZERO>(r, G, fv, fr, A, dA, Ab, el, W, lane, red);
-    default: return step_rows<DB, -1, COL, ZERO>(r, G, fv, fr, A, dA, Ab, el, W, lane, red);
-  }
-}
-
-// The fields of component steps [g0, g0 + nsteps) into h[step * 32] (this
-// sample's column), the steps shared out over the warps.
-__device__ __forceinline__ void step_fields(const GenDev& G, int g0, int nsteps, const int8_t* s, float* h, int el,
-                                            int W) {
-#pragma unroll 2
-  for (int st = el; st < nsteps; st += W) {
-    const int* F = G.fprog + G.fstep[g0 + st];
-    h[st * 32] = field_of(G, F[1], F[2], s);
-  }
+  return mx;
 }
 
 // A read that only brings its line into L1; landed() ends its wait.
@@ -574,99 +548,198 @@ __device__ __forceinline__ int touch(const void* p) {
   return v;
 }
 __device__ __forceinline__ void landed(int v) { asm volatile("" ::"r"(v)); }
-
-// li.tile = 32; place: bit 0 tables and fields in shared memory, bit 1 the
-// derivatives too, else in this CTA's slice of gscr.
+// Touch what the task of record rec reads first, a line a lane: bond products,
+// maps, fields.  A plan's data is read once per tile, so without this every
+// task starts with a chain of L2 reads.
 template <bool DB>
-__global__ void __launch_bounds__(32 * G2_MAXW, 2) general_rows_kernel(const InstDev* __restrict__ inst,
-                                                                       const LaunchInfo li, int arena, int steps,
-                                                                       int place, const int8_t* __restrict__ spins,
-                                                                       double* __restrict__ logZR,
-                                                                       double* __restrict__ dbeta,
-                                                                       float* __restrict__ gscr) {
-  extern __shared__ float sm[];
-  __shared__ float red[2][G2_MAXW * 32];
-  const int k = find_inst(li, blockIdx.x);
-  const InstDev& I = inst[k];
-  if (I.kind != 2) return;
-  const int lane = threadIdx.x & 31, el = threadIdx.x >> 5, W = blockDim.x >> 5;
-  const int b0 = (blockIdx.x - li.tile_begin[k]) * 32, b = b0 + lane;
-  const float beta = (float)li.beta[k];
-  const int D = I.D, Dp = padded_bytes(D);
-  const size_t mf = g2_main_floats(arena, steps), df = (size_t)arena * 32;
-  const size_t per = ((place & 1) ? 0 : mf) + (DB && !(place & 2) ? df : 0);
-  float* sp = sm;
-  float* gp = gscr + (size_t)blockIdx.x * per;
-  float* A;
-  if (place & 1) A = sp, sp += mf;
-  else A = gp, gp += mf;
-  float* dA = nullptr;
-  if (DB) {
-    if (place & 2) dA = sp, sp += df;
-    else dA = gp;
-  }
-  float* h = A + (size_t)arena * 32 + lane;
-  A += lane;
-  if (DB) dA += lane;
-  int8_t* ssp = reinterpret_cast<int8_t*>(sp);
-  const GenDev& G = I.gen;
-  stage_spins(ssp, spins + I.spin_units * li.batch + (long long)b0 * D, min(32, li.batch - b0), 32, D, Dp);
-  __syncthreads();
-  const int8_t* s = ssp + lane * Dp;
-  const bool tab = li.gen_tab && G.n_tab > 0 && G.n_tab <= li.batch;  // tables built for this call
-  double lz = 0.0, dl = 0.0;
-  int par = 0;
-  for (int c = 0; c < G.n_comp; ++c) {
-    const int* cr = G.ctab + 5 * c;
-    if (tab && cr[4] >= 0) {  // a tabulated component: one lookup
-      const int x = boundary_index(G, cr, s);
-      lz += G.tab_lz[cr[4] + x];
-      if (DB) dl += G.tab_db[cr[4] + x];
-      continue;
+__device__ __forceinline__ int touch_task(const GenDev& G, int rec, int lane) {
+  const int w0 = field(rec, 0), m = w0 & 255, nin = (w0 >> 8) & 255, M = 1 << m, x = field(rec, 6) + (lane & 1) * M;
+  const int ppo = field(rec, 2), mo = field(rec, 3), fb = field(rec, 8), fc = field(rec, 9);
+  const int j = lane >> 1;
+  const void* p = nullptr;
+  if (j == 0) p = G.pp + ppo + x;
+  else if (j == 1) p = DB ? G.pp + G.n_pp + ppo + x : nullptr;
+  else if (j == 2) p = fc == 0 ? nullptr : (lane & 1) ? static_cast<const void*>(G.fldJ + fb) : G.fld + 2 * fb;
+  else if (j - 3 < nin && j < 9) p = G.map + mo + (j - 3) * 2 * M + x;
+  return p ? touch(p) : 0;
+}
+
+// One level after the other, into A (and dA): FULL every table's own place,
+// otherwise the level arena.  he[step]: this sample's field and the table's
+// exponent.  red: the cut steps' maxima.  skip: leave out tabulated components.
+// A, dA, he and red point at this lane's column.
+template <bool DB, bool FULL>
+__device__ __forceinline__ void level_sweep(const GenDev& G, const int8_t* s, float beta, float* A, float* dA,
+                                            float2* he, float* red, bool skip, int wi, int NW, int lane) {
+  const int t_end = G.n_lev > 0 ? G.llev[3 * G.n_lev - 1] : 0;
+  auto record = [&](int t) {
+    return t < t_end && lane < TNVAN_LTASK ? __ldg(G.ltask + (size_t)t * TNVAN_LTASK + lane) : 0;
+  };
+  int first = record(wi);
+  for (int l = 0; l < G.n_lev; ++l) {
+    const int t0 = G.llev[3 * l], tc = G.llev[3 * l + 1], t1 = G.llev[3 * l + 2];
+    int nxt = first, far = record(t0 + wi + NW);
+    first = record(t1 + wi);  // of the next level
+    for (int t = t0 + wi; t < t1; t += NW) {
+      const int rec = nxt;
+      nxt = far;
+      far = record(t + 2 * NW);
+      const int tc0 = t + NW < t1 ? touch_task<DB>(G, nxt, lane) : 0;
+      const int w0 = field(rec, 0), m = w0 & 255, nin = (w0 >> 8) & 255;
+      if (skip && (w0 >> 16)) continue;
+      const int ppo = field(rec, 2), mo = field(rec, 3), out = field(rec, FULL ? 5 : 4);
+      const int x0 = field(rec, 6), nx = field(rec, 7), slot = field(rec, 10);
+      const int in[3] = {field(rec, FULL ? 17 : 14), field(rec, FULL ? 18 : 15), field(rec, FULL ? 19 : 16)};
+      const float h = field_of(G, field(rec, 8), field(rec, 9), s), ah = fabsf(h);
+      const float fv[2] = {expf(beta * (h - ah)), expf(beta * (-h - ah))};
+      const float fr[2] = {h - ah, -h - ah};
+      const int* lin = G.lin + field(rec, 13) + (FULL ? 1 : 0);
+      const bool fin = slot < 0;
+      float mx;
+      constexpr int U3 = DB ? LV_U / 2 : LV_U;  // within 128 registers
+      if (nx <= 2) {
+        switch (nin) {
+          case 0: mx = level_entries<DB, 0, 2>(G, m, nin, ppo, mo, out, in, lin, x0, nx, fv, fr, A, dA, fin); break;
+          case 1: mx = level_entries<DB, 1, 2>(G, m, nin, ppo, mo, out, in, lin, x0, nx, fv, fr, A, dA, fin); break;
+          case 2: mx = level_entries<DB, 2, 2>(G, m, nin, ppo, mo, out, in, lin, x0, nx, fv, fr, A, dA, fin); break;
+          default: mx = level_entries<DB, -1, 2>(G, m, nin, ppo, mo, out, in, lin, x0, nx, fv, fr, A, dA, fin); break;
+        }
+      } else {
+        switch (nin) {
+          case 0: mx = level_entries<DB, 0, LV_U>(G, m, nin, ppo, mo, out, in, lin, x0, nx, fv, fr, A, dA, fin); break;
+          case 1: mx = level_entries<DB, 1, LV_U>(G, m, nin, ppo, mo, out, in, lin, x0, nx, fv, fr, A, dA, fin); break;
+          case 2: mx = level_entries<DB, 2, LV_U>(G, m, nin, ppo, mo, out, in, lin, x0, nx, fv, fr, A, dA, fin); break;
+          case 3: mx = level_entries<DB, 3, U3>(G, m, nin, ppo, mo, out, in, lin, x0, nx, fv, fr, A, dA, fin); break;
+          default: mx = level_entries<DB, -1, 2>(G, m, nin, ppo, mo, out, in, lin, x0, nx, fv, fr, A, dA, fin); break;
+        }
+      }
+      const int step = field(rec, 1);
+      if (fin) {
+        he[step * 32] = make_float2(h, __int_as_float(exponent_of(mx)));
+      } else {
+        const int ch = field(rec, 11) >> 16;
+        red[(slot + ch) * 32] = mx;
+        if (ch == 0) he[step * 32].x = h;
+      }
+      landed(tc0);
     }
-    const int* H = G.fprog + G.fhdr[c];
-    const int nsteps = H[0], fin = H[1], g0 = G.comp_step0[c];
-    step_fields(G, g0, nsteps, s, h, el, W);
+    landed(t1 + wi < t_end ? touch_task<DB>(G, first, lane) : 0);
     __syncthreads();
-    int esum = 0;
-    float hs = 0.f, hc = 0.f;  // as run_component
-    StepBlock blk, nxt = load_block<0>(G, g0 + min(lane, nsteps - 1));
-    for (int st = 0; st < nsteps; ++st) {
-      const int j = st & 31;
-      if (j == 0) {
-        blk = nxt;
-        nxt = load_block<0>(G, g0 + min(st + 32 + lane, nsteps - 1));
+    if (tc == t0) continue;
+    for (int t = t0 + wi; t < tc; t += NW) {  // the cut steps' scales
+      const int rec = lane < TNVAN_LTASK ? __ldg(G.ltask + (size_t)t * TNVAN_LTASK + lane) : 0;
+      if (skip && (field(rec, 0) >> 16)) continue;
+      const int out = field(rec, FULL ? 5 : 4), x0 = field(rec, 6), nx = field(rec, 7);
+      const int slot = field(rec, 10), nch = field(rec, 11) & 0xffff, ch = field(rec, 11) >> 16, step = field(rec, 1);
+      float mx = red[slot * 32];
+      for (int j = 1; j < nch; ++j) mx = fmaxf(mx, red[(slot + j) * 32]);
+      const int e = exponent_of(mx);
+      const float sc = pow2i(-e);
+      if (ch == 0) he[step * 32].y = __int_as_float(e);
+#pragma unroll 4
+      for (int x = x0; x < x0 + nx; ++x) {
+        A[(out + x) * 32] *= sc;
+        if (DB) dA[(out + x) * 32] *= sc;
       }
-      const Step r = block_step(blk, j, 32);
-      const float hv = h[st * 32], ah = fabsf(hv);
-      {
-        const float y = ah - hc;
-        const float t2 = hs + y;
-        hc = (t2 - hs) - y;
-        hs = t2;
+    }
+    __syncthreads();
+  }
+}
+
+// place: bit 0 A in shared memory, bit 1 dA too, else in this CTA's slice of
+// gscr (as he always is).  tiles: li's CTAs, taken in turn by the launched ones.
+template <bool DB>
+__global__ void __launch_bounds__(512, 1) general_levels_kernel(const InstDev* __restrict__ inst, const LaunchInfo li,
+                                                                int live, int steps, int red_slots, int place,
+                                                                const int8_t* __restrict__ spins,
+                                                                double* __restrict__ logZR, double* __restrict__ dbeta,
+                                                                float* __restrict__ gscr) {
+  extern __shared__ float sm[];
+  __shared__ double term[16][32], dterm[DB ? 16 : 1][32];
+  const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5, NW = blockDim.x >> 5;
+  const size_t af = (size_t)live * 32;
+  float* sp = sm;
+  float* gp = gscr + (size_t)blockIdx.x * general_levels_cta_floats(live, steps, DB, place);
+  float2* he = reinterpret_cast<float2*>(gp) + lane;
+  gp += (size_t)steps * 64;
+  float* A;
+  float* dA = nullptr;
+  if (place & 1) A = sp, sp += af;
+  else A = gp, gp += af;
+  if (DB) {
+    if (place & 2) dA = sp, sp += af;
+    else dA = gp;
+    dA += lane;
+  }
+  A += lane;
+  float* red = sp + lane;
+  int8_t* ssp = reinterpret_cast<int8_t*>(sp + (size_t)red_slots * 32);
+  for (int blk = blockIdx.x; blk < li.tile_begin[li.n_inst]; blk += gridDim.x) {
+    const int k = find_inst(li, blk);
+    const InstDev& I = inst[k];
+    const GenDev& G = I.gen;
+    const int b0 = (blk - li.tile_begin[k]) * 32, b = b0 + lane;
+    const float beta = (float)li.beta[k];
+    const int D = I.D, Dp = padded_bytes(D);
+    stage_spins(ssp, spins + I.spin_units * li.batch + (long long)b0 * D, min(32, li.batch - b0), 32, D, Dp);
+    __syncthreads();
+    const int8_t* s = ssp + lane * Dp;
+    const bool tab = li.gen_tab && G.n_tab > 0 && G.n_tab <= li.batch;  // tables built for this call
+    if (!tab || G.n_tabc < G.n_comp) level_sweep<DB, false>(G, s, beta, A, dA, he, red, tab, wi, NW, lane);
+    double lz = 0.0, dl = 0.0;
+    for (int c0 = 0; c0 < G.n_comp; c0 += NW) {  // the components' terms, added up in their order
+      const int c = c0 + wi;
+      if (c < G.n_comp) {
+        const int* cr = G.ctab + 5 * c;
+        if (tab && cr[4] >= 0) {  // a tabulated component: one lookup
+          const int x = boundary_index(G, cr, s);
+          term[wi][lane] = G.tab_lz[cr[4] + x];
+          if (DB) dterm[wi][lane] = G.tab_db[cr[4] + x];
+        } else {
+          const int g0 = G.comp_step0[c], g1 = G.comp_step0[c + 1], z0 = G.lroot[2 * c];
+          int esum = 0;
+          float hs = 0.f, hc = 0.f;  // as run_component
+          for (int g = g0; g < g1; g += 8) {
+            float2 q[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) q[j] = he[min(g + j, g1 - 1) * 32];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+              if (g + j >= g1) break;
+              const float y = fabsf(q[j].x) - hc;
+              const float t2 = hs + y;
+              hc = (t2 - hs) - y;
+              hs = t2;
+              esum += __float_as_int(q[j].y);
+            }
+          }
+          const double hsum = (double)hs - (double)hc;
+          const float z = A[z0 * 32];
+          term[wi][lane] = (double)beta * hsum + (double)esum * 0.69314718055994530942 + (double)logf(z);
+          if (DB) dterm[wi][lane] = hsum + (double)(dA[z0 * 32] / z);
+        }
       }
-      const float fv[2] = {expf(beta * (hv - ah)), expf(beta * (-hv - ah))};
-      const float fr[2] = {hv - ah, -hv - ah};
-      esum += step_rows_any<DB, 0, false>(r, G, fv, fr, A, dA, nullptr, el, W, lane, red[par]);
-      par ^= 1;
+      __syncthreads();
+      if (wi == 0)
+        for (int j = 0; j < min(NW, G.n_comp - c0); ++j) {
+          lz += term[j][lane];
+          if (DB) dl += dterm[j][lane];
+        }
       __syncthreads();
     }
-    const double hsum = (double)hs - (double)hc;
-    const float z = A[fin * 32];
-    lz += (double)beta * hsum + (double)esum * 0.69314718055994530942 + (double)logf(z);
-    if (DB) dl += hsum + (double)(dA[fin * 32] / z);
-    __syncthreads();  // the tables and fields are free for the next component
+    if (wi == 0 && b < li.batch) {
+      float e1 = 0.f;
+      for (int e = 0; e < I.n_ww; ++e) {
+        const EdgeWW q = I.ww[e];
+        e1 = fmaf(q.J, (float)(s[q.a] * s[q.b]), e1);
+      }
+      const double chf = G.c_hat;
+      const long long o = (long long)k * li.batch + b;
+      if (logZR) logZR[o] = lz + li.beta[k] * (chf + (double)e1);
+      if (DB) dbeta[o] = dl + chf + (double)e1;
+    }
+    __syncthreads();  // spins free for the next tile
   }
-  if (el != 0 || b >= li.batch) return;
-  float e1 = 0.f;
-  for (int e = 0; e < I.n_ww; ++e) {
-    const EdgeWW q = I.ww[e];
-    e1 = fmaf(q.J, (float)(s[q.a] * s[q.b]), e1);
-  }
-  const double chf = G.c_hat;
-  const long long o = (long long)k * li.batch + b;
-  if (logZR) logZR[o] = lz + li.beta[k] * (chf + (double)e1);
-  if (DB) dbeta[o] = dl + chf + (double)e1;
 }
 
 // The tables of the tabulated components (at most TNVAN_TAB_MAX_K width-set
@@ -986,89 +1059,98 @@ __global__ void __launch_bounds__(128, U0 > 1 ? 4 : 8) general_dJ_kernel(const I
 }
 
 // ---------------------------------------------------------------------------
-// The reverse sweep with lane = sample (see general_rows_kernel), 32 samples
-// and 16 warps per CTA.  general_dJ_kernel's order of every sum is kept, so
-// d/dJ has the same bits in both forms: a bond's sum over a step's entries is
-// made of W (4 or 8, that kernel's lanes per sample) chains x = w, w + W, ...,
-// each added over the 32 / W samples of a group, then over the chains by the
-// same tree, the groups' rows in turn into one row per 128 / W samples.
-//
-// Tables and adjoints (1.3 MB for 32 samples of the n = 500 graph) stay in
-// global memory, i.e. L2, so a step is a chain of dependent L2 reads: record ->
-// maps -> tables -> g -> adjoints.  The next step's record, bond products, maps
-// and table rows are therefore read into L1 a step ahead (touch), and all 16
-// warps share out the extended indices, the bonds and the gathered entries.
-// 4,096 samples of the n = 500 graph, width 8: 1,769 us against 2,380 in the
-// lane-group form; without the reads ahead and with W warps only, 2,287.
+// The reverse sweep by levels (see general_levels_kernel): a forward sweep keeps
+// every table, then from the last level back the g values of a level's steps,
+// and after a barrier its bonds and its inputs' adjoints, each a warp's task.
+// general_dJ_kernel's order of every sum is kept, so d/dJ has the same bits in
+// both forms: a bond's sum over a step's entries is made of W (that kernel's
+// lanes per sample: 2, 4 or 8) chains x = w, w + W, ..., each added over the
+// 32 / W samples of a group, then over the chains by the same tree, into the
+// group's row; levels_dJ_reduce_kernel adds four groups' rows in turn, as that
+// kernel's CTA did.  An edge has one bond in the plan, so rows are written, not
+// added to.
 // ---------------------------------------------------------------------------
-#define G2_DJ_WARPS 16
 
-// Touch what step r will read: threads 0-31 bond products, 32-127 n_maps maps
-// of its extended indices, 128 and 129 its record, and each thread a row of its
-// inputs' tables (T) and, with ADJ, of their adjoints.
-struct Touched {
-  int a, b, c;
-};
-template <bool ADJ>
-__device__ __forceinline__ Touched touch_step(const GenDev& G, const Step& r, const int (&kk)[3], int n_maps,
-                                              const float* A, const float* Ab, int t) {
-  const int E = 2 << r.m;
-  Touched v = {0, 0, 0};
-  if (t < 32) {
-    if (t * 32 < E + 32) v.a = touch(G.pp + r.ppo + min(t * 32, E - 1));
-  } else if (t < 128) {
-    const int nm = n_maps * E, o = (t - 32) * 64;
-    if (nm > 0 && o < nm + 64) v.a = touch(G.map + r.mo + min(o, nm - 1));
-  } else if (ADJ && t < 130) {
-    v.a = touch(G.fprog + r.f + (t == 128 ? 0 : 8));
-  }
-  int q = t;
+// g of the extended indices of entries x0 .. x0 + nx - 1, into gb.
+template <int NIN>
+__device__ __forceinline__ void level_g(const GenDev& G, int m, int nin, int ppo, int mo, const int (&in)[3],
+                                        const int* lin, int x0, int nx, const float (&fv)[2], const float* A,
+                                        const float* Ab, float* gb, float scl) {
+  constexpr int U = NIN >= 0 && NIN <= 2 ? 4 : 2;
+  const int M = 1 << m, E = 2 * M, x1 = x0 + nx;
+  const float* pp = G.pp + ppo;
+  const unsigned short* mp = G.map + mo;
+  for (int xb = x0; xb < x1; xb += U) {
+    float p[U][2], ab[U], val[NIN > 0 ? NIN : 1][U][2];
 #pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    if (i >= r.nin) break;
-    const int n = 1 << kk[i];
-    if (q >= 0 && q < n) {
-      v.b = touch(A + (r.in[i] + q) * 32);
-      if (ADJ) v.c = touch(Ab + (r.in[i] + q) * 32);
+    for (int u = 0; u < U; ++u) {
+      const int x = min(xb + u, x1 - 1);
+      ab[u] = Ab[x * 32];
+#pragma unroll
+      for (int sg = 0; sg < 2; ++sg) {
+        p[u][sg] = __ldg(pp + (x | (sg << m)));
+#pragma unroll
+        for (int i = 0; i < NIN; ++i) val[i][u][sg] = A[(in[i] + __ldg(mp + i * E + (x | (sg << m)))) * 32];
+      }
     }
-    q -= n;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int x = xb + u;
+      if (x >= x1) continue;
+#pragma unroll
+      for (int sg = 0; sg < 2; ++sg) {
+        float v = fv[sg] * p[u][sg];
+        if constexpr (NIN >= 0) {
+#pragma unroll
+          for (int i = 0; i < NIN; ++i) v *= val[i][u][sg];
+        } else {
+          for (int i = 0; i < nin; ++i) v *= A[(lin[2 * i] + mp[i * E + (x | (sg << m))]) * 32];
+        }
+        gb[(x | (sg << m)) * 32] = (ab[u] * scl) * v;
+      }
+    }
   }
-  return v;
 }
 
-// g of the extended indices ext = w0, w0 + NW, ... of a step, into gb.
-template <int NIN>
-__device__ __forceinline__ void rows_g(const Step& r, const GenDev& G, const float (&fv)[2], const float* A,
-                                       const float* Ab, float* gb, float scl, int w0, int NW) {
-  const int M = 1 << r.m, E = 2 * M;
-  const float* pp = G.pp + r.ppo;
-  const unsigned short* mp = G.map + r.mo;
-  for (int e0 = w0; e0 < E; e0 += NW * GEN_U) {
-    float p[GEN_U], ab[GEN_U], val[NIN > 0 ? NIN : 1][GEN_U];
+// The adjoints of n entries of an input: each gathers the g of the R extended
+// indices that read it, in index order (RR = R: four entries' loads at once).
+template <int RR>
+__device__ __forceinline__ void gather_g(const float* g, const unsigned short* inv, const float* av, float* ab, int n,
+                                         int R) {
+  if constexpr (RR > 0) {
+    for (int e0 = 0; e0 < n; e0 += 4) {
+      float a[4], v[4][RR];
 #pragma unroll
-    for (int u = 0; u < GEN_U; ++u) {
-      const int ext = e0 + u * NW;
-      p[u] = ab[u] = 0.f;
+      for (int u = 0; u < 4; ++u) {
+        const int e = min(e0 + u, n - 1);
+        a[u] = av[e * 32];
 #pragma unroll
-      for (int i = 0; i < NIN; ++i) val[i][u] = 0.f;
-      if (ext >= E) continue;
-      p[u] = __ldg(pp + ext);
-      ab[u] = Ab[(r.out + (ext & (M - 1))) * 32];
-#pragma unroll
-      for (int i = 0; i < NIN; ++i) val[i][u] = A[(r.in[i] + __ldg(mp + i * E + ext)) * 32];
-    }
-#pragma unroll
-    for (int u = 0; u < GEN_U; ++u) {
-      const int ext = e0 + u * NW;
-      if (ext >= E) continue;
-      float v = ((ext >> r.m) & 1 ? fv[1] : fv[0]) * p[u];
-      if constexpr (NIN >= 0) {
-#pragma unroll
-        for (int i = 0; i < NIN; ++i) v *= val[i][u];
-      } else {
-        for (int i = 0; i < r.nin; ++i) v *= A[(G.fprog[r.f + 9 + 3 * i + 1] + mp[i * E + ext]) * 32];
+        for (int f = 0; f < RR; ++f) v[u][f] = g[__ldg(inv + e * RR + f) * 32];
       }
-      gb[ext * 32] = (ab[u] * scl) * v;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        if (e0 + u >= n) continue;
+        float sum = 0.f;
+#pragma unroll
+        for (int f = 0; f < RR; ++f) sum += v[u][f];
+        ab[(e0 + u) * 32] = a[u] > 0.f ? 0.f + sum / a[u] : 0.f;
+      }
+    }
+  } else {
+#pragma unroll 2
+    for (int e = 0; e < n; ++e) {
+      const float a = av[e * 32];
+      float sum = 0.f;
+      for (int f = 0; f + 4 <= R; f += 4) {
+        float v[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) v[j] = g[__ldg(inv + e * R + f + j) * 32];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) sum += v[j];
+      }
+      if (R < 4)
+        for (int f = 0; f < R; ++f) sum += g[inv[e * R + f] * 32];
+      ab[e * 32] = a > 0.f ? 0.f + sum / a : 0.f;
     }
   }
 }
@@ -1100,173 +1182,169 @@ __device__ __forceinline__ void bond_chains(const float* gb, int m, int pos, flo
     }
   }
 }
-// The chains, each times mul and added over the groups' samples, added up; into
-// edge e of each group's row (ne4 floats).
+// The chains, times wscale (and sgn), added over the groups' samples and over the
+// chains; to edge e of each group's row.
 template <int W>
-__device__ __forceinline__ void bond_add(const float (&v)[W], float wscale, float sgn, bool signed_, float* acc,
-                                         int ne4, int e, int lane) {
+__device__ __forceinline__ void bond_store(const float (&v)[W], float wscale, float sgn, bool field_bond, float* rows,
+                                           int stride, int e, int lane) {
   float u[W];
 #pragma unroll
   for (int w = 0; w < W; ++w) {
     const float q = wscale * v[w];
-    u[w] = group_samples<W>(signed_ ? q * sgn : q);
+    u[w] = group_samples<W>(field_bond ? q * sgn : q);
   }
-  if (W == 8) {
 #pragma unroll
-    for (int w = 0; w < 4; ++w) u[w] += u[w + W / 2];
-  }
-  u[0] += u[2];
-  u[1] += u[3];
-  const float sum = u[0] + u[1];
-  if (e >= 0 && (lane & (32 / W - 1)) == 0) acc[lane / (32 / W) * ne4 + e] += sum;
+  for (int o = W / 2; o >= 1; o >>= 1)
+#pragma unroll
+    for (int w = 0; w < o; ++w) u[w] += u[w + o];
+  if (e >= 0 && (lane & (32 / W - 1)) == 0) rows[(size_t)(lane / (32 / W)) * stride + e] = 0.f + u[0];
 }
 
-// Dynamic shared memory: g values [gmax][32], bond sums [W][n_edges], spins.
-// Tables, adjoints, scales and fields ((2 arena + 2 steps) x 32 floats) in this
-// CTA's slice of gscr.
+// place: bit 0 g values in shared memory, bit 1 the adjoints too, bit 2 the
+// tables too, else in this CTA's slice of gscr.  rows of part: W per tile.
 template <int W>
-__global__ void __launch_bounds__(32 * G2_DJ_WARPS, 1) general_rows_dJ_kernel(
-    const InstDev* __restrict__ inst, const LaunchInfo li, int arena, int steps, int gmax,
-    const int8_t* __restrict__ spins, float* __restrict__ part, int part_stride, float* __restrict__ gscr) {
+__global__ void __launch_bounds__(512, 1) general_levels_dJ_kernel(const InstDev* __restrict__ inst, const LaunchInfo li,
+                                                                   int total, int live, int gmax, int steps,
+                                                                   int red_slots, int place,
+                                                                   const int8_t* __restrict__ spins,
+                                                                   float* __restrict__ part, int part_stride,
+                                                                   float* __restrict__ gscr) {
   extern __shared__ float sm[];
-  __shared__ float red[2][G2_DJ_WARPS * 32];
-  const int k = find_inst(li, blockIdx.x);
-  const InstDev& I = inst[k];
-  if (I.kind != 2) return;
-  constexpr int NW = G2_DJ_WARPS;
-  const int t = threadIdx.x, lane = t & 31, wi = t >> 5;
-  const int c_idx = blockIdx.x - li.tile_begin[k];
-  const int b0 = c_idx * 32, b = b0 + lane;
-  const float beta = (float)li.beta[k];
-  const int D = I.D, Dp = padded_bytes(D), ne = I.n_edges, ne4 = (ne + 3) & ~3;
-  float* A0 = gscr + (size_t)blockIdx.x * (size_t)(2 * arena + 2 * steps) * 32;
-  float* A = A0 + lane;
-  float* Ab0 = A0 + (size_t)arena * 32;
-  float* Ab = Ab0 + lane;
-  float* sc = Ab + (size_t)arena * 32;
-  float* h = sc + (size_t)steps * 32;
-  float* gb = sm + lane;
-  float* acc = sm + gmax * 32;  // [W groups][ne4]
-  int8_t* ssp = reinterpret_cast<int8_t*>(acc + W * ne4);
-  const GenDev& G = I.gen;
-  for (int e = t; e < W * ne4; e += 32 * NW) acc[e] = 0.f;
-  stage_spins(ssp, spins + I.spin_units * li.batch + (long long)b0 * D, min(32, li.batch - b0), 32, D, Dp);
-  __syncthreads();
-  const int8_t* s = ssp + lane * Dp;
-  // per-sample weight of the bond sums (importance multipliers when given)
-  const float wscale =
-      b < li.batch ? beta / (float)li.batch * (li.wmul ? li.wmul[(long long)k * li.batch + b] : 1.f) : 0.f;
-  int par = 0;
-  for (int c = 0; c < G.n_comp; ++c) {
-    const int* H = G.fprog + G.fhdr[c];
-    const int nsteps = H[0], fin = H[2], g0 = G.comp_step0[c];
-    step_fields(G, g0, nsteps, s, h, wi, NW);
+  const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5, NW = blockDim.x >> 5;
+  float* sp = sm;
+  float* gp = gscr + (size_t)blockIdx.x * general_levels_dJ_cta_floats(total, live, gmax, steps, place);
+  float2* he = reinterpret_cast<float2*>(gp) + lane;
+  gp += (size_t)steps * 64;
+  auto take = [&](bool shared, int rows) {
+    float*& q = shared ? sp : gp;
+    float* r = q + lane;
+    q += (size_t)rows * 32;
+    return r;
+  };
+  float* gb = take(place & 1, gmax);
+  float* Ab = take(place & 2, live);
+  float* A = take(place & 4, total);
+  float* red = take(true, red_slots);
+  int8_t* ssp = reinterpret_cast<int8_t*>(sp);
+  for (int blk = blockIdx.x; blk < li.tile_begin[li.n_inst]; blk += gridDim.x) {
+    const int k = find_inst(li, blk);
+    const InstDev& I = inst[k];
+    const GenDev& G = I.gen;
+    const int b0 = (blk - li.tile_begin[k]) * 32, b = b0 + lane;
+    const float beta = (float)li.beta[k];
+    const int D = I.D, Dp = padded_bytes(D);
+    float* rows = part + (size_t)blk * W * part_stride;
+    for (int e = threadIdx.x; e < W * part_stride; e += blockDim.x) rows[e] = 0.f;
+    stage_spins(ssp, spins + I.spin_units * li.batch + (long long)b0 * D, min(32, li.batch - b0), 32, D, Dp);
     __syncthreads();
-    const float fr[2] = {0.f, 0.f};
-    int kk[3];
-    {
-      StepBlock blk = load_block<1>(G, g0 + min(lane, nsteps - 1)), nxt = blk;
-      float hv = h[0];
-      for (int st = 0; st < nsteps; ++st) {
-        const int j = st & 31;
-        if (j == 0) {
-          blk = nxt;
-          nxt = load_block<1>(G, g0 + min(st + 32 + lane, nsteps - 1));
+    const int8_t* s = ssp + lane * Dp;
+    // per-sample weight of the bond sums (importance multipliers when given)
+    const float wscale =
+        b < li.batch ? beta / (float)li.batch * (li.wmul ? li.wmul[(long long)k * li.batch + b] : 1.f) : 0.f;
+    level_sweep<false, true>(G, s, beta, A, nullptr, he, red, false, wi, NW, lane);
+    for (int c = wi; c < G.n_comp; c += NW) Ab[G.lroot[2 * c] * 32] = 1.f / A[G.lroot[2 * c + 1] * 32];
+    __syncthreads();
+    auto level_first = [&](int l) {  // this warp's first task of level l
+      const int t = l < 0 ? 0 : G.llev[3 * l] + wi;
+      return l >= 0 && t < G.llev[3 * l + 2] && lane < TNVAN_LTASK ? __ldg(G.ltask + (size_t)t * TNVAN_LTASK + lane) : 0;
+    };
+    int first = level_first(G.n_lev - 1);
+    for (int l = G.n_lev - 1; l >= 0; --l) {
+      const int t0 = G.llev[3 * l], t1 = G.llev[3 * l + 2];
+      auto record = [&](int t) {
+        return t < t1 && lane < TNVAN_LTASK ? __ldg(G.ltask + (size_t)t * TNVAN_LTASK + lane) : 0;
+      };
+      int nxt = first, far = record(t0 + wi + NW);
+      for (int t = t0 + wi; t < t1; t += NW) {
+        const int rec = nxt;
+        nxt = far;
+        far = record(t + 2 * NW);
+        const int tc0 = t + NW < t1 ? touch_task<false>(G, nxt, lane) : 0;
+        const int w0 = field(rec, 0), m = w0 & 255, nin = (w0 >> 8) & 255;
+        const int ppo = field(rec, 2), mo = field(rec, 3), x0 = field(rec, 6), nx = field(rec, 7);
+        const int in[3] = {field(rec, 17), field(rec, 18), field(rec, 19)};
+        const int* lin = G.lin + field(rec, 13) + 1;
+        const float2 q = he[field(rec, 1) * 32];
+        const float h = q.x, ah = fabsf(h), scl = pow2i(-__float_as_int(q.y));
+        const float fv[2] = {expf(beta * (h - ah)), expf(beta * (-h - ah))};
+        const float* ab = Ab + field(rec, 4) * 32;
+        float* g = gb + field(rec, 12) * 32;
+        switch (nin) {
+          case 0: level_g<0>(G, m, nin, ppo, mo, in, lin, x0, nx, fv, A, ab, g, scl); break;
+          case 1: level_g<1>(G, m, nin, ppo, mo, in, lin, x0, nx, fv, A, ab, g, scl); break;
+          case 2: level_g<2>(G, m, nin, ppo, mo, in, lin, x0, nx, fv, A, ab, g, scl); break;
+          case 3: level_g<3>(G, m, nin, ppo, mo, in, lin, x0, nx, fv, A, ab, g, scl); break;
+          default: level_g<-1>(G, m, nin, ppo, mo, in, lin, x0, nx, fv, A, ab, g, scl); break;
         }
-        const Step r = block_step(blk, j, 32);
-        const Step rn = block_step(j == 31 ? nxt : blk, (j + 1) & 31, 32);
-        next_widths(j == 31 ? nxt : blk, (j + 1) & 31, kk);
-        const float hn = h[min(st + 1, nsteps - 1) * 32], ah = fabsf(hv);
-        const Touched tc = touch_step<false>(G, rn, kk, rn.nin, A0, Ab0, t);
-        const float fv[2] = {expf(beta * (hv - ah)), expf(beta * (-hv - ah))};
-        const int e = step_rows_any<false, 1, true>(r, G, fv, fr, A, nullptr, Ab, wi, NW, lane, red[par]);
-        par ^= 1;
-        if (wi == 0) sc[st * 32] = pow2i(-e);
-        hv = hn;
-        landed(tc.a), landed(tc.b);
-        __syncthreads();
-      }
-    }
-    if (wi == 0) Ab[fin * 32] = 1.f / A[fin * 32];
-    __syncthreads();
-    StepBlock blk, nxt = load_block<1>(G, g0 + max(nsteps - 1 - lane, 0));
-    float hv = h[(nsteps - 1) * 32], scl = sc[(nsteps - 1) * 32];
-    for (int st = nsteps - 1, j0 = 0; st >= 0; --st, ++j0) {
-      const int jb = j0 & 31;
-      if (jb == 0) {
-        blk = nxt;
-        nxt = load_block<1>(G, g0 + max(st - 32 - lane, 0));
-      }
-      const Step r = block_step(blk, jb, 32);
-      const Step rn = block_step(jb == 31 ? nxt : blk, (jb + 1) & 31, 32);
-      next_widths(jb == 31 ? nxt : blk, (jb + 1) & 31, kk);
-      const float hn = h[max(st - 1, 0) * 32], scn = sc[max(st - 1, 0) * 32], ah = fabsf(hv);
-      const Touched tc = touch_step<true>(G, rn, kk, 2 * rn.nin, A0, Ab0, t);
-      const int* F = G.fprog + r.f;
-      const int fb = F[1], fc = F[2], np = min(F[4], TNVAN_MAX_ELIM_W);
-      const int* pr = F + 9 + 3 * r.nin;
-      const float fv[2] = {expf(beta * (hv - ah)), expf(beta * (-hv - ah))};
-      switch (r.nin) {
-        case 0: rows_g<0>(r, G, fv, A, Ab, gb, scl, wi, NW); break;
-        case 1: rows_g<1>(r, G, fv, A, Ab, gb, scl, wi, NW); break;
-        case 2: rows_g<2>(r, G, fv, A, Ab, gb, scl, wi, NW); break;
-        default: rows_g<-1>(r, G, fv, A, Ab, gb, scl, wi, NW); break;
+        landed(tc0);
       }
       __syncthreads();
-      // bonds, a warp each from the last warp on: one for the fields (if any),
-      // one for each pair
-      const int nq = np + (fc > 0);
-      for (int q = NW - 1 - wi; q < nq; q += NW) {
-        float v[W];
-        const int j = q - (fc > 0);
-        if (j < 0) {
-          bond_chains<W>(gb, r.m, -1, v);
-          for (int f = 0; f < fc; ++f)
-            bond_add<W>(v, wscale, (float)s[G.fld[2 * (fb + f)]], true, acc, ne4, G.fld[2 * (fb + f) + 1], lane);
+      const int u0 = G.blev[2 * l], u1 = G.blev[2 * l + 1];
+      auto back = [&](int t) {
+        return t < u1 && lane < TNVAN_BTASK ? __ldg(G.btask + (size_t)t * TNVAN_BTASK + lane) : 0;
+      };
+      int bnxt = back(u0 + wi);
+      first = level_first(l - 1);
+      for (int t = u0 + wi; t < u1; t += NW) {
+        const int rec = bnxt;
+        bnxt = back(t + NW);
+        const int w0 = field(rec, 0), kind = w0 & 255, r1 = field(rec, 1), r3 = field(rec, 3), r4 = field(rec, 4);
+        const float* g = gb + field(rec, 2) * 32;
+        if (kind == 2) {  // input adjoints: each entry gathers the g of the extended indices that read it
+          const int R = w0 >> 8, e0 = field(rec, 6);
+          const unsigned short* inv = G.map + field(rec, 5);
+          float* ab = Ab + (r3 + e0) * 32;
+          const float* av = A + (r4 + e0) * 32;
+          if (R == 2) gather_g<2>(g, inv, av, ab, r1, R);
+          else if (R == 4) gather_g<4>(g, inv, av, ab, r1, R);
+          else gather_g<0>(g, inv, av, ab, r1, R);
         } else {
-          bond_chains<W>(gb, r.m, pr[2 * j + 1], v);
-          bond_add<W>(v, wscale, 1.f, false, acc, ne4, G.pairE[pr[2 * j]], lane);
-        }
-      }
-      // input adjoints: each entry gathers the g of the extended indices that read it
-      const int E = 2 << r.m;
-      const unsigned short* mp = G.map + r.mo;
-      for (int i = 0; i < r.nin; ++i) {
-        const int in = F[9 + 3 * i + 1], ki = F[9 + 3 * i + 2];
-        const int R = E >> ki;
-        const unsigned short* inv = mp + (r.nin + i) * E;
-#pragma unroll 2
-        for (int e = wi; e < (1 << ki); e += NW) {
-          const float av = A[(in + e) * 32];
-          float sum = 0.f;
-          for (int f = 0; f + 4 <= R; f += 4) {  // in index order, four loads in flight
-            float q[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) q[j] = gb[__ldg(inv + e * R + f + j) * 32];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) sum += q[j];
+          float v[W];
+          bond_chains<W>(g, r1, kind == 0 ? -1 : r3, v);
+          if (kind == 0) {
+            for (int f = r3; f < r3 + r4; ++f)
+              bond_store<W>(v, wscale, (float)s[G.fld[2 * f]], true, rows, part_stride, G.fld[2 * f + 1], lane);
+          } else {
+            bond_store<W>(v, wscale, 1.f, false, rows, part_stride, G.pairE[r4], lane);
           }
-          if (R < 4)
-            for (int f = 0; f < R; ++f) sum += gb[inv[e * R + f] * 32];
-          if (av > 0.f) Ab[(in + e) * 32] += sum / av;
         }
       }
-      hv = hn, scl = scn;
-      landed(tc.a), landed(tc.b), landed(tc.c);
+      landed(touch_task<false>(G, first, lane));
       __syncthreads();
     }
   }
-  // one row per 128 / W samples: its four groups in turn
-  const int rows = W / 4, n_rows = (li.batch + 128 / W - 1) / (128 / W);
-  const long long row0 = (long long)k * n_rows + (long long)c_idx * rows;
-  for (int q = 0; q < rows && c_idx * rows + q < n_rows; ++q) {
-    float* row = part + (row0 + q) * part_stride;
-    for (int e = t; e < ne; e += 32 * NW) {
-      float v = 0.f;
-      for (int w = 0; w < 4; ++w) v += acc[(4 * q + w) * ne4 + e];
-      row[e] = v;
-    }
+}
+
+// d/dJ from the group rows: 32 edges a CTA, 16 slices of the rows of four groups
+// each, added in slice order.
+template <int W>
+__global__ void __launch_bounds__(512) levels_dJ_reduce_kernel(const InstDev* __restrict__ inst, const LaunchInfo li,
+                                                               const float* __restrict__ part, int part_stride,
+                                                               double* __restrict__ dJ) {
+  __shared__ double acc[16][32];
+  const int k = blockIdx.y;
+  const InstDev& I = inst[k];
+  const int lane = threadIdx.x & 31, sl = threadIdx.x >> 5, e = blockIdx.x * 32 + lane;
+  if (I.kind != 2 || blockIdx.x * 32 >= I.n_edges) return;
+  const int ng = (li.tile_begin[k + 1] - li.tile_begin[k]) * W, nr = (ng + 3) / 4;
+  const float* p = part + (size_t)li.tile_begin[k] * W * part_stride + min(e, I.n_edges - 1);
+  const int r0 = (int)((long long)nr * sl / 16), r1 = (int)((long long)nr * (sl + 1) / 16);
+  double s = 0.0;
+#pragma unroll 4
+  for (int r = r0; r < r1; ++r) {
+    float q[4], v = 0.f;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) q[j] = 4 * r + j < ng ? p[(size_t)(4 * r + j) * part_stride] : 0.f;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v += q[j];
+    s += (double)v;
   }
+  acc[sl][lane] = s;
+  __syncthreads();
+  if (sl != 0 || e >= I.n_edges) return;
+  s = 0.0;
+  for (int j = 0; j < 16; ++j) s += acc[j][lane];
+  dJ[I.edge_off + e] += s;
 }
 
 __global__ void general_dJ_reduce_kernel(const InstDev* __restrict__ inst, const LaunchInfo li,
@@ -1315,47 +1393,69 @@ cudaError_t launch_general_dJ(const InstDev* d_inst, const LaunchInfo& li, int s
   return cudaGetLastError();
 }
 
-int general_rows_smem_bytes(int arena, int steps, int D, bool db, int place) {
+// Warps a CTA of the level kernels: a level's tasks, within 16; with more tiles
+// than SMs half or a quarter of them in as many more CTAs an SM, where the
+// shared memory allows it, so that one CTA's barriers are another's work.
+static int levels_warps(int nblk, int tasks, int smem_bytes) {
+  const int fit = 227 * 1024 / (smem_bytes + 10 * 1024);
+  int w = tasks > 8 ? 16 : 8;
+  while (w > 4 && nblk > 152 * (16 / w) && fit >= 2 * (16 / w)) w /= 2;
+  return w;
+}
+// CTAs that fit the chip at once: 128 registers a thread and the shared memory.
+static int levels_ctas(int nblk, int warps, int smem_bytes) {
+  const int per_sm = std::max(1, std::min(16 / warps, 227 * 1024 / (smem_bytes + 10 * 1024)));
+  return std::min(nblk, 152 * per_sm);
+}
+static int spin_bytes(int D) {
   int w4 = (D + 3) / 4;
   if ((w4 & 1) == 0) ++w4;
-  return (int)(4 * (((place & 1) ? g2_main_floats(arena, steps) : 0) + (db && (place & 2) ? (size_t)arena * 32 : 0))) +
-         32 * 4 * w4;
+  return 32 * 4 * w4;
 }
-size_t general_rows_scratch_floats(int arena, int steps, bool db, int place, int nblk) {
-  return (((place & 1) ? 0 : g2_main_floats(arena, steps)) + (db && !(place & 2) ? (size_t)arena * 32 : 0)) * nblk;
+int general_levels_smem_bytes(int live, int red_slots, int D, bool db, int place) {
+  return 128 * (((place & 1) ? live : 0) + (db && (place & 2) ? live : 0) + red_slots) + spin_bytes(D);
 }
-cudaError_t launch_general_rows(const InstDev* d_inst, const LaunchInfo& li, int smem_bytes, int W, int arena,
-                                int steps, int place, const int8_t* spins, double* logZR, double* dbeta, float* gscr,
-                                cudaStream_t s) {
+size_t general_levels_scratch_floats(int live, int steps, bool db, int place, int nblk, int tasks, int smem_bytes) {
+  return general_levels_cta_floats(live, steps, db, place) * levels_ctas(nblk, levels_warps(nblk, tasks, smem_bytes), smem_bytes);
+}
+cudaError_t launch_general_levels(const InstDev* d_inst, const LaunchInfo& li, int smem_bytes, int live, int steps,
+                                  int red_slots, int tasks, int place, const int8_t* spins, double* logZR,
+                                  double* dbeta, float* gscr, cudaStream_t s) {
   const int nblk = li.tile_begin[li.n_inst];
   if (nblk == 0) return cudaSuccess;
-  auto kern = dbeta ? general_rows_kernel<true> : general_rows_kernel<false>;
+  auto kern = dbeta ? general_levels_kernel<true> : general_levels_kernel<false>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
   if (e != cudaSuccess) return e;
-  kern<<<nblk, 32 * W, smem_bytes, s>>>(d_inst, li, arena, steps, place, spins, logZR, dbeta, gscr);
+  const int nw = levels_warps(nblk, tasks, smem_bytes);
+  kern<<<levels_ctas(nblk, nw, smem_bytes), 32 * nw, smem_bytes, s>>>(d_inst, li, live, steps, red_slots, place, spins,
+                                                                    logZR, dbeta, gscr);
   return cudaGetLastError();
 }
-
-int general_rows_dJ_smem_bytes(int D, int n_edges, int gmax, int W) {
-  int w4 = (D + 3) / 4;
-  if ((w4 & 1) == 0) ++w4;
-  return 4 * (gmax * 32 + W * ((n_edges + 3) & ~3)) + 32 * 4 * w4;
+int general_levels_dJ_smem_bytes(int total, int live, int gmax, int red_slots, int D, int place) {
+  return 128 * (((place & 1) ? gmax : 0) + ((place & 2) ? live : 0) + ((place & 4) ? total : 0) + red_slots) +
+         spin_bytes(D);
 }
-size_t general_rows_dJ_scratch_floats(int arena, int steps, int nblk) {
-  return (size_t)(2 * arena + 2 * steps) * 32 * nblk;
+size_t general_levels_dJ_scratch_floats(int total, int live, int gmax, int steps, int place, int nblk, int tasks,
+                                        int smem_bytes) {
+  return general_levels_dJ_cta_floats(total, live, gmax, steps, place) *
+         levels_ctas(nblk, levels_warps(nblk, tasks, smem_bytes), smem_bytes);
 }
-cudaError_t launch_general_rows_dJ(const InstDev* d_inst, const LaunchInfo& li, const LaunchInfo& lr, int smem_bytes,
-                                   int W, int arena, int steps, int gmax, const int8_t* spins, float* part,
-                                   int part_stride, double* dJ, float* gscr, cudaStream_t s) {
+cudaError_t launch_general_levels_dJ(const InstDev* d_inst, const LaunchInfo& li, int smem_bytes, int W, int total,
+                                     int live, int gmax, int steps, int red_slots, int tasks, int place, int max_edges,
+                                     const int8_t* spins, float* part, int part_stride, double* dJ, float* gscr,
+                                     cudaStream_t s) {
   const int nblk = li.tile_begin[li.n_inst];
   if (nblk == 0) return cudaSuccess;
-  auto kern = W == 8 ? general_rows_dJ_kernel<8> : general_rows_dJ_kernel<4>;
+  auto kern = W == 8 ? general_levels_dJ_kernel<8> : (W == 4 ? general_levels_dJ_kernel<4> : general_levels_dJ_kernel<2>);
+  auto red = W == 8 ? levels_dJ_reduce_kernel<8> : (W == 4 ? levels_dJ_reduce_kernel<4> : levels_dJ_reduce_kernel<2>);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
   if (e != cudaSuccess) return e;
-  kern<<<nblk, 32 * G2_DJ_WARPS, smem_bytes, s>>>(d_inst, li, arena, steps, gmax, spins, part, part_stride, gscr);
+  const int nw = levels_warps(nblk, tasks, smem_bytes);
+  kern<<<levels_ctas(nblk, nw, smem_bytes), 32 * nw, smem_bytes, s>>>(d_inst, li, total, live, gmax, steps, red_slots,
+                                                                    place, spins, part, part_stride, gscr);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  general_dJ_reduce_kernel<<<dim3(4, lr.n_inst), 256, 0, s>>>(d_inst, lr, part, part_stride, dJ);
+  red<<<dim3((max_edges + 31) / 32, li.n_inst), 512, 0, s>>>(d_inst, li, part, part_stride, dJ);
   return cudaGetLastError();
 }
 
