@@ -3446,9 +3446,11 @@ int contract_all(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* d
     // By levels where the kernel's buffers can be had (a capture allocates
     // nothing), whatever the sizes: from 33 to 32,768 samples of random regular
     // graphs (n = 128 to 500, widths 1 to 8) 1.1 to 6 times faster than groups of
-    // lanes, with one exception: d/dbeta of tables of 4 to 8 entries on average
+    // lanes, with two exceptions: d/dbeta of tables of 4 to 8 entries on average
     // over more than four rounds of CTAs (n = 500, width 4, 32,768 samples: 803 us
-    // by levels, 653 in lane groups).
+    // by levels, 653 in lane groups); and few steps left beside the components'
+    // tables (45 of 136 steps, 65,536 samples: 177 us by levels, 132 in lane
+    // groups; with 373 of 374 left 77 against 320).
     const LevelPlan lp = level_plan(ctx);
     LaunchInfo lw;
     if ((rc = fill_launch(ctx, betas, batch, 32, lw))) return rc;
@@ -3465,10 +3467,15 @@ int contract_all(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* d
       if (lsm <= LEVEL_SMEM || !place) break;
     }
     double mean = 1;
+    int untab = 0;  // steps left beside the tables
     for (const Instance& in : ctx->inst)
-      if (in.kind == 2) mean = std::max(mean, in.g_mean_entries);
+      if (in.kind == 2) {
+        mean = std::max(mean, in.g_mean_entries);
+        const bool tab = in.g_ntab > 0 && in.g_ntab <= batch;
+        untab = std::max(untab, tab ? in.gl_untab : (int)in.gfstep.size());
+      }
     const bool by_levels =
-        lsm <= LEVEL_SMEM && !(db && mean >= 4 && mean < 8 && acc > 4 * 152) &&
+        lsm <= LEVEL_SMEM && !(db && mean >= 4 && mean < 8 && acc > 4 * 152) && !(lg.gen_tab > 0 && untab <= 64) &&
         try_gen_scratch(ctx, 0, general_levels_scratch_floats(lp.live, lp.steps, db, place, acc, lp.tasks, lsm), s);
     if (glob && (!by_levels || lg.gen_tab > 0) &&
         (rc = ensure_gen_scratch(ctx, 0, general_scratch_floats(lg, arena, GL, db), s)))
@@ -3799,6 +3806,9 @@ void plan_levels(Instance& in, const std::vector<int>& prog, const std::vector<i
   in.glin.swap(lin);
   in.glroot.swap(root);
   in.gl_levels = L;
+  in.gl_untab = 0;
+  for (int c = 0; c < nc; ++c)
+    if (ctab[5 * c + 4] < 0) in.gl_untab += comp_step0[c + 1] - comp_step0[c];
   in.gl_live = (arena + 3) & ~3;
   in.gl_total = total;
   in.gl_gmax = gmax;
