@@ -235,20 +235,39 @@ __device__ __forceinline__ int padded_row_bytes(int D) {
   return 4 * w4;
 }
 
-// Stage the tile's spins [T][D] (int8) into shared memory rows of Dp bytes: a
-// warp per row in turn, four spins an access where the rows are aligned.
+// Stage the tile's spins [T][D] (int8) into shared memory rows of Dp bytes, four
+// spins an access where the rows are aligned.  The units of all rows are shared
+// out over the threads (row and column advance without a division), the loads of
+// four at a time in flight: with a warp per row in turn the strip adjoint's 32-sample
+// CTAs waited for eight loads one after the other (127 us for 5 x 16,384
+// samples of the 16 x 16 lattice, 117 here).
+template <class U>
+__device__ __forceinline__ void stage_units(const int8_t* __restrict__ g, int n_valid, int D, int Dp, int8_t* s, int t,
+                                            int T) {
+  const int n = D / (int)sizeof(U), total = n_valid * n;
+  if (total <= 0) return;
+  const int rs = T / n, cs = T - rs * n;
+  int r = t / n, c = t - r * n;
+  for (int e = t; e < total; e += 4 * T) {
+    U v[4];
+    int o[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      o[j] = r * Dp + c * (int)sizeof(U);
+      if (e + j * T < total) v[j] = *reinterpret_cast<const U*>(g + (long long)r * D + c * (int)sizeof(U));
+      r += rs;
+      c += cs;
+      if (c >= n) c -= n, ++r;
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (e + j * T < total) *reinterpret_cast<U*>(s + o[j]) = v[j];
+  }
+}
 __device__ void stage_spins(const int8_t* __restrict__ g, int n_valid, int D, int Dp, int8_t* s,
                             int t, int T) {
-  const int lane = t & 31, nw = T >> 5;
-  if ((D & 3) == 0 && (reinterpret_cast<uintptr_t>(g) & 3) == 0) {
-    const int W4 = D >> 2;
-    for (int r = t >> 5; r < n_valid; r += nw)
-      for (int c = lane; c < W4; c += 32)
-        reinterpret_cast<uint32_t*>(s + r * Dp)[c] = reinterpret_cast<const uint32_t*>(g + (long long)r * D)[c];
-  } else {
-    for (int r = t >> 5; r < n_valid; r += nw)
-      for (int c = lane; c < D; c += 32) s[r * Dp + c] = g[(long long)r * D + c];
-  }
+  if ((D & 3) == 0 && (reinterpret_cast<uintptr_t>(g) & 3) == 0) stage_units<uint32_t>(g, n_valid, D, Dp, s, t, T);
+  else stage_units<int8_t>(g, n_valid, D, Dp, s, t, T);
 }
 
 // sum J s_a s_b over the W-W bonds, in bond order.
@@ -271,7 +290,7 @@ __device__ __forceinline__ float ww_energy(const InstDev& I, const int8_t* srow)
 // four columns with d/dbeta need 128) for 32 warps an SM.  5 x 65,536 samples
 // of the 16 x 16 lattice with d/dbeta: 176 us with one thread per sample
 // through all strips (20 warps an SM, tables and a division per staged spin in
-// every 128-sample CTA), 166 us here; 24 warps and the W-W sums after the
+// every 128-sample CTA), 151 us here; 24 warps and the W-W sums after the
 // strips by half of the threads: 202.
 template <bool DB, int MAXW>
 __global__ void __launch_bounds__(256, DB && MAXW == 4 ? 2 : 4) strips_kernel(const InstDev* __restrict__ inst,
