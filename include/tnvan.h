@@ -358,8 +358,9 @@ int tnvan_magnetisation(tnvan_ctx* ctx, const double* betas, int batch, const in
  * padded to 16 as Dp; 128 + G + (H1 + 16) + (H2 + 16) <= 512 columns with
  * G = Dp when D is not a multiple of 16, else Dp + 16) and whose tiles fit
  * 227 KB of shared memory (every such width set does with H1 = H2 = 128) run
- * the fused tcgen05 backward; the other instances of the same call run the
- * tensor-core GEMM chain (TF32 / BF16 operands, FP32 accumulate) or, where the
+ * the fused tcgen05 backward; the other instances of the same call run on the
+ * tensor cores layer by layer (BF16 with layers of <= 256 units in one kernel,
+ * else as a GEMM chain; TF32 / BF16 operands, FP32 accumulate) or, where the
  * autotuner found it faster, the FP32 SIMT backward.
  *   d_grad_params   device float [total params] out, packed layout of
  *                   tnvan_n_params (overwritten; masked entries are 0).
@@ -416,7 +417,7 @@ int tnvan_train_step(tnvan_ctx* ctx, const double* betas, int batch, uint64_t se
  * 12, 16 or 32), whether tnvan_sample_contract_adjoint overlaps sampling
  * and the strip adjoint on side streams (2 = on, 1 = off), and, for networks
  * the fused BF16 backward does not take, whether the TF32 / BF16 backward
- * runs as the tensor-core GEMM chain (1) or as the FP32 SIMT backward (2,
+ * runs as the tensor-core chain (1) or as the FP32 SIMT backward (2,
  * exact to FP32 and faster for small networks) -- with CUDA events on
  * `stream`, and keeps
  * the fastest in the context for later calls.  With the overlapped schedule

