@@ -91,12 +91,15 @@ struct FusedBwdArgs {
 };
 
 // Bytes of the buffer dX and then dA2 share (D padded): dA2 is written once
-// the products reading dX are done.  The MN-major view of dX (M = 128 of its
-// D columns) reads up to 2 KB past the dX tile when D < 128; the buffer
-// covers that.
-__host__ __device__ inline int fused_bwd_xbuf(int D, int H2) {
-  const int a = 256 * D + 2048, b = 256 * H2;
-  return a > b ? a : b;
+// the products reading dX are done.  An MN-major A operand spans 128 columns
+// whatever the tile holds: of a C-column tile the last 8-row group starts at
+// 240 C and is read for 2,048 bytes, past the tile where C < 128.  The buffer
+// covers that for dX and dA2 and, behind the A2 tile that dA1 overwrites
+// (128 x H1 in 256 (H2 + 16) bytes), for dA1.
+__host__ __device__ inline int fused_bwd_xbuf(int D, int H1, int H2) {
+  const int x = 256 * D + 2048, a2 = 240 * H2 + 2048, a1 = 240 * H1 + 2048 - 256 * (H2 + 16);
+  const int m = x > a2 ? x : a2;
+  return m > a1 ? m : a1;
 }
 
 // Shared memory bytes for (D, H1, H2).
@@ -104,7 +107,7 @@ __host__ __device__ inline int fused_bwd_smem(int D0, int H1, int H2) {
   const int D = (D0 + 15) & ~15;
   const int w = H1 * D + H2 * H1 + D * H2;              // weights
   const int a = 128 * ((D + 16) + (H1 + 16) + (H2 + 16));  // S, A1, A2/dA1
-  return 2 * (w + a) + fused_bwd_xbuf(D, H2) + 4 * (H1 + H2 + D) + 64;  // + dX/dA2, biases, barriers, TMEM slot
+  return 2 * (w + a) + fused_bwd_xbuf(D, H1, H2) + 4 * (H1 + H2 + D) + 64;  // + dX/dA2, biases, barriers, TMEM slot
 }
 
 __global__ void __launch_bounds__(128 * BWD_WG, 1) bwd_fused_kernel(const InstDev* __restrict__ inst,
@@ -133,7 +136,7 @@ __global__ void __launch_bounds__(128 * BWD_WG, 1) bwd_fused_kernel(const InstDe
   unsigned char* sA1 = p; p += 128 * (H1 + 16) * 2;
   unsigned char* sA2 = p; p += 128 * (H2 + 16) * 2;  // later dA1 (128 x H1)
   unsigned char* sdX = p;                             // dX, then dA2 in the same buffer
-  unsigned char* sdA2 = p; p += fused_bwd_xbuf(Dp, H2);
+  unsigned char* sdA2 = p; p += fused_bwd_xbuf(Dp, H1, H2);
   float* sb1 = reinterpret_cast<float*>(p); p += 4 * H1;  // biases
   float* sb2 = reinterpret_cast<float*>(p); p += 4 * H2;
   float* sbo = reinterpret_cast<float*>(p); p += 4 * Dp;  // padded: the barriers below stay 8-byte aligned
