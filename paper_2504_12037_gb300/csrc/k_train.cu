@@ -190,17 +190,18 @@ __device__ __forceinline__ double ff_to_double(FF x) { return (double)x.hi + (do
 // s1, s2: float-float sums of l - K and (l - K)^2; se: the sum of exp(l - e ln 2)
 // in FP64, e an integer (m, once a chunk's sums are written) near its largest
 // l / ln 2 (Eq. 9's log Z_IS is a logsumexp of the l_b, kept in FP64
-// throughout).
+// throughout); far: the sum of exp(l - m) instead, m the chunk's largest l.
 struct TupleFF {
   int n, bad;
   FF s1, s2;
   double m, se;
+  int far;
 };
 __device__ __forceinline__ FF shfl_ff(FF x, int o) {
   return FF{__shfl_xor_sync(0xffffffffu, x.hi, o), __shfl_xor_sync(0xffffffffu, x.lo, o)};
 }
 // partial tuples in a 6-double slot: n, bad, s1, s2 in words 0..5, m and se
-// in doubles 3 and 4
+// in doubles 3 and 4, far in word 10
 __device__ __forceinline__ void st_tuple_ff(double* slot, const TupleFF& t) {
   float* f = reinterpret_cast<float*>(slot);
   reinterpret_cast<int*>(f)[0] = t.n;
@@ -208,12 +209,13 @@ __device__ __forceinline__ void st_tuple_ff(double* slot, const TupleFF& t) {
   f[2] = t.s1.hi, f[3] = t.s1.lo, f[4] = t.s2.hi, f[5] = t.s2.lo;
   slot[3] = t.m;
   slot[4] = t.se;
+  reinterpret_cast<int*>(f)[10] = t.far;
 }
 __device__ __forceinline__ TupleFF ld_tuple_ff(const double* slot) {
   const float* f = reinterpret_cast<const float*>(slot);
   const int* q = reinterpret_cast<const int*>(slot);
   return TupleFF{__ldcg(q), __ldcg(q + 1), FF{__ldcg(f + 2), __ldcg(f + 3)}, FF{__ldcg(f + 4), __ldcg(f + 5)},
-                 __ldcg(slot + 3), __ldcg(slot + 4)};
+                 __ldcg(slot + 3), __ldcg(slot + 4), __ldcg(q + 10)};
 }
 // Floats as integers of the same order (and back).
 __device__ __forceinline__ int ordered(float f) {
@@ -248,7 +250,11 @@ __device__ __forceinline__ double scale_log(int e) { return (double)e * 0.693147
 // exponentials, and what depends on the batch size alone (its log, reciprocals)
 // comes from the host.  1,024 samples: 14.8 us with FP64 maxima, an exp per
 // chunk and one thread merging the warps, 11 us here (3 x 4,096: 15.1 and
-// 11).
+// 11).  A chunk whose largest l lies where FP32 no longer places it within the
+// exponentials' range (|l| > RED_FAR: its spacing there is 64) takes the FP64
+// maximum as its scale, and an instance with such a chunk rescales by
+// exponentials.
+#define RED_FAR 6e8f
 struct BatchConsts {  // of n samples: 1 / n, 1 / (n - 1) (0 for n = 1), ln n, 1 / sqrt n
   double inv_n, inv_n1, ln_n, rsqrt_n;
 };
@@ -267,6 +273,7 @@ __global__ void __launch_bounds__(256) reduce_kernel(const LaunchInfo li, int n_
   const int lo = p * chunk, hi = min(B, lo + chunk);
   const int l = threadIdx.x & 31, nw = blockDim.x >> 5;
   __shared__ int redi[8];
+  __shared__ double redd[8];
   __shared__ TupleFF red[8];
   __shared__ int last;
   // pass 1: the chunk's largest finite l
@@ -280,12 +287,25 @@ __global__ void __launch_bounds__(256) reduce_kernel(const LaunchInfo li, int n_
   __syncthreads();
   mi = redi[0];
   for (int w = 1; w < nw; ++w) mi = max(mi, redi[w]);
-  // no finite l: any scale (the sums stay zero)
   const float top = from_ordered(mi);
-  const int e2 = top > -INFINITY ? (int)fminf(fmaxf(ceilf(top * 1.44269504f), -1e9f), 1e9f) : 0;
-  const double mx = scale_log(e2);
+  const bool far = !(fabsf(top) <= RED_FAR);  // the same for the CTA; also no finite l
+  const int e2 = far ? 0 : (int)ceilf(top * 1.44269504f);
+  double mx = scale_log(e2);
+  if (far) {
+    double md = -INFINITY;
+    for (int b = lo + threadIdx.x; b < hi; b += blockDim.x) {
+      const double ld = logZR[base + b] - (double)logq[base + b];
+      if (isfinite(ld)) md = fmax(md, ld);
+    }
+    for (int o = 16; o > 0; o >>= 1) md = fmax(md, __shfl_xor_sync(0xffffffffu, md, o));
+    if (l == 0) redd[threadIdx.x >> 5] = md;
+    __syncthreads();
+    mx = redd[0];
+    for (int w = 1; w < nw; ++w) mx = fmax(mx, redd[w]);
+    if (!isfinite(mx)) mx = 0.0;  // no finite l: any scale (the sums stay zero)
+  }
   // pass 2: exp sums at that scale, moment sums, counts
-  TupleFF acc = {0, 0, {0.f, 0.f}, {0.f, 0.f}, 0.0, 0.0};
+  TupleFF acc = {0, 0, {0.f, 0.f}, {0.f, 0.f}, 0.0, 0.0, 0};
   for (int b = lo + threadIdx.x; b < hi; b += blockDim.x) {
     const double z = logZR[base + b];
     const float q = logq[base + b];
@@ -305,10 +325,11 @@ __global__ void __launch_bounds__(256) reduce_kernel(const LaunchInfo li, int n_
   __syncthreads();
   if (threadIdx.x < 32) {
     TupleFF r = red[l < nw ? l : 0];
-    if (l >= nw) r = TupleFF{0, 0, {0.f, 0.f}, {0.f, 0.f}, 0.0, 0.0};
+    if (l >= nw) r = TupleFF{0, 0, {0.f, 0.f}, {0.f, 0.f}, 0.0, 0.0, 0};
     for (int o = 4; o > 0; o >>= 1) add_lane(r, o);
     if (l == 0) {
-      r.m = (double)e2;
+      r.m = far ? mx : (double)e2;
+      r.far = far;
       st_tuple_ff(part + ((long long)k * n_part + p) * 6, r);
       __threadfence();
       last = atomicAdd(counters + k, 1) == n_part - 1;
@@ -319,15 +340,26 @@ __global__ void __launch_bounds__(256) reduce_kernel(const LaunchInfo li, int n_
   const double inv_beta = 1.0 / li.beta[k];
   __threadfence();
   // the instance's chunks: lane l holds chunks l and l + 32
-  TupleFF r = {0, 0, {0.f, 0.f}, {0.f, 0.f}, 0.0, 0.0};
+  TupleFF r = {0, 0, {0.f, 0.f}, {0.f, 0.f}, 0.0, 0.0, 0};
   TupleFF r2 = r;
   if (l < n_part) r = ld_tuple_ff(part + ((long long)k * n_part + l) * 6);
   if (l + 32 < n_part) r2 = ld_tuple_ff(part + ((long long)k * n_part + l + 32) * 6);
-  const int ea = r.n ? (int)r.m : INT_MIN, eb = r2.n ? (int)r2.m : INT_MIN;
-  const int E = __reduce_max_sync(0xffffffffu, max(ea, eb));
-  r.se = r.n ? scalbn(r.se, max(ea - E, -2000)) : 0.0;
+  double top_l;  // log of the sums' common scale
+  if (!__any_sync(0xffffffffu, (r.n && r.far) || (r2.n && r2.far))) {
+    const int ea = r.n ? (int)r.m : INT_MIN, eb = r2.n ? (int)r2.m : INT_MIN;
+    const int E = __reduce_max_sync(0xffffffffu, max(ea, eb));
+    top_l = scale_log(E);
+    r.se = r.n ? scalbn(r.se, max(ea - E, -2000)) : 0.0;
+    r2.se = r2.n ? scalbn(r2.se, max(eb - E, -2000)) : 0.0;
+  } else {
+    const double ma = r.far ? r.m : scale_log((int)r.m), mb = r2.far ? r2.m : scale_log((int)r2.m);
+    top_l = fmax(r.n ? ma : -INFINITY, r2.n ? mb : -INFINITY);
+    for (int o = 16; o > 0; o >>= 1) top_l = fmax(top_l, __shfl_xor_sync(0xffffffffu, top_l, o));
+    r.se = r.n ? r.se * exp(ma - top_l) : 0.0;
+    r2.se = r2.n ? r2.se * exp(mb - top_l) : 0.0;
+  }
   if (n_part > 32) {
-    r.se += r2.n ? scalbn(r2.se, max(eb - E, -2000)) : 0.0;
+    r.se += r2.se;
     r.n += r2.n;
     r.bad += r2.bad;
     r.s1 = ff_add(r.s1, r2.s1);
@@ -354,7 +386,7 @@ __global__ void __launch_bounds__(256) reduce_kernel(const LaunchInfo li, int n_
   if (l != 0) return;
   const double nan = __longlong_as_double(0x7FF8000000000000ll);
   const double mean = n_ ? ff_to_double(K) + mean_d : nan;
-  const double lz = n_ ? scale_log(E) + f - ln_n : nan;
+  const double lz = n_ ? top_l + f - ln_n : nan;
   double* st = stats + 8 * k;
   st[0] = -mean * inv_beta;
   st[1] = -lz * inv_beta;
