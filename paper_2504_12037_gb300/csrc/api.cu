@@ -742,7 +742,7 @@ struct FusedBwdPlan {
   int smem;
   long long max_elems;
 };
-int plan_fused_bwd(tnvan_ctx* ctx, const double* betas, int batch, FusedBwdPlan& p);
+int plan_fused_bwd(tnvan_ctx* ctx, const double* betas, int batch, FusedBwdPlan& p, cudaStream_t s);
 // Backward and Adam of each instance chunk, queued behind that chunk's
 // adjoint and Eq. 9 reduction (whose mean is Eq. 10's baseline) in the
 // overlapped schedule.
@@ -759,15 +759,55 @@ int sample_contract_adjoint_impl(tnvan_ctx* ctx, const double* betas, int batch,
 
 }  // namespace
 
-int ensure_ws(tnvan_ctx* ctx, size_t bytes) {
-  if (bytes <= ctx->ws_bytes) return TNVAN_OK;
-  if (ctx->d_ws) cudaFree(ctx->d_ws);
-  ctx->d_ws = nullptr;
-  ctx->ws_bytes = 0;
-  cudaError_t e = cudaMalloc(&ctx->d_ws, bytes);
-  if (e != cudaSuccess) return fail(ctx, TNVAN_E_NOMEM, "cudaMalloc(workspace, %zu B): %s", bytes, cudaGetErrorString(e));
-  ctx->ws_bytes = bytes;
+static bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) == cudaSuccess) return st != cudaStreamCaptureStatusNone;
+  cudaGetLastError();  // the legacy stream beside a capture
+  return true;
+}
+
+// A buffer that a replay of a captured graph may read or write stays until the
+// context goes; one that no graph has seen is freed.
+template <class T>
+static void let_go(tnvan_ctx* ctx, GrowBuf<T>& b) {
+  if (b.p && b.captured) ctx->outgrown.push_back(b.p);
+  else if (b.p) cudaFree(b.p);
+  b = GrowBuf<T>();
+}
+// At least n elements for a call on stream s.
+template <class T>
+static int grow(tnvan_ctx* ctx, GrowBuf<T>& b, size_t n, cudaStream_t s, const char* what) {
+  if (!b.captured && b.p) b.captured = capturing(s);  // also where it is outgrown inside the capture
+  if (n > b.n) {
+    let_go(ctx, b);
+    cudaError_t e = cudaMalloc(&b.p, n * sizeof(T));
+    if (e != cudaSuccess) {
+      b.p = nullptr;
+      return fail(ctx, TNVAN_E_NOMEM, "cudaMalloc(%s, %zu B): %s", what, n * sizeof(T), cudaGetErrorString(e));
+    }
+    b.n = n;
+    b.captured = capturing(s);
+  }
   return TNVAN_OK;
+}
+// The same for a form that has another to fall back on: false where the buffer
+// would have to grow inside a capture or cannot.
+template <class T>
+static bool try_grow(tnvan_ctx* ctx, GrowBuf<T>& b, size_t n, cudaStream_t s) {
+  const bool cap = capturing(s);
+  if (n > b.n) {
+    if (cap) return false;
+    T* p = nullptr;  // the old buffer stays until the new one is there
+    if (cudaMalloc(&p, n * sizeof(T)) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    let_go(ctx, b);
+    b.p = p;
+    b.n = n;
+  }
+  b.captured = b.captured || cap;
+  return true;
 }
 
 size_t chain_ws_elems(const tnvan_ctx* ctx, int batch, ChainWs* cw);
@@ -856,8 +896,8 @@ int backward_tc(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* d_
   const int n = (int)ctx->inst.size();
   // instances the fused backward handles in the same call are left out
   auto skip = [&](int k) { return skip_fused && ctx->inst[k].dev.made.fused_ok; };
-  if ((rc = ensure_ws(ctx, tc_ws_floats(ctx, batch) * sizeof(float)))) return rc;
-  float* ws = static_cast<float*>(ctx->d_ws);
+  if ((rc = grow(ctx, ctx->ws, tc_ws_floats(ctx, batch) * sizeof(float), s, "workspace"))) return rc;
+  float* ws = reinterpret_cast<float*>(ctx->ws.p);
   struct Bufs { float *A1, *A2, *dX, *dA2, *dA1, *w; };
   std::vector<Bufs> bf(n);
   size_t off = 0;
@@ -976,7 +1016,7 @@ int backward_tc(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* d_
     const int occ = std::max(1, std::min(227 * 1024 / (chain_wgrad_smem_bytes(max_n) + 1024), 512 / std::max(32, 2 * max_n)));
     *splits_out = std::max(1, std::min({TC_SPLITS, (batch + 127) / 128, 152 * occ / std::max(acc, 1)}));
     PROF("gemm_wgrad", s);
-    CK(launch_chain_wgrad(ctx->d_inst, lc, cw, *splits_out, max_n, ctx->d_grad_packed, part_stride, s),
+    CK(launch_chain_wgrad(ctx->d_inst, lc, cw, *splits_out, max_n, ctx->grad_packed.p, part_stride, s),
        "weight gradient kernel");
     return TNVAN_OK;
   } else {
@@ -1057,7 +1097,7 @@ int backward_tc(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* d_
   }
   // stage 6: weight gradients, split over the batch into TC_SPLITS partial slices
   splits = *splits_out;
-  float* part = ctx->d_grad_packed;
+  float* part = ctx->grad_packed.p;
   for (int k = 0; k < n; ++k) {
     if (skip(k)) continue;
     const Instance& in = ctx->inst[k];
@@ -1152,15 +1192,12 @@ int tnvan_destroy(tnvan_ctx* ctx) {
   if (ctx->d_inst) cudaFree(ctx->d_inst);
   if (ctx->d_stats) cudaFree(ctx->d_stats);
   if (ctx->d_status) cudaFree(ctx->d_status);
-  if (ctx->d_grad_packed) cudaFree(ctx->d_grad_packed);
-  if (ctx->d_ws) cudaFree(ctx->d_ws);
   if (ctx->d_obs) cudaFree(ctx->d_obs);
-  if (ctx->d_dj_part) cudaFree(ctx->d_dj_part);
-  if (ctx->d_wide_part) cudaFree(ctx->d_wide_part);
   if (ctx->prof_ref) cudaEventDestroy(ctx->prof_ref);
-  for (float* p : ctx->d_gen_scratch)
+  for (void* p : {(void*)ctx->ws.p, (void*)ctx->grad_packed.p, (void*)ctx->dj_part.p, (void*)ctx->gen_scratch[0].p,
+                  (void*)ctx->gen_scratch[1].p, (void*)ctx->wide_part.p})
     if (p) cudaFree(p);
-  for (float* p : ctx->gen_scratch_old) cudaFree(p);
+  for (void* p : ctx->outgrown) cudaFree(p);
   delete ctx;
   return TNVAN_OK;
 }
@@ -1866,17 +1903,6 @@ int tnvan_instance_info(const tnvan_ctx* ctx, int instance, int32_t* info) {
   return TNVAN_OK;
 }
 
-static int ensure_dj_part(tnvan_ctx* ctx, size_t floats) {
-  if (floats <= ctx->dj_part_floats) return TNVAN_OK;
-  if (ctx->d_dj_part) cudaFree(ctx->d_dj_part);
-  ctx->d_dj_part = nullptr;
-  ctx->dj_part_floats = 0;
-  cudaError_t e = cudaMalloc(&ctx->d_dj_part, floats * sizeof(float));
-  if (e != cudaSuccess) return fail(ctx, TNVAN_E_NOMEM, "cudaMalloc(d/dJ partials): %s", cudaGetErrorString(e));
-  ctx->dj_part_floats = floats;
-  return TNVAN_OK;
-}
-
 // Elimination launch shape: GL lanes share a sample and a CTA has 128
 // threads, so 128 / GL samples.  GL is the largest power of two not above the
 // instances' mean table size, doubled once when the batch alone would give
@@ -1902,61 +1928,6 @@ bool gen_tables_global(int S, F smem) {
 }
 }  // extern "C++"
 
-// Global table scratch of the elimination kernels (which: 0 forward, 1
-// reverse sweep); grows only, kept for the context's lifetime.
-static bool capturing(cudaStream_t s) {
-  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(s, &st) == cudaSuccess) return st != cudaStreamCaptureStatusNone;
-  cudaGetLastError();  // the legacy stream beside a capture
-  return true;
-}
-static int ensure_gen_scratch(tnvan_ctx* ctx, int which, size_t floats, cudaStream_t s) {
-  if (floats > ctx->gen_scratch_floats[which]) {
-    // a captured graph may hold the old buffer: kept until the context goes
-    if (ctx->d_gen_scratch[which] && ctx->gen_scratch_captured[which])
-      ctx->gen_scratch_old.push_back(ctx->d_gen_scratch[which]);
-    else if (ctx->d_gen_scratch[which])
-      cudaFree(ctx->d_gen_scratch[which]);
-    ctx->d_gen_scratch[which] = nullptr;
-    ctx->gen_scratch_floats[which] = 0;
-    ctx->gen_scratch_captured[which] = false;
-    cudaError_t e = cudaMalloc(&ctx->d_gen_scratch[which], floats * sizeof(float));
-    if (e != cudaSuccess)
-      return fail(ctx, TNVAN_E_NOMEM, "cudaMalloc(elimination tables, %zu floats): %s", floats, cudaGetErrorString(e));
-    ctx->gen_scratch_floats[which] = floats;
-  }
-  if (!ctx->gen_scratch_captured[which]) ctx->gen_scratch_captured[which] = capturing(s);
-  return TNVAN_OK;
-}
-// The same for a form that has another to fall back on: false where the buffer
-// would have to grow inside a capture or cannot.
-static bool try_gen_scratch(tnvan_ctx* ctx, int which, size_t floats, cudaStream_t s) {
-  if (floats > ctx->gen_scratch_floats[which]) {
-    if (capturing(s)) return false;
-    float* p = nullptr;  // the old buffer stays until the new one is there
-    if (cudaMalloc(&p, floats * sizeof(float)) != cudaSuccess) {
-      cudaGetLastError();
-      return false;
-    }
-    if (ctx->d_gen_scratch[which] && ctx->gen_scratch_captured[which])
-      ctx->gen_scratch_old.push_back(ctx->d_gen_scratch[which]);
-    else if (ctx->d_gen_scratch[which])
-      cudaFree(ctx->d_gen_scratch[which]);
-    ctx->d_gen_scratch[which] = p;
-    ctx->gen_scratch_floats[which] = floats;
-    ctx->gen_scratch_captured[which] = false;
-  }
-  return ensure_gen_scratch(ctx, which, floats, s) == TNVAN_OK;
-}
-
-static bool try_dj_part(tnvan_ctx* ctx, size_t floats, cudaStream_t s) {
-  if (floats <= ctx->dj_part_floats) return true;
-  if (capturing(s)) return false;
-  if (ensure_dj_part(ctx, floats) == TNVAN_OK) return true;
-  cudaGetLastError();
-  return false;
-}
-
 // What the level kernels of a launch need: the largest over the instances.
 struct LevelPlan {
   int live = 0, total = 0, gmax = 0, red = 0, tasks = 0, steps = 0;
@@ -1976,34 +1947,11 @@ static LevelPlan level_plan(const tnvan_ctx* ctx) {
 }
 constexpr int LEVEL_SMEM = 216 * 1024;  // and 8 KB of their own
 
-// Per-strip results of the wide-strip kernels [n_inst][batch][strips]; grows only.
-static int ensure_wide_part(tnvan_ctx* ctx, size_t n) {
-  if (n <= ctx->wide_part_n) return TNVAN_OK;
-  if (ctx->d_wide_part) cudaFree(ctx->d_wide_part);
-  ctx->d_wide_part = nullptr;
-  ctx->wide_part_n = 0;
-  cudaError_t e = cudaMalloc(&ctx->d_wide_part, n * sizeof(double));
-  if (e != cudaSuccess) return fail(ctx, TNVAN_E_NOMEM, "cudaMalloc(wide strips, %zu): %s", n, cudaGetErrorString(e));
-  ctx->wide_part_n = n;
-  return TNVAN_OK;
-}
-
 static int wide_max_strips(const tnvan_ctx* ctx) {
   int ms = 0;
   for (const Instance& in : ctx->inst)
     if (in.kind == 2) ms = std::max(ms, in.dev.n_wide);
   return ms;
-}
-
-static int ensure_grad_ws(tnvan_ctx* ctx, size_t floats) {
-  if (floats <= ctx->grad_packed_floats) return TNVAN_OK;
-  if (ctx->d_grad_packed) cudaFree(ctx->d_grad_packed);
-  ctx->d_grad_packed = nullptr;
-  ctx->grad_packed_floats = 0;
-  cudaError_t e = cudaMalloc(&ctx->d_grad_packed, floats * sizeof(float));
-  if (e != cudaSuccess) return fail(ctx, TNVAN_E_NOMEM, "cudaMalloc(gradient partials, %zu floats): %s", floats, cudaGetErrorString(e));
-  ctx->grad_packed_floats = floats;
-  return TNVAN_OK;
 }
 
 // Partial gradient rows of the FP32 backward.
@@ -2018,17 +1966,18 @@ int tnvan_reserve(tnvan_ctx* ctx, int max_batch) {
   DeviceGuard g(ctx->device);
   int rc = check_ready(ctx, false);
   if (rc) return rc;
-  rc = ensure_grad_ws(ctx, grad_ws_floats(ctx, std::max(max_batch, 1)));
+  const cudaStream_t s = nullptr;
+  rc = grow(ctx, ctx->grad_packed, grad_ws_floats(ctx, std::max(max_batch, 1)), s, "gradient partials");
   if (rc) return rc;
   {
     long long maxp = 0;
     for (const Instance& in : ctx->inst) maxp = std::max(maxp, in.n_params);
     const int splits = std::max(1, std::min(TC_SPLITS, (std::max(max_batch, 1) + 127) / 128));
-    rc = ensure_grad_ws(ctx, std::max(grad_ws_floats(ctx, std::max(max_batch, 1)),
-                                      (size_t)splits * ctx->inst.size() * (size_t)maxp));
+    rc = grow(ctx, ctx->grad_packed, std::max(grad_ws_floats(ctx, std::max(max_batch, 1)),
+                                      (size_t)splits * ctx->inst.size() * (size_t)maxp), s, "gradient partials");
     if (rc) return rc;
-    rc = ensure_ws(ctx, std::max(tc_ws_floats(ctx, std::max(max_batch, 1)),
-                                 bwd32_ws_floats(ctx, std::max(max_batch, 1), nullptr)) * sizeof(float));
+    rc = grow(ctx, ctx->ws, std::max(tc_ws_floats(ctx, std::max(max_batch, 1)),
+                                 bwd32_ws_floats(ctx, std::max(max_batch, 1), nullptr)) * sizeof(float), s, "workspace");
     if (rc) return rc;
     int max_edges = 0, ctas = 0;
     for (const Instance& in : ctx->inst) {
@@ -2036,10 +1985,12 @@ int tnvan_reserve(tnvan_ctx* ctx, int max_batch) {
       // elimination instances: up to 8 rows per 32 samples
       ctas += in.kind == 2 ? 8 * ((std::max(max_batch, 1) + 31) / 32) : (std::max(max_batch, 1) + 127) / 128;
     }
-    rc = ensure_dj_part(ctx, (size_t)ctas * ((max_edges + 3) & ~3));
+    rc = grow(ctx, ctx->dj_part, (size_t)ctas * ((max_edges + 3) & ~3), s, "d/dJ partials");
     if (rc) return rc;
     const int ms = wide_max_strips(ctx);
-    if (ms > 0 && (rc = ensure_wide_part(ctx, ctx->inst.size() * (size_t)std::max(max_batch, 1) * ms))) return rc;
+    if (ms > 0 &&
+        (rc = grow(ctx, ctx->wide_part, ctx->inst.size() * (size_t)std::max(max_batch, 1) * ms, s, "wide strips")))
+      return rc;
   }
   ctx->reserved_batch = std::max(ctx->reserved_batch, max_batch);
   CK(cudaDeviceSynchronize(), "reserve");
@@ -2120,7 +2071,8 @@ static int sample_adjoint_overlapped(tnvan_ctx* ctx, const double* betas, int ba
     max_edges = std::max(max_edges, in.m);
   }
   const int stride = (max_edges + 3) & ~3;
-  if (d_dJ && (rc = ensure_dj_part(ctx, (size_t)la.tile_begin[la.n_inst] * stride))) return rc;
+  if (d_dJ && (rc = grow(ctx, ctx->dj_part, (size_t)la.tile_begin[la.n_inst] * stride, s, "d/dJ partials")))
+    return rc;
   if ((rc = ensure_side_streams(ctx))) return rc;
   LaunchInfo lr;
   if (chunk_stats && (rc = fill_launch(ctx, betas, batch, 1, lr))) return rc;
@@ -2149,7 +2101,7 @@ static int sample_adjoint_overlapped(tnvan_ctx* ctx, const double* betas, int ba
     {
       PROF("strips_adj", ctx->side_lo[c]);
       CK(launch_strips_adj(ctx->d_inst, la, adj_smem, adj_lv, d_spins, d_logZR, d_dbeta,
-                           d_dJ ? ctx->d_dj_part : nullptr, stride, nullptr, ctx->side_lo[c], la.tile_begin[k0],
+                           d_dJ ? ctx->dj_part.p : nullptr, stride, nullptr, ctx->side_lo[c], la.tile_begin[k0],
                            la.tile_begin[k1], adj_ws),
          "strip adjoint kernel");
     }
@@ -2163,12 +2115,12 @@ static int sample_adjoint_overlapped(tnvan_ctx* ctx, const double* betas, int ba
       const FusedBwdPlan& fp = *cb->plan;
       {
         PROF("bwd_fused", ctx->side_lo[c]);
-        CK(launch_bwd_fused(ctx->d_inst, fp.lf, fp.smem, d_spins, d_logZR, d_logq, ctx->d_stats, ctx->d_grad_packed,
+        CK(launch_bwd_fused(ctx->d_inst, fp.lf, fp.smem, d_spins, d_logZR, d_logq, ctx->d_stats, ctx->grad_packed.p,
                             fp.max_elems, ctx->d_status, ctx->side_lo[c], fp.lf.tile_begin[k0], fp.lf.tile_begin[k1]),
            "fused backward kernel");
       }
       PROF("grad_reduce", ctx->side_lo[c]);
-      CK(launch_grad_reduce(ctx->d_inst, fp.lf, ctx->d_grad_packed, (int)fp.max_elems, cb->d_grad, ctx->side_lo[c],
+      CK(launch_grad_reduce(ctx->d_inst, fp.lf, ctx->grad_packed.p, (int)fp.max_elems, cb->d_grad, ctx->side_lo[c],
                             cb->adam, k0, k1),
          "gradient reduce kernel");
     }
@@ -2185,7 +2137,7 @@ static int sample_adjoint_overlapped(tnvan_ctx* ctx, const double* betas, int ba
     }
     {
       PROF("strips_dJ_reduce", sr);
-      CK(launch_strips_dJ_reduce(ctx->d_inst, la, ctx->d_dj_part, stride, d_dJ, sr, true), "d/dJ reduce");
+      CK(launch_strips_dJ_reduce(ctx->d_inst, la, ctx->dj_part.p, stride, d_dJ, sr, true), "d/dJ reduce");
     }
     if (defer_dj) CK(cudaEventRecord(ctx->dj_ev, sr), "d/dJ event");
   }
@@ -2246,7 +2198,7 @@ int tnvan_train_step(tnvan_ctx* ctx, const double* betas, int batch, uint64_t se
   const AdamArgs a = adam_args(ctx, d_m, d_v, lr, beta1, beta2, eps, t);
   FusedBwdPlan fp;
   ChunkBackward cb{&fp, d_grad_params, &a};
-  if (all_fused && (rc = plan_fused_bwd(ctx, betas, batch, fp))) return rc;
+  if (all_fused && (rc = plan_fused_bwd(ctx, betas, batch, fp, s))) return rc;
   if (d_dbeta || d_dJ)
     rc = sample_contract_adjoint_impl(ctx, betas, batch, seed, step, precision, d_spins, d_logq, d_logZR, d_dbeta,
                                       d_dJ, s, &dj_deferred, &stats_done, all_fused ? &cb : nullptr, &bwd_done);
@@ -2540,8 +2492,9 @@ int tnvan_magnetisation(tnvan_ctx* ctx, const double* betas, int batch, const in
     CK(launch_general_pp(ctx->d_inst, lg, nsteps, s), "elimination bond products");
     float* gs = nullptr;
     if (glob) {
-      if ((rc = ensure_gen_scratch(ctx, 0, general_mom_scratch_floats(lg, arena, GL), s))) return rc;
-      gs = ctx->d_gen_scratch[0];
+      if ((rc = grow(ctx, ctx->gen_scratch[0], general_mom_scratch_floats(lg, arena, GL), s, "elimination tables")))
+        return rc;
+      gs = ctx->gen_scratch[0].p;
     }
     CK(launch_general_mom(ctx->d_inst, lg, sm, arena, GL, d_spins, mean, var, gs, s), "elimination moments kernel");
   }
@@ -2610,16 +2563,16 @@ int backward_impl(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* 
     if (ctx->inst[k].dev.made.fused_ok) fused_bits[k >> 5] |= 1u << (k & 31);
   if (any_fused) {
     FusedBwdPlan fp;
-    if ((rc = plan_fused_bwd(ctx, betas, batch, fp))) return rc;
+    if ((rc = plan_fused_bwd(ctx, betas, batch, fp, s))) return rc;
     {
       PROF("bwd_fused", s);
-      CK(launch_bwd_fused(ctx->d_inst, fp.lf, fp.smem, d_spins, d_logZR, d_logq, ctx->d_stats, ctx->d_grad_packed,
+      CK(launch_bwd_fused(ctx->d_inst, fp.lf, fp.smem, d_spins, d_logZR, d_logq, ctx->d_stats, ctx->grad_packed.p,
                           fp.max_elems, ctx->d_status, s),
          "fused backward kernel");
     }
     {
       PROF("grad_reduce", s);
-      CK(launch_grad_reduce(ctx->d_inst, fp.lf, ctx->d_grad_packed, (int)fp.max_elems, d_grad_params, s, adam),
+      CK(launch_grad_reduce(ctx->d_inst, fp.lf, ctx->grad_packed.p, (int)fp.max_elems, d_grad_params, s, adam),
          "gradient reduce kernel");
     }
   }
@@ -2628,7 +2581,9 @@ int backward_impl(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* 
   const bool simt = precision == TNVAN_FP32 || (!all_fused && ctx->tune_bwd_form == 2);
   if (!all_fused && !simt) {
     int splits = std::max(1, std::min(TC_SPLITS, (batch + 127) / 128));
-    if ((rc = ensure_grad_ws(ctx, (size_t)splits * ctx->inst.size() * (size_t)max_elems))) return rc;
+    if ((rc = grow(ctx, ctx->grad_packed, (size_t)splits * ctx->inst.size() * (size_t)max_elems, s,
+                   "gradient partials")))
+      return rc;
     if ((rc = backward_tc(ctx, betas, batch, d_spins, d_logZR, d_logq, precision == TNVAN_BF16,
                           (int)max_elems, s, any_fused, &splits)))
       return rc;
@@ -2638,7 +2593,7 @@ int backward_impl(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* 
     for (int j = 0; j < TNVAN_MAX_INST / 32; ++j) lr.skip[j] = fused_bits[j];
     {
       PROF("grad_reduce", s);
-      CK(launch_grad_reduce(ctx->d_inst, lr, ctx->d_grad_packed, (int)max_elems, d_grad_params, s, adam),
+      CK(launch_grad_reduce(ctx->d_inst, lr, ctx->grad_packed.p, (int)max_elems, d_grad_params, s, adam),
          "gradient reduce kernel");
     }
   }
@@ -2669,9 +2624,9 @@ int backward_impl(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* 
     lb.tile_begin[lb.n_inst] = acc;
     for (int j = 0; j < TNVAN_MAX_INST / 32; ++j) lb.skip[j] = fused_bits[j];
     Bwd32Ws bw;
-    if ((rc = ensure_grad_ws(ctx, grad_ws_floats(ctx, batch)))) return rc;
-    if ((rc = ensure_ws(ctx, bwd32_ws_floats(ctx, batch, &bw) * sizeof(float)))) return rc;
-    bw.base = static_cast<float*>(ctx->d_ws);
+    if ((rc = grow(ctx, ctx->grad_packed, grad_ws_floats(ctx, batch), s, "gradient partials"))) return rc;
+    if ((rc = grow(ctx, ctx->ws, bwd32_ws_floats(ctx, batch, &bw) * sizeof(float), s, "workspace"))) return rc;
+    bw.base = reinterpret_cast<float*>(ctx->ws.p);
     {
       PROF("backward", s);
       CK(launch_bwd32_delta(ctx->d_inst, lb, bw, res, bwd32_smem_bytes(max_units, res ? max_res : 0), d_spins, d_logZR,
@@ -2680,14 +2635,14 @@ int backward_impl(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* 
     }
     {
       PROF("backward_wgrad", s);
-      CK(launch_bwd32_wgrad(ctx->d_inst, lb, bw, max_blocks, splits, ctx->d_grad_packed, max_elems, s),
+      CK(launch_bwd32_wgrad(ctx->d_inst, lb, bw, max_blocks, splits, ctx->grad_packed.p, max_elems, s),
          "weight gradient kernel");
     }
     LaunchInfo lr = lb;
     for (int k = 0; k <= lr.n_inst; ++k) lr.tile_begin[k] = k * splits;
     {
       PROF("grad_reduce", s);
-      CK(launch_grad_reduce(ctx->d_inst, lr, ctx->d_grad_packed, (int)max_elems, d_grad_params, s, adam),
+      CK(launch_grad_reduce(ctx->d_inst, lr, ctx->grad_packed.p, (int)max_elems, d_grad_params, s, adam),
          "gradient reduce kernel");
     }
   }
@@ -2695,7 +2650,7 @@ int backward_impl(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* 
   return TNVAN_OK;
 }
 
-int plan_fused_bwd(tnvan_ctx* ctx, const double* betas, int batch, FusedBwdPlan& p) {
+int plan_fused_bwd(tnvan_ctx* ctx, const double* betas, int batch, FusedBwdPlan& p, cudaStream_t s) {
   int rc;
   p.max_elems = 0;
   p.smem = 0;
@@ -2723,7 +2678,8 @@ int plan_fused_bwd(tnvan_ctx* ctx, const double* betas, int batch, FusedBwdPlan&
   }
   p.lf.tile_begin[p.lf.n_inst] = acc;
   p.lf.tile = per;
-  return ensure_grad_ws(ctx, (size_t)p.lf.tile_begin[p.lf.n_inst] * (size_t)p.max_elems);
+  return grow(ctx, ctx->grad_packed, (size_t)p.lf.tile_begin[p.lf.n_inst] * (size_t)p.max_elems, s,
+              "gradient partials");
 }
 
 AdamArgs adam_args(const tnvan_ctx* ctx, float* d_m, float* d_v, double lr, double beta1, double beta2, double eps,
@@ -3404,9 +3360,9 @@ int contract_all(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* d
       for (const WideStripDev& sd : in.wide.strips) ++cnt[sd.w <= 5 ? 0 : sd.w - 5];
       for (int c = 0; c < 8; ++c) per_class[c] = std::max(per_class[c], cnt[c]);
     }
-    if ((rc = ensure_wide_part(ctx, (size_t)lw.n_inst * batch * ms))) return rc;
+    if ((rc = grow(ctx, ctx->wide_part, (size_t)lw.n_inst * batch * ms, s, "wide strips"))) return rc;
     PROF("wide_strips", s);
-    CK(launch_wide(ctx->d_inst, lw, per_class, ms, rows, d_spins, ctx->d_wide_part, d_logZR, s), "wide-strip kernels");
+    CK(launch_wide(ctx->d_inst, lw, per_class, ms, rows, d_spins, ctx->wide_part.p, d_logZR, s), "wide-strip kernels");
     k2 = rest;
   }
   if (k2) {
@@ -3476,11 +3432,12 @@ int contract_all(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* d
       }
     const bool by_levels =
         lsm <= LEVEL_SMEM && !(db && mean >= 4 && mean < 8 && acc > 4 * 152) && !(lg.gen_tab > 0 && untab <= 64) &&
-        try_gen_scratch(ctx, 0, general_levels_scratch_floats(lp.live, lp.steps, db, place, acc, lp.tasks, lsm), s);
+        try_grow(ctx, ctx->gen_scratch[0],
+                 general_levels_scratch_floats(lp.live, lp.steps, db, place, acc, lp.tasks, lsm), s);
     if (glob && (!by_levels || lg.gen_tab > 0) &&
-        (rc = ensure_gen_scratch(ctx, 0, general_scratch_floats(lg, arena, GL, db), s)))
+        (rc = grow(ctx, ctx->gen_scratch[0], general_scratch_floats(lg, arena, GL, db), s, "elimination tables")))
       return rc;
-    float* gs = ctx->d_gen_scratch[0];
+    float* gs = ctx->gen_scratch[0].p;
     if (lg.gen_tab > 0) {
       PROF("general_tables", s);
       CK(launch_general_tables(ctx->d_inst, lg, sm, db, GL, glob ? gs : nullptr, s), "general tables kernel");
@@ -3533,11 +3490,12 @@ int run_adjoint(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* d_
     for (const Instance& in : ctx->inst)
       if (in.kind == 0) max_edges = std::max(max_edges, in.m);
     const int stride = (max_edges + 3) & ~3;
-    if (d_dJ && (rc = ensure_dj_part(ctx, (size_t)la.tile_begin[la.n_inst] * stride))) return rc;
+    if (d_dJ && (rc = grow(ctx, ctx->dj_part, (size_t)la.tile_begin[la.n_inst] * stride, s, "d/dJ partials")))
+      return rc;
     CK(launch_strip_tables(ctx->d_inst, la, 0, la.n_inst, s), "strip tables");
     PROF(d_dJ ? "strips_adj" : "strips_dbeta", s);
     CK(launch_strips_adj(ctx->d_inst, la, adj_smem, adj_lv, d_spins, d_logZR, d_dbeta,
-                         d_dJ ? ctx->d_dj_part : nullptr, stride, d_dJ, s, 0, -1, adj_ws),
+                         d_dJ ? ctx->dj_part.p : nullptr, stride, d_dJ, s, 0, -1, adj_ws),
        "strip adjoint kernel");
   }
   if (d_dJ) {
@@ -3593,33 +3551,34 @@ int run_adjoint(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* d_
           lsm = general_levels_dJ_smem_bytes(lp.total, lp.live, lp.gmax, lp.red, Dm, place);
           if (lsm <= LEVEL_SMEM || !place) break;
         }
-        if (GL >= 2 && lsm <= LEVEL_SMEM && try_dj_part(ctx, (size_t)acc * GL * stride, s) &&
-            try_gen_scratch(ctx, 1,
-                            general_levels_dJ_scratch_floats(lp.total, lp.live, lp.gmax, lp.steps, place, acc, lp.tasks, lsm),
-                            s)) {
+        if (GL >= 2 && lsm <= LEVEL_SMEM && try_grow(ctx, ctx->dj_part, (size_t)acc * GL * stride, s) &&
+            try_grow(ctx, ctx->gen_scratch[1],
+                     general_levels_dJ_scratch_floats(lp.total, lp.live, lp.gmax, lp.steps, place, acc, lp.tasks, lsm),
+                     s)) {
           {
             PROF("general_pp", s);
             CK(launch_general_pp(ctx->d_inst, lg, nsteps, s), "elimination bond products");
           }
           PROF("general_dJ", s);
           CK(launch_general_levels_dJ(ctx->d_inst, lw, lsm, GL, lp.total, lp.live, lp.gmax, lp.steps, lp.red, lp.tasks,
-                                      place, me, d_spins, ctx->d_dj_part, stride, d_dJ, ctx->d_gen_scratch[1], s),
+                                      place, me, d_spins, ctx->dj_part.p, stride, d_dJ, ctx->gen_scratch[1].p, s),
              "general adjoint kernel");
           return TNVAN_OK;
         }
-        if ((rc = ensure_dj_part(ctx, (size_t)lg.tile_begin[lg.n_inst] * stride))) return rc;
+        if ((rc = grow(ctx, ctx->dj_part, (size_t)lg.tile_begin[lg.n_inst] * stride, s, "d/dJ partials"))) return rc;
         float* gs = nullptr;
         if (glob) {
-          if ((rc = ensure_gen_scratch(ctx, 1, general_dJ_scratch_floats(per, T, GL, lg.tile_begin[lg.n_inst]), s)))
+          if ((rc = grow(ctx, ctx->gen_scratch[1], general_dJ_scratch_floats(per, T, GL, lg.tile_begin[lg.n_inst]), s,
+                         "elimination tables")))
             return rc;
-          gs = ctx->d_gen_scratch[1];
+          gs = ctx->gen_scratch[1].p;
         }
         {
           PROF("general_pp", s);
           CK(launch_general_pp(ctx->d_inst, lg, nsteps, s), "elimination bond products");
         }
         PROF("general_dJ", s);
-        CK(launch_general_dJ(ctx->d_inst, lg, sm, arena, steps, gmax, GL, d_spins, ctx->d_dj_part, stride, d_dJ, gs,
+        CK(launch_general_dJ(ctx->d_inst, lg, sm, arena, steps, gmax, GL, d_spins, ctx->dj_part.p, stride, d_dJ, gs,
                              s),
            "general adjoint kernel");
       }

@@ -371,6 +371,16 @@ struct tnvan_prof_rec {
   long long launches = 0;
 };
 
+namespace tnvan {
+// A device buffer of a context: n elements at p, grows only.
+template <class T>
+struct GrowBuf {
+  T* p = nullptr;
+  size_t n = 0;
+  bool captured = false;  // a captured graph may hold p
+};
+}  // namespace tnvan
+
 struct tnvan_ctx {
   int device = 0;
   const unsigned long long* step_dev = nullptr;  // tnvan_set_step_counter
@@ -402,19 +412,13 @@ struct tnvan_ctx {
   double* d_stats = nullptr;         // [n_inst][8] + partial tuples (training path)
   double* d_stats_fe = nullptr;      // the same for tnvan_free_energy (inside d_stats' allocation)
   int* d_status = nullptr;           // [4] device status words, then [TNVAN_MAX_INST] reduction counters
-  size_t ws_bytes = 0;
-  void* d_ws = nullptr;              // general workspace
+  tnvan::GrowBuf<unsigned char> ws;      // general workspace
   int reserved_batch = 0;
-  float* d_grad_packed = nullptr;    // packed-layout gradient partials
-  size_t grad_packed_floats = 0;
-  float* d_dj_part = nullptr;        // d/dJ partial rows [CTA][max edges]
-  size_t dj_part_floats = 0;
-  float* d_gen_scratch[2] = {nullptr, nullptr};  // global elimination tables: forward, reverse sweep
-  size_t gen_scratch_floats[2] = {0, 0};
-  bool gen_scratch_captured[2] = {false, false};  // a captured graph may hold the buffer
-  std::vector<float*> gen_scratch_old;            // such buffers, outgrown
-  double* d_wide_part = nullptr;  // per-strip log Z of the wide-strip kernels
-  size_t wide_part_n = 0;
+  tnvan::GrowBuf<float> grad_packed;     // packed-layout gradient partials
+  tnvan::GrowBuf<float> dj_part;         // d/dJ partial rows [CTA][max edges]
+  tnvan::GrowBuf<float> gen_scratch[2];  // global elimination tables: forward, reverse sweep
+  tnvan::GrowBuf<double> wide_part;      // per-strip log Z of the wide-strip kernels
+  std::vector<void*> outgrown;           // buffers a captured graph may still use
   void* d_obs = nullptr;             // tnvan_observables: weights, d/dbeta, sums
   size_t obs_bytes = 0;
 };
