@@ -3400,13 +3400,27 @@ int contract_all(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* d
       if (in.kind == 2 && in.g_ntab > 0 && in.g_ntab <= batch)
         lg.gen_tab = std::max(lg.gen_tab, in.g_ntab);
     // By levels where the kernel's buffers can be had (a capture allocates
-    // nothing), whatever the sizes: from 33 to 32,768 samples of random regular
-    // graphs (n = 128 to 500, widths 1 to 8) 1.1 to 6 times faster than groups of
-    // lanes, with two exceptions: d/dbeta of tables of 4 to 8 entries on average
-    // over more than four rounds of CTAs (n = 500, width 4, 32,768 samples: 803 us
-    // by levels, 653 in lane groups); and few steps left beside the components'
-    // tables (45 of 136 steps, 65,536 samples: 177 us by levels, 132 in lane
-    // groups; with 373 of 374 left 77 against 320).
+    // nothing): 1,000 to 65,536 samples of random regular graphs (n = 128 to 1,000,
+    // widths 1 to 12) take 0.23 to 1.0 times the lane groups' time as long as
+    // those keep their tables in shared memory, which leaves them few CTAs an SM.
+    // With global tables lane groups have 16 CTAs an SM to hide the tables'
+    // latency, and the level kernel's rounds of one CTA an SM lose
+    //   - with d/dbeta and both of its own table sets in global memory too, from
+    //     the second round on (n = 1,000, 14,000 samples, by levels and in lane
+    //     groups: width 8 2,889 and 2,920 us, width 10 7,805 and 6,135, width 12
+    //     23,424 and 18,571; 4,096 samples 793 and 1,194, 2,010 and 2,637, 6,378
+    //     and 8,274);
+    //   - over more than four rounds where a group has at most four lanes (n =
+    //     1,000, 65,536 samples without d/dbeta: width 2 1,736 and 986, width 4
+    //     3,021 and 2,249; 20,000 samples 820 and 1,153, 1,081 and 1,525; eight
+    //     lanes, n = 600 of degree 4, 65,536 samples: 2,643 and 2,875).
+    // Lane groups also skip a tabulated component's steps at no cost, where the
+    // levels stay as many: they win with at most 64 steps left over more than four
+    // rounds (45 of 83 steps, 65,536 samples: 125 us by levels and 99 in lane
+    // groups; 8,192 samples 44 and 75), and without d/dbeta with up to 80 % of the
+    // steps left over more than eight (n = 500, 234 of 327 steps, 65,536 samples:
+    // 433 and 331, with d/dbeta 571 and 784; 20,000 samples 218 and 275; 141 of
+    // 143 left, 65,536 samples: 282 and 405).
     const LevelPlan lp = level_plan(ctx);
     LaunchInfo lw;
     if ((rc = fill_launch(ctx, betas, batch, 32, lw))) return rc;
@@ -3422,16 +3436,17 @@ int contract_all(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* d
       lsm = general_levels_smem_bytes(lp.live, lp.red, Dm, db, place);
       if (lsm <= LEVEL_SMEM || !place) break;
     }
-    double mean = 1;
     int untab = 0;  // steps left beside the tables
     for (const Instance& in : ctx->inst)
       if (in.kind == 2) {
-        mean = std::max(mean, in.g_mean_entries);
         const bool tab = in.g_ntab > 0 && in.g_ntab <= batch;
         untab = std::max(untab, tab ? in.gl_untab : (int)in.gfstep.size());
       }
+    const bool groups_hide = glob && (place ? GL <= 4 && acc > 4 * 152 : db && acc > 152);
+    const bool groups_skip = lg.gen_tab > 0 && (untab <= 64 ? acc > 4 * 152
+                                                            : !db && acc > 8 * 152 && 10 * untab <= 8 * lp.steps);
     const bool by_levels =
-        lsm <= LEVEL_SMEM && !(db && mean >= 4 && mean < 8 && acc > 4 * 152) && !(lg.gen_tab > 0 && untab <= 64) &&
+        lsm <= LEVEL_SMEM && !groups_hide && !groups_skip &&
         try_grow(ctx, ctx->gen_scratch[0],
                  general_levels_scratch_floats(lp.live, lp.steps, db, place, acc, lp.tasks, lsm), s);
     if (glob && (!by_levels || lg.gen_tab > 0) &&

@@ -1,0 +1,76 @@
+"""Which form an elimination call takes (by levels or in lane groups), read off
+the kernels a capture records, and that both forms give the same bits, also where
+the level form keeps its tables in global memory."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2504_12037_gb300 import tnvan as tv
+from paper_2504_12037_gb300 import workloads as wl
+from paper_2504_12037_gb300.model import TNVAN
+
+from gpu_helpers import to_dev_spins
+
+pytestmark = [pytest.mark.gpu, pytest.mark.filterwarnings("ignore:DEBUG")]
+
+
+def _recorded(fn, path):
+    """Names (mangled) of the kernels `fn` launches, from a capture's graph."""
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    graph.enable_debug_mode()
+    with torch.cuda.graph(graph, capture_error_mode="relaxed"):
+        fn()
+    graph.debug_dump(str(path))
+    return path.read_text()
+
+
+def _form(text):
+    levels, groups = "general_levels_kernel" in text, "14general_kernel" in text
+    assert levels != groups
+    return "levels" if levels else "groups"
+
+
+# tables and derivatives of two levels in global memory; tables in shared memory, derivatives in global;
+# both in shared memory with four lanes a sample; tables only, four lanes a sample
+@pytest.mark.parametrize("n,d,wu,db,small,large", [
+    (1000, 3, 10, True, 4800, 4896), (500, 3, 8, True, 4864, 4865), (500, 3, 4, True, 19456, 32768),
+    (1000, 3, 4, True, 19456, 32768), (1000, 3, 4, False, 4096, 32768)])
+def test_forms_agree(n, d, wu, db, small, large, tmp_path):
+    g = wl.random_regular(n, d, 77 + n + d)
+    W, order, _, _ = tv.find_width_set(g.n, g.ei, g.ej, wu, restarts=1, seed=1)
+    model = TNVAN([g], [W], [16], [0.8], seed=3, elim_orders=[order])
+    s = to_dev_spins(np.random.default_rng(5).choice([-1, 1], size=large * len(W)).astype(np.int8))
+
+    def run(b):
+        lz = torch.full((b,), float("nan"), dtype=torch.float64, device="cuda")
+        dl = torch.full((b,), float("nan"), dtype=torch.float64, device="cuda") if db else None
+
+        def call():
+            model.ctx.contract(model.betas, b, s[:b * len(W)], tv.FP32, lz, dl)
+
+        call()
+        torch.cuda.synchronize()
+        out = (lz.clone(), dl.clone() if db else lz.clone())
+        return out, _form(_recorded(call, tmp_path / f"{b}.dot"))
+
+    (lz0, dl0), form0 = run(small)
+    (lz1, dl1), form1 = run(large)
+    assert (form0, form1) == ("levels", "groups")
+    assert torch.isfinite(lz1).all() and torch.isfinite(dl1).all()
+    assert torch.equal(lz0, lz1[:small]) and torch.equal(dl0, dl1[:small])
+
+
+def test_large_untabulated_call_stays_by_levels(tmp_path):
+    """Lane groups keep the tables in shared memory: few CTAs an SM, slower at any batch."""
+    g = wl.random_regular(500, 3, 77 + 503)
+    W, order, _, _ = tv.find_width_set(g.n, g.ei, g.ej, 4, restarts=1, seed=1)
+    model = TNVAN([g], [W], [16], [0.8], seed=3, elim_orders=[order])
+    b = 20000
+    s = to_dev_spins(np.random.default_rng(5).choice([-1, 1], size=b * len(W)).astype(np.int8))
+    lz, dl = torch.empty(2, b, dtype=torch.float64, device="cuda")
+
+    def call():
+        model.ctx.contract(model.betas, b, s, tv.FP32, lz, dl)
+
+    call()
+    assert _form(_recorded(call, tmp_path / "g.dot")) == "levels"
