@@ -95,6 +95,27 @@ __device__ __forceinline__ StepBlock load_block(const GenDev& G, int g) {
   b.h = 0.f;
   return b;
 }
+// The same read by each lane for itself: with one or two lanes a sample, and many
+// CTAs to hide the reads, cheaper than the shuffles (65,536 samples, log Z_R and
+// d/dbeta: n = 1,000 of width 2 985 and 1,439 us with shuffles, 926 and 1,263
+// here; with four lanes, 32,768 samples of width 4, 1,088 and 1,567 against 1,190
+// and 1,522).
+template <int COL>
+__device__ __forceinline__ Step read_step(const GenDev& G, int g, const int8_t* s) {
+  Step r;
+  r.f = G.fstep[g];
+  const int* F = G.fprog + r.f;
+  r.m = F[0];
+  r.nin = F[3];
+  r.ppo = F[5];
+  r.mo = F[6];
+  r.out = F[7 + COL];
+  r.in[0] = r.nin > 0 ? F[9 + COL] : 0;
+  r.in[1] = r.nin > 1 ? F[12 + COL] : 0;
+  r.in[2] = r.nin > 2 ? F[15 + COL] : 0;
+  r.h = field_of(G, F[1], F[2], s);
+  return r;
+}
 template <int COL>
 __device__ __forceinline__ StepBlock load_block(const GenDev& G, int g, const int8_t* s) {
   StepBlock b = load_block<COL>(G, g);
@@ -303,7 +324,7 @@ __device__ __forceinline__ int step_table_any(const Step& r, const GenDev& G, co
 // Component c for the sample whose tables start at A; forward, live offsets.
 // Adds log Z_c (and with DB its beta-derivative) to lz / dl on lane 0 of the
 // group.
-template <bool DB, int U0>
+template <bool DB, int U0, bool DIRECT>
 __device__ __forceinline__ void run_component(const GenDev& G, int c, const int8_t* s, float* A, float* dA, int RS,
                                               int lane, int GL, float beta, double& lz, double& dl) {
   const int* H = G.fprog + G.fhdr[c];
@@ -317,8 +338,8 @@ __device__ __forceinline__ void run_component(const GenDev& G, int c, const int8
   StepBlock blk;
   for (int st = 0; st < nsteps; ++st) {
     const int j = st & (GL - 1);
-    if (j == 0) blk = load_block<0>(G, g0 + min(st + lane, nsteps - 1), s);
-    const Step r = block_step(blk, j, GL);
+    if (!DIRECT && j == 0) blk = load_block<0>(G, g0 + min(st + lane, nsteps - 1), s);
+    const Step r = DIRECT ? read_step<0>(G, g0 + st, s) : block_step(blk, j, GL);
     const float h = r.h, ah = fabsf(h);
     {
       const float y = ah - hc;
@@ -355,7 +376,7 @@ __device__ __forceinline__ void stage_spins(int8_t* ssp, const int8_t* gsp, int 
 }
 
 // li.tile = samples per CTA (S); blockDim.x = S * GL.
-template <bool DB, int U0>
+template <bool DB, int U0, bool DIRECT>
 __global__ void __launch_bounds__(128, U0 > 1 ? 4 : 8) general_kernel(const InstDev* __restrict__ inst,
                                                       const LaunchInfo li, int arena_floats, int GL,
                                                       const int8_t* __restrict__ spins,
@@ -392,7 +413,7 @@ __global__ void __launch_bounds__(128, U0 > 1 ? 4 : 8) general_kernel(const Inst
       lz += G.tab_lz[cr[4] + x];
       if (DB) dl += G.tab_db[cr[4] + x];
     } else {
-      run_component<DB, U0>(G, c, s, A, dA, RS, lane, GL, beta, lz, dl);
+      run_component<DB, U0, DIRECT>(G, c, s, A, dA, RS, lane, GL, beta, lz, dl);
     }
   }
   if (lane != 0 || b >= li.batch) return;
@@ -801,7 +822,7 @@ __global__ void __launch_bounds__(128) general_tab_kernel(const InstDev* __restr
       for (int j = 0; j < cr[2]; ++j) s[G.bpos[cr[3] + j]] = ((x >> j) & 1) ? -1 : 1;
     __syncwarp();
     double lz = 0.0, dl = 0.0;
-    run_component<DB, GEN_U>(G, want, s, A, dA, RS, lane, GL, beta, lz, dl);
+    run_component<DB, GEN_U, false>(G, want, s, A, dA, RS, lane, GL, beta, lz, dl);
     if (mine && live && lane == 0) {
       G.tab_lz[g] = lz;
       if (DB) G.tab_db[g] = dl;
@@ -1501,9 +1522,11 @@ cudaError_t launch_general(const InstDev* d_inst, const LaunchInfo& li, int smem
   if (nblk == 0) return cudaSuccess;
   // li.seed carries the arena size (floats) for this launch
   const int arena = (int)(li.seed & 0xffffffffull);
-  const bool few = nblk <= GEN_FEW;
-  auto kern = dbeta ? (few ? general_kernel<true, GEN_U> : general_kernel<true, 1>)
-                    : (few ? general_kernel<false, GEN_U> : general_kernel<false, 1>);
+  const bool few = nblk <= GEN_FEW, direct = GL <= 2;
+  auto kern = dbeta ? (few ? general_kernel<true, GEN_U, false>
+                           : (direct ? general_kernel<true, 1, true> : general_kernel<true, 1, false>))
+                    : (few ? general_kernel<false, GEN_U, false>
+                           : (direct ? general_kernel<false, 1, true> : general_kernel<false, 1, false>));
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
   if (e != cudaSuccess) return e;
   kern<<<nblk, li.tile * GL, smem_bytes, s>>>(d_inst, li, arena, GL, spins, logZR, dbeta, garena);

@@ -31,10 +31,11 @@ def _form(text):
 
 
 # tables and derivatives of two levels in global memory; tables in shared memory, derivatives in global;
-# both in shared memory with four lanes a sample; tables only, four lanes a sample
+# both in shared memory with four lanes a sample; tables only, four lanes a sample; two lanes a sample
 @pytest.mark.parametrize("n,d,wu,db,small,large", [
     (1000, 3, 10, True, 4800, 4896), (500, 3, 8, True, 4864, 4865), (500, 3, 4, True, 19456, 32768),
-    (1000, 3, 4, True, 19456, 32768), (1000, 3, 4, False, 4096, 32768)])
+    (1000, 3, 4, True, 19456, 32768), (1000, 3, 4, False, 4096, 32768),
+    (1000, 3, 2, True, 4096, 65536), (1000, 3, 2, False, 4096, 65536)])
 def test_forms_agree(n, d, wu, db, small, large, tmp_path):
     g = wl.random_regular(n, d, 77 + n + d)
     W, order, _, _ = tv.find_width_set(g.n, g.ei, g.ej, wu, restarts=1, seed=1)
