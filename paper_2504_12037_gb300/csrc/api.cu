@@ -1,4 +1,5 @@
 // C-ABI of the TNVAN GB300 library: context, host planner, launch sequencing.
+#include <limits.h>
 #include <math.h>
 #include <stdarg.h>
 #include <stdio.h>
@@ -1931,11 +1932,13 @@ bool gen_tables_global(int S, F smem) {
 // What the level kernels of a launch need: the largest over the instances.
 struct LevelPlan {
   int live = 0, total = 0, gmax = 0, red = 0, tasks = 0, steps = 0;
+  bool ok = true;  // every instance has a level schedule
 };
 static LevelPlan level_plan(const tnvan_ctx* ctx) {
   LevelPlan p;
   for (const Instance& in : ctx->inst) {
     if (in.kind != 2) continue;
+    p.ok = p.ok && in.gl_ok;
     p.live = std::max(p.live, in.gl_live);
     p.total = std::max(p.total, in.gl_total);
     p.gmax = std::max(p.gmax, in.gl_gmax);
@@ -3446,7 +3449,7 @@ int contract_all(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* d
     const bool groups_skip = lg.gen_tab > 0 && (untab <= 64 ? acc > 4 * 152
                                                             : !db && acc > 8 * 152 && 10 * untab <= 8 * lp.steps);
     const bool by_levels =
-        lsm <= LEVEL_SMEM && !groups_hide && !groups_skip &&
+        lp.ok && lsm <= LEVEL_SMEM && !groups_hide && !groups_skip &&
         try_grow(ctx, ctx->gen_scratch[0],
                  general_levels_scratch_floats(lp.live, lp.steps, db, place, acc, lp.tasks, lsm), s);
     if (glob && (!by_levels || lg.gen_tab > 0) &&
@@ -3546,6 +3549,8 @@ int run_adjoint(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* d_
             gen_tables_global(T, [&](int t, bool g) { return general_dJ_smem_bytes(per, Dm, me, t, GL, g); });
         const int sm = general_dJ_smem_bytes(per, Dm, me, T, GL, glob);
         if (sm > 227 * 1024) return fail(ctx, TNVAN_E_UNSUPPORTED, "elimination adjoint needs %d B of shared memory", sm);
+        if ((long long)arena * (T + 32 / GL) > INT_MAX)  // a CTA's tables: 32-bit indices
+          return fail(ctx, TNVAN_E_UNSUPPORTED, "elimination adjoint of %d table entries", arena);
         LaunchInfo lg;
         if ((rc = fill_launch(ctx, betas, batch, T, lg))) return rc;
         lg.wmul = wmul;
@@ -3566,7 +3571,7 @@ int run_adjoint(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* d_
           lsm = general_levels_dJ_smem_bytes(lp.total, lp.live, lp.gmax, lp.red, Dm, place);
           if (lsm <= LEVEL_SMEM || !place) break;
         }
-        if (GL >= 2 && lsm <= LEVEL_SMEM && try_grow(ctx, ctx->dj_part, (size_t)acc * GL * stride, s) &&
+        if (GL >= 2 && lp.ok && lsm <= LEVEL_SMEM && try_grow(ctx, ctx->dj_part, (size_t)acc * GL * stride, s) &&
             try_grow(ctx, ctx->gen_scratch[1],
                      general_levels_dJ_scratch_floats(lp.total, lp.live, lp.gmax, lp.steps, place, acc, lp.tasks, lsm),
                      s)) {
@@ -3691,6 +3696,15 @@ void plan_levels(Instance& in, const std::vector<int>& prog, const std::vector<i
   const int L = S ? deepest + 1 : 0;
   std::vector<std::vector<int>> lev(L);
   for (int st = 0; st < S; ++st) lev[deepest - depth[st]].push_back(st);
+  // the kernels' table indices are 32-bit, 32 samples a row
+  long long entries = 0;
+  for (int st = 0; st < S; ++st) entries += 1LL << F[fs[st]];
+  in.gl_ok = 2 * entries <= INT_MAX / 32;
+  if (!in.gl_ok) {
+    for (std::vector<int>* v : {&in.glt, &in.glb, &in.gltl, &in.glbl, &in.glin, &in.glroot}) v->clear();
+    in.gl_levels = in.gl_live = in.gl_total = in.gl_gmax = in.gl_red = in.gl_tasks = in.gl_untab = 0;
+    return;
+  }
   std::vector<int> live(S), full(S), goff(S), size(L + 1, 0), m(S);
   int total = 0, arena = 0, gmax = 0;
   for (int l = 0; l < L; ++l)

@@ -345,6 +345,7 @@ struct Instance {
   std::vector<unsigned short> gmap;       // input index maps (GenDev::map)
   int g_npp = 0;
   std::vector<int> glt, gltl, glb, glbl, glin, glroot;  // level schedule (GenDev)
+  bool gl_ok = false;  // (index ranges allow it)
   int gl_levels = 0, gl_live = 0, gl_total = 0, gl_gmax = 0, gl_red = 0, gl_tasks = 0, gl_untab = 0;
   double g_mean_entries = 1;  // mean table size (entries) of the elimination steps
   int g_max_steps = 0;

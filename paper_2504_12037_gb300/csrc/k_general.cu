@@ -1387,12 +1387,16 @@ cudaError_t launch_general_pp(const InstDev* d_inst, const LaunchInfo& li, int m
   return cudaGetLastError();
 }
 
+// Shared memory sizes count in 64 bits: tables of a few 10^7 entries (a 12 x 1,024
+// strip) pass 2^31 bytes, and a wrapped size would look as if they fitted.
+static int clamp_bytes(long long b) { return (int)std::min<long long>(b, INT_MAX); }
+
 // per-sample floats: 2 * arena + steps + gmax (tables, adjoints, scales, g)
 int general_dJ_smem_bytes(int per_sample, int D, int n_edges, int T, int GL, bool glob) {
   int w4 = (D + 3) / 4;
   if ((w4 & 1) == 0) ++w4;
-  return (glob ? 0 : per_sample * gen_row_stride(T, GL) * 4) + (T * GL / 32) * ((n_edges + 3) & ~3) * 4 +
-         T * 4 * w4;
+  return clamp_bytes((glob ? 0 : 4LL * per_sample * gen_row_stride(T, GL)) +
+                     4LL * (T * GL / 32) * ((n_edges + 3) & ~3) + T * 4 * w4);
 }
 
 size_t general_dJ_scratch_floats(int per_sample, int T, int GL, int nblk) {
@@ -1434,7 +1438,8 @@ static int spin_bytes(int D) {
   return 32 * 4 * w4;
 }
 int general_levels_smem_bytes(int live, int red_slots, int D, bool db, int place) {
-  return 128 * (((place & 1) ? live : 0) + (db && (place & 2) ? live : 0) + red_slots) + spin_bytes(D);
+  const long long rows = ((place & 1) ? live : 0LL) + (db && (place & 2) ? live : 0) + red_slots;
+  return clamp_bytes(128 * rows + spin_bytes(D));
 }
 size_t general_levels_scratch_floats(int live, int steps, bool db, int place, int nblk, int tasks, int smem_bytes) {
   return general_levels_cta_floats(live, steps, db, place) * levels_ctas(nblk, levels_warps(nblk, tasks, smem_bytes), smem_bytes);
@@ -1453,8 +1458,8 @@ cudaError_t launch_general_levels(const InstDev* d_inst, const LaunchInfo& li, i
   return cudaGetLastError();
 }
 int general_levels_dJ_smem_bytes(int total, int live, int gmax, int red_slots, int D, int place) {
-  return 128 * (((place & 1) ? gmax : 0) + ((place & 2) ? live : 0) + ((place & 4) ? total : 0) + red_slots) +
-         spin_bytes(D);
+  const long long rows = ((place & 1) ? gmax : 0LL) + ((place & 2) ? live : 0) + ((place & 4) ? total : 0) + red_slots;
+  return clamp_bytes(128 * rows + spin_bytes(D));
 }
 size_t general_levels_dJ_scratch_floats(int total, int live, int gmax, int steps, int place, int nblk, int tasks,
                                         int smem_bytes) {
@@ -1503,7 +1508,7 @@ cudaError_t launch_general_tables(const InstDev* d_inst, const LaunchInfo& li, i
 int general_smem_bytes(int arena, int D, int T, int GL, bool db, bool glob) {
   int w4 = (D + 3) / 4;
   if ((w4 & 1) == 0) ++w4;
-  return (glob ? 0 : arena * gen_row_stride(T, GL) * 4 * (db ? 2 : 1)) + T * 4 * w4;
+  return clamp_bytes((glob ? 0 : 4LL * arena * gen_row_stride(T, GL) * (db ? 2 : 1)) + T * 4 * w4);
 }
 
 // Scratch of the global-table mode: one [arena][row stride] slice (two with
@@ -1633,7 +1638,7 @@ __global__ void __launch_bounds__(128) general_mom_kernel(const InstDev* __restr
 int general_mom_smem_bytes(int arena, int D, int T, int GL, bool glob) {
   int w4 = (D + 3) / 4;
   if ((w4 & 1) == 0) ++w4;
-  return (glob ? 0 : arena * gen_row_stride(T, GL) * 4 * 3) + T * 4 * w4;
+  return clamp_bytes((glob ? 0 : 12LL * arena * gen_row_stride(T, GL)) + T * 4 * w4);
 }
 
 size_t general_mom_scratch_floats(const LaunchInfo& li, int arena, int GL) {
