@@ -1481,6 +1481,7 @@ cudaError_t launch_general_levels_dJ(const InstDev* d_inst, const LaunchInfo& li
                                                                     place, spins, part, part_stride, gscr);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
+  if (max_edges == 0) return cudaSuccess;  // graphs without bonds
   red<<<dim3((max_edges + 31) / 32, li.n_inst), 512, 0, s>>>(d_inst, li, part, part_stride, dJ);
   return cudaGetLastError();
 }
