@@ -179,7 +179,12 @@ int tnvan_instance_info(const tnvan_ctx* ctx, int instance, int32_t* info);
 
 /* Pre-allocate the context's internal workspaces for batches up to
  * max_batch so that later calls allocate nothing (needed before capturing
- * calls into a CUDA graph).  Synchronous. */
+ * calls into a CUDA graph; tnvan_observables and tnvan_magnetisation, which
+ * wait for host results and cannot be captured, grow workspaces of their own).
+ * Elimination tables that do not fit device memory are left out: calls that
+ * need them then take another form or return TNVAN_E_NOMEM.  A workspace that a
+ * captured call uses is kept until tnvan_destroy when a later, larger call
+ * outgrows it.  Synchronous. */
 int tnvan_reserve(tnvan_ctx* ctx, int max_batch);
 
 /* Algorithm 1 steps (a)-(b) for every instance, in one pass on `stream`:

@@ -1950,6 +1950,144 @@ static LevelPlan level_plan(const tnvan_ctx* ctx) {
 }
 constexpr int LEVEL_SMEM = 216 * 1024;  // and 8 KB of their own
 
+// Launch shapes of an elimination call: the lane-group form's (lg, GL, sm;
+// group_floats of global tables) and the level form's (lw, place, lsm;
+// level_floats of scratch).  levels: the level form where its buffers can be had.
+struct GenForward {
+  LaunchInfo lg, lw;
+  LevelPlan lp;
+  int GL = 1, sm = 0, nsteps = 0, place = 0, lsm = 0;
+  bool db = false, glob = false, levels = false;
+  size_t group_floats = 0, level_floats = 0;
+};
+
+// skip_wide: instances the wide-strip kernel contracts get no tiles.
+int plan_gen_forward(tnvan_ctx* ctx, const double* betas, int batch, bool db, bool skip_wide, GenForward& p) {
+  int rc, arena = 0, Dm = 0;
+  for (const Instance& in : ctx->inst)
+    if (in.kind == 2) {
+      arena = std::max(arena, in.g_max_live);
+      Dm = std::max(Dm, (int)in.W.size());
+      p.nsteps = std::max(p.nsteps, (int)in.gfstep.size());
+    }
+  p.db = db;
+  const int GL = p.GL = gen_lanes(ctx, batch, 16), T = 128 / GL;
+  p.glob = gen_tables_global(T, [&](int t, bool g) { return general_smem_bytes(arena, Dm, t, GL, db, g); });
+  p.sm = general_smem_bytes(arena, Dm, T, GL, db, p.glob);
+  if (p.sm > 227 * 1024) return fail(ctx, TNVAN_E_UNSUPPORTED, "elimination tables need %d B of shared memory", p.sm);
+  LaunchInfo &lg = p.lg, &lw = p.lw;
+  if ((rc = fill_launch(ctx, betas, batch, T, lg)) || (rc = fill_launch(ctx, betas, batch, 32, lw))) return rc;
+  lg.seed = (unsigned long long)arena;
+  // components with small boundaries: tables when they are smaller than the batch
+  for (const Instance& in : ctx->inst)
+    if (in.kind == 2 && in.g_ntab > 0 && in.g_ntab <= batch) lg.gen_tab = std::max(lg.gen_tab, in.g_ntab);
+  lw.gen_tab = lg.gen_tab;
+  int gacc = 0, acc = 0;
+  for (int k = 0; k < lg.n_inst; ++k) {
+    const Instance& in = ctx->inst[k];
+    const bool out = skip_wide && in.kind == 2 && in.dev.n_wide > 0;
+    lg.tile_begin[k] = gacc;
+    lw.tile_begin[k] = acc;
+    if (!out) gacc += (batch + T - 1) / T;
+    if (!out && in.kind == 2) acc += (batch + 31) / 32;
+  }
+  lg.tile_begin[lg.n_inst] = gacc;
+  lw.tile_begin[lw.n_inst] = acc;
+  p.lp = level_plan(ctx);
+  for (p.place = db ? 3 : 1;; p.place >>= 1) {
+    p.lsm = general_levels_smem_bytes(p.lp.live, p.lp.red, Dm, db, p.place);
+    if (p.lsm <= LEVEL_SMEM || !p.place) break;
+  }
+  int untab = 0;  // steps left beside the tables
+  for (const Instance& in : ctx->inst)
+    if (in.kind == 2) {
+      const bool tab = in.g_ntab > 0 && in.g_ntab <= batch;
+      untab = std::max(untab, tab ? in.gl_untab : (int)in.gfstep.size());
+    }
+  // By levels where the kernel's buffers can be had (a capture allocates
+  // nothing): 1,000 to 65,536 samples of random regular graphs (n = 128 to 1,000,
+  // widths 1 to 12) take 0.23 to 1.0 times the lane groups' time as long as
+  // those keep their tables in shared memory, which leaves them few CTAs an SM.
+  // With global tables lane groups have 16 CTAs an SM to hide the tables'
+  // latency, and the level kernel's rounds of one CTA an SM lose
+  //   - with d/dbeta and both of its own table sets in global memory too, from
+  //     the second round on (n = 1,000, 14,000 samples, by levels and in lane
+  //     groups: width 8 2,889 and 2,920 us, width 10 7,805 and 6,135, width 12
+  //     23,424 and 18,571; 4,096 samples 793 and 1,194, 2,010 and 2,637, 6,378
+  //     and 8,274);
+  //   - over more than four rounds where a group has at most four lanes (n =
+  //     1,000, 65,536 samples without d/dbeta: width 2 1,736 and 986, width 4
+  //     3,021 and 2,249; 20,000 samples 820 and 1,153, 1,081 and 1,525; eight
+  //     lanes, n = 600 of degree 4, 65,536 samples: 2,643 and 2,875).
+  // Lane groups also skip a tabulated component's steps at no cost, where the
+  // levels stay as many: they win with at most 64 steps left over more than four
+  // rounds (45 of 83 steps, 65,536 samples: 125 us by levels and 99 in lane
+  // groups; 8,192 samples 44 and 75), and without d/dbeta with up to 80 % of the
+  // steps left over more than eight (n = 500, 234 of 327 steps, 65,536 samples:
+  // 433 and 331, with d/dbeta 571 and 784; 20,000 samples 218 and 275; 141 of
+  // 143 left, 65,536 samples: 282 and 405).
+  const bool groups_hide = p.glob && (p.place ? GL <= 4 && acc > 4 * 152 : db && acc > 152);
+  const bool groups_skip =
+      lg.gen_tab > 0 && (untab <= 64 ? acc > 4 * 152 : !db && acc > 8 * 152 && 10 * untab <= 8 * p.lp.steps);
+  p.levels = p.lp.ok && p.lsm <= LEVEL_SMEM && !groups_hide && !groups_skip;
+  if (p.levels)
+    p.level_floats = general_levels_scratch_floats(p.lp.live, p.lp.steps, db, p.place, acc, p.lp.tasks, p.lsm);
+  if (p.glob) p.group_floats = general_scratch_floats(lg, arena, GL, db);
+  return TNVAN_OK;
+}
+
+// The same of the reverse sweep; rows of d/dJ partials: level_rows, or one a CTA
+// of lg, of `stride` floats.
+struct GenAdjoint {
+  LaunchInfo lg, lw;
+  LevelPlan lp;
+  int GL = 1, sm = 0, nsteps = 0, place = 0, lsm = 0, arena = 0, steps = 0, gmax = 0, me = 0, stride = 0;
+  bool glob = false, levels = false;
+  size_t group_floats = 0, level_floats = 0, level_rows = 0;
+};
+
+int plan_gen_adjoint(tnvan_ctx* ctx, const double* betas, int batch, GenAdjoint& p) {
+  int rc, Dm = 0, mw = 0;
+  for (const Instance& in : ctx->inst)
+    if (in.kind == 2) {
+      p.arena = std::max(p.arena, in.g_max_entries);
+      p.steps = std::max(p.steps, in.g_max_steps);
+      Dm = std::max(Dm, (int)in.W.size());
+      p.me = std::max(p.me, in.m);
+      p.nsteps = std::max(p.nsteps, (int)in.gfstep.size());
+      mw = std::max(mw, in.max_width);
+    }
+  p.gmax = 2 << mw;  // g of one step: 2^(m+1) extended indices
+  p.stride = (p.me + 3) & ~3;
+  const int per = 2 * p.arena + p.steps + p.gmax;
+  const int GL = p.GL = gen_lanes(ctx, batch, 8), T = 128 / GL;
+  p.glob = gen_tables_global(T, [&](int t, bool g) { return general_dJ_smem_bytes(per, Dm, p.me, t, GL, g); });
+  p.sm = general_dJ_smem_bytes(per, Dm, p.me, T, GL, p.glob);
+  if (p.sm > 227 * 1024) return fail(ctx, TNVAN_E_UNSUPPORTED, "elimination adjoint needs %d B of shared memory", p.sm);
+  if ((long long)p.arena * (T + 32 / GL) > INT_MAX)  // a CTA's tables: 32-bit indices
+    return fail(ctx, TNVAN_E_UNSUPPORTED, "elimination adjoint of %d table entries", p.arena);
+  if ((rc = fill_launch(ctx, betas, batch, T, p.lg)) || (rc = fill_launch(ctx, betas, batch, 32, p.lw))) return rc;
+  int acc = 0;
+  for (int k = 0; k <= p.lw.n_inst; ++k) {
+    p.lw.tile_begin[k] = acc;
+    if (k < p.lw.n_inst && ctx->inst[k].kind == 2) acc += (batch + 31) / 32;
+  }
+  // by levels where the sum order allows it (2, 4 or 8 lanes per sample)
+  p.lp = level_plan(ctx);
+  for (p.place = 7;; p.place >>= 1) {
+    p.lsm = general_levels_dJ_smem_bytes(p.lp.total, p.lp.live, p.lp.gmax, p.lp.red, Dm, p.place);
+    if (p.lsm <= LEVEL_SMEM || !p.place) break;
+  }
+  p.levels = GL >= 2 && p.lp.ok && p.lsm <= LEVEL_SMEM;
+  if (p.levels) {
+    p.level_rows = (size_t)acc * GL;
+    p.level_floats = general_levels_dJ_scratch_floats(p.lp.total, p.lp.live, p.lp.gmax, p.lp.steps, p.place, acc,
+                                                      p.lp.tasks, p.lsm);
+  }
+  if (p.glob) p.group_floats = general_dJ_scratch_floats(per, T, GL, p.lg.tile_begin[p.lg.n_inst]);
+  return TNVAN_OK;
+}
+
 static int wide_max_strips(const tnvan_ctx* ctx) {
   int ms = 0;
   for (const Instance& in : ctx->inst)
@@ -1964,36 +2102,84 @@ static size_t grad_ws_floats(const tnvan_ctx* ctx, int batch) {
   return (size_t)bwd32_splits(ctx, batch) * ctx->inst.size() * (size_t)maxp;
 }
 
+// The batches up to max_batch at which a launch shape of the elimination calls
+// changes, and max_batch: every buffer a smaller batch needs is largest at one
+// of these.
+static std::vector<int> gen_batches(const tnvan_ctx* ctx, int max_batch) {
+  std::vector<int> b = {max_batch};
+  auto add = [&](long long v) {
+    if (v >= 1 && v < max_batch) b.push_back((int)v);
+  };
+  for (int gl = 1; gl <= 16; gl *= 2) add((1 << 17) / gl - 1);  // gen_lanes
+  long long gen = 0, nowide = 0;
+  for (const Instance& in : ctx->inst)
+    if (in.kind == 2) {
+      ++gen;
+      nowide += in.dev.n_wide == 0;
+      add(in.g_ntab - 1);
+    }
+  for (int r : {1, 4, 8})  // the dispatch's rounds of tiles of 32 samples
+    for (long long n : {gen, nowide})
+      if (n > 0) add(32 * (r * 152 / n));
+  return b;
+}
+
 int tnvan_reserve(tnvan_ctx* ctx, int max_batch) {
   if (!ctx || max_batch < 0) return TNVAN_E_ARG;
   DeviceGuard g(ctx->device);
   int rc = check_ready(ctx, false);
   if (rc) return rc;
   const cudaStream_t s = nullptr;
-  rc = grow(ctx, ctx->grad_packed, grad_ws_floats(ctx, std::max(max_batch, 1)), s, "gradient partials");
+  const int B = std::max(max_batch, 1), n = (int)ctx->inst.size(), tiles = (B + 127) / 128;
+  // gradient partials: rows of the FP32 backward, of the tensor-core chain, and of
+  // the fused backward (plan_fused_bwd; a smaller batch may be cut into more CTAs)
+  long long maxp = 0;
+  for (const Instance& in : ctx->inst) maxp = std::max(maxp, (in.n_params + 3) & ~3LL);
+  const size_t cut = std::min(tiles, ctx->tune_bwd_ctas ? ctx->tune_bwd_ctas : (148 + n - 1) / std::max(n, 1));
+  const size_t fused_rows = n * cut + (n > 1 ? std::max<size_t>(cut, (tiles + 1) / 2) - cut : 0);
+  const size_t tc_rows = (size_t)std::max(1, std::min(TC_SPLITS, tiles)) * n;
+  rc = grow(ctx, ctx->grad_packed, std::max(grad_ws_floats(ctx, B), std::max(fused_rows, tc_rows) * (size_t)maxp), s,
+            "gradient partials");
   if (rc) return rc;
-  {
-    long long maxp = 0;
-    for (const Instance& in : ctx->inst) maxp = std::max(maxp, in.n_params);
-    const int splits = std::max(1, std::min(TC_SPLITS, (std::max(max_batch, 1) + 127) / 128));
-    rc = grow(ctx, ctx->grad_packed, std::max(grad_ws_floats(ctx, std::max(max_batch, 1)),
-                                      (size_t)splits * ctx->inst.size() * (size_t)maxp), s, "gradient partials");
-    if (rc) return rc;
-    rc = grow(ctx, ctx->ws, std::max(tc_ws_floats(ctx, std::max(max_batch, 1)),
-                                 bwd32_ws_floats(ctx, std::max(max_batch, 1), nullptr)) * sizeof(float), s, "workspace");
-    if (rc) return rc;
-    int max_edges = 0, ctas = 0;
-    for (const Instance& in : ctx->inst) {
-      max_edges = std::max(max_edges, in.m);
-      // elimination instances: up to 8 rows per 32 samples
-      ctas += in.kind == 2 ? 8 * ((std::max(max_batch, 1) + 31) / 32) : (std::max(max_batch, 1) + 127) / 128;
+  rc = grow(ctx, ctx->ws, std::max(tc_ws_floats(ctx, B), bwd32_ws_floats(ctx, B, nullptr)) * sizeof(float), s,
+            "workspace");
+  if (rc) return rc;
+  int max_edges = 0;
+  size_t rows = 0;
+  for (const Instance& in : ctx->inst) {
+    max_edges = std::max(max_edges, in.m);
+    // d/dJ partials: a row per 32 samples at least; elimination instances up to 8
+    rows += (size_t)(in.kind == 2 ? 8 : 1) * ((B + 31) / 32);
+  }
+  rc = grow(ctx, ctx->dj_part, rows * ((max_edges + 3) & ~3), s, "d/dJ partials");
+  if (rc) return rc;
+  const int ms = wide_max_strips(ctx);
+  if (ms > 0 && (rc = grow(ctx, ctx->wide_part, ctx->inst.size() * (size_t)B * ms, s, "wide strips"))) return rc;
+  // elimination tables; where they cannot be had, the calls that need them say so
+  // or take the other form, as without a reservation
+  bool gen = false, wide = false;
+  for (const Instance& in : ctx->inst) {
+    gen = gen || in.kind == 2;
+    wide = wide || (in.kind == 2 && in.dev.n_wide > 0);
+  }
+  if (gen) {
+    const std::vector<double> ones(n, 1.0);
+    size_t levels[2] = {0, 0}, groups[2] = {0, 0};
+    for (int b : gen_batches(ctx, B)) {
+      for (bool db : {false, true}) {
+        GenForward p;
+        if (plan_gen_forward(ctx, ones.data(), b, db, wide && !db, p)) continue;
+        levels[0] = std::max(levels[0], p.level_floats);
+        if (!p.levels || p.lg.gen_tab > 0) groups[0] = std::max(groups[0], p.group_floats);
+      }
+      GenAdjoint p;
+      if (plan_gen_adjoint(ctx, ones.data(), b, p)) continue;
+      levels[1] = std::max(levels[1], p.level_floats);
+      if (!p.levels) groups[1] = std::max(groups[1], p.group_floats);
     }
-    rc = grow(ctx, ctx->dj_part, (size_t)ctas * ((max_edges + 3) & ~3), s, "d/dJ partials");
-    if (rc) return rc;
-    const int ms = wide_max_strips(ctx);
-    if (ms > 0 &&
-        (rc = grow(ctx, ctx->wide_part, ctx->inst.size() * (size_t)std::max(max_batch, 1) * ms, s, "wide strips")))
-      return rc;
+    for (int k = 0; k < 2; ++k)
+      if (!try_grow(ctx, ctx->gen_scratch[k], std::max(levels[k], groups[k]), s))
+        try_grow(ctx, ctx->gen_scratch[k], std::min(levels[k], groups[k]), s);
   }
   ctx->reserved_batch = std::max(ctx->reserved_batch, max_batch);
   CK(cudaDeviceSynchronize(), "reserve");
@@ -3369,104 +3555,29 @@ int contract_all(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* d
     k2 = rest;
   }
   if (k2) {
-    int arena = 0, Dm = 0, nsteps = 0;
-    for (const Instance& in : ctx->inst)
-      if (in.kind == 2) {
-        arena = std::max(arena, in.g_max_live);
-        Dm = std::max(Dm, (int)in.W.size());
-        nsteps = std::max(nsteps, (int)in.gfstep.size());
-      }
-    const bool db = d_dbeta != nullptr;
-    const int GL = gen_lanes(ctx, batch, 16), T = 128 / GL;
-    const bool glob =
-        gen_tables_global(T, [&](int t, bool g) { return general_smem_bytes(arena, Dm, t, GL, db, g); });
-    const int sm = general_smem_bytes(arena, Dm, T, GL, db, glob);
-    if (sm > 227 * 1024) return fail(ctx, TNVAN_E_UNSUPPORTED, "elimination tables need %d B of shared memory", sm);
-    LaunchInfo lg;
-    if ((rc = fill_launch(ctx, betas, batch, T, lg))) return rc;
-    lg.seed = (unsigned long long)arena;
-    if (any_wide) {  // instances the wide-strip kernel has contracted get no tiles
-      int acc = 0;
-      for (int k = 0; k < lg.n_inst; ++k) {
-        const int nt = lg.tile_begin[k + 1] - lg.tile_begin[k];
-        lg.tile_begin[k] = acc;
-        if (!(ctx->inst[k].kind == 2 && ctx->inst[k].dev.n_wide > 0)) acc += nt;
-      }
-      lg.tile_begin[lg.n_inst] = acc;
-    }
+    GenForward p;
+    if ((rc = plan_gen_forward(ctx, betas, batch, d_dbeta != nullptr, any_wide, p))) return rc;
     {
       PROF("general_pp", s);
-      CK(launch_general_pp(ctx->d_inst, lg, nsteps, s), "elimination bond products");
+      CK(launch_general_pp(ctx->d_inst, p.lg, p.nsteps, s), "elimination bond products");
     }
-    // components with small boundaries: tables when they are smaller than the batch
-    for (const Instance& in : ctx->inst)
-      if (in.kind == 2 && in.g_ntab > 0 && in.g_ntab <= batch)
-        lg.gen_tab = std::max(lg.gen_tab, in.g_ntab);
-    // By levels where the kernel's buffers can be had (a capture allocates
-    // nothing): 1,000 to 65,536 samples of random regular graphs (n = 128 to 1,000,
-    // widths 1 to 12) take 0.23 to 1.0 times the lane groups' time as long as
-    // those keep their tables in shared memory, which leaves them few CTAs an SM.
-    // With global tables lane groups have 16 CTAs an SM to hide the tables'
-    // latency, and the level kernel's rounds of one CTA an SM lose
-    //   - with d/dbeta and both of its own table sets in global memory too, from
-    //     the second round on (n = 1,000, 14,000 samples, by levels and in lane
-    //     groups: width 8 2,889 and 2,920 us, width 10 7,805 and 6,135, width 12
-    //     23,424 and 18,571; 4,096 samples 793 and 1,194, 2,010 and 2,637, 6,378
-    //     and 8,274);
-    //   - over more than four rounds where a group has at most four lanes (n =
-    //     1,000, 65,536 samples without d/dbeta: width 2 1,736 and 986, width 4
-    //     3,021 and 2,249; 20,000 samples 820 and 1,153, 1,081 and 1,525; eight
-    //     lanes, n = 600 of degree 4, 65,536 samples: 2,643 and 2,875).
-    // Lane groups also skip a tabulated component's steps at no cost, where the
-    // levels stay as many: they win with at most 64 steps left over more than four
-    // rounds (45 of 83 steps, 65,536 samples: 125 us by levels and 99 in lane
-    // groups; 8,192 samples 44 and 75), and without d/dbeta with up to 80 % of the
-    // steps left over more than eight (n = 500, 234 of 327 steps, 65,536 samples:
-    // 433 and 331, with d/dbeta 571 and 784; 20,000 samples 218 and 275; 141 of
-    // 143 left, 65,536 samples: 282 and 405).
-    const LevelPlan lp = level_plan(ctx);
-    LaunchInfo lw;
-    if ((rc = fill_launch(ctx, betas, batch, 32, lw))) return rc;
-    lw.gen_tab = lg.gen_tab;
-    int acc = 0;
-    for (int k = 0; k < lw.n_inst; ++k) {  // no tiles for other kinds and what the wide-strip kernel has contracted
-      lw.tile_begin[k] = acc;
-      if (ctx->inst[k].kind == 2 && lg.tile_begin[k + 1] > lg.tile_begin[k]) acc += (batch + 31) / 32;
-    }
-    lw.tile_begin[lw.n_inst] = acc;
-    int place = db ? 3 : 1, lsm = 0;
-    for (;; place >>= 1) {
-      lsm = general_levels_smem_bytes(lp.live, lp.red, Dm, db, place);
-      if (lsm <= LEVEL_SMEM || !place) break;
-    }
-    int untab = 0;  // steps left beside the tables
-    for (const Instance& in : ctx->inst)
-      if (in.kind == 2) {
-        const bool tab = in.g_ntab > 0 && in.g_ntab <= batch;
-        untab = std::max(untab, tab ? in.gl_untab : (int)in.gfstep.size());
-      }
-    const bool groups_hide = glob && (place ? GL <= 4 && acc > 4 * 152 : db && acc > 152);
-    const bool groups_skip = lg.gen_tab > 0 && (untab <= 64 ? acc > 4 * 152
-                                                            : !db && acc > 8 * 152 && 10 * untab <= 8 * lp.steps);
-    const bool by_levels =
-        lp.ok && lsm <= LEVEL_SMEM && !groups_hide && !groups_skip &&
-        try_grow(ctx, ctx->gen_scratch[0],
-                 general_levels_scratch_floats(lp.live, lp.steps, db, place, acc, lp.tasks, lsm), s);
-    if (glob && (!by_levels || lg.gen_tab > 0) &&
-        (rc = grow(ctx, ctx->gen_scratch[0], general_scratch_floats(lg, arena, GL, db), s, "elimination tables")))
+    const bool by_levels = p.levels && try_grow(ctx, ctx->gen_scratch[0], p.level_floats, s);
+    if ((!by_levels || p.lg.gen_tab > 0) &&
+        (rc = grow(ctx, ctx->gen_scratch[0], p.group_floats, s, "elimination tables")))
       return rc;
     float* gs = ctx->gen_scratch[0].p;
-    if (lg.gen_tab > 0) {
+    if (p.lg.gen_tab > 0) {
       PROF("general_tables", s);
-      CK(launch_general_tables(ctx->d_inst, lg, sm, db, GL, glob ? gs : nullptr, s), "general tables kernel");
+      CK(launch_general_tables(ctx->d_inst, p.lg, p.sm, p.db, p.GL, p.glob ? gs : nullptr, s),
+         "general tables kernel");
     }
     PROF(d_dbeta ? "general_dbeta" : "general", s);
     if (by_levels)
-      CK(launch_general_levels(ctx->d_inst, lw, lsm, lp.live, lp.steps, lp.red, lp.tasks, place, d_spins, d_logZR,
-                               d_dbeta, gs, s),
+      CK(launch_general_levels(ctx->d_inst, p.lw, p.lsm, p.lp.live, p.lp.steps, p.lp.red, p.lp.tasks, p.place, d_spins,
+                               d_logZR, d_dbeta, gs, s),
          "general kernel");
     else
-      CK(launch_general(ctx->d_inst, lg, sm, GL, d_spins, d_logZR, d_dbeta, glob ? gs : nullptr, s),
+      CK(launch_general(ctx->d_inst, p.lg, p.sm, p.GL, d_spins, d_logZR, d_dbeta, p.glob ? gs : nullptr, s),
          "general kernel");
   }
   return TNVAN_OK;
@@ -3529,78 +3640,33 @@ int run_adjoint(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* d_
         PROF("dense_dJ", s);
         CK(launch_dense(ctx->d_inst, lt, precision, d_spins, nullptr, nullptr, d_dJ, s), "dense adjoint kernel");
       }
-      int arena = 0, steps = 0, Dm = 0, me = 0, nsteps = 0, mw = 0;
       bool any_gen = false;
-      for (const Instance& in : ctx->inst)
-        if (in.kind == 2) {
-          any_gen = true;
-          arena = std::max(arena, in.g_max_entries);
-          steps = std::max(steps, in.g_max_steps);
-          Dm = std::max(Dm, (int)in.W.size());
-          me = std::max(me, in.m);
-          nsteps = std::max(nsteps, (int)in.gfstep.size());
-          mw = std::max(mw, in.max_width);
-        }
+      for (const Instance& in : ctx->inst) any_gen = any_gen || in.kind == 2;
       if (any_gen) {
-        const int gmax = 2 << mw;  // g of one step: 2^(m+1) extended indices
-        const int per = 2 * arena + steps + gmax;
-        const int GL = gen_lanes(ctx, batch, 8), T = 128 / GL;
-        const bool glob =
-            gen_tables_global(T, [&](int t, bool g) { return general_dJ_smem_bytes(per, Dm, me, t, GL, g); });
-        const int sm = general_dJ_smem_bytes(per, Dm, me, T, GL, glob);
-        if (sm > 227 * 1024) return fail(ctx, TNVAN_E_UNSUPPORTED, "elimination adjoint needs %d B of shared memory", sm);
-        if ((long long)arena * (T + 32 / GL) > INT_MAX)  // a CTA's tables: 32-bit indices
-          return fail(ctx, TNVAN_E_UNSUPPORTED, "elimination adjoint of %d table entries", arena);
-        LaunchInfo lg;
-        if ((rc = fill_launch(ctx, betas, batch, T, lg))) return rc;
-        lg.wmul = wmul;
-        const int stride = (me + 3) & ~3;
-        // by levels where the sum order allows it (2, 4 or 8 lanes per sample) and
-        // the kernel's buffers can be had
-        const LevelPlan lp = level_plan(ctx);
-        LaunchInfo lw;
-        if ((rc = fill_launch(ctx, betas, batch, 32, lw))) return rc;
-        lw.wmul = wmul;
-        int acc = 0;
-        for (int k = 0; k <= lw.n_inst; ++k) {
-          lw.tile_begin[k] = acc;
-          if (k < lw.n_inst && ctx->inst[k].kind == 2) acc += (batch + 31) / 32;
-        }
-        int place = 7, lsm = 0;
-        for (;; place >>= 1) {
-          lsm = general_levels_dJ_smem_bytes(lp.total, lp.live, lp.gmax, lp.red, Dm, place);
-          if (lsm <= LEVEL_SMEM || !place) break;
-        }
-        if (GL >= 2 && lp.ok && lsm <= LEVEL_SMEM && try_grow(ctx, ctx->dj_part, (size_t)acc * GL * stride, s) &&
-            try_grow(ctx, ctx->gen_scratch[1],
-                     general_levels_dJ_scratch_floats(lp.total, lp.live, lp.gmax, lp.steps, place, acc, lp.tasks, lsm),
-                     s)) {
-          {
-            PROF("general_pp", s);
-            CK(launch_general_pp(ctx->d_inst, lg, nsteps, s), "elimination bond products");
-          }
-          PROF("general_dJ", s);
-          CK(launch_general_levels_dJ(ctx->d_inst, lw, lsm, GL, lp.total, lp.live, lp.gmax, lp.steps, lp.red, lp.tasks,
-                                      place, me, d_spins, ctx->dj_part.p, stride, d_dJ, ctx->gen_scratch[1].p, s),
-             "general adjoint kernel");
-          return TNVAN_OK;
-        }
-        if ((rc = grow(ctx, ctx->dj_part, (size_t)lg.tile_begin[lg.n_inst] * stride, s, "d/dJ partials"))) return rc;
-        float* gs = nullptr;
-        if (glob) {
-          if ((rc = grow(ctx, ctx->gen_scratch[1], general_dJ_scratch_floats(per, T, GL, lg.tile_begin[lg.n_inst]), s,
-                         "elimination tables")))
-            return rc;
-          gs = ctx->gen_scratch[1].p;
-        }
+        GenAdjoint p;
+        if ((rc = plan_gen_adjoint(ctx, betas, batch, p))) return rc;
+        p.lg.wmul = p.lw.wmul = wmul;
+        const bool by_levels = p.levels && try_grow(ctx, ctx->dj_part, p.level_rows * p.stride, s) &&
+                               try_grow(ctx, ctx->gen_scratch[1], p.level_floats, s);
+        if (!by_levels &&
+            ((rc = grow(ctx, ctx->dj_part, (size_t)p.lg.tile_begin[p.lg.n_inst] * p.stride, s, "d/dJ partials")) ||
+             (rc = grow(ctx, ctx->gen_scratch[1], p.group_floats, s, "elimination tables"))))
+          return rc;
         {
           PROF("general_pp", s);
-          CK(launch_general_pp(ctx->d_inst, lg, nsteps, s), "elimination bond products");
+          CK(launch_general_pp(ctx->d_inst, p.lg, p.nsteps, s), "elimination bond products");
         }
         PROF("general_dJ", s);
-        CK(launch_general_dJ(ctx->d_inst, lg, sm, arena, steps, gmax, GL, d_spins, ctx->dj_part.p, stride, d_dJ, gs,
-                             s),
-           "general adjoint kernel");
+        float* gs = ctx->gen_scratch[1].p;
+        if (by_levels)
+          CK(launch_general_levels_dJ(ctx->d_inst, p.lw, p.lsm, p.GL, p.lp.total, p.lp.live, p.lp.gmax, p.lp.steps,
+                                      p.lp.red, p.lp.tasks, p.place, p.me, d_spins, ctx->dj_part.p, p.stride, d_dJ, gs,
+                                      s),
+             "general adjoint kernel");
+        else
+          CK(launch_general_dJ(ctx->d_inst, p.lg, p.sm, p.arena, p.steps, p.gmax, p.GL, d_spins, ctx->dj_part.p,
+                               p.stride, d_dJ, p.glob ? gs : nullptr, s),
+             "general adjoint kernel");
       }
     }
   }
