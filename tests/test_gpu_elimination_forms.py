@@ -61,6 +61,48 @@ def test_forms_agree(n, d, wu, db, small, large, tmp_path):
     assert torch.equal(lz0, lz1[:small]) and torch.equal(dl0, dl1[:small])
 
 
+@pytest.mark.parametrize("n,d,wu,insts,batch", [
+    (64, 3, 1, 3, 33), (128, 3, 3, 1, 130), (90, 3, 4, 2, 65), (60, 3, 7, 2, 300), (500, 3, 8, 1, 200)])
+def test_adjoint_forms_agree(n, d, wu, insts, batch, tmp_path):
+    """A capture that finds no buffers records lane groups; log Z_R and d/dbeta have the same bits, d/dJ is
+    added up over the batch in FP64 in another order."""
+    gs = [wl.random_regular(n + 8 * k, d, 11 + n + d + k) for k in range(insts)]
+    plans = [tv.find_width_set(g.n, g.ei, g.ej, wu, restarts=1, seed=1)[:2] for g in gs]
+    model = TNVAN(gs, [W for W, _ in plans], [16], [0.7 + 0.2 * k for k in range(insts)], seed=3,
+                  elim_orders=[o for _, o in plans])
+    D, m = sum(model.D), sum(model.n_edges)
+    s = to_dev_spins(np.random.default_rng(n).choice([-1, 1], size=batch * D).astype(np.int8))
+    model.ctx.reserve(1)
+    lz, lz1, db = torch.full((3, insts * batch), float("nan"), dtype=torch.float64, device="cuda")
+    dJ = torch.full((m,), float("nan"), dtype=torch.float64, device="cuda")
+    lq, grad = torch.zeros(insts * batch, device="cuda"), torch.empty_like(model.params)
+
+    def call():
+        model.ctx.contract(model.betas, batch, s, tv.FP32, lz)
+        model.ctx.contract(model.betas, batch, s, tv.FP32, lz1, db)
+        model.ctx.backward(model.betas, batch, s, lz, lq, tv.FP32, grad, None, dJ)
+
+    def run(path):
+        graph = torch.cuda.CUDAGraph(keep_graph=True)
+        graph.enable_debug_mode()
+        with torch.cuda.graph(graph, capture_error_mode="relaxed"):
+            call()
+        graph.debug_dump(str(path))
+        graph.instantiate()
+        graph.replay()
+        torch.cuda.synchronize()
+        text = path.read_text()
+        return _form(text), "general_levels_dJ_kernel" in text, [t.clone() for t in (lz, lz1, db, dJ)]
+
+    form0, dj0, out0 = run(tmp_path / "groups.dot")
+    call()  # allocates
+    form1, dj1, out1 = run(tmp_path / "levels.dot")
+    assert (form0, dj0, form1, dj1) == ("groups", False, "levels", True)
+    for a, b in zip(out0[:3], out1[:3]):
+        assert torch.isfinite(b).all() and torch.equal(a, b)
+    assert float((out0[3] - out1[3]).abs().max()) <= 1e-14 * max(1.0, float(out1[3].abs().max()))
+
+
 def test_large_untabulated_call_stays_by_levels(tmp_path):
     """Lane groups keep the tables in shared memory: few CTAs an SM, slower at any batch."""
     g = wl.random_regular(500, 3, 77 + 503)
