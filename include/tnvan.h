@@ -431,7 +431,9 @@ int tnvan_train_step(tnvan_ctx* ctx, const double* betas, int batch, uint64_t se
  * in a CUDA graph on a private stream and replayed, with learning rate 0 and
  * scratch moments, so the networks are left as they were.  out (host
  * int32[7], may be NULL) receives the choices in that order (0 = heuristic,
- * not tuned).
+ * not tuned); the first two are the fastest of the fixed counts below, also
+ * where the context keeps its own count by batch size because that is the same
+ * or faster.
  * Synchronous; allocates and frees temporary device buffers.
  * Errors: TNVAN_E_ARG, TNVAN_E_STATE, TNVAN_E_NOMEM, TNVAN_E_CUDA. */
 int tnvan_autotune(tnvan_ctx* ctx, const double* betas, int batch, int precision, void* stream,

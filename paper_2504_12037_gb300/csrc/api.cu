@@ -644,6 +644,12 @@ int pick_sample_tile(const tnvan_ctx* ctx, int batch) {
 }
 
 
+// Samples per CTA of the strip contraction by rule: 32 where that is what it
+// takes to share few samples out over the SMs.
+int pick_strip_tile(const tnvan_ctx* ctx, int batch) {
+  return (long long)ctx->inst.size() * ((batch + 127) / 128) < 152 ? 32 : 128;
+}
+
 // Launch shape of the strip adjoint: one thread per sample with T in
 // {128, 96, 64, 32} samples per CTA (all strips in turn), or one warp per
 // strip over 32 samples per CTA (ws_threads = 32 x strips; tuning value 1).
@@ -2979,23 +2985,30 @@ int tnvan_autotune(tnvan_ctx* ctx, const double* betas, int batch, int precision
     ctx->tune_tc_plan = best;
     ctx->tune_tc_form = best >= 0 ? best_form : 0;
   }
+  // the fixed counts reported; the context keeps its own rule (0) where that is
+  // the same launch or faster
+  int fixed_sample = ctx->tune_sample_tile, fixed_strip = ctx->tune_strip_tile;
   if (!tc_sampler) {
     int best = 0;
-    float best_ms = 1e30f;
-    for (int T : {16, 32, 64}) {
-      if (max_sample_smem(ctx, T) > 227 * 1024) continue;
+    float best_ms = 1e30f, rule_ms = 0.f;
+    for (int T : {0, 16, 32, 64}) {
+      if (T && max_sample_smem(ctx, T) > 227 * 1024) continue;
       ctx->tune_sample_tile = T;
       float ms = 0.f;
       if ((rc = time_it(sample, &ms))) {
         cleanup();
         return rc;
       }
-      if (ms < best_ms) {
+      if (!T) {
+        rule_ms = ms;
+      } else if (ms < best_ms) {
         best_ms = ms;
         best = T;
       }
     }
-    ctx->tune_sample_tile = best;
+    fixed_sample = best;
+    ctx->tune_sample_tile = 0;
+    if (best && best_ms < rule_ms && best != pick_sample_tile(ctx, batch)) ctx->tune_sample_tile = best;
   }
   if ((rc = sample())) {  // spins for the contraction and backward candidates
     cleanup();
@@ -3005,8 +3018,8 @@ int tnvan_autotune(tnvan_ctx* ctx, const double* betas, int batch, int precision
   for (const Instance& in : ctx->inst) any_strip = any_strip || in.kind == 0;
   if (any_strip) {
     int best = 0;
-    float best_ms = 1e30f;
-    for (int T : {32, 64, 128}) {
+    float best_ms = 1e30f, rule_ms = 0.f;
+    for (int T : {0, 32, 64, 128}) {
       ctx->tune_strip_tile = T;
       float ms = 0.f;
       auto contract = [&]() { return tnvan_contract(ctx, betas, batch, sp, precision, lz, nullptr, stream); };
@@ -3014,12 +3027,16 @@ int tnvan_autotune(tnvan_ctx* ctx, const double* betas, int batch, int precision
         cleanup();
         return rc;
       }
-      if (ms < best_ms) {
+      if (!T) {
+        rule_ms = ms;
+      } else if (ms < best_ms) {
         best_ms = ms;
         best = T;
       }
     }
-    ctx->tune_strip_tile = best;
+    fixed_strip = best;
+    ctx->tune_strip_tile = 0;
+    if (best_ms < rule_ms && best != pick_strip_tile(ctx, batch)) ctx->tune_strip_tile = best;
   }
   bool fused = precision == TNVAN_BF16;
   for (const Instance& in : ctx->inst) fused = fused && in.dev.made.fused_ok;
@@ -3209,8 +3226,8 @@ int tnvan_autotune(tnvan_ctx* ctx, const double* betas, int batch, int precision
     cudaFree(db);
   }
   if (out) {
-    out[0] = ctx->tune_sample_tile;
-    out[1] = ctx->tune_strip_tile;
+    out[0] = fixed_sample;
+    out[1] = fixed_strip;
     out[2] = ctx->tune_bwd_ctas;
     out[3] = ctx->tune_adj_tile;
     out[4] = tc_plan_value(ctx, ctx->tune_tc_plan);
@@ -3497,8 +3514,7 @@ int contract_all(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* d
         for (const StripDev& sd : in.strip.strips) max_w = std::max(max_w, sd.w);
       }
     if (sm > 227 * 1024) return fail(ctx, TNVAN_E_UNSUPPORTED, "strip tables need %d B of shared memory", sm);
-    // few samples: 32 a CTA, so that more SMs share them
-    if (!ctx->tune_strip_tile && (long long)li.n_inst * ((batch + 127) / 128) < 152) stile = 32;
+    if (!ctx->tune_strip_tile) stile = pick_strip_tile(ctx, batch);
     for (;; stile /= 2) {
       sm = 0;
       for (const Instance& in : ctx->inst)
