@@ -10,8 +10,8 @@
 //   v <- D_y v       D_y(x) = product over the row's bonds that x leaves
 //                    unsatisfied (J s s' < 0, W neighbours included) of
 //                    exp(-2 beta |J|): every factor is at most 1;
-//   v <- v / 2^e     e the exponent of the row's largest entry.
-// ln Z_strip = ln sum_x v(x) + ln 2 sum e + beta sum |J| over the strip's
+//   v <- v 2^k       where the row's largest entry has left [2^20, 2^81).
+// ln Z_strip = ln sum_x v(x) - ln 2 sum k + beta sum |J| over the strip's
 // bonds; log Z_R adds beta sum over W-W bonds J s s' (Eq. 4).
 //
 // The 2^w states of a row are spread over the warp: bits 0-4 of a state on the
@@ -24,9 +24,12 @@
 // D_y of a state is a product over the bonds in column order, the W neighbours
 // after bond 3 and last.  Its lane part is formed once per lane and row; the
 // register part along the binary tree of j's bits, so a state costs about
-// three products and not a chain of nine conditional ones.  The power of two
-// of the row before rides on the lane part.  The factors are tabulated per
-// strip row and beta (wide_tab_kernel).  Every value is rounded as in the
+// three products and not a chain of nine conditional ones.  Entries 2^-149 times
+// the largest have to survive a row (at low temperature a frustrated row can
+// make the next row's largest of them), so scales go into v, not into D, and
+// before the largest entry falls below 1; keeping it near 2^50 leaves most rows
+// without a scaling pass.  The factors are tabulated per strip row and beta
+// (wide_tab_kernel).  Every value is rounded as in the
 // plain chain of products: at high temperature the same few products recur in
 // every row, so their rounding is systematic and moves log Z.
 // Bound by the FP32 pipe and shared memory alike (w + 4 operations and 4
@@ -140,6 +143,20 @@ __device__ __forceinline__ int row_exponent(const float (&v)[NPL]) {
   return exponent_of(mx);
 }
 
+// Brings the largest entry, of exponent e, back to 2^50 where it has left the
+// range; e2 counts the powers of two taken out.
+#define WIDE_EXP 50
+template <int NPL>
+__device__ __forceinline__ void rescale(float (&v)[NPL], int& e, int& e2) {
+  if (e >= WIDE_EXP - 30 && e <= WIDE_EXP + 30) return;  // the same for the warp
+  const int k = min(WIDE_EXP - e, 127);  // no entry left: any
+  const float sc = pow2i(k);
+#pragma unroll
+  for (int j = 0; j < NPL; ++j) v[j] *= sc;
+  e += k;
+  e2 -= k;
+}
+
 // Which lane bits a bond of the lane part leaves unsatisfied: bits i, i + 1.
 __device__ __forceinline__ bool unsat(uint32_t x, int i, uint32_t neg_bit) {
   return (((x >> i) ^ (x >> (i + 1))) & 1u) != (neg_bit & 1u);
@@ -160,14 +177,14 @@ __device__ __forceinline__ void diag_tree(float (&v)[NPL], float p, const float 
   }
 }
 
-// D of a row on v, times sc (FIRST: v = D sc).
+// D of a row on v (FIRST: v = 2^WIDE_EXP D).
 template <int NPL, bool FIRST>
 __device__ __forceinline__ void diag(float (&v)[NPL], const float* __restrict__ row, int w, uint32_t wantL,
-                                     uint32_t wantR, bool hasL, bool hasR, float sc, int lane) {
+                                     uint32_t wantR, bool hasL, bool hasR, int lane) {
   const float4 u03 = __ldg(reinterpret_cast<const float4*>(row));
   const float u[4] = {u03.x, u03.y, u03.z, u03.w};
   const uint32_t neg = __float_as_uint(__ldg(row + 28)), x0 = (uint32_t)lane;
-  float pl = sc;
+  float pl = FIRST ? pow2i(WIDE_EXP) : 1.f;
 #pragma unroll
   for (int c = 0; c < 4; ++c)
     if (c + 1 < w && unsat(x0, c, neg >> c)) pl *= u[c];
@@ -218,10 +235,10 @@ __device__ __forceinline__ void wide_chain(const WideStripDev& sd, const WideRow
     hr = __ballot_sync(0xffffffffu, pR >= 0);
   };
   neighbours(0);
-  diag<NPL, true>(v, tab, w, wl & 1u, wr & 1u, hl & 1u, hr & 1u, 1.f, lane);
+  diag<NPL, true>(v, tab, w, wl & 1u, wr & 1u, hl & 1u, hr & 1u, lane);
   int e = row_exponent(v);
-  e2 = e;
-  float sc = pow2i(-e);
+  e2 = -WIDE_EXP;
+  rescale(v, e, e2);
   for (int y = 1; y < sd.L; ++y) {
     if ((y & 31) == 0) neighbours(y);
     const uint32_t b = 1u << (y & 31);
@@ -246,11 +263,12 @@ __device__ __forceinline__ void wide_chain(const WideStripDev& sd, const WideRow
     vert<NPL, 4>(v, tc.y);
     vert<NPL, 5>(v, tc.z);
     vert<NPL, 6>(v, tc.w);
-    diag<NPL, false>(v, row, w, (wl & b) ? 1u : 0u, (wr & b) ? 1u : 0u, hl & b, hr & b, sc, lane);
+    diag<NPL, false>(v, row, w, (wl & b) ? 1u : 0u, (wr & b) ? 1u : 0u, hl & b, hr & b, lane);
     e = row_exponent(v);
-    e2 += e;
-    sc = pow2i(-e);
+    rescale(v, e, e2);
   }
+  const float sc = pow2i(-e);
+  e2 += e;
   float z = 0.f;
 #pragma unroll
   for (int j = 0; j < NPL; ++j) z += v[j] * sc;
