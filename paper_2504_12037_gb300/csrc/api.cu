@@ -3831,10 +3831,9 @@ void plan_levels(Instance& in, const std::vector<int>& prog, const std::vector<i
     for (const Task& t : ts) {
       const int st = t.st, f = fs[st], nin = F[f + 3];
       const bool tabbed = ctab[5 * comp[st] + 4] >= 0;
-      int r[TNVAN_LTASK] = {m[st] | ((tabbed ? 1 : 0) << 16), st, F[f + 5], F[f + 6], live[st], full[st],
+      int r[TNVAN_LTASK] = {m[st] | ((tabbed ? 1 : 0) << 8) | (nin << 9), st, F[f + 5], F[f + 6], live[st], full[st],
                             t.x0, t.nx, F[f + 1], F[f + 2], t.nch > 1 ? slot[st] : -1, t.nch | (t.ch << 16), goff[st],
                             (int)lin.size()};
-      r[20] = nin;  // any number: the hub of a star has one per leaf
       for (int i = 0; i < nin; ++i) {
         if (i < 3) r[14 + i] = live[inputs[st][i]], r[17 + i] = full[inputs[st][i]];
         lin.push_back(live[inputs[st][i]]);

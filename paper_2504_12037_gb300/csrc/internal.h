@@ -227,11 +227,10 @@ struct GenDev {
   // Level schedule: levels of steps that only need earlier levels' tables, as
   // tasks of one warp.  llev[3 l]: first task, end of those of cut steps, end;
   // blev[2 l]: first and end of the reverse sweep's tasks.  ltask (24 ints):
-  //   m | tabulated << 16, step, pp_off, map_off, out (level arena),
+  //   m | tabulated << 8 | n_in << 9, step, pp_off, map_off, out (level arena),
   //   out (all tables), x0, entries, fld_begin, fld_count, first slot of the cut
   //   step's maxima (-1: not cut), tasks of the step | this one << 16, g offset
-  //   in the level, lin offset, 3 x input (level arena), 3 x input (all tables),
-  //   n_in.
+  //   in the level, lin offset, 3 x input (level arena), 3 x input (all tables).
   // btask (8 ints): 0, m, g offset, fld_begin, fld_count | 1, m, g offset, pos_u,
   //   pair_id | 2 | R << 8, entries, g offset, input (level arena), input (all
   //   tables), its inverse map from entry e0 on, e0.

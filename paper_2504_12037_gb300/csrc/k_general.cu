@@ -574,7 +574,7 @@ __device__ __forceinline__ void landed(int v) { asm volatile("" ::"r"(v)); }
 // task starts with a chain of L2 reads.
 template <bool DB>
 __device__ __forceinline__ int touch_task(const GenDev& G, int rec, int lane) {
-  const int w0 = field(rec, 0), m = w0 & 255, nin = field(rec, 20), M = 1 << m, x = field(rec, 6) + (lane & 1) * M;
+  const int w0 = field(rec, 0), m = w0 & 255, nin = w0 >> 9, M = 1 << m, x = field(rec, 6) + (lane & 1) * M;
   const int ppo = field(rec, 2), mo = field(rec, 3), fb = field(rec, 8), fc = field(rec, 9);
   const int j = lane >> 1;
   const void* p = nullptr;
@@ -606,8 +606,8 @@ __device__ __forceinline__ void level_sweep(const GenDev& G, const int8_t* s, fl
       nxt = far;
       far = record(t + 2 * NW);
       const int tc0 = t + NW < t1 ? touch_task<DB>(G, nxt, lane) : 0;
-      const int w0 = field(rec, 0), m = w0 & 255, nin = field(rec, 20);
-      if (skip && (w0 >> 16)) continue;
+      const int w0 = field(rec, 0), m = w0 & 255, nin = w0 >> 9;  // any number: the hub of a star has one per leaf
+      if (skip && ((w0 >> 8) & 1)) continue;
       const int ppo = field(rec, 2), mo = field(rec, 3), out = field(rec, FULL ? 5 : 4);
       const int x0 = field(rec, 6), nx = field(rec, 7), slot = field(rec, 10);
       const int in[3] = {field(rec, FULL ? 17 : 14), field(rec, FULL ? 18 : 15), field(rec, FULL ? 19 : 16)};
@@ -649,7 +649,7 @@ __device__ __forceinline__ void level_sweep(const GenDev& G, const int8_t* s, fl
     if (tc == t0) continue;
     for (int t = t0 + wi; t < tc; t += NW) {  // the cut steps' scales
       const int rec = lane < TNVAN_LTASK ? __ldg(G.ltask + (size_t)t * TNVAN_LTASK + lane) : 0;
-      if (skip && (field(rec, 0) >> 16)) continue;
+      if (skip && ((field(rec, 0) >> 8) & 1)) continue;
       const int out = field(rec, FULL ? 5 : 4), x0 = field(rec, 6), nx = field(rec, 7);
       const int slot = field(rec, 10), nch = field(rec, 11) & 0xffff, ch = field(rec, 11) >> 16, step = field(rec, 1);
       float mx = red[slot * 32];
@@ -1281,7 +1281,7 @@ __global__ void __launch_bounds__(512, 1) general_levels_dJ_kernel(const InstDev
         nxt = far;
         far = record(t + 2 * NW);
         const int tc0 = t + NW < t1 ? touch_task<false>(G, nxt, lane) : 0;
-        const int w0 = field(rec, 0), m = w0 & 255, nin = field(rec, 20);
+        const int w0 = field(rec, 0), m = w0 & 255, nin = w0 >> 9;
         const int ppo = field(rec, 2), mo = field(rec, 3), x0 = field(rec, 6), nx = field(rec, 7);
         const int in[3] = {field(rec, 17), field(rec, 18), field(rec, 19)};
         const int* lin = G.lin + field(rec, 13) + 1;
