@@ -830,10 +830,10 @@ size_t tc_ws_floats(const tnvan_ctx* ctx, int batch) {
   return std::max(tot + (size_t)ctx->inst.size() * batch + 16, (chain_ws_elems(ctx, batch, nullptr) + 1) / 2);
 }
 
-// FP32 backward (k_bwd32.cu): its unit-major rows, the batch rounded up to the
-// 32 samples of a tile.
-size_t bwd32_ws_floats(const tnvan_ctx* ctx, int batch, Bwd32Ws* bw) {
-  const size_t ldb = ((size_t)batch + 31) & ~size_t(31);
+// FP32 backward (k_bwd32.cu): its unit-major rows for nb samples, rounded up to
+// the 32 of a tile.
+size_t bwd32_ws_floats(const tnvan_ctx* ctx, int nb, Bwd32Ws* bw) {
+  const size_t ldb = ((size_t)nb + 31) & ~size_t(31);
   size_t off = 0;
   for (size_t k = 0; k < ctx->inst.size(); ++k) {
     const Instance& in = ctx->inst[k];
@@ -842,6 +842,14 @@ size_t bwd32_ws_floats(const tnvan_ctx* ctx, int batch, Bwd32Ws* bw) {
   }
   if (bw) bw->ldb = (long long)ldb;
   return off;
+}
+// Samples of the batch it takes at a time: as many as keep those rows within 1
+// GB (84,000 of five 64-128-128-64 networks, ten times what fills the GPU), so
+// that a large batch needs no more memory.
+int bwd32_window(const tnvan_ctx* ctx, int batch) {
+  const size_t per = bwd32_ws_floats(ctx, 32, nullptr);  // a tile of every instance
+  const size_t tiles = std::max<size_t>(1, (size_t(1) << 28) / std::max<size_t>(per, 1));
+  return (int)std::min<size_t>((size_t)std::max(batch, 1), 32 * tiles);
 }
 
 // Weight blocks of an instance and the slices of the batch the FP32 weight
@@ -2101,11 +2109,15 @@ static int wide_max_strips(const tnvan_ctx* ctx) {
   return ms;
 }
 
-// Partial gradient rows of the FP32 backward.
+// Partial gradient rows of the FP32 backward: slices of every window.
+static int bwd32_rows(const tnvan_ctx* ctx, int batch) {
+  const int win = bwd32_window(ctx, batch);
+  return bwd32_splits(ctx, win) * (int)((std::max(batch, 1) + (long long)win - 1) / win);
+}
 static size_t grad_ws_floats(const tnvan_ctx* ctx, int batch) {
   long long maxp = 0;
   for (const Instance& in : ctx->inst) maxp = std::max(maxp, in.n_params);
-  return (size_t)bwd32_splits(ctx, batch) * ctx->inst.size() * (size_t)maxp;
+  return (size_t)bwd32_rows(ctx, batch) * ctx->inst.size() * (size_t)maxp;
 }
 
 // The batches up to max_batch at which a launch shape of the elimination calls
@@ -2147,7 +2159,7 @@ int tnvan_reserve(tnvan_ctx* ctx, int max_batch) {
   rc = grow(ctx, ctx->grad_packed, std::max(grad_ws_floats(ctx, B), std::max(fused_rows, tc_rows) * (size_t)maxp), s,
             "gradient partials");
   if (rc) return rc;
-  rc = grow(ctx, ctx->ws, std::max(tc_ws_floats(ctx, B), bwd32_ws_floats(ctx, B, nullptr)) * sizeof(float), s,
+  rc = grow(ctx, ctx->ws, std::max(tc_ws_floats(ctx, B), bwd32_ws_floats(ctx, bwd32_window(ctx, B), nullptr)) * sizeof(float), s,
             "workspace");
   if (rc) return rc;
   int max_edges = 0;
@@ -2795,7 +2807,7 @@ int backward_impl(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* 
   if (simt) {
     LaunchInfo lb;
     if ((rc = fill_launch(ctx, betas, batch, 32, lb))) return rc;
-    const int splits = bwd32_splits(ctx, batch);
+    const int win = bwd32_window(ctx, batch), splits = bwd32_splits(ctx, win), n_rows = bwd32_rows(ctx, batch);
     int n_run = 0, max_units = 0, max_blocks = 0, max_res = 0;
     for (int k = 0; k < lb.n_inst; ++k) {
       const Instance& in = ctx->inst[k];
@@ -2807,34 +2819,38 @@ int backward_impl(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* 
     }
     // the networks this backward is sized for (any that fit 880 units of a 32-sample tile)
     if (max_units > 880) return fail(ctx, TNVAN_E_CUDA, "backward kernel: invalid argument (%d units)", max_units);
-    // weights resident in shared memory, one CTA per SM, where they fit beside
-    // two tiles and every CTA has work for both of its halves
-    const int tiles = (batch + 31) / 32, per = std::max(1, 152 / std::max(n_run, 1));
-    const bool res = bwd32_smem_bytes(max_units, max_res) <= 227 * 1024 && tiles >= 2 * per;
-    int acc = 0;
-    for (int k = 0; k < lb.n_inst; ++k) {  // the fused instances are left out (no CTAs, not reduced)
-      lb.tile_begin[k] = acc;
-      if (!((fused_bits[k >> 5] >> (k & 31)) & 1u)) acc += res ? per : tiles;
-    }
-    lb.tile_begin[lb.n_inst] = acc;
     for (int j = 0; j < TNVAN_MAX_INST / 32; ++j) lb.skip[j] = fused_bits[j];
     Bwd32Ws bw;
     if ((rc = grow(ctx, ctx->grad_packed, grad_ws_floats(ctx, batch), s, "gradient partials"))) return rc;
-    if ((rc = grow(ctx, ctx->ws, bwd32_ws_floats(ctx, batch, &bw) * sizeof(float), s, "workspace"))) return rc;
+    if ((rc = grow(ctx, ctx->ws, bwd32_ws_floats(ctx, win, nullptr) * sizeof(float), s, "workspace"))) return rc;
     bw.base = reinterpret_cast<float*>(ctx->ws.p);
-    {
-      PROF("backward", s);
-      CK(launch_bwd32_delta(ctx->d_inst, lb, bw, res, bwd32_smem_bytes(max_units, res ? max_res : 0), d_spins, d_logZR,
-                            d_logq, ctx->d_stats, s),
-         "backward kernel");
-    }
-    {
+    for (int b0 = 0, w = 0; w * splits < n_rows; b0 += win, ++w) {
+      bw.b0 = b0;
+      bw.nb = std::min(win, batch - b0);
+      bwd32_ws_floats(ctx, bw.nb, &bw);
+      // weights resident in shared memory, one CTA per SM, where they fit beside
+      // two tiles and every CTA has work for both of its halves
+      const int tiles = (bw.nb + 31) / 32, per = std::max(1, 152 / std::max(n_run, 1));
+      const bool res = bwd32_smem_bytes(max_units, max_res) <= 227 * 1024 && tiles >= 2 * per;
+      int acc = 0;
+      for (int k = 0; k < lb.n_inst; ++k) {  // the fused instances are left out (no CTAs, not reduced)
+        lb.tile_begin[k] = acc;
+        if (!((fused_bits[k >> 5] >> (k & 31)) & 1u)) acc += res ? per : tiles;
+      }
+      lb.tile_begin[lb.n_inst] = acc;
+      {
+        PROF("backward", s);
+        CK(launch_bwd32_delta(ctx->d_inst, lb, bw, res, bwd32_smem_bytes(max_units, res ? max_res : 0), d_spins,
+                              d_logZR, d_logq, ctx->d_stats, s),
+           "backward kernel");
+      }
       PROF("backward_wgrad", s);
-      CK(launch_bwd32_wgrad(ctx->d_inst, lb, bw, max_blocks, splits, ctx->grad_packed.p, max_elems, s),
+      CK(launch_bwd32_wgrad(ctx->d_inst, lb, bw, max_blocks, splits, n_rows, w * splits, ctx->grad_packed.p, max_elems,
+                            s),
          "weight gradient kernel");
     }
     LaunchInfo lr = lb;
-    for (int k = 0; k <= lr.n_inst; ++k) lr.tile_begin[k] = k * splits;
+    for (int k = 0; k <= lr.n_inst; ++k) lr.tile_begin[k] = k * n_rows;
     {
       PROF("grad_reduce", s);
       CK(launch_grad_reduce(ctx->d_inst, lr, ctx->grad_packed.p, (int)max_elems, d_grad_params, s, adam),

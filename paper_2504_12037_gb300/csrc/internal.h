@@ -525,12 +525,13 @@ cudaError_t launch_reduce(const InstDev* d_inst, const LaunchInfo& li, const dou
 // merged into stats[8k + 0..7] for their union (fixed order).
 cudaError_t launch_merge_stats(const LaunchInfo& li, int n_parts, const double* parts, double* stats,
                                cudaStream_t s);
-// FP32 backward (k_bwd32.cu): per-instance unit-major rows of the hidden values
-// and deltas, [2 D + 2 H1 + 2 H2][ldb] at base + off[k] (ldb: the batch rounded
-// up to 32).
+// FP32 backward (k_bwd32.cu), samples b0 .. b0 + nb - 1 of the batch: per-instance
+// unit-major rows of the hidden values and deltas, [2 D + 2 H1 + 2 H2][ldb] at
+// base + off[k] (ldb: nb rounded up to 32).
 struct Bwd32Ws {
   float* base;
   long long ldb;
+  int b0, nb;
   long long off[TNVAN_MAX_INST];
 };
 // Hidden values, dX and deltas of every tile of 32 samples: li.tile_begin counts
@@ -541,11 +542,12 @@ cudaError_t launch_bwd32_delta(const InstDev* d_inst, const LaunchInfo& li, cons
                                cudaStream_t s);
 int bwd32_res_floats(int D, int nh, int H1, int H2);
 int bwd32_smem_bytes(int max_units, int res);
-// The weight gradients of the batch's `splits` slices, slice z of instance k
-// (not skipped) in partial row k * splits + z; max_blocks: the most 64 x 64
+// The weight gradients of `splits` slices of those samples, slice z of instance k
+// (not skipped) in partial row k * rows + row0 + z; max_blocks: the most 64 x 64
 // weight blocks of an instance.
 cudaError_t launch_bwd32_wgrad(const InstDev* d_inst, const LaunchInfo& li, const Bwd32Ws& bw, int max_blocks,
-                               int splits, float* partials, long long part_stride, cudaStream_t s);
+                               int splits, int rows, int row0, float* partials, long long part_stride,
+                               cudaStream_t s);
 // Adam's state and hyper-parameters for one launch (moments in the packed
 // all-instances gradient layout).  With t_dev the step is t_base + *t_dev and
 // bc1/bc2 are formed on the device.

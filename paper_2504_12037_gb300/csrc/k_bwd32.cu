@@ -419,13 +419,13 @@ __global__ void __launch_bounds__(RES ? 512 : 256, RES ? 1 : 2)
   float* A1 = S + D * B3_TP;
   float* A2 = A1 + H1 * B3_TP;  // three rows past each are readable (the last quad of a fan-in)
   __syncthreads();
-  const int ntile = (li.batch + B3_TS - 1) / B3_TS;
+  const int ntile = (bw.nb + B3_TS - 1) / B3_TS;
   const int rank = blockIdx.x - li.tile_begin[k], nblk = li.tile_begin[k + 1] - li.tile_begin[k];
   const double wscale = -1.0 / (li.beta[k] * stats_batch(stats + 8 * k));
   for (int it = RES ? 2 * rank + half : rank; it < ntile; it += RES ? 2 * nblk : ntile) {
-    const long long b0 = (long long)it * B3_TS;
-    const Rows g = rows_of(md, bw.base + bw.off[k] + b0, bw.ldb);
-    const int nv = min(B3_TS, li.batch - (int)b0);
+    const long long b0 = bw.b0 + (long long)it * B3_TS;
+    const Rows g = rows_of(md, bw.base + bw.off[k] + (long long)it * B3_TS, bw.ldb);
+    const int nv = min(B3_TS, bw.nb - it * B3_TS);
     if (tid < B3_TS) {
       const long long o = (long long)k * li.batch + b0 + tid;
       wb[tid] = tid < nv ? (float)(wscale * (logZR[o] - (double)logq[o] - stats[8 * k + 4])) : 0.f;
@@ -458,7 +458,7 @@ __global__ void __launch_bounds__(RES ? 512 : 256, RES ? 1 : 2)
 // 32 samples are summed first and then added to the running sum.  Blocks
 // wholly outside the MADE mask are left out (their entries are never read).
 __global__ void __launch_bounds__(128, 4) bwd32_wgrad_kernel(const InstDev* __restrict__ inst, const LaunchInfo li,
-                                                             const Bwd32Ws bw, int splits,
+                                                             const Bwd32Ws bw, int splits, int rows, int row0,
                                                              float* __restrict__ partials, long long part_stride) {
   __shared__ __align__(16) float As[2][64 * B3_TP], Bs[2][64 * B3_TP];
   const int k = blockIdx.z;
@@ -546,7 +546,7 @@ __global__ void __launch_bounds__(128, 4) bwd32_wgrad_kernel(const InstDev* __re
     }
     __syncthreads();
   }
-  float* G = partials + ((long long)k * splits + blockIdx.y) * part_stride + md.layer[l].dst_off;
+  float* G = partials + ((long long)k * rows + row0 + blockIdx.y) * part_stride + md.layer[l].dst_off;
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     const int m = m0 + ml + 8 * i;
@@ -574,9 +574,11 @@ cudaError_t launch_bwd32_delta(const InstDev* d_inst, const LaunchInfo& li, cons
 }
 
 cudaError_t launch_bwd32_wgrad(const InstDev* d_inst, const LaunchInfo& li, const Bwd32Ws& bw, int max_blocks,
-                               int splits, float* partials, long long part_stride, cudaStream_t s) {
+                               int splits, int rows, int row0, float* partials, long long part_stride,
+                               cudaStream_t s) {
   if (li.n_inst == 0 || max_blocks == 0) return cudaSuccess;
-  bwd32_wgrad_kernel<<<dim3(max_blocks, splits, li.n_inst), 128, 0, s>>>(d_inst, li, bw, splits, partials, part_stride);
+  bwd32_wgrad_kernel<<<dim3(max_blocks, splits, li.n_inst), 128, 0, s>>>(d_inst, li, bw, splits, rows, row0, partials,
+                                                                        part_stride);
   return cudaGetLastError();
 }
 
