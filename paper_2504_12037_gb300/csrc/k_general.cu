@@ -195,11 +195,13 @@ __device__ __forceinline__ float group_max(float v, int GL) {
 // registers until their scale is known (one table write instead of a write, a
 // read and a write).
 #define GEN_U 4
-// Launches of more CTAs than this take one entry at a time in half of the
-// registers instead: there the CTAs in flight hide the latency, and the batch's
-// dropped entries are only instructions (n = 500 of degree 3, width 4, with
-// d/dbeta: 32,768 samples in 1,024 CTAs 1,068 us four at a time, 653 one at a
-// time; 4,096 samples in 256 CTAs 434 us four at a time, 526 one at a time).
+// Launches of more CTAs than this (all that the dispatch sends here by itself;
+// a capture that finds no buffers for the level kernels brings small ones too)
+// take one entry at a time in half of the registers instead: there the CTAs in
+// flight hide the latency, and the batch's dropped entries are only instructions
+// (n = 500 of degree 3, width 4, with d/dbeta: 32,768 samples in 1,024 CTAs 1,068
+// us four at a time, 653 one at a time; 4,096 samples in 256 CTAs 434 us four at
+// a time, 526 one at a time).
 #define GEN_FEW (2 * 152)
 template <bool DB, int NIN, int COL, bool ZERO, int U0>
 __device__ __forceinline__ int step_table(const Step& r, const GenDev& G, const float (&fv)[2], const float (&fr)[2],
@@ -1083,13 +1085,14 @@ __global__ void __launch_bounds__(128, U0 > 1 ? 4 : 8) general_dJ_kernel(const I
 // The reverse sweep by levels (see general_levels_kernel): a forward sweep keeps
 // every table, then from the last level back the g values of a level's steps,
 // and after a barrier its bonds and its inputs' adjoints, each a warp's task.
-// general_dJ_kernel's order of every sum is kept, so d/dJ has the same bits in
-// both forms: a bond's sum over a step's entries is made of W (that kernel's
-// lanes per sample: 2, 4 or 8) chains x = w, w + W, ..., each added over the
-// 32 / W samples of a group, then over the chains by the same tree, into the
-// group's row; levels_dJ_reduce_kernel adds four groups' rows in turn, as that
-// kernel's CTA did.  An edge has one bond in the plan, so rows are written, not
-// added to.
+// general_dJ_kernel's order of every FP32 sum is kept, so a group's row has the
+// same bits in both forms (the rows are then added up in FP64, here by slices,
+// there one after the other: d/dJ agrees to 1e-15): a bond's sum over a step's
+// entries is made of W (that kernel's lanes per sample: 2, 4 or 8) chains x = w,
+// w + W, ..., each added over the 32 / W samples of a group, then over the chains
+// by the same tree, into the group's row; levels_dJ_reduce_kernel adds four
+// groups' rows in turn, as that kernel's CTA did.  An edge has one bond in the
+// plan, so rows are written, not added to.
 // ---------------------------------------------------------------------------
 
 // g of the extended indices of entries x0 .. x0 + nx - 1, into gb.

@@ -35,7 +35,8 @@
 // Bound by the FP32 pipe and shared memory alike (w + 4 operations and 4
 // shared accesses a state and row); 40 x 40 ferromagnet, 6 x 1,000 samples:
 // 5.15 ms with conditional products per state, a sample per CTA and shuffles,
-// 2.13 ms in this form.
+// 2.14 ms in this form (2.12 with the scales on the next row's diagonal, which
+// lost the small entries, 2.24 with a scaling pass for every row below 1).
 #include "common.cuh"
 
 namespace tnvan {
