@@ -619,30 +619,53 @@ int max_sample_smem(const tnvan_ctx* ctx, int tile) {
   return m;
 }
 
-// Samples per CTA of the FP32 sampler (a multiple of 8, four threads each).
-// A CTA takes as long as its D dependent steps while fewer than about 16 warps
-// share an SM, then as long as their instructions; so the tile is the one that
-// needs the least (waves of CTAs) x max(16, warps per SM) -- a tile that
+// Samples per CTA of the FP32 sampler with four threads a sample (a multiple of
+// 8).  A CTA takes as long as its D dependent steps while fewer than about 16
+// warps share an SM, then as long as their instructions; so the tile is the one
+// that needs the least (waves of CTAs) x max(16, warps per SM) -- a tile that
 // leaves a nearly empty last wave costs a whole pass of D steps.  Of equals
 // the smaller CTA.
+struct SampleShape {
+  int tile, threads;  // samples per CTA, threads per sample (4 or 1)
+};
+// Waves of CTAs of that shape, each counted as its warps per SM, `few` at least.
+double sample_waves(const tnvan_ctx* ctx, int batch, SampleShape p, int few) {
+  // (registers: 768 threads with four a sample, 640 with one)
+  const int smem = max_sample_smem(ctx, p.tile), fit = (p.threads == 4 ? 192 : 640) / p.tile;
+  const int occ = std::max(1, std::min({227 * 1024 / (smem + 1024), fit, 32}));
+  const long long nblk = (long long)ctx->inst.size() * ((batch + p.tile - 1) / p.tile), slots = 152LL * occ;
+  const long long full = nblk / slots, rest = nblk % slots;
+  const double warps = p.tile * p.threads / 32.0;
+  return full * std::max<double>(few, occ * warps) + (rest ? std::max<double>(few, (rest + 151) / 152 * warps) : 0.0);
+}
 int pick_sample_tile(const tnvan_ctx* ctx, int batch) {
   if (ctx->tune_sample_tile && max_sample_smem(ctx, ctx->tune_sample_tile) <= 227 * 1024) return ctx->tune_sample_tile;
-  const long long n = (long long)ctx->inst.size();
   int best = 8;
-  long long best_cost = -1;
-  for (int T = 8; T <= 192; T += 8) {
-    const int smem = max_sample_smem(ctx, T);
-    if (smem > 227 * 1024) break;
-    const int occ = std::max(1, std::min({227 * 1024 / (smem + 1024), 192 / T, 32}));
-    const long long nblk = n * ((batch + T - 1) / T), slots = 152LL * occ;
-    const long long full = nblk / slots, rest = nblk % slots;
-    const long long warps = (long long)occ * T / 8, last = ((rest + 151) / 152) * T / 8;
-    const long long cost = full * std::max(16LL, warps) + (rest ? std::max(16LL, last) : 0);
+  double best_cost = -1;
+  for (int T = 8; T <= 192 && max_sample_smem(ctx, T) <= 227 * 1024; T += 8) {
+    const double cost = sample_waves(ctx, batch, {T, 4}, 16);
     if (best_cost < 0 || cost < best_cost) best = T, best_cost = cost;
   }
   return best;
 }
-
+// Four threads a sample or one: four shorten a thread's chain (sample_len, its
+// instructions over all steps), but all four form every logit, and few units a
+// step leave some idle, so that with the GPU full a small network costs up to
+// three times the instructions (327,680 samples, log q: no hidden layer, D = 30,
+// 1 thread 0.29 of the time with 4; 64-64, D = 14, 1.14 times; 128-128, D = 64,
+// 1.19 times; 6,000 samples 1.0 to 1.8 times).  The lower of length x waves, a
+// wave of fewer than 12 warps an SM counted as 12, one thread where it is within
+// 10 %: over 770 combinations of network, D and samples 0.6 % from the faster form
+// on average, within 10 % in all but 14, and 30 % at most.
+SampleShape pick_sample_shape(const tnvan_ctx* ctx, int batch) {
+  const SampleShape four = {pick_sample_tile(ctx, batch), 4};
+  SampleShape one = {ctx->tune_sample_tile, 1};
+  if (!one.tile) one.tile = max_sample_smem(ctx, 64) <= 113 * 1024 ? 64 : 32;
+  if (one.tile % 32 || max_sample_smem(ctx, one.tile) > 227 * 1024) return four;
+  double len1 = 0, len4 = 0;
+  for (const Instance& in : ctx->inst) len1 += in.sample_len[0], len4 += in.sample_len[1];
+  return len1 * sample_waves(ctx, batch, one, 12) < 1.1 * len4 * sample_waves(ctx, batch, four, 12) ? one : four;
+}
 
 // Samples per CTA of the strip contraction by rule: 32 where that is what it
 // takes to share few samples out over the SMs.
@@ -1492,8 +1515,15 @@ int tnvan_set_made(tnvan_ctx* ctx, int instance, int n_hidden, const int32_t* wi
     auto pad4 = [&]() {
       while (src.size() % 4) src.push_back(-1);
     };
+    // instructions of one thread over all steps, one and four threads a sample:
+    // 16 or 4 multiply-adds with their loads an input of a block, 3 an in-group
+    // product, 140 a step's logit, draw and random number
+    double* len = in.sample_len;
+    len[0] = len[1] = 0;
     auto add_blocks = [&](int n_in, int lo, int hi, long long wofs, int stride) {
       const int off = (int)src.size();
+      len[0] += (hi - lo + 15) / 16 * (21.0 * n_in + 30);
+      len[1] += (hi - lo + 15) / 16 * (6.0 * n_in + 12);
       for (int c = lo; c < hi; c += 16)
         for (int j = 0; j < n_in; ++j)
           for (int q = 0; q < 16; ++q) {
@@ -1529,6 +1559,15 @@ int tnvan_set_made(tnvan_ctx* ctx, int instance, int n_hidden, const int32_t* wi
         const int clo = n_hidden == 0 ? i0 : (n_hidden == 1 ? u1lo : u2lo);
         const int chi = n_hidden == 0 ? i1 : (n_hidden == 1 ? u1hi : u2hi);
         to = add_tile(i0, i1, clo, chi, md.layer[n_hidden].dst_off, Hl);
+        for (int t = 0; t < 2; ++t) {
+          const int ns = t ? 4 : 1;
+          for (int i = i0; i < i1; ++i) {
+            const int a = before(c1, i), b = before(c1, i + 1), c = before(c2, i), d = before(c2, i + 1);
+            len[t] += (b - a + ns - 1) / ns * (3.0 * (i - i0) + 10) + (d - c + ns - 1) / ns * (3.0 * (b - u1lo) + 10);
+            len[t] += 3.0 * ((n_hidden == 0 ? i : (n_hidden == 1 ? b : d)) - clo) + 140;
+          }
+          len[t] += 60;
+        }
       }
       pad4();
       const int gsize = (int)src.size() - gstart;
@@ -3024,7 +3063,7 @@ int tnvan_autotune(tnvan_ctx* ctx, const double* betas, int batch, int precision
     }
     fixed_sample = best;
     ctx->tune_sample_tile = 0;
-    if (best && best_ms < rule_ms && best != pick_sample_tile(ctx, batch)) ctx->tune_sample_tile = best;
+    if (best && best_ms < rule_ms && best != pick_sample_shape(ctx, batch).tile) ctx->tune_sample_tile = best;
   }
   if ((rc = sample())) {  // spins for the contraction and backward candidates
     cleanup();
@@ -3499,13 +3538,14 @@ int run_sampler(tnvan_ctx* ctx, const double* betas, int batch, uint64_t seed, u
     }
     return TNVAN_OK;
   }
-  const int tile = pick_sample_tile(ctx, batch);
+  const SampleShape p = pick_sample_shape(ctx, batch);
   LaunchInfo li;
-  if ((rc = fill_launch(ctx, betas, batch, tile, li))) return rc;
+  if ((rc = fill_launch(ctx, betas, batch, p.tile, li))) return rc;
   li.seed = seed;
   li.step = step;
   PROF(given ? "log_prob" : "sample", s);
-  CK(launch_sample(ctx->d_inst, li, max_sample_smem(ctx, tile), d_spins, d_logq, given, s), "sample kernel");
+  CK(launch_sample(ctx->d_inst, li, p.threads, max_sample_smem(ctx, p.tile), d_spins, d_logq, given, s),
+     "sample kernel");
   return TNVAN_OK;
 }
 

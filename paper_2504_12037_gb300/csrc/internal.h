@@ -344,6 +344,7 @@ struct Instance {
   std::vector<unsigned short> gmap;       // input index maps (GenDev::map)
   int g_npp = 0;
   std::vector<int> glt, gltl, glb, glbl, glin, glroot;  // level schedule (GenDev)
+  double sample_len[2] = {0, 0};  // FP32 sampler: a thread's instructions, one and four threads a sample
   bool gl_ok = false;  // (index ranges allow it)
   int gl_levels = 0, gl_live = 0, gl_total = 0, gl_gmax = 0, gl_red = 0, gl_tasks = 0, gl_untab = 0;
   double g_mean_entries = 1;  // mean table size (entries) of the elimination steps
@@ -429,8 +430,9 @@ namespace tnvan {
 enum { PACK_FLAT = 1, PACK_TILES = 2, PACK_SIMT = 4, PACK_TC = 8, PACK_TCG = 16, PACK_CHAIN = 32 };
 __host__ __device__ long long pack_elems(const MadeDev& md, int mask);
 cudaError_t launch_pack_all(const InstDev* d_inst, int n_inst, const long long* counts, int mask, cudaStream_t s);
-cudaError_t launch_sample(const InstDev* d_inst, const LaunchInfo& li, int smem_bytes,
-                          int8_t* spins, float* logq, const int8_t* given, cudaStream_t s);
+// threads: per sample, 4 or 1 (li.tile then a multiple of 32)
+cudaError_t launch_sample(const InstDev* d_inst, const LaunchInfo& li, int threads, int smem_bytes, int8_t* spins,
+                          float* logq, const int8_t* given, cudaStream_t s);
 cudaError_t launch_strips(const InstDev* d_inst, const LaunchInfo& li, int smem_bytes, int max_strips, int max_w,
                           const int8_t* spins, double* logZR, double* dbeta, cudaStream_t s);
 int strip_con_smem_bytes(const Instance& in, int tile, bool db);

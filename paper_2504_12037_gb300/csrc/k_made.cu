@@ -246,29 +246,34 @@ cudaError_t launch_pack_all(const InstDev* d_inst, int n_inst, const long long* 
 
 // Pre-activations of the units [lo, hi) of one layer for the current group,
 // 16 units a block: acc[q] = bias[q] + sum_j blk[j][q] act[j] in input order,
-// four units to each of the sample's four threads (one activation load and
-// one 16-byte weight load per four FMAs).  Results go to pre[unit][T].
+// 16 / NS units to each of the sample's NS threads (one activation load and a
+// 16-byte weight load per four FMAs).  Results go to pre[unit][T].
+template <int NS>
 __device__ __forceinline__ void layer_preact(const float* blocks, int off, int n_in, int lo, int hi,
                                              const float* __restrict__ bias, const float* act, int T, int sub,
                                              float* pre) {
+  constexpr int U = 16 / NS;
   for (int c = lo; c < hi; c += 16) {
-    const int q0 = c + 4 * sub;
+    const int q0 = c + U * sub;
     if (q0 >= hi) break;
-    const float4* w4 = reinterpret_cast<const float4*>(blocks + off + (long long)(c - lo) * n_in) + sub;
-    float acc[4];
+    const float4* w4 = reinterpret_cast<const float4*>(blocks + off + (long long)(c - lo) * n_in) + U / 4 * sub;
+    float acc[U];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) acc[q] = q0 + q < hi ? __ldg(bias + q0 + q) : 0.f;
-#pragma unroll 8
+    for (int q = 0; q < U; ++q) acc[q] = q0 + q < hi ? __ldg(bias + q0 + q) : 0.f;
+#pragma unroll(NS == 1 ? 2 : 8)
     for (int j = 0; j < n_in; ++j) {
       const float x = act[j * T];
-      const float4 a = w4[4 * j];
-      acc[0] = fmaf(a.x, x, acc[0]);
-      acc[1] = fmaf(a.y, x, acc[1]);
-      acc[2] = fmaf(a.z, x, acc[2]);
-      acc[3] = fmaf(a.w, x, acc[3]);
+#pragma unroll
+      for (int q = 0; q < U; q += 4) {
+        const float4 a = w4[4 * j + q / 4];
+        acc[q] = fmaf(a.x, x, acc[q]);
+        acc[q + 1] = fmaf(a.y, x, acc[q + 1]);
+        acc[q + 2] = fmaf(a.z, x, acc[q + 2]);
+        acc[q + 3] = fmaf(a.w, x, acc[q + 3]);
+      }
     }
 #pragma unroll
-    for (int q = 0; q < 4; ++q)
+    for (int q = 0; q < U; ++q)
       if (q0 + q < hi) pre[(q0 + q - lo) * T] = acc[q];
   }
 }
@@ -280,8 +285,8 @@ __device__ __forceinline__ float chain_dot(float a, const float* w, const float*
   return a;
 }
 
-// Ancestral sampling (Eq. 8), four threads per sample (8 samples a warp), T
-// samples per CTA.
+// Ancestral sampling (Eq. 8), NS = 4 or 1 threads per sample (8 or 32 samples a
+// warp), T samples per CTA.
 // Hidden units are degree-sorted, so output i (degree i+1) needs exactly the
 // inputs 0..i-1, the layer-1 units of degree <= i and the layer-2 units of
 // degree <= i, each evaluated once: one masked forward pass in total.
@@ -292,26 +297,30 @@ __device__ __forceinline__ float chain_dot(float a, const float* w, const float*
 //            every input known before the group (register tiled, 16 units);
 //   phase B: the group's steps one by one, adding the in-group contributions
 //            and drawing s_i = +1 iff u < sigmoid(x_i).
-// The units of a phase are shared out over a sample's four threads (each
-// unit's sum stays one thread's chain, in input order); the logit and the draw
-// are formed by all four alike.  Bound by latency: D dependent steps, whose
-// hidden values limit the samples a CTA's shared memory holds, so warps in
-// flight come from splitting the samples; 5 x 4,099 samples of the 64-128-128-64
-// network took 0.26 ms with one thread per sample, 0.12 ms here.
+// The units of a phase are shared out over a sample's NS threads (each unit's
+// sum stays one thread's chain, in input order, so both give the same bits);
+// the logit and the draw are formed by all alike.  Bound by latency: D dependent
+// steps, whose hidden values limit the samples a CTA's shared memory holds, so
+// warps in flight come from splitting the samples; 5 x 4,099 samples of the
+// 64-128-128-64 network take 0.26 ms with one thread per sample, 0.12 with four.
+// Small networks on a full GPU are bound by issue, where one thread is up to
+// three times faster (pick_sample_shape).
 // With `given` non-null the spins are read from it (teacher forcing).
 // Shared memory: [unit][T] S [D], A1 [H1], A2 [H2], P1 [ug1], P2 [ug2],
 // PO [ugo]; then the weight block [wmax] and one mbarrier.
-__global__ void __launch_bounds__(768) sample_kernel(const InstDev* __restrict__ inst,
-                                                      const LaunchInfo li,
-                                                      int8_t* __restrict__ spins,
-                                                      float* __restrict__ logq,
-                                                      const int8_t* __restrict__ given) {
+template <int NS>
+__global__ void __launch_bounds__(192 * NS) sample_kernel(const InstDev* __restrict__ inst,
+                                                          const LaunchInfo li,
+                                                          int8_t* __restrict__ spins,
+                                                          float* __restrict__ logq,
+                                                          const int8_t* __restrict__ given) {
   extern __shared__ __align__(16) float sm[];
   const int k = find_inst(li, blockIdx.x);
   const InstDev& I = inst[k];
   const MadeDev& md = I.made;
-  const int T = li.tile, lane = threadIdx.x & 31, sub = lane >> 3;
-  const int t = (threadIdx.x >> 5) * 8 + (lane & 7);
+  constexpr int SW = 32 / NS;  // samples a warp
+  const int T = li.tile, lane = threadIdx.x & 31, sub = lane / SW;
+  const int t = (threadIdx.x >> 5) * SW + lane % SW;
   const int b = (blockIdx.x - li.tile_begin[k]) * T + t;
   const int D = md.D, nh = md.nh, H1 = md.H1, H2 = md.H2;
   float* S = sm;
@@ -350,11 +359,11 @@ __global__ void __launch_bounds__(768) sample_kernel(const InstDev* __restrict__
       return;
     }
     // phase A
-    if (nh >= 1) layer_preact(Wsm, G[6], i0, u1lo, u1hi, bias1, S + t, T, sub, P1 + t);
-    if (nh >= 2) layer_preact(Wsm, G[7], u1lo, u2lo, u2hi, bias2, A1 + t, T, sub, P2 + t);
+    if (nh >= 1) layer_preact<NS>(Wsm, G[6], i0, u1lo, u1hi, bias1, S + t, T, sub, P1 + t);
+    if (nh >= 2) layer_preact<NS>(Wsm, G[7], u1lo, u2lo, u2hi, bias2, A1 + t, T, sub, P2 + t);
     {
       const int n_in = nh == 0 ? i0 : (nh == 1 ? u1lo : u2lo);
-      layer_preact(Wsm, G[8], n_in, i0, i1, biaso, src + t, T, sub, PO + t);
+      layer_preact<NS>(Wsm, G[8], n_in, i0, i1, biaso, src + t, T, sub, PO + t);
     }
     __syncwarp();
     // phase B
@@ -369,13 +378,13 @@ __global__ void __launch_bounds__(768) sample_kernel(const InstDev* __restrict__
         rnd = philox4x32_10(
             make_uint4((uint32_t)b, (uint32_t)(i >> 2), step32, (uint32_t)k), key);
       if (nh >= 1 && i >= 1) {
-        for (int u = md.c1[i - 1] + sub; u < md.c1[i]; u += 4)
+        for (int u = md.c1[i - 1] + sub; u < md.c1[i]; u += NS)
           A1[u * T + t] = fmaxf(chain_dot(P1[(u - u1lo) * T + t], TW1 + (u - u1lo) * gi, S + i0 * T + t, T, i - i0), 0.f);
         __syncwarp();
       }
       if (nh >= 2 && i >= 1) {
         const int n1i = md.c1[i];
-        for (int v = md.c2[i - 1] + sub; v < md.c2[i]; v += 4)
+        for (int v = md.c2[i - 1] + sub; v < md.c2[i]; v += NS)
           A2[v * T + t] =
               fmaxf(chain_dot(P2[(v - u2lo) * T + t], TW2 + (v - u2lo) * n1, A1 + u1lo * T + t, T, n1i - u1lo), 0.f);
         __syncwarp();
@@ -396,7 +405,7 @@ __global__ void __launch_bounds__(768) sample_kernel(const InstDev* __restrict__
   if (valid) {
     if (spins) {
       int8_t* out = spins + I.spin_units * li.batch + (long long)b * D;
-      for (int i = sub; i < D; i += 4) out[i] = (int8_t)S[i * T + t];
+      for (int i = sub; i < D; i += NS) out[i] = (int8_t)S[i * T + t];
     }
     if (sub == 0) logq[(long long)k * li.batch + b] = lq;
   }
@@ -408,14 +417,14 @@ int sample_smem_bytes(const Instance& in, int tile) {
                ((md.wmax + 3) & ~3) * sizeof(float) + 16);
 }
 
-cudaError_t launch_sample(const InstDev* d_inst, const LaunchInfo& li, int smem_bytes,
-                          int8_t* spins, float* logq, const int8_t* given, cudaStream_t s) {
+cudaError_t launch_sample(const InstDev* d_inst, const LaunchInfo& li, int threads, int smem_bytes, int8_t* spins,
+                          float* logq, const int8_t* given, cudaStream_t s) {
   int nblk = li.tile_begin[li.n_inst];
   if (nblk == 0) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(sample_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       smem_bytes);
+  auto kern = threads == 4 ? sample_kernel<4> : sample_kernel<1>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
   if (e != cudaSuccess) return e;
-  sample_kernel<<<nblk, 4 * li.tile, smem_bytes, s>>>(d_inst, li, spins, logq, given);
+  kern<<<nblk, threads * li.tile, smem_bytes, s>>>(d_inst, li, spins, logq, given);
   return cudaGetLastError();
 }
 
