@@ -2072,6 +2072,10 @@ int plan_gen_forward(tnvan_ctx* ctx, const double* betas, int batch, bool db, bo
   //     1,000, 65,536 samples without d/dbeta: width 2 1,736 and 986, width 4
   //     3,021 and 2,249; 20,000 samples 820 and 1,153, 1,081 and 1,525; eight
   //     lanes, n = 600 of degree 4, 65,536 samples: 2,643 and 2,875).
+  // The same few lanes win over more than four rounds where a level has at most
+  // four tasks on average, fewer than a CTA's warps, wherever the tables are
+  // (ladder of 50 spins, 36 steps in 20 levels, 65,536 samples: 94 and 56 us, with
+  // d/dbeta 137 and 75; 8,000 samples 32 and 41).
   // Lane groups also skip a tabulated component's steps at no cost, where the
   // levels stay as many: they win with at most 64 steps left over more than four
   // rounds (45 of 83 steps, 65,536 samples: 125 us by levels and 99 in lane
@@ -2079,7 +2083,8 @@ int plan_gen_forward(tnvan_ctx* ctx, const double* betas, int batch, bool db, bo
   // steps left over more than eight (n = 500, 234 of 327 steps, 65,536 samples:
   // 433 and 331, with d/dbeta 571 and 784; 20,000 samples 218 and 275; 141 of
   // 143 left, 65,536 samples: 282 and 405).
-  const bool groups_hide = p.glob && (p.place ? GL <= 4 && acc > 4 * 152 : db && acc > 152);
+  const bool groups_hide = (p.glob && !p.place && db && acc > 152) ||
+                           (GL <= 4 && acc > 4 * 152 && ((p.glob && p.place) || p.lp.tasks <= 4));
   const bool groups_skip =
       lg.gen_tab > 0 && (untab <= 64 ? acc > 4 * 152 : !db && acc > 8 * 152 && 10 * untab <= 8 * p.lp.steps);
   p.levels = p.lp.ok && p.lsm <= LEVEL_SMEM && !groups_hide && !groups_skip;

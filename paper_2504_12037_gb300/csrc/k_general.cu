@@ -772,7 +772,7 @@ __global__ void __launch_bounds__(512, 1) general_levels_kernel(const InstDev* _
 // enter c) and runs c's program alone, so that tab_lz[toff_c + x] = log Z_c
 // and tab_db[..] its beta-derivative.  Built per call (they depend on beta)
 // when they are smaller than the batch.
-template <bool DB>
+template <bool DB, bool DIRECT>
 __global__ void __launch_bounds__(128) general_tab_kernel(const InstDev* __restrict__ inst, const LaunchInfo li,
                                                           int arena_floats, int GL, float* __restrict__ garena) {
   extern __shared__ float sm[];
@@ -824,7 +824,7 @@ __global__ void __launch_bounds__(128) general_tab_kernel(const InstDev* __restr
       for (int j = 0; j < cr[2]; ++j) s[G.bpos[cr[3] + j]] = ((x >> j) & 1) ? -1 : 1;
     __syncwarp();
     double lz = 0.0, dl = 0.0;
-    run_component<DB, GEN_U, false>(G, want, s, A, dA, RS, lane, GL, beta, lz, dl);
+    run_component<DB, DIRECT ? 1 : GEN_U, DIRECT>(G, want, s, A, dA, RS, lane, GL, beta, lz, dl);
     if (mine && live && lane == 0) {
       G.tab_lz[g] = lz;
       if (DB) G.tab_db[g] = dl;
@@ -1496,16 +1496,12 @@ cudaError_t launch_general_tables(const InstDev* d_inst, const LaunchInfo& li, i
   if (li.gen_tab <= 0) return cudaSuccess;
   const int arena = (int)(li.seed & 0xffffffffull);
   const dim3 tg((unsigned)((li.gen_tab + li.tile - 1) / li.tile), li.n_inst);
-  cudaError_t e;
-  if (db) {
-    e = cudaFuncSetAttribute(general_tab_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
-    if (e != cudaSuccess) return e;
-    general_tab_kernel<true><<<tg, li.tile * GL, smem_bytes, s>>>(d_inst, li, arena, GL, garena);
-  } else {
-    e = cudaFuncSetAttribute(general_tab_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
-    if (e != cudaSuccess) return e;
-    general_tab_kernel<false><<<tg, li.tile * GL, smem_bytes, s>>>(d_inst, li, arena, GL, garena);
-  }
+  const bool direct = GL <= 2;
+  auto kern = db ? (direct ? general_tab_kernel<true, true> : general_tab_kernel<true, false>)
+                 : (direct ? general_tab_kernel<false, true> : general_tab_kernel<false, false>);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
+  if (e != cudaSuccess) return e;
+  kern<<<tg, li.tile * GL, smem_bytes, s>>>(d_inst, li, arena, GL, garena);
   return cudaGetLastError();
 }
 

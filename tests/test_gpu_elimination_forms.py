@@ -61,6 +61,32 @@ def test_forms_agree(n, d, wu, db, small, large, tmp_path):
     assert torch.equal(lz0, lz1[:small]) and torch.equal(dl0, dl1[:small])
 
 
+@pytest.mark.parametrize("db", [False, True])
+def test_ladder_forms_agree(db, tmp_path):
+    """Few tasks a level: lane groups over many samples, tables in shared memory."""
+    n, w = 50, 5
+    ij = [(v, v + w) for v in range(n - w)] + [(v, v + 1) for v in range(n - 1) if (v + 1) % w]
+    ei, ej = (np.asarray(x, np.int32) for x in zip(*ij))
+    g = wl.Graph(n, ei, ej, np.random.default_rng(1).normal(size=len(ij)))
+    W = np.random.default_rng(7).choice(n, 14, replace=False).astype(np.int32)
+    model = TNVAN([g], [W], [8], [0.8], seed=1)
+    small, large = 8000, 65536
+    s = to_dev_spins(np.random.default_rng(2).choice([-1, 1], size=large * len(W)).astype(np.int8))
+    got = []
+    for b in (small, large):
+        lz, dl = torch.full((2, b), float("nan"), dtype=torch.float64, device="cuda")
+
+        def call():
+            model.ctx.contract(model.betas, b, s[:b * len(W)], tv.FP32, lz, dl if db else None)
+
+        call()
+        torch.cuda.synchronize()
+        got.append((_form(_recorded(call, tmp_path / f"{b}.dot")), lz, dl if db else lz))
+    assert [f for f, _, _ in got] == ["levels", "groups"]
+    for a, c in zip(got[0][1:], got[1][1:]):
+        assert torch.isfinite(c).all() and torch.equal(a, c[:small])
+
+
 @pytest.mark.parametrize("n,d,wu,insts,batch", [
     (64, 3, 1, 3, 33), (128, 3, 3, 1, 130), (90, 3, 4, 2, 65), (60, 3, 7, 2, 300), (500, 3, 8, 1, 200)])
 def test_adjoint_forms_agree(n, d, wu, insts, batch, tmp_path):
