@@ -667,6 +667,7 @@ SampleShape pick_sample_shape(const tnvan_ctx* ctx, int batch) {
   return len1 * sample_waves(ctx, batch, one, 12) < 1.1 * len4 * sample_waves(ctx, batch, four, 12) ? one : four;
 }
 
+constexpr int SOLO_MAX = 128;
 // Samples per CTA of the strip contraction by rule: 32 where that is what it
 // takes to share few samples out over the SMs.
 int pick_strip_tile(const tnvan_ctx* ctx, int batch) {
@@ -3567,19 +3568,27 @@ int contract_all(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* d
   LaunchInfo li;
   if ((rc = fill_launch(ctx, betas, batch, tile, li))) return rc;
   if (k0) {
-    int stile = tile, sm = 0, max_strips = 0, max_w = 1;
+    int stile = tile, sm = 0, max_strips = 0, max_w = 1, work = 0;
     for (const Instance& in : ctx->inst)
       if (in.kind == 0) {
+        int states = 0;  // of all rows of a sample's strips
+        for (const StripDev& sd : in.strip.strips) states += sd.L << sd.w;
+        work = std::max(work, states);
         sm = std::max(sm, strip_smem_bytes(in, stile));  // the limit this call has always had
         max_strips = std::max(max_strips, (int)in.strip.strips.size());
         for (const StripDev& sd : in.strip.strips) max_w = std::max(max_w, sd.w);
       }
     if (sm > 227 * 1024) return fail(ctx, TNVAN_E_UNSUPPORTED, "strip tables need %d B of shared memory", sm);
-    if (!ctx->tune_strip_tile) stile = pick_strip_tile(ctx, batch);
+    // short strips over more than two rounds of 128 samples an SM: a thread per sample
+    // through all of them (SOLO). Up to 128 states 0.71 to 0.86 times the time of
+    // (strip, 32 samples) pairs at 5 x 65,536 samples, 1.2 at 64 to 1,000 (9 x 9 with
+    // stride 2: 53 against 62 us, 17 against 12)
+    const bool solo = work <= SOLO_MAX && (long long)ctx->inst.size() * batch > 2 * 152 * 128;
+    if (!ctx->tune_strip_tile && !solo) stile = pick_strip_tile(ctx, batch);
     for (;; stile /= 2) {
       sm = 0;
       for (const Instance& in : ctx->inst)
-        if (in.kind == 0) sm = std::max(sm, strip_con_smem_bytes(in, stile, d_dbeta != nullptr));
+        if (in.kind == 0) sm = std::max(sm, strip_con_smem_bytes(in, stile, d_dbeta != nullptr, solo));
       if (sm <= 227 * 1024 || stile <= 8) break;
     }
     LaunchInfo ls;
@@ -3589,7 +3598,7 @@ int contract_all(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* d
       if (k < ls.n_inst && ctx->inst[k].kind == 0) acc += (batch + stile - 1) / stile;
     }
     PROF(d_dbeta ? (d_logZR ? "strips+dbeta" : "strips_dbeta") : "strips", s);
-    CK(launch_strips(ctx->d_inst, ls, sm, max_strips, max_w, d_spins, d_logZR, d_dbeta, s), "strip kernel");
+    CK(launch_strips(ctx->d_inst, ls, sm, max_strips, max_w, solo, d_spins, d_logZR, d_dbeta, s), "strip kernel");
   }
   if (k1) {
     PROF(d_dbeta ? "dense_dbeta" : "dense", s);

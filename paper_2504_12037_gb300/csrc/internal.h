@@ -433,9 +433,9 @@ cudaError_t launch_pack_all(const InstDev* d_inst, int n_inst, const long long* 
 // threads: per sample, 4 or 1 (li.tile then a multiple of 32)
 cudaError_t launch_sample(const InstDev* d_inst, const LaunchInfo& li, int threads, int smem_bytes, int8_t* spins,
                           float* logq, const int8_t* given, cudaStream_t s);
-cudaError_t launch_strips(const InstDev* d_inst, const LaunchInfo& li, int smem_bytes, int max_strips, int max_w,
+cudaError_t launch_strips(const InstDev* d_inst, const LaunchInfo& li, int smem_bytes, int max_strips, int max_w, bool solo,
                           const int8_t* spins, double* logZR, double* dbeta, cudaStream_t s);
-int strip_con_smem_bytes(const Instance& in, int tile, bool db);
+int strip_con_smem_bytes(const Instance& in, int tile, bool db, bool solo);
 cudaError_t launch_strips_adj(const InstDev* d_inst, const LaunchInfo& li, int smem_bytes, int lv_floats,
                               const int8_t* spins, double* logZR, double* dbeta, float* part, int part_stride,
                               double* dJ, cudaStream_t s, int blk_begin = 0, int blk_end = -1, int ws_threads = 0);

@@ -292,7 +292,10 @@ __device__ __forceinline__ float ww_energy(const InstDev& I, const int8_t* srow)
 // through all strips (20 warps an SM, tables and a division per staged spin in
 // every 128-sample CTA), 151 us here; 24 warps and the W-W sums after the
 // strips by half of the threads: 202.
-template <bool DB, int MAXW>
+// SOLO: a thread takes its sample through all strips, without the results in
+// shared memory and their barrier, which cost more than short strips' chains
+// (log Z_R of 5 x 65,536 samples of the 5 x 5 lattice 29 us in pairs, 19 solo).
+template <bool DB, int MAXW, bool SOLO>
 __global__ void __launch_bounds__(256, DB && MAXW == 4 ? 2 : 4) strips_kernel(const InstDev* __restrict__ inst,
                                                                              const LaunchInfo li,
                                                                              const int8_t* __restrict__ spins,
@@ -310,7 +313,18 @@ __global__ void __launch_bounds__(256, DB && MAXW == 4 ? 2 : 4) strips_kernel(co
   double* pl = reinterpret_cast<double*>(sm + (DB ? I.strip_tab_floats : strip_tab_offset(I, ns, false)));
   float* pd = reinterpret_cast<float*>(pl + ns * T);
   float* pe = pd + (DB ? ns * T : 0);
-  int8_t* ssp = reinterpret_cast<int8_t*>(pe + T);
+  int8_t* ssp = SOLO ? reinterpret_cast<int8_t*>(pl) : reinterpret_cast<int8_t*>(pe + T);
+  // ln Z of strip st for the sample of row srow, and its beta-derivative
+  auto chain = [&](int st, const int8_t* srow, double& l, float& d) {
+    const StripDev& sd = I.strips[st];
+    const StripTab tb = strip_tab_at(sm + strip_tab_offset(I, st, DB), sd.w, sd.L, DB);
+    switch (sd.w) {
+      case 1: strip_chain<1, DB>(tb, sd.L, srow, l, d); break;
+      case 2: strip_chain<2, DB>(tb, sd.L, srow, l, d); break;
+      case 3: strip_chain<3, DB>(tb, sd.L, srow, l, d); break;
+      default: if (MAXW >= 4) strip_chain<MAXW, DB>(tb, sd.L, srow, l, d); break;
+    }
+  };
   const int GS = T < 32 ? T : 32, G = T / GS;  // samples of a group, groups of a tile
   const int rank = blockIdx.x - li.tile_begin[k], nblk = li.tile_begin[k + 1] - li.tile_begin[k];
   const int ntile = (li.batch + T - 1) / T;
@@ -318,6 +332,26 @@ __global__ void __launch_bounds__(256, DB && MAXW == 4 ? 2 : 4) strips_kernel(co
     const int b0 = tile * T, n_valid = min(T, li.batch - b0);
     stage_spins(spins + I.spin_units * li.batch + (long long)b0 * D, n_valid, D, Dp, ssp, t, NT);
     __syncthreads();
+    if constexpr (SOLO) {
+      for (int i = t; i < n_valid; i += NT) {
+        const int8_t* srow = ssp + i * Dp;
+        double lz = 0.0, dl = 0.0, chat = 0.0;
+        for (int st = 0; st < ns; ++st) {
+          double l = 0.0;
+          float d = 0.f;
+          chain(st, srow, l, d);
+          lz += l;
+          if (DB) dl += d;
+          chat += I.strips[st].c_hat;
+        }
+        const float e1 = ww_energy(I, srow);  // -beta E_1(s) = beta e1
+        const long long o = (long long)k * li.batch + b0 + i;
+        if (logZR) logZR[o] = lz + li.beta[k] * (chat + (double)e1);
+        if (DB) dbeta[o] = dl + chat + (double)e1;
+      }
+      __syncthreads();  // spins free for the next tile
+      continue;
+    }
     for (int it = t >> 5; it < (ns + 1) * G; it += NT >> 5) {
       const int st = it / G, i = (it - st * G) * GS + lane;
       if (lane >= GS || i >= n_valid) continue;
@@ -326,16 +360,9 @@ __global__ void __launch_bounds__(256, DB && MAXW == 4 ? 2 : 4) strips_kernel(co
         pe[i] = ww_energy(I, srow);
         continue;
       }
-      const StripDev& sd = I.strips[st];
-      const StripTab tb = strip_tab_at(sm + strip_tab_offset(I, st, DB), sd.w, sd.L, DB);
       double l = 0.0;
       float d = 0.f;
-      switch (sd.w) {
-        case 1: strip_chain<1, DB>(tb, sd.L, srow, l, d); break;
-        case 2: strip_chain<2, DB>(tb, sd.L, srow, l, d); break;
-        case 3: strip_chain<3, DB>(tb, sd.L, srow, l, d); break;
-        default: if (MAXW >= 4) strip_chain<MAXW, DB>(tb, sd.L, srow, l, d); break;
-      }
+      chain(st, srow, l, d);
       pl[st * T + i] = l;
       if (DB) pd[st * T + i] = d;
     }
@@ -357,7 +384,7 @@ __global__ void __launch_bounds__(256, DB && MAXW == 4 ? 2 : 4) strips_kernel(co
 }
 
 // Shared memory of strips_kernel for `tile` samples.
-int strip_con_smem_bytes(const Instance& in, int tile, bool db) {
+int strip_con_smem_bytes(const Instance& in, int tile, bool db, bool solo) {
   int w4 = ((int)in.W.size() + 3) / 4;
   if ((w4 & 1) == 0) ++w4;
   int tabn = in.dev.strip_tab_floats;
@@ -365,7 +392,7 @@ int strip_con_smem_bytes(const Instance& in, int tile, bool db) {
     tabn = 0;
     for (const StripDev& sd : in.strip.strips) tabn += strip_tab_floats_adj(sd.w, sd.L);
   }
-  return 4 * tabn + ((int)in.strip.strips.size() * (db ? 12 : 8) + 4) * tile + tile * 4 * w4;
+  return 4 * tabn + (solo ? 0 : (int)in.strip.strips.size() * (db ? 12 : 8) + 4) * tile + tile * 4 * w4;
 }
 
 int strip_smem_bytes(const Instance& in, int tile) {
@@ -376,15 +403,18 @@ int strip_smem_bytes(const Instance& in, int tile) {
 }
 
 cudaError_t launch_strips(const InstDev* d_inst, const LaunchInfo& li, int smem_bytes, int max_strips, int max_w,
-                          const int8_t* spins, double* logZR, double* dbeta, cudaStream_t s) {
+                          bool solo, const int8_t* spins, double* logZR, double* dbeta, cudaStream_t s) {
   if (li.tile_begin[li.n_inst] == 0) return cudaSuccess;
   void (*kern)(const InstDev*, const LaunchInfo, const int8_t*, double*, double*) =
-      dbeta ? (max_w > 3 ? strips_kernel<true, 4> : strips_kernel<true, 3>)
-            : (max_w > 3 ? strips_kernel<false, 4> : strips_kernel<false, 3>);
+      dbeta ? (max_w > 3 ? (solo ? strips_kernel<true, 4, true> : strips_kernel<true, 4, false>)
+                         : (solo ? strips_kernel<true, 3, true> : strips_kernel<true, 3, false>))
+            : (max_w > 3 ? (solo ? strips_kernel<false, 4, true> : strips_kernel<false, 4, false>)
+                         : (solo ? strips_kernel<false, 3, true> : strips_kernel<false, 3, false>));
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
   if (e != cudaSuccess) return e;
-  // a warp per item of a tile, at most 8
-  const int pairs = (max_strips + 1) * ((li.tile + 31) / 32), threads = 32 * (pairs < 1 ? 1 : (pairs < 8 ? pairs : 8));
+  // a warp per item of a tile, at most 8; solo a thread a sample
+  const int pairs = (solo ? 1 : max_strips + 1) * ((li.tile + 31) / 32);
+  const int threads = 32 * (pairs < 1 ? 1 : (pairs < 8 ? pairs : 8));
   int occ = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, threads, smem_bytes);
   if (e != cudaSuccess) return e;
