@@ -412,9 +412,10 @@ cudaError_t launch_strips(const InstDev* d_inst, const LaunchInfo& li, int smem_
                          : (solo ? strips_kernel<false, 3, true> : strips_kernel<false, 3, false>));
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
   if (e != cudaSuccess) return e;
-  // a warp per item of a tile, at most 8; solo a thread a sample
+  // a warp per item of a tile, 4 to 8 (fewer fetch the spins too slowly: 5 x 1,000 samples
+  // of 120 W spins and no strip 18.6 us by one warp a CTA, 16.7 by four); solo a thread a sample
   const int pairs = (solo ? 1 : max_strips + 1) * ((li.tile + 31) / 32);
-  const int threads = 32 * (pairs < 1 ? 1 : (pairs < 8 ? pairs : 8));
+  const int threads = 32 * (pairs < 4 ? 4 : (pairs < 8 ? pairs : 8));
   int occ = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, threads, smem_bytes);
   if (e != cudaSuccess) return e;
