@@ -876,6 +876,23 @@ int bwd32_window(const tnvan_ctx* ctx, int batch) {
   return (int)std::min<size_t>((size_t)std::max(batch, 1), 32 * tiles);
 }
 
+// Small networks take one kernel (bwd32_small_kernel): its CTAs' samples, about
+// two CTAs per SM over all instances, and the most rows batches up to this one
+// need (a smaller one may be cut into more CTAs).
+bool bwd32_small(const tnvan_ctx* ctx) {
+  for (const Instance& in : ctx->inst)
+    if (in.n_params > BWD32_SMALL) return false;
+  return true;
+}
+int bwd32_small_ctas(const tnvan_ctx* ctx) { return std::max(1, 304 / std::max((int)ctx->inst.size(), 1)); }
+int bwd32_chunk(const tnvan_ctx* ctx, int batch) {
+  const long long per = bwd32_small_ctas(ctx), chunk = (std::max(batch, 1) + per - 1) / per;
+  return (int)((chunk + 31) / 32 * 32);
+}
+int bwd32_small_rows(const tnvan_ctx* ctx, int batch) {
+  return (int)std::min<long long>(bwd32_small_ctas(ctx), (std::max(batch, 1) + 31LL) / 32);
+}
+
 // Weight blocks of an instance and the slices of the batch the FP32 weight
 // gradients run over: about four CTAs per SM over all instances (the kernel's
 // occupancy, one wave), slices of at least 64 samples.
@@ -2162,7 +2179,12 @@ static int bwd32_rows(const tnvan_ctx* ctx, int batch) {
 static size_t grad_ws_floats(const tnvan_ctx* ctx, int batch) {
   long long maxp = 0;
   for (const Instance& in : ctx->inst) maxp = std::max(maxp, in.n_params);
-  return (size_t)bwd32_rows(ctx, batch) * ctx->inst.size() * (size_t)maxp;
+  const int rows = bwd32_small(ctx) ? bwd32_small_rows(ctx, batch) : bwd32_rows(ctx, batch);
+  return (size_t)rows * ctx->inst.size() * (size_t)maxp;
+}
+// Workspace of the FP32 backward's rows (none for the one kernel).
+static size_t grad_rows_floats(const tnvan_ctx* ctx, int batch) {
+  return bwd32_small(ctx) ? 0 : bwd32_ws_floats(ctx, bwd32_window(ctx, batch), nullptr);
 }
 
 // The batches up to max_batch at which a launch shape of the elimination calls
@@ -2204,7 +2226,7 @@ int tnvan_reserve(tnvan_ctx* ctx, int max_batch) {
   rc = grow(ctx, ctx->grad_packed, std::max(grad_ws_floats(ctx, B), std::max(fused_rows, tc_rows) * (size_t)maxp), s,
             "gradient partials");
   if (rc) return rc;
-  rc = grow(ctx, ctx->ws, std::max(tc_ws_floats(ctx, B), bwd32_ws_floats(ctx, bwd32_window(ctx, B), nullptr)) * sizeof(float), s,
+  rc = grow(ctx, ctx->ws, std::max(tc_ws_floats(ctx, B), grad_rows_floats(ctx, B)) * sizeof(float), s,
             "workspace");
   if (rc) return rc;
   int max_edges = 0;
@@ -2849,7 +2871,34 @@ int backward_impl(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* 
          "gradient reduce kernel");
     }
   }
-  if (simt) {
+  if (simt && bwd32_small(ctx)) {
+    const int chunk = bwd32_chunk(ctx, batch);
+    LaunchInfo lb;
+    if ((rc = fill_launch(ctx, betas, batch, 32, lb))) return rc;
+    lb.tile = chunk;
+    int acc = 0, max_units = 0;
+    for (int k = 0; k < lb.n_inst; ++k) {  // the fused instances are left out (no CTAs, not reduced)
+      const Instance& in = ctx->inst[k];
+      lb.tile_begin[k] = acc;
+      if ((fused_bits[k >> 5] >> (k & 31)) & 1u) continue;
+      acc += (int)((batch + (long long)chunk - 1) / chunk);
+      max_units = std::max(max_units, (int)in.W.size() + in.H[0] + in.H[1]);
+    }
+    lb.tile_begin[lb.n_inst] = acc;
+    for (int j = 0; j < TNVAN_MAX_INST / 32; ++j) lb.skip[j] = fused_bits[j];
+    if ((rc = grow(ctx, ctx->grad_packed, grad_ws_floats(ctx, batch), s, "gradient partials"))) return rc;
+    {
+      PROF("backward", s);
+      CK(launch_bwd32_small(ctx->d_inst, lb, bwd32_small_smem(max_units), d_spins, d_logZR, d_logq, ctx->d_stats,
+                            ctx->grad_packed.p, max_elems, s),
+         "backward kernel");
+    }
+    {
+      PROF("grad_reduce", s);
+      CK(launch_grad_reduce(ctx->d_inst, lb, ctx->grad_packed.p, (int)max_elems, d_grad_params, s, adam),
+         "gradient reduce kernel");
+    }
+  } else if (simt) {
     LaunchInfo lb;
     if ((rc = fill_launch(ctx, betas, batch, 32, lb))) return rc;
     const int win = bwd32_window(ctx, batch), splits = bwd32_splits(ctx, win), n_rows = bwd32_rows(ctx, batch);

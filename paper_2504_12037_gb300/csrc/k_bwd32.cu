@@ -10,7 +10,8 @@
 // weight gradient in global memory and added to it every 32 samples, with one
 // output per thread, took 1.51 ms for 5 x 16,384 samples of that network;
 // these two take 0.28 + 0.15 ms (0.35 + 0.15 with streamed weights; the
-// multiply-adds alone take 0.11).
+// multiply-adds alone take 0.11).  For networks of at most BWD32_SMALL
+// parameters that one kernel (bwd32_small_kernel) is the faster form and stays.
 #include <math.h>
 
 #include <type_traits>
@@ -558,6 +559,168 @@ __global__ void __launch_bounds__(128, 4) bwd32_wgrad_kernel(const InstDev* __re
     }
   }
   if (n0 == 0 && tid < 64 && m0 + tid < M) G[(long long)M * N + m0 + tid] = bsum;
+}
+
+// ---------------------------------------------------------------------------
+// Small networks: all of it in one kernel, a chunk of li.tile samples per CTA, 32
+// at a time, a warp's lanes on the samples and the warps on the units; the
+// chunk's weight gradient is kept in the CTA's row of `partials`, in L2.  What
+// bounds it is the chain of barriers between the layers; the two kernels above
+// add a launch and the rows' way through memory, which such a network's few
+// multiply-adds do not repay (us here and there): one 5-16 network, 250 samples
+// 25 and 33; five over 64,000 samples of 5 units and no hidden layer 172 and 228,
+// of 5-16 281 and 394, of 14-17-9 (557 parameters) 433 and 570.  Above 1,000
+// parameters they gain: 14-40 (1,174) 572 in one kernel when that took 368 for 5-40,
+// and 466 in two.  The outer product stays a function with a loop of
+// four samples a turn: unrolled in place it took 106 registers and 20 to 25 %
+// more time.
+// Forward sums as forward_layer adds them; per weight the sum over 32 samples,
+// added to the chunk's.
+// ---------------------------------------------------------------------------
+namespace {
+
+constexpr int SM_TP = 33;  // row stride of its [unit][sample] tiles
+
+__device__ __forceinline__ float small_dot(const float* __restrict__ w, const float* col, int n) {
+  float a[4] = {0.f, 0.f, 0.f, 0.f};
+  int j = 0;
+  for (; j + 4 <= n; j += 4)
+#pragma unroll
+    for (int p = 0; p < 4; ++p) a[p] = fmaf(__ldg(w + j + p), col[(j + p) * SM_TP], a[p]);
+  for (; j < n; ++j) a[0] = fmaf(__ldg(w + j), col[j * SM_TP], a[0]);
+  return (a[0] + a[1]) + (a[2] + a[3]);
+}
+
+// sum_{i = i0}^{n-1} col[i] w[i * stride]
+__device__ __forceinline__ float small_dot_t(const float* __restrict__ w, int stride, const float* col, int i0, int n) {
+  float a0 = 0.f, a1 = 0.f;
+  int i = i0;
+  for (; i + 2 <= n; i += 2) {
+    a0 = fmaf(__ldg(w + i * stride), col[i * SM_TP], a0);
+    a1 = fmaf(__ldg(w + (i + 1) * stride), col[(i + 1) * SM_TP], a1);
+  }
+  if (i < n) a0 = fmaf(__ldg(w + i * stride), col[i * SM_TP], a0);
+  return a0 + a1;
+}
+
+// G[m][n] (+)= sum_t delta[m][t] act[n][t], and the bias sums after it; 4 x 4 weights a thread.
+__device__ __noinline__ void small_outer(float* __restrict__ G, const float* delta, const float* act, int M, int N, bool first) {
+  const int mb = (M + 3) >> 2, nb = (N + 3) >> 2;
+  for (int blk = threadIdx.x; blk < mb * nb; blk += blockDim.x) {
+    const int m0 = (blk / nb) << 2, n0 = (blk % nb) << 2;
+    float acc[4][4] = {};
+#pragma unroll 4
+    for (int t = 0; t < B3_TS; ++t) {
+      float a[4], b[4];
+#pragma unroll
+      for (int r = 0; r < 4; ++r) a[r] = m0 + r < M ? delta[(m0 + r) * SM_TP + t] : 0.f;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) b[c] = n0 + c < N ? act[(n0 + c) * SM_TP + t] : 0.f;
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[r][c] = fmaf(a[r], b[c], acc[r][c]);
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        if (m0 + r < M && n0 + c < N) {
+          float* g = G + (m0 + r) * N + n0 + c;
+          *g = first ? acc[r][c] : *g + acc[r][c];
+        }
+  }
+  float* gb = G + M * N;
+  for (int m = threadIdx.x; m < M; m += blockDim.x) {
+    float sum = 0.f;
+#pragma unroll 4
+    for (int t = 0; t < B3_TS; ++t) sum += delta[m * SM_TP + t];
+    gb[m] = first ? sum : gb[m] + sum;
+  }
+}
+
+}  // namespace
+
+__global__ void __launch_bounds__(256)
+    bwd32_small_kernel(const InstDev* __restrict__ inst, const LaunchInfo li, const int8_t* __restrict__ spins,
+                       const double* __restrict__ logZR, const float* __restrict__ logq,
+                       const double* __restrict__ stats, float* __restrict__ partials, long long part_stride) {
+  extern __shared__ __align__(16) float sm[];
+  const int k = find_inst(li, blockIdx.x);
+  const InstDev& I = inst[k];
+  const MadeDev& md = I.made;
+  const int D = md.D, nh = md.nh, H1 = md.H1, H2 = md.H2;
+  const int tid = threadIdx.x, nth = blockDim.x, t = tid & 31, q = tid >> 5, nq = nth >> 5;
+  float* S = sm;  // spins, hidden values, dX and the deltas
+  float* A1 = S + D * SM_TP;
+  float* A2 = A1 + H1 * SM_TP;
+  float* X = A2 + H2 * SM_TP;
+  float* dA2 = X + D * SM_TP;
+  float* dA1 = dA2 + H2 * SM_TP;
+  const float *last = nh == 0 ? S : (nh == 1 ? A1 : A2), *W1 = md.packed + md.layer[0].dst_off;
+  const float* W2 = nh >= 2 ? md.packed + md.layer[1].dst_off : nullptr;
+  const float *Wo = md.packed + md.layer[nh].dst_off, *b1 = W1 + H1 * D, *b2 = W2 + H2 * H1, *bo = Wo + D * md.Hl;
+  const int Hl = md.Hl, *deg1 = nh >= 1 ? md.layer[0].deg_out : nullptr, *deg2 = nh >= 2 ? md.layer[1].deg_out : nullptr;
+  const int *c1 = md.c1, *c2 = md.c2, *cl = nh == 1 ? c1 : c2;
+  const double wscale = -1.0 / (li.beta[k] * stats_batch(stats + 8 * k)), mean = stats[8 * k + 4];
+  float* G = partials + (long long)blockIdx.x * part_stride;
+  float *G1 = G + md.layer[0].dst_off, *G2 = nh >= 2 ? G + md.layer[1].dst_off : nullptr, *Go = G + md.layer[nh].dst_off;
+  const int8_t* sp = spins + I.spin_units * li.batch;
+  const int chunk = li.tile, b_lo = (blockIdx.x - li.tile_begin[k]) * chunk, n = min(li.batch - b_lo, chunk);
+  for (int c = 0; c < n; c += B3_TS) {
+    const int b0 = b_lo + c, nv = min(B3_TS, n - c);
+    for (int e = tid; e < B3_TS * D; e += nth) {
+      const int tt = e / D, i = e - tt * D;
+      S[i * SM_TP + tt] = tt < nv ? (float)sp[(long long)b0 * D + e] : 0.f;
+    }
+    __syncthreads();
+    if (nh >= 1) {
+      for (int o = q; o < H1; o += nq)
+        A1[o * SM_TP + t] = fmaxf(__ldg(b1 + o) + small_dot(W1 + o * D, S + t, deg1[o]), 0.f);
+      __syncthreads();
+    }
+    if (nh >= 2) {
+      for (int o = q; o < H2; o += nq)
+        A2[o * SM_TP + t] = fmaxf(__ldg(b2 + o) + small_dot(W2 + o * H1, A1 + t, c1[deg2[o]]), 0.f);
+      __syncthreads();
+    }
+    const long long at = (long long)k * li.batch + b0 + t;
+    const float wb = t < nv ? (float)(wscale * (logZR[at] - (double)logq[at] - mean)) : 0.f;
+    for (int i = q; i < D; i += nq) {
+      const float x = __ldg(bo + i) + small_dot(Wo + i * Hl, last + t, nh == 0 ? i : cl[i]), sv = S[i * SM_TP + t];
+      X[i * SM_TP + t] = wb * sv / (1.f + expf(sv * x));
+    }
+    __syncthreads();
+    if (nh >= 2) {
+      for (int o = q; o < H2; o += nq)
+        dA2[o * SM_TP + t] = A2[o * SM_TP + t] > 0.f ? small_dot_t(Wo + o, Hl, X + t, deg2[o], D) : 0.f;
+      __syncthreads();
+      for (int j = q; j < H1; j += nq)
+        dA1[j * SM_TP + t] = A1[j * SM_TP + t] > 0.f ? small_dot_t(W2 + j, H1, dA2 + t, c2[deg1[j] - 1], H2) : 0.f;
+      __syncthreads();
+    } else if (nh == 1) {
+      for (int j = q; j < H1; j += nq)
+        dA1[j * SM_TP + t] = A1[j * SM_TP + t] > 0.f ? small_dot_t(Wo + j, Hl, X + t, deg1[j], D) : 0.f;
+      __syncthreads();
+    }
+    small_outer(Go, X, last, D, Hl, c == 0);
+    if (nh >= 2) small_outer(G2, dA2, A1, H2, H1, c == 0);
+    if (nh >= 1) small_outer(G1, dA1, S, H1, D, c == 0);
+    __syncthreads();  // tiles free for the next samples
+  }
+}
+
+int bwd32_small_smem(int max_units) { return 2 * max_units * SM_TP * (int)sizeof(float); }
+
+cudaError_t launch_bwd32_small(const InstDev* d_inst, const LaunchInfo& li, int smem, const int8_t* spins,
+                               const double* logZR, const float* logq, const double* stats, float* partials,
+                               long long part_stride, cudaStream_t s) {
+  const int nblk = li.tile_begin[li.n_inst];
+  if (nblk == 0) return cudaSuccess;
+  cudaError_t e = cudaFuncSetAttribute(bwd32_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  bwd32_small_kernel<<<nblk, 256, smem, s>>>(d_inst, li, spins, logZR, logq, stats, partials, part_stride);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_bwd32_delta(const InstDev* d_inst, const LaunchInfo& li, const Bwd32Ws& bw, bool resident, int smem,
