@@ -552,7 +552,7 @@ cudaError_t launch_bwd32_wgrad(const InstDev* d_inst, const LaunchInfo& li, cons
                                cudaStream_t s);
 // Networks of at most BWD32_SMALL parameters, in one kernel: a chunk of li.tile
 // samples per CTA, its weight gradient in the partial row of the CTA.
-constexpr long long BWD32_SMALL = 1024;
+constexpr long long BWD32_SMALL = 1536;
 int bwd32_small_smem(int max_units);
 cudaError_t launch_bwd32_small(const InstDev* d_inst, const LaunchInfo& li, int smem, const int8_t* spins,
                                const double* logZR, const float* logq, const double* stats, float* partials,

@@ -569,11 +569,12 @@ __global__ void __launch_bounds__(128, 4) bwd32_wgrad_kernel(const InstDev* __re
 // add a launch and the rows' way through memory, which such a network's few
 // multiply-adds do not repay (us here and there): one 5-16 network, 250 samples
 // 25 and 33; five over 64,000 samples of 5 units and no hidden layer 172 and 228,
-// of 5-16 281 and 394, of 14-17-9 (557 parameters) 433 and 570.  Above 1,000
-// parameters they gain: 14-40 (1,174) 572 in one kernel when that took 368 for 5-40,
-// and 466 in two.  The outer product stays a function with a loop of
-// four samples a turn: unrolled in place it took 106 registers and 20 to 25 %
-// more time.
+// of 5-16 281 and 394, of 40-17-9 (1,259 parameters) 524 and 597.  Above that
+// the wide layers lose at large batches what the launch gains at small ones:
+// 40 units and no hidden layer (1,640) 25 and 31 at 60 samples, 365 and 324 at
+// 5 x 64,000; 1-32-48 (1,697) 621 and 504.  The outer product stays a function
+// with a loop of four samples a turn: unrolled in place it took 106 registers and
+// 20 to 25 % more time.
 // Forward sums as forward_layer adds them; per weight the sum over 32 samples,
 // added to the chunk's.
 // ---------------------------------------------------------------------------
