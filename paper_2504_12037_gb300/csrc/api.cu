@@ -876,14 +876,27 @@ int bwd32_window(const tnvan_ctx* ctx, int batch) {
   return (int)std::min<size_t>((size_t)std::max(batch, 1), 32 * tiles);
 }
 
-// Small networks take one kernel (bwd32_small_kernel): its CTAs' samples, about
-// two CTAs per SM over all instances, and the most rows batches up to this one
-// need (a smaller one may be cut into more CTAs).
+// 64 x 64 weight blocks of an instance, over which the weight gradients run.
+int bwd32_blocks(const Instance& in) {
+  int nb = 0;
+  for (int l = 0; l <= in.nh; ++l)
+    nb += ((in.dev.made.layer[l].nout + 63) / 64) * ((in.dev.made.layer[l].nin + 63) / 64);
+  return nb;
+}
+
+// Small networks take one kernel (bwd32_small_kernel), and so do those whose
+// weight blocks are mostly empty (5 x 64,000 samples: 256 units on 3 spins 855
+// against 1,579 us, 100 on 8, 427 parameters a block, 567 against 722; 9 on 100,
+// 477, 744 against 674), where the tiles fit.
 bool bwd32_small(const tnvan_ctx* ctx) {
   for (const Instance& in : ctx->inst)
-    if (in.n_params > BWD32_SMALL) return false;
+    if (in.n_params > std::max(BWD32_SMALL, 450LL * bwd32_blocks(in)) ||
+        (int)in.W.size() + in.H[0] + in.H[1] > BWD32_UNITS)
+      return false;
   return true;
 }
+// Its CTAs' samples, about two CTAs per SM over all instances, and the most rows
+// batches up to this one need (a smaller one may be cut into more CTAs).
 int bwd32_small_ctas(const tnvan_ctx* ctx) { return std::max(1, 304 / std::max((int)ctx->inst.size(), 1)); }
 int bwd32_chunk(const tnvan_ctx* ctx, int batch) {
   const long long per = bwd32_small_ctas(ctx), chunk = (std::max(batch, 1) + per - 1) / per;
@@ -893,15 +906,9 @@ int bwd32_small_rows(const tnvan_ctx* ctx, int batch) {
   return (int)std::min<long long>(bwd32_small_ctas(ctx), (std::max(batch, 1) + 31LL) / 32);
 }
 
-// Weight blocks of an instance and the slices of the batch the FP32 weight
-// gradients run over: about four CTAs per SM over all instances (the kernel's
-// occupancy, one wave), slices of at least 64 samples.
-int bwd32_blocks(const Instance& in) {
-  int nb = 0;
-  for (int l = 0; l <= in.nh; ++l)
-    nb += ((in.dev.made.layer[l].nout + 63) / 64) * ((in.dev.made.layer[l].nin + 63) / 64);
-  return nb;
-}
+// The slices of the batch the FP32 weight gradients run over: about four CTAs per
+// SM over all instances (the kernel's occupancy, one wave), slices of at least 64
+// samples.
 int bwd32_splits(const tnvan_ctx* ctx, int batch) {
   int blocks = 0;
   for (const Instance& in : ctx->inst) blocks += bwd32_blocks(in);
@@ -2912,7 +2919,7 @@ int backward_impl(tnvan_ctx* ctx, const double* betas, int batch, const int8_t* 
       max_res = std::max(max_res, bwd32_res_floats((int)in.W.size(), in.nh, in.H[0], in.H[1]));
     }
     // the networks this backward is sized for (any that fit 880 units of a 32-sample tile)
-    if (max_units > 880) return fail(ctx, TNVAN_E_CUDA, "backward kernel: invalid argument (%d units)", max_units);
+    if (max_units > BWD32_UNITS) return fail(ctx, TNVAN_E_CUDA, "backward kernel: invalid argument (%d units)", max_units);
     for (int j = 0; j < TNVAN_MAX_INST / 32; ++j) lb.skip[j] = fused_bits[j];
     Bwd32Ws bw;
     if ((rc = grow(ctx, ctx->grad_packed, grad_ws_floats(ctx, batch), s, "gradient partials"))) return rc;

@@ -550,9 +550,11 @@ int bwd32_smem_bytes(int max_units, int res);
 cudaError_t launch_bwd32_wgrad(const InstDev* d_inst, const LaunchInfo& li, const Bwd32Ws& bw, int max_blocks,
                                int splits, int rows, int row0, float* partials, long long part_stride,
                                cudaStream_t s);
-// Networks of at most BWD32_SMALL parameters, in one kernel: a chunk of li.tile
-// samples per CTA, its weight gradient in the partial row of the CTA.
+// Small networks in one kernel (always up to BWD32_SMALL parameters): a chunk of
+// li.tile samples per CTA, its weight gradient in the partial row of the CTA.  No
+// FP32 backward takes more than BWD32_UNITS spins and hidden units.
 constexpr long long BWD32_SMALL = 1536;
+constexpr int BWD32_UNITS = 880;
 int bwd32_small_smem(int max_units);
 cudaError_t launch_bwd32_small(const InstDev* d_inst, const LaunchInfo& li, int smem, const int8_t* spins,
                                const double* logZR, const float* logq, const double* stats, float* partials,

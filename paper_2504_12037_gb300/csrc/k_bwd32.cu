@@ -10,8 +10,8 @@
 // weight gradient in global memory and added to it every 32 samples, with one
 // output per thread, took 1.51 ms for 5 x 16,384 samples of that network;
 // these two take 0.28 + 0.15 ms (0.35 + 0.15 with streamed weights; the
-// multiply-adds alone take 0.11).  For networks of at most BWD32_SMALL
-// parameters that one kernel (bwd32_small_kernel) is the faster form and stays.
+// multiply-adds alone take 0.11).  For small networks one kernel
+// (bwd32_small_kernel) is the faster form and stays.
 #include <math.h>
 
 #include <type_traits>
@@ -605,7 +605,8 @@ __device__ __forceinline__ float small_dot_t(const float* __restrict__ w, int st
 }
 
 // G[m][n] (+)= sum_t delta[m][t] act[n][t], and the bias sums after it; 4 x 4 weights a thread.
-__device__ __noinline__ void small_outer(float* __restrict__ G, const float* delta, const float* act, int M, int N, bool first) {
+__device__ __noinline__ void small_outer(float* __restrict__ G, const float* delta, const float* act, int M, int N,
+                                         bool first) {
   const int mb = (M + 3) >> 2, nb = (N + 3) >> 2;
   for (int blk = threadIdx.x; blk < mb * nb; blk += blockDim.x) {
     const int m0 = (blk / nb) << 2, n0 = (blk % nb) << 2;
@@ -661,11 +662,14 @@ __global__ void __launch_bounds__(256)
   const float *last = nh == 0 ? S : (nh == 1 ? A1 : A2), *W1 = md.packed + md.layer[0].dst_off;
   const float* W2 = nh >= 2 ? md.packed + md.layer[1].dst_off : nullptr;
   const float *Wo = md.packed + md.layer[nh].dst_off, *b1 = W1 + H1 * D, *b2 = W2 + H2 * H1, *bo = Wo + D * md.Hl;
-  const int Hl = md.Hl, *deg1 = nh >= 1 ? md.layer[0].deg_out : nullptr, *deg2 = nh >= 2 ? md.layer[1].deg_out : nullptr;
+  const int* deg1 = nh >= 1 ? md.layer[0].deg_out : nullptr;
+  const int* deg2 = nh >= 2 ? md.layer[1].deg_out : nullptr;
+  const int Hl = md.Hl;
   const int *c1 = md.c1, *c2 = md.c2, *cl = nh == 1 ? c1 : c2;
   const double wscale = -1.0 / (li.beta[k] * stats_batch(stats + 8 * k)), mean = stats[8 * k + 4];
   float* G = partials + (long long)blockIdx.x * part_stride;
-  float *G1 = G + md.layer[0].dst_off, *G2 = nh >= 2 ? G + md.layer[1].dst_off : nullptr, *Go = G + md.layer[nh].dst_off;
+  float *G1 = G + md.layer[0].dst_off, *Go = G + md.layer[nh].dst_off;
+  float* G2 = nh >= 2 ? G + md.layer[1].dst_off : nullptr;
   const int8_t* sp = spins + I.spin_units * li.batch;
   const int chunk = li.tile, b_lo = (blockIdx.x - li.tile_begin[k]) * chunk, n = min(li.batch - b_lo, chunk);
   for (int c = 0; c < n; c += B3_TS) {

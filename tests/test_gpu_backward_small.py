@@ -1,4 +1,5 @@
-"""The FP32 backward of networks of at most 1,536 parameters in one kernel: against
+"""The FP32 backward of small networks in one kernel (at most 1,536 parameters, or at
+most 450 per 64 x 64 block of weights): against
 the oracle, against the general form (which a larger network beside them makes the
 call take), and which of them a call launches."""
 import numpy as np
@@ -49,10 +50,11 @@ def _one_kernel(fn, path):
     return one
 
 
-# the smallest network, both sides of the line (1,482 and 1,560 parameters), 502 units; batches of one sample, of one chunk and
-# a sample, of chunks of 64 and a ragged one
+# the smallest network, both sides of the line (1,482 and 1,560 parameters), 502 units, wide
+# thin layers up to 880 units; batches of one sample, of one chunk and a sample, of chunks of 64 and a ragged one
 @pytest.mark.parametrize("D,hidden,batch,one", [
-    (1, [], 1, True), (38, [], 33, True), (39, [], 33, False), (1, [501], 70, True), (14, [17, 9], 4865, True),
+    (1, [], 1, True), (38, [], 33, True), (39, [], 33, False), (1, [501], 70, True), (3, [256], 500, True),
+    (400, [4], 97, True), (100, [9], 64, False), (876, [4], 40, True), (14, [17, 9], 4865, True),
     (5, [3, 2], 9999, True), (300, [1], 31, True), (2, [4, 33], 64, True)])
 def test_matches_oracle(D, hidden, batch, one, tmp_path):
     Ds = [D, D]
